@@ -129,30 +129,34 @@ int f64_vjp_variants();
 const KernelEntry &f64_vjp_kernel(int variant, bool zeps);
 
 // -------------------------------------------------- spatial order (order.cu)
-constexpr int SORT_CHUNK = 2048;  // keys per warp-chunk of the radix sort
 struct OrderScratch {
-    double *box;        // [1024][6]: bounding-box partials of up to 1023 blocks, then the folded box
+    double *box;        // [1024][6]: bounding-box partials
     unsigned *keys[2];  // [n] Morton keys (ping-pong)
     int *vals[2];       // [n] body indices (ping-pong)
-    unsigned *hist;     // [256][chunks] digit counts / offsets, then scan partials
+    unsigned *hist;     // sort_hist_entries: per pass [tiles][256] digit counts, then digit totals
 };
-int sort_chunks(int n);
-size_t sort_hist_entries(int n);  // entries of OrderScratch::hist for n bodies
+size_t sort_hist_entries(int n);  // entries of OrderScratch::hist for up to n bodies
+// Where a sort packs the bodies in sorted order: float32 hi/lo pairs
+// (Phi.w = m, Plo.w = log2(m)) when Phi, else float64 when P64, else nothing.
+struct SortedPack {
+    const double *pos = nullptr, *mass = nullptr;
+    float4 *Phi = nullptr, *Plo = nullptr;
+    double4 *P64 = nullptr;
+};
 // perm_out[k] = body at Morton rank k (stable in body index); `kernels` = launches made.
 cudaError_t launch_morton_sort(cudaStream_t s, int n, const double *pos, OrderScratch &o,
-                               int *perm_out, int &kernels);
+                               int *perm_out, const SortedPack &pack, int &kernels);
 // Tree-code order: 30-bit Morton keys (float64 quantisation), stable radix
 // sort; sorted keys end in o.keys[0], box_out = {lo_x, lo_y, lo_z, ext}.
 cudaError_t launch_tree_sort(cudaStream_t s, int n, const double *pos, OrderScratch &o,
-                             int *perm_out, double *box_out, int &kernels);
+                             int *perm_out, double *box_out, const SortedPack &pack, int &kernels);
 // Stable sort of bodies by an integer key below 2^(8 passes) (k32, or k64
 // when k32 is NULL; values below 2^31): perm_out[k] = the k-th body.
 cudaError_t launch_key_sort(cudaStream_t s, int n, const int *k32, const long long *k64,
                             int passes, OrderScratch &o, int *perm_out, int &kernels);
-// Phi[k], Plo[k] = float32 hi/lo packing of body perm[k] (perm NULL = identity);
-// Phi.w = m, Plo.w = log2(m).
+// Phi[k], Plo[k] = float32 hi/lo packing of body k; Phi.w = m, Plo.w = log2(m).
 cudaError_t launch_pack_hilo(cudaStream_t s, int n, const double *pos, const double *mass,
-                             const int *perm, float4 *Phi, float4 *Plo);
+                             float4 *Phi, float4 *Plo);
 
 // ------------------------------------------------------ tree code (tree.cu)
 // Octree over bodies in 30-bit Morton order.  Node arrays hold `cap` entries;
@@ -364,10 +368,8 @@ cudaError_t launch_rank_counts(cudaStream_t s, int n, const int *rank, int P,
 cudaError_t launch_hi_box(cudaStream_t s, int n, const float4 *P, float *box);
 
 // ------------------------------------------------- O(n) kernels (integrate.cu)
-cudaError_t launch_pack_f32(cudaStream_t s, int n, const double *pos, const double *mass, float4 *P);
-// P[k] = (x, y, z, m) of body perm[k] (perm NULL = identity).
-cudaError_t launch_pack_f64(cudaStream_t s, int n, const double *pos, const double *mass, double4 *P,
-                            const int *perm = nullptr);
+// P[k] = (x, y, z, m) of body k.
+cudaError_t launch_pack_f64(cudaStream_t s, int n, const double *pos, const double *mass, double4 *P);
 // v += half_dt a; x += dt v; then repack into P (double4) when f64, into the
 // float32 hi/lo pair (P, Plo) otherwise; P == NULL skips the packing.  Records
 // (x, v) before the update when rec_* is set.

@@ -310,23 +310,20 @@ nb_status pack(nb_ctx *c, cudaStream_t s, int64_t n, const double *pos, const do
 {
     if (n == 0) return NB_OK;
     c->perm_active = allow_order && use_order(c, n);
-    if (is_f64(c)) {
-        if (c->perm_active) {
-            int k = 0;
-            NB_CUDA(c, nb::launch_morton_sort(s, (int)n, pos, c->order, c->perm, k));
-            c->launches += k;
-        }
-        NB_LAUNCHED(c, nb::launch_pack_f64(s, (int)n, pos, mass, (double4 *)c->pack,
-                                           c->perm_active ? c->perm : nullptr));
-        return NB_OK;
-    }
+    nb::SortedPack pk{pos, mass, nullptr, nullptr, nullptr};
+    if (is_f64(c))
+        pk.P64 = (double4 *)c->pack;
+    else
+        pk.Phi = (float4 *)c->pack, pk.Plo = lo_half(c);
     if (c->perm_active) {
         int k = 0;
-        NB_CUDA(c, nb::launch_morton_sort(s, (int)n, pos, c->order, c->perm, k));
+        NB_CUDA(c, nb::launch_morton_sort(s, (int)n, pos, c->order, c->perm, pk, k));
         c->launches += k;
+    } else if (is_f64(c)) {
+        NB_LAUNCHED(c, nb::launch_pack_f64(s, (int)n, pos, mass, pk.P64));
+    } else {
+        NB_LAUNCHED(c, nb::launch_pack_hilo(s, (int)n, pos, mass, pk.Phi, pk.Plo));
     }
-    NB_LAUNCHED(c, nb::launch_pack_hilo(s, (int)n, pos, mass, c->perm_active ? c->perm : nullptr,
-                                        (float4 *)c->pack, lo_half(c)));
     return NB_OK;
 }
 
@@ -784,10 +781,9 @@ nb_status tree_build_enqueue(nb_ctx *c, cudaStream_t s, int64_t n, const double 
 {
     int k = 0;
     TreeTimer tm(c, nb::PROF_TREE_BUILD, s);
-    NB_CUDA(c, nb::launch_tree_sort(s, (int)n, pos, c->order, c->tree_perm, c->tree_box, k));
+    const nb::SortedPack pk{pos, mass, c->tree_P, c->tree_Plo, nullptr};
+    NB_CUDA(c, nb::launch_tree_sort(s, (int)n, pos, c->order, c->tree_perm, c->tree_box, pk, k));
     c->launches += k;
-    NB_LAUNCHED(c, nb::launch_pack_hilo(s, (int)n, pos, mass, c->tree_perm, c->tree_P,
-                                        c->tree_Plo));
     NB_CUDA(c, nb::launch_tree_build(s, c->tree, (int)n, c->order.keys[0], c->tree_box, pos, mass,
                                      c->tree_perm, leaf_cap, c->err, k));
     c->launches += k;
@@ -865,17 +861,7 @@ nb_status fmm_forces_run(nb_ctx *c, int64_t n, const double *pos, const double *
     cudaStream_t s = c->stream;
     int k = 0;
     c->let_n = 0;  // the local tree of nb_let_build is replaced
-    {
-        TreeTimer tm(c, nb::PROF_TREE_BUILD, s);
-        NB_CUDA(c, nb::launch_tree_sort(s, (int)n, pos, c->order, c->tree_perm, c->tree_box, k));
-        c->launches += k;
-        NB_LAUNCHED(c, nb::launch_pack_hilo(s, (int)n, pos, mass, c->tree_perm, c->tree_P,
-                                            c->tree_Plo));
-        NB_CUDA(c, nb::launch_tree_build(s, c->tree, (int)n, c->order.keys[0], c->tree_box, pos,
-                                         mass, c->tree_perm, leaf_cap, c->err, k));
-        c->launches += k;
-        tm.done();
-    }
+    NB_TRY(tree_build_enqueue(c, s, n, pos, mass, leaf_cap));
     for (int attempt = 0;; ++attempt) {
         nb::FmmParams p;
         p.tree = c->tree;

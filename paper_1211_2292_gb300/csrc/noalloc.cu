@@ -194,7 +194,7 @@ extern "C" nb_status nb_forces_noalloc(int64_t n, const double *pos, const doubl
     // rather than trusting the previous call's contents.
     cudaError_t e = cudaMemsetAsync(counters, 0, (size_t)n_itiles * sizeof(unsigned), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(err, 0, sizeof(int), s);
-    if (e == cudaSuccess) e = nb::launch_pack_hilo(s, (int)n, pos, mass, nullptr, Phi, Plo);
+    if (e == cudaSuccess) e = nb::launch_pack_hilo(s, (int)n, pos, mass, Phi, Plo);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return fail(NB_ECUDA, "memset or pack launch failed");

@@ -4,17 +4,18 @@
 // relative to an origin at the centre of the i-tile (see force_f32.cu).  This
 // only helps close pairs when an i-tile is spatially compact, so for large N
 // the bodies are processed in Morton (Z-curve) order:
-//   1. bounding box of all positions (per-block partials, re-reduced by every
+//   1. bounding box of all positions (per-block partials, folded by every
 //      block of the next kernel: no atomics, deterministic);
 //   2. 24-bit Morton key per body (8 bits per axis over the cube that holds
 //      the box);
-//   3. stable LSD radix sort of (key, body index), three 8-bit passes: per
-//      warp-chunk digit histograms, one exclusive scan in (digit, chunk)
-//      order, then a stable scatter that ranks equal digits within a warp
-//      with __match_any_sync, chunk keys taken strictly in order;
+//   3. stable LSD radix sort of (key, body index), 8 bits per pass: tiles of
+//      consecutive keys, one block each, ranked per warp with
+//      __match_any_sync, ordered in shared memory and written out in runs;
+//      each pass also counts the next pass's digits per destination tile;
 //   4. packing in sorted order as float32 hi/lo pairs:
 //      P_hi = (fl(x), fl(y), fl(z), fl(m)),
-//      P_lo = (fl(x - fl(x)), ..., fl(log2 m)) (log2 m for the log-domain pairs).
+//      P_lo = (fl(x - fl(x)), ..., fl(log2 m)) (log2 m for the log-domain pairs),
+//      or as float64 (x, y, z, m), by the sort's last pass.
 // Every step is deterministic, so the order and the forces are reproducible.
 #include <cuda_runtime.h>
 #include <float.h>
@@ -26,8 +27,7 @@ namespace nb {
 namespace {
 
 constexpr int OTPB = 256;
-constexpr int MAX_BOX_PARTS = 1023;            // box partials; the folded box follows them
-constexpr int BOX_FINAL = 6 * MAX_BOX_PARTS;  // {min x,y,z, max x,y,z} in the box scratch
+constexpr int MAX_BOX_PARTS = 304;  // box partials, each folded by every block of the next kernel
 
 __device__ __forceinline__ unsigned spread8(unsigned v)
 {
@@ -71,37 +71,69 @@ __global__ void __launch_bounds__(OTPB) bbox_kernel(int n, const double *__restr
     if (threadIdx.x < 6) parts[6 * (size_t)blockIdx.x + threadIdx.x] = sh[threadIdx.x][0];
 }
 
-// One block of 6 warps: warp c folds component c of the box partials into
-// parts[BOX_FINAL + c].
-__global__ void __launch_bounds__(192) box_fold_kernel(double *__restrict__ parts, int nparts)
+// The box {min x,y,z, max x,y,z} of the partials, folded by every block for
+// itself (at most MAX_BOX_PARTS x 48 bytes from L2, ~1 us; a launch of its own
+// took as long and its gap more).
+__device__ __forceinline__ void fold_box(const double *__restrict__ parts, int nparts,
+                                         double (&box)[6])
 {
+    __shared__ double sh[6];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const bool is_min = warp < 3;
-    double v = is_min ? DBL_MAX : -DBL_MAX;
-    for (int b = lane; b < nparts; b += 32) {
-        const double p = parts[6 * (size_t)b + warp];
-        v = is_min ? fmin(v, p) : fmax(v, p);
-    }
+    if (warp < 6) {
+        const bool is_min = warp < 3;
+        double v = is_min ? DBL_MAX : -DBL_MAX;
+#pragma unroll 4
+        for (int b = lane; b < nparts; b += 32) {
+            const double p = parts[6 * (size_t)b + warp];
+            v = is_min ? fmin(v, p) : fmax(v, p);
+        }
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        const double o = __shfl_xor_sync(0xffffffffu, v, off);
-        v = is_min ? fmin(v, o) : fmax(v, o);
+        for (int off = 16; off > 0; off >>= 1) {
+            const double o = __shfl_xor_sync(0xffffffffu, v, off);
+            v = is_min ? fmin(v, o) : fmax(v, o);
+        }
+        if (lane == 0) sh[warp] = v;
     }
-    if (lane == 0) parts[BOX_FINAL + warp] = v;
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < 6; ++c) box[c] = sh[c];
+}
+
+// Keys of a tile for the sort's first pass: the tile's digit counts into row
+// blockIdx.x of the first pass, the later passes' rows zeroed (each pass adds
+// the next one's counts).  key(i) gives body i's key; i is its value.
+template <class F>
+__device__ __forceinline__ void emit_keys(int n, int tile, int rows, int passes,
+                                          unsigned *__restrict__ keys,
+                                          unsigned *__restrict__ hist, F &&key)
+{
+    __shared__ unsigned cnt[256];
+    cnt[threadIdx.x] = 0u;
+    __syncthreads();
+    const int base = blockIdx.x * tile, m = min(tile, n - base);
+    for (int q = threadIdx.x; q < m; q += OTPB) {
+        const unsigned k = key(base + q);
+        keys[base + q] = k;
+        atomicAdd(&cnt[k & 255u], 1u);
+    }
+    __syncthreads();
+    hist[(size_t)blockIdx.x * 256 + threadIdx.x] = cnt[threadIdx.x];
+    for (int p = 1; p < passes; ++p)
+        hist[((size_t)p * rows + blockIdx.x) * 256 + threadIdx.x] = 0u;
 }
 
 // Morton keys (8 bits per axis) in the folded box.
 __global__ void __launch_bounds__(OTPB) morton_kernel(int n, const double *__restrict__ pos,
-                                                       const double *__restrict__ parts,
+                                                       const double *__restrict__ parts, int nparts,
+                                                       int tile, int rows,
                                                        unsigned *__restrict__ keys,
-                                                       int *__restrict__ vals)
+                                                       unsigned *__restrict__ hist)
 {
     double box[6];
-#pragma unroll
-    for (int c = 0; c < 6; ++c) box[c] = parts[BOX_FINAL + c];
+    fold_box(parts, nparts, box);
     const double ext = fmax(fmax(box[3] - box[0], box[4] - box[1]), box[5] - box[2]);
     const double scale = ext > 0.0 ? 256.0 / ext : 0.0;
-    for (int i = blockIdx.x * OTPB + threadIdx.x; i < n; i += gridDim.x * OTPB) {
+    emit_keys(n, tile, rows, 3, keys, hist, [&](int i) {
         unsigned q[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
@@ -109,9 +141,8 @@ __global__ void __launch_bounds__(OTPB) morton_kernel(int n, const double *__res
             t = fmin(fmax(t, 0.0), 255.0);
             q[c] = (unsigned)t;
         }
-        keys[i] = spread8(q[0]) | (spread8(q[1]) << 1) | (spread8(q[2]) << 2);
-        vals[i] = i;
-    }
+        return spread8(q[0]) | (spread8(q[1]) << 1) | (spread8(q[2]) << 2);
+    });
 }
 
 __device__ __forceinline__ unsigned spread10(unsigned v)
@@ -131,13 +162,13 @@ __device__ __forceinline__ unsigned spread10(unsigned v)
 // ext} for the tree kernels.
 __global__ void __launch_bounds__(OTPB) morton30_kernel(int n, const double *__restrict__ pos,
                                                          const double *__restrict__ parts,
+                                                         int nparts, int tile, int rows,
                                                          unsigned *__restrict__ keys,
-                                                         int *__restrict__ vals,
+                                                         unsigned *__restrict__ hist,
                                                          double *__restrict__ box_out)
 {
     double box[6];
-#pragma unroll
-    for (int c = 0; c < 6; ++c) box[c] = parts[BOX_FINAL + c];
+    fold_box(parts, nparts, box);
     double ext = box[3] - box[0];
     if (box[4] - box[1] > ext) ext = box[4] - box[1];
     if (box[5] - box[2] > ext) ext = box[5] - box[2];
@@ -149,152 +180,216 @@ __global__ void __launch_bounds__(OTPB) morton30_kernel(int n, const double *__r
         box_out[2] = box[2];
         box_out[3] = ext;
     }
-    for (int i = blockIdx.x * OTPB + threadIdx.x; i < n; i += gridDim.x * OTPB) {
+    emit_keys(n, tile, rows, 4, keys, hist, [&](int i) {
         unsigned q[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             const double t = __dmul_rn(__dsub_rn(pos[3 * (size_t)i + c], box[c]), scale);
             q[c] = t >= 1023.0 ? 1023u : (t <= 0.0 ? 0u : (unsigned)t);
         }
-        keys[i] = spread10(q[0]) | (spread10(q[1]) << 1) | (spread10(q[2]) << 2);
-        vals[i] = i;
-    }
+        return spread10(q[0]) | (spread10(q[1]) << 1) | (spread10(q[2]) << 2);
+    });
 }
 
-// Digit histogram per warp-chunk of SORT_CHUNK keys: hist[d * nchunks + chunk].
-__global__ void __launch_bounds__(OTPB) radix_hist_kernel(int n, const unsigned *__restrict__ keys,
-                                                           int shift, int nchunks,
-                                                           unsigned *__restrict__ hist)
-{
-    __shared__ unsigned cnt[OTPB / 32][256];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int d = lane; d < 256; d += 32) cnt[warp][d] = 0u;
-    __syncwarp();
-    const int chunk = blockIdx.x * (OTPB / 32) + warp;
-    if (chunk < nchunks) {
-        const int base = chunk * SORT_CHUNK;
-        const int end = min(base + SORT_CHUNK, n);
-        for (int i = base + lane; i < end; i += 32) atomicAdd(&cnt[warp][(keys[i] >> shift) & 255u], 1u);
-        __syncwarp();
-        for (int d = lane; d < 256; d += 32) hist[(size_t)d * nchunks + chunk] = cnt[warp][d];
-    }
-}
-
-// In-place exclusive scan of hist[0..total) over several blocks: block b
-// sums its segment of BSCAN_TILE entries into part[b] (radix_part_kernel),
-// then scans it starting from the sum of the segments before it.
-__global__ void __launch_bounds__(1024) radix_part_kernel(const unsigned *__restrict__ hist,
-                                                          int total, unsigned *__restrict__ part)
-{
-    __shared__ unsigned ws[32];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int base = blockIdx.x * BSCAN_TILE;
-    unsigned v = 0u;
-    for (int q = threadIdx.x; q < BSCAN_TILE; q += 1024)
-        if (base + q < total) v += hist[base + q];
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    if (lane == 0) ws[warp] = v;
-    __syncthreads();
-    if (warp == 0) {
-        v = ws[lane];
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-        if (lane == 0) part[blockIdx.x] = v;
-    }
-}
-
-__global__ void __launch_bounds__(1024) radix_scan_kernel(unsigned *__restrict__ hist, int total,
-                                                          const unsigned *__restrict__ part)
-{
-    __shared__ unsigned tile[BSCAN_TILE + BSCAN_TILE / 32];
-    __shared__ unsigned wsum[32];
-    __shared__ unsigned offset;
-    if (threadIdx.x < 32) {
-        unsigned v = 0u;
-        for (int b = threadIdx.x; b < (int)blockIdx.x; b += 32) v += part[b];
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-        if (threadIdx.x == 0) offset = v;
-    }
-    __syncthreads();
-    const int base = blockIdx.x * BSCAN_TILE;
-    block_scan_exclusive<unsigned>(hist + base, hist + base, min(BSCAN_TILE, total - base), tile,
-                                   wsum, offset);
-}
-
-inline void launch_radix_scan(cudaStream_t s, unsigned *hist, int total)
-{
-    const int blocks = (total + BSCAN_TILE - 1) / BSCAN_TILE;
-    radix_part_kernel<<<blocks, 1024, 0, s>>>(hist, total, hist + total);
-    radix_scan_kernel<<<blocks, 1024, 0, s>>>(hist, total, hist + total);
-}
-
-// Stable scatter: one warp per chunk, keys taken 32 at a time in order.
-__global__ void __launch_bounds__(OTPB) radix_scatter_kernel(int n,
-                                                              const unsigned *__restrict__ kin,
-                                                              const int *__restrict__ vin,
-                                                              unsigned *__restrict__ kout,
-                                                              int *__restrict__ vout, int shift,
-                                                              int nchunks,
-                                                              const unsigned *__restrict__ offs)
-{
-    __shared__ unsigned run[OTPB / 32][256];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int chunk = blockIdx.x * (OTPB / 32) + warp;
-    if (chunk >= nchunks) return;  // whole warp leaves together
-    for (int d = lane; d < 256; d += 32) run[warp][d] = offs[(size_t)d * nchunks + chunk];
-    __syncwarp();
-    const int base = chunk * SORT_CHUNK;
-    const int end = min(base + SORT_CHUNK, n);
-    const unsigned lt = (1u << lane) - 1u;
-    for (int r = base; r < end; r += 32) {
-        const int i = r + lane;
-        const bool valid = i < end;
-        const unsigned k = valid ? kin[i] : 0u;
-        const unsigned d = valid ? ((k >> shift) & 255u) : 256u + (unsigned)lane;
-        const unsigned peers = __match_any_sync(0xffffffffu, d);
-        unsigned off = 0u;
-        if (valid) off = run[warp][d] + (unsigned)__popc(peers & lt);
-        __syncwarp();
-        if (valid && (__ffs(peers) - 1) == lane) run[warp][d] += (unsigned)__popc(peers);
-        __syncwarp();
-        if (valid) {
-            kout[off] = k;
-            vout[off] = vin[i];
-        }
-    }
-}
-
-// Keys of a plain integer sort: keys[i] = k32[i] or k64[i] (values below
-// 2^31), vals[i] = i.
+// Keys of a plain integer sort: k32[i] or k64[i] (values below 2^31).
 __global__ void __launch_bounds__(OTPB) key_init_kernel(int n, const int *__restrict__ k32,
                                                          const long long *__restrict__ k64,
+                                                         int tile, int rows, int passes,
                                                          unsigned *__restrict__ keys,
-                                                         int *__restrict__ vals)
+                                                         unsigned *__restrict__ hist)
 {
-    for (int i = blockIdx.x * OTPB + threadIdx.x; i < n; i += gridDim.x * OTPB) {
-        keys[i] = k32 ? (unsigned)k32[i] : (unsigned)k64[i];
-        vals[i] = i;
+    emit_keys(n, tile, rows, passes, keys, hist,
+              [&](int i) { return k32 ? (unsigned)k32[i] : (unsigned)k64[i]; });
+}
+
+// Per digit: exclusive scan of its counts over the tiles (rows), in place, and
+// the digit's total.  A block takes 32 digits (a lane each), its 32 warps a
+// range of rows each.
+__global__ void __launch_bounds__(1024) radix_rows_kernel(unsigned *__restrict__ hist, int rows,
+                                                          unsigned *__restrict__ total)
+{
+    __shared__ unsigned ws[32][33];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int d = blockIdx.x * 32 + lane;
+    const int per = (rows + 31) / 32, r0 = min(rows, warp * per), r1 = min(rows, r0 + per);
+    unsigned v = 0u;
+#pragma unroll 8
+    for (int r = r0; r < r1; ++r) v += hist[(size_t)r * 256 + d];
+    ws[warp][lane] = v;
+    __syncthreads();
+    unsigned run = 0u, all = 0u;
+#pragma unroll
+    for (int w = 0; w < 32; ++w) {
+        if (w == warp) run = all;
+        all += ws[w][lane];
+    }
+    if (warp == 0) total[d] = all;
+#pragma unroll 8
+    for (int r = r0; r < r1; ++r) {
+        const unsigned c = hist[(size_t)r * 256 + d];
+        hist[(size_t)r * 256 + d] = run;
+        run += c;
     }
 }
 
-// Pack body perm[k] at slot k as float32 hi/lo pairs.
-__global__ void __launch_bounds__(OTPB) pack_hilo_kernel(int n, const double *__restrict__ pos,
-                                                          const double *__restrict__ mass,
-                                                          const int *__restrict__ perm,
-                                                          float4 *__restrict__ Phi,
-                                                          float4 *__restrict__ Plo)
+// Exclusive scan over the block's 256 threads.
+__device__ __forceinline__ unsigned scan256(unsigned v, unsigned (&ws)[OTPB / 32])
 {
-    for (int k = blockIdx.x * OTPB + threadIdx.x; k < n; k += gridDim.x * OTPB) {
-        const int i = perm ? perm[k] : k;
-        const double *x = pos + 3 * (size_t)i;
-        const float hx = (float)x[0], hy = (float)x[1], hz = (float)x[2];
-        const double m = mass[i];
-        Phi[k] = make_float4(hx, hy, hz, (float)m);
-        Plo[k] = make_float4((float)(x[0] - (double)hx), (float)(x[1] - (double)hy),
-                             (float)(x[2] - (double)hz), (float)log2(m));
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    unsigned incl = v;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const unsigned t = __shfl_up_sync(0xffffffffu, incl, off);
+        if (lane >= off) incl += t;
     }
+    if (lane == 31) ws[warp] = incl;
+    __syncthreads();
+    unsigned below = 0u;
+#pragma unroll
+    for (int w = 0; w < OTPB / 32; ++w)
+        if (w < warp) below += ws[w];
+    __syncthreads();  // ws may be reused
+    return below + incl - v;
+}
+
+// Body i packed at slot k: float32 hi/lo pairs, or float64, or not at all.
+__device__ __forceinline__ void put_body(const SortedPack &p, size_t k, int i)
+{
+    if (p.Phi) {
+        const double *x = p.pos + 3 * (size_t)i;
+        const float hx = (float)x[0], hy = (float)x[1], hz = (float)x[2];
+        const double m = p.mass[i];
+        p.Phi[k] = make_float4(hx, hy, hz, (float)m);
+        p.Plo[k] = make_float4((float)(x[0] - (double)hx), (float)(x[1] - (double)hy),
+                               (float)(x[2] - (double)hz), (float)log2(m));
+    } else if (p.P64) {
+        const double *x = p.pos + 3 * (size_t)i;
+        p.P64[k] = make_double4(x[0], x[1], x[2], p.mass[i]);
+    }
+}
+
+struct SortPass {
+    int n, rows, shift;
+    const unsigned *kin;
+    const int *vin;          // NULL: the value is the index (first pass)
+    unsigned *kout;          // NULL: the sorted keys are not wanted
+    int *vout;
+    const unsigned *hist;    // this pass's counts, [rows][256]
+    const unsigned *total;   // digit totals when radix_rows_kernel scanned hist, else NULL
+    unsigned *next;          // the next pass's counts, NULL in the last one
+    SortedPack pack;         // last pass: the bodies packed in sorted order
+};
+
+// One tile of one pass.  What bounds it at a tree's sizes (2^14 to 2^20 keys,
+// all in L2) is latency and the number of blocks: a warp ranks 32 keys at a
+// time with __match_any_sync against its own counters (stable: warps, rounds
+// and lanes are in key order), the tile is put in order in shared memory and
+// written in runs.  Up to SORT_SELF_ROWS tiles every block sums the tiles'
+// counts for itself; beyond, radix_rows_kernel has.  Against warps that took
+// 2048 keys each (2 to 64 blocks; two scan launches per pass, packing in a
+// launch of its own) a tree evaluation takes 2413 us instead of 2822 for four
+// steps of 20000 bodies, 4282 instead of 4408 at 2^20 bodies; the order itself
+// 106 us less at 16384 bodies, all with the same results.
+template <int IPT>
+__global__ void __launch_bounds__(OTPB) radix_scatter_kernel(const SortPass a)
+{
+    constexpr int TILE = OTPB * IPT, NW = OTPB / 32;
+    __shared__ __align__(16) unsigned cnt[NW][256];
+    __shared__ unsigned skey[TILE];
+    __shared__ int sval[TILE];
+    __shared__ unsigned gofs[256];
+    __shared__ unsigned ws[NW];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, t = threadIdx.x;
+    const unsigned lt = (1u << lane) - 1u;
+    const int tile0 = blockIdx.x * TILE, m = min(TILE, a.n - tile0);
+    const int wbase = warp * 32 * IPT;  // this warp's first key in the tile
+
+    unsigned k[IPT];
+    int v[IPT], rank[IPT];
+#pragma unroll
+    for (int r = 0; r < IPT; ++r) {
+        const int q = wbase + 32 * r + lane;
+        k[r] = q < m ? a.kin[tile0 + q] : 0u;
+        v[r] = q < m ? (a.vin ? a.vin[tile0 + q] : tile0 + q) : 0;
+    }
+    // counts of digit t before this tile, and in all tiles
+    unsigned pre, tot;
+    if (a.total) {
+        pre = a.hist[(size_t)blockIdx.x * 256 + t];
+        tot = a.total[t];
+    } else {
+        uint4 s4 = make_uint4(0u, 0u, 0u, 0u), p4 = s4;
+        const uint4 *h4 = reinterpret_cast<const uint4 *>(a.hist);
+#pragma unroll 8
+        for (int r = t >> 6; r < a.rows; r += OTPB / 64) {
+            const uint4 c = h4[(size_t)r * 64 + (t & 63)];
+            s4.x += c.x; s4.y += c.y; s4.z += c.z; s4.w += c.w;
+            if (r < (int)blockIdx.x) {
+                p4.x += c.x; p4.y += c.y; p4.z += c.z; p4.w += c.w;
+            }
+        }
+        uint4 *c4 = reinterpret_cast<uint4 *>(&cnt[0][0]);  // rows 0..3 all tiles, 4..7 before
+        c4[t] = s4;
+        c4[OTPB + t] = p4;
+        __syncthreads();
+        tot = cnt[0][t] + cnt[1][t] + cnt[2][t] + cnt[3][t];
+        pre = cnt[4][t] + cnt[5][t] + cnt[6][t] + cnt[7][t];
+        __syncthreads();
+    }
+#pragma unroll
+    for (int w = 0; w < NW; ++w) cnt[w][t] = 0u;
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < IPT; ++r) {
+        const bool valid = wbase + 32 * r + lane < m;
+        const unsigned d = valid ? ((k[r] >> a.shift) & 255u) : 256u;
+        const unsigned peers = __match_any_sync(0xffffffffu, d);
+        rank[r] = valid ? (int)(cnt[warp][d] + __popc(peers & lt)) : 0;
+        __syncwarp();
+        if (valid && (peers & lt) == 0u) cnt[warp][d] += (unsigned)__popc(peers);
+        __syncwarp();
+    }
+    __syncthreads();
+    {  // digit t: each warp's first place in the ordered tile, and the way from there to the output
+        unsigned run = 0u;
+#pragma unroll
+        for (int w = 0; w < NW; ++w) run += cnt[w][t];
+        unsigned place = scan256(run, ws);
+        gofs[t] = scan256(tot, ws) + pre - place;
+#pragma unroll
+        for (int w = 0; w < NW; ++w) {
+            const unsigned c = cnt[w][t];
+            cnt[w][t] = place;
+            place += c;
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < IPT; ++r) {
+        if (wbase + 32 * r + lane < m) {
+            const unsigned q = cnt[warp][(k[r] >> a.shift) & 255u] + (unsigned)rank[r];
+            skey[q] = k[r];
+            sval[q] = v[r];
+        }
+    }
+    __syncthreads();
+#pragma unroll 4
+    for (int q = t; q < m; q += OTPB) {
+        const unsigned key = skey[q];
+        const int i = sval[q];
+        const unsigned off = gofs[(key >> a.shift) & 255u] + (unsigned)q;
+        if (a.kout) a.kout[off] = key;
+        a.vout[off] = i;
+        if (a.next)
+            atomicAdd(a.next + (size_t)(off / TILE) * 256 + ((key >> (a.shift + 8)) & 255u), 1u);
+        else
+            put_body(a.pack, off, i);
+    }
+}
+
+__global__ void __launch_bounds__(OTPB) pack_hilo_kernel(int n, const SortedPack p)
+{
+    for (int k = blockIdx.x * OTPB + threadIdx.x; k < n; k += gridDim.x * OTPB) put_body(p, k, k);
 }
 
 inline int grid_for(int n)
@@ -303,66 +398,98 @@ inline int grid_for(int n)
     return g < 1 ? 1 : (g > 4096 ? 4096 : g);
 }
 
-}  // namespace
+// Tiles of the sort: small ones up to 2^16 keys, so that a few thousand keys
+// still spread over many blocks; up to SORT_SELF_ROWS tiles sum each other's
+// counts themselves (a block reads 1 KB per tile: above 64 tiles that costs
+// more than the launch that scans them).
+constexpr int SORT_SMALL = 4, SORT_LARGE = 16, SORT_SMALL_N = 1 << 16, SORT_SELF_ROWS = 64;
+inline int sort_ipt(int n) { return n <= SORT_SMALL_N ? SORT_SMALL : SORT_LARGE; }
+inline int sort_rows(int n)
+{
+    const int tile = OTPB * sort_ipt(n);
+    return (n + tile - 1) / tile;
+}
 
-int sort_chunks(int n) { return (n + SORT_CHUNK - 1) / SORT_CHUNK; }
+// Passes 0..passes-1 over the keys in o.keys[0] (their counts for the first
+// pass in o.hist): the order into perm_out, the sorted keys (if wanted) into
+// o.keys[passes & 1].
+void sort_passes(cudaStream_t s, int n, int passes, OrderScratch &o, int *perm_out, bool want_keys,
+                 const SortedPack &pack, int &kernels)
+{
+    const int rows = sort_rows(n);
+    unsigned *total = o.hist + (size_t)passes * rows * 256;
+    int cur = 0;
+    for (int pass = 0; pass < passes; ++pass) {
+        const bool last = pass == passes - 1;
+        unsigned *hist = o.hist + (size_t)pass * rows * 256;
+        SortPass a;
+        a.n = n;
+        a.rows = rows;
+        a.shift = 8 * pass;
+        a.kin = o.keys[cur];
+        a.vin = pass == 0 ? nullptr : o.vals[cur];
+        a.kout = last && !want_keys ? nullptr : o.keys[cur ^ 1];
+        a.vout = last ? perm_out : o.vals[cur ^ 1];
+        a.hist = hist;
+        a.total = nullptr;
+        a.next = last ? nullptr : hist + (size_t)rows * 256;
+        a.pack = pack;
+        if (rows > SORT_SELF_ROWS) {
+            radix_rows_kernel<<<8, 1024, 0, s>>>(hist, rows, total);
+            ++kernels;
+            a.total = total;
+        }
+        if (sort_ipt(n) == SORT_SMALL)
+            radix_scatter_kernel<SORT_SMALL><<<rows, OTPB, 0, s>>>(a);
+        else
+            radix_scatter_kernel<SORT_LARGE><<<rows, OTPB, 0, s>>>(a);
+        ++kernels;
+        cur ^= 1;
+    }
+}
+
+inline int box_parts(int n)
+{
+    const int g = grid_for(n);
+    return g < MAX_BOX_PARTS ? g : MAX_BOX_PARTS;
+}
+
+}  // namespace
 
 size_t sort_hist_entries(int n)
 {
-    // digit counts, then one partial sum per scan block
-    const size_t total = (size_t)256 * sort_chunks(n);
-    return total + (total + BSCAN_TILE - 1) / BSCAN_TILE + 32;
+    // 256 counts per tile for each of at most 4 passes, then the digit totals;
+    // fewer bodies than n may make up to 64 of the small tiles
+    const size_t large = ((size_t)n + OTPB * SORT_LARGE - 1) / (OTPB * SORT_LARGE);
+    const size_t rows = large > 64 ? large : 64;
+    return (4 * rows + 1) * 256;
 }
 
 cudaError_t launch_morton_sort(cudaStream_t s, int n, const double *pos, OrderScratch &o,
-                               int *perm_out, int &kernels)
+                               int *perm_out, const SortedPack &pack, int &kernels)
 {
     kernels = 0;
     if (n <= 0) return cudaSuccess;
-    const int nparts = grid_for(n) < MAX_BOX_PARTS ? grid_for(n) : MAX_BOX_PARTS;
+    const int nparts = box_parts(n), rows = sort_rows(n);
     bbox_kernel<<<nparts, OTPB, 0, s>>>(n, pos, o.box);
-    box_fold_kernel<<<1, 192, 0, s>>>(o.box, nparts);
-    morton_kernel<<<grid_for(n), OTPB, 0, s>>>(n, pos, o.box, o.keys[0], o.vals[0]);
-    kernels += 3;
-    const int nchunks = sort_chunks(n);
-    const int blocks = (nchunks + OTPB / 32 - 1) / (OTPB / 32);
-    int cur = 0;
-    for (int pass = 0; pass < 3; ++pass) {
-        const int shift = 8 * pass;
-        radix_hist_kernel<<<blocks, OTPB, 0, s>>>(n, o.keys[cur], shift, nchunks, o.hist);
-        launch_radix_scan(s, o.hist, 256 * nchunks);
-        int *vout = pass == 2 ? perm_out : o.vals[cur ^ 1];
-        radix_scatter_kernel<<<blocks, OTPB, 0, s>>>(n, o.keys[cur], o.vals[cur], o.keys[cur ^ 1],
-                                                     vout, shift, nchunks, o.hist);
-        kernels += 4;
-        cur ^= 1;
-    }
+    morton_kernel<<<rows, OTPB, 0, s>>>(n, pos, o.box, nparts, OTPB * sort_ipt(n), rows, o.keys[0],
+                                        o.hist);
+    kernels += 2;
+    sort_passes(s, n, 3, o, perm_out, false, pack, kernels);
     return cudaGetLastError();
 }
 
 cudaError_t launch_tree_sort(cudaStream_t s, int n, const double *pos, OrderScratch &o,
-                             int *perm_out, double *box_out, int &kernels)
+                             int *perm_out, double *box_out, const SortedPack &pack, int &kernels)
 {
     kernels = 0;
     if (n <= 0) return cudaSuccess;
-    const int nparts = grid_for(n) < MAX_BOX_PARTS ? grid_for(n) : MAX_BOX_PARTS;
+    const int nparts = box_parts(n), rows = sort_rows(n);
     bbox_kernel<<<nparts, OTPB, 0, s>>>(n, pos, o.box);
-    box_fold_kernel<<<1, 192, 0, s>>>(o.box, nparts);
-    morton30_kernel<<<grid_for(n), OTPB, 0, s>>>(n, pos, o.box, o.keys[0], o.vals[0], box_out);
-    kernels += 3;
-    const int nchunks = sort_chunks(n);
-    const int blocks = (nchunks + OTPB / 32 - 1) / (OTPB / 32);
-    int cur = 0;
-    for (int pass = 0; pass < 4; ++pass) {  // 30-bit keys: 4 passes, sorted keys end in keys[0]
-        const int shift = 8 * pass;
-        radix_hist_kernel<<<blocks, OTPB, 0, s>>>(n, o.keys[cur], shift, nchunks, o.hist);
-        launch_radix_scan(s, o.hist, 256 * nchunks);
-        int *vout = pass == 3 ? perm_out : o.vals[cur ^ 1];
-        radix_scatter_kernel<<<blocks, OTPB, 0, s>>>(n, o.keys[cur], o.vals[cur], o.keys[cur ^ 1],
-                                                     vout, shift, nchunks, o.hist);
-        kernels += 4;
-        cur ^= 1;
-    }
+    morton30_kernel<<<rows, OTPB, 0, s>>>(n, pos, o.box, nparts, OTPB * sort_ipt(n), rows,
+                                          o.keys[0], o.hist, box_out);
+    kernels += 2;
+    sort_passes(s, n, 4, o, perm_out, true, pack, kernels);  // sorted keys end in keys[0]
     return cudaGetLastError();
 }
 
@@ -371,29 +498,19 @@ cudaError_t launch_key_sort(cudaStream_t s, int n, const int *k32, const long lo
 {
     kernels = 0;
     if (n <= 0) return cudaSuccess;
-    key_init_kernel<<<grid_for(n), OTPB, 0, s>>>(n, k32, k64, o.keys[0], o.vals[0]);
+    const int rows = sort_rows(n);
+    key_init_kernel<<<rows, OTPB, 0, s>>>(n, k32, k64, OTPB * sort_ipt(n), rows, passes, o.keys[0],
+                                          o.hist);
     ++kernels;
-    const int nchunks = sort_chunks(n);
-    const int blocks = (nchunks + OTPB / 32 - 1) / (OTPB / 32);
-    int cur = 0;
-    for (int pass = 0; pass < passes; ++pass) {
-        const int shift = 8 * pass;
-        radix_hist_kernel<<<blocks, OTPB, 0, s>>>(n, o.keys[cur], shift, nchunks, o.hist);
-        launch_radix_scan(s, o.hist, 256 * nchunks);
-        int *vout = pass == passes - 1 ? perm_out : o.vals[cur ^ 1];
-        radix_scatter_kernel<<<blocks, OTPB, 0, s>>>(n, o.keys[cur], o.vals[cur], o.keys[cur ^ 1],
-                                                     vout, shift, nchunks, o.hist);
-        kernels += 4;
-        cur ^= 1;
-    }
+    sort_passes(s, n, passes, o, perm_out, false, SortedPack{}, kernels);
     return cudaGetLastError();
 }
 
 cudaError_t launch_pack_hilo(cudaStream_t s, int n, const double *pos, const double *mass,
-                             const int *perm, float4 *Phi, float4 *Plo)
+                             float4 *Phi, float4 *Plo)
 {
     if (n <= 0) return cudaSuccess;
-    pack_hilo_kernel<<<grid_for(n), OTPB, 0, s>>>(n, pos, mass, perm, Phi, Plo);
+    pack_hilo_kernel<<<grid_for(n), OTPB, 0, s>>>(n, SortedPack{pos, mass, Phi, Plo, nullptr});
     return cudaGetLastError();
 }
 
