@@ -137,11 +137,13 @@ struct OrderScratch {
 };
 size_t sort_hist_entries(int n);  // entries of OrderScratch::hist for up to n bodies
 // Where a sort packs the bodies in sorted order: float32 hi/lo pairs
-// (Phi.w = m, Plo.w = log2(m)) when Phi, else float64 when P64, else nothing.
+// (Phi.w = m, Plo.w = log2(m) when logm, else 0) when Phi, else float64 when
+// P64, else nothing.
 struct SortedPack {
     const double *pos = nullptr, *mass = nullptr;
     float4 *Phi = nullptr, *Plo = nullptr;
     double4 *P64 = nullptr;
+    bool logm = false;  // the log-domain pair kernels will read Plo.w
 };
 // perm_out[k] = body at Morton rank k (stable in body index); `kernels` = launches made.
 cudaError_t launch_morton_sort(cudaStream_t s, int n, const double *pos, OrderScratch &o,
@@ -165,9 +167,9 @@ cudaError_t launch_pack_hilo(cudaStream_t s, int n, const double *pos, const dou
 // from `first` in octant order (nchild == 0: leaf).
 struct TreeView {
     int cap;
-    int *meta;            // [tree_meta_ints()] per-level node counts and bases, overflow flag
-    int *start, *end, *level, *nchild, *first, *offs;
-    int *parent, *arrive;     // parent node (-1 at the root); children counted in by the moments
+    int *meta;            // [tree_meta_ints()] per-level node counts and bases
+    int *start, *end, *level, *nchild, *first;
+    int *parent, *arrive;     // parent node (-1 at the root); bodies counted in by the moments
     unsigned *prefix;
     double *M, *com;      // float64 monopoles: mass, centre of mass [cap][3]
     float4 *box_lo, *box_hi;  // float32 cell cube corners; .w = nchild, first (int bits)
@@ -216,9 +218,10 @@ int tree_meta_ints();
 // Upper bound on the node count of a tree over n bodies with leaves of at
 // most leaf_cap bodies (no build can exceed it).
 int64_t tree_node_bound(int64_t n, int leaf_cap);
-// Build over sorted keys (launch_tree_sort), float64 moments, float32 walk data.
+// Build over the sorted keys launch_tree_sort left in o.keys[0] (o.vals[0] and
+// o.hist are scratch), float64 moments, float32 walk data.
 // box = {lo_x, lo_y, lo_z, ext} from launch_tree_sort.
-cudaError_t launch_tree_build(cudaStream_t s, const TreeView &t, int n, const unsigned *keys,
+cudaError_t launch_tree_build(cudaStream_t s, const TreeView &t, int n, const OrderScratch &o,
                               const double *box, const double *pos, const double *mass,
                               const int *perm, int leaf_cap, int *err, int &kernels);
 cudaError_t launch_tree_walk(cudaStream_t s, const TreeWalkParams &p, bool zeps, int &kernels);

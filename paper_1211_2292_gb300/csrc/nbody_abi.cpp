@@ -310,7 +310,7 @@ nb_status pack(nb_ctx *c, cudaStream_t s, int64_t n, const double *pos, const do
 {
     if (n == 0) return NB_OK;
     c->perm_active = allow_order && use_order(c, n);
-    nb::SortedPack pk{pos, mass, nullptr, nullptr, nullptr};
+    nb::SortedPack pk{pos, mass, nullptr, nullptr, nullptr, true};
     if (is_f64(c))
         pk.P64 = (double4 *)c->pack;
     else
@@ -496,10 +496,10 @@ T *dev_alloc(nb_ctx *c, size_t count, nb_status &st)
 void free_tree_nodes(nb_ctx *c)
 {
     nb::TreeView &t = c->tree;
-    void *arrays[] = {t.start, t.end,   t.level,  t.nchild, t.first, t.offs, t.parent,
+    void *arrays[] = {t.start, t.end,   t.level,  t.nchild, t.first, t.parent,
                       t.arrive, t.prefix, t.M,  t.com,    t.box_lo, t.box_hi, t.chi, t.clo};
     for (void *a : arrays) cudaFree(a);
-    t.start = t.end = t.level = t.nchild = t.first = t.offs = t.parent = t.arrive = nullptr;
+    t.start = t.end = t.level = t.nchild = t.first = t.parent = t.arrive = nullptr;
     t.prefix = nullptr;
     t.M = t.com = nullptr;
     t.box_lo = t.box_hi = t.chi = t.clo = nullptr;
@@ -622,7 +622,7 @@ nb_status ensure_tree(nb_ctx *c, int leaf_cap)
     free_tree_nodes(c);
     nb::TreeView &t = c->tree;
     const size_t m = (size_t)need;
-    int **ints[] = {&t.start, &t.end, &t.level, &t.nchild, &t.first, &t.offs, &t.parent, &t.arrive};
+    int **ints[] = {&t.start, &t.end, &t.level, &t.nchild, &t.first, &t.parent, &t.arrive};
     for (int **a : ints)
         if (st == NB_OK) *a = dev_alloc<int>(c, m, st);
     if (st == NB_OK) t.prefix = dev_alloc<unsigned>(c, m, st);
@@ -781,10 +781,10 @@ nb_status tree_build_enqueue(nb_ctx *c, cudaStream_t s, int64_t n, const double 
 {
     int k = 0;
     TreeTimer tm(c, nb::PROF_TREE_BUILD, s);
-    const nb::SortedPack pk{pos, mass, c->tree_P, c->tree_Plo, nullptr};
+    const nb::SortedPack pk{pos, mass, c->tree_P, c->tree_Plo, nullptr, false};
     NB_CUDA(c, nb::launch_tree_sort(s, (int)n, pos, c->order, c->tree_perm, c->tree_box, pk, k));
     c->launches += k;
-    NB_CUDA(c, nb::launch_tree_build(s, c->tree, (int)n, c->order.keys[0], c->tree_box, pos, mass,
+    NB_CUDA(c, nb::launch_tree_build(s, c->tree, (int)n, c->order, c->tree_box, pos, mass,
                                      c->tree_perm, leaf_cap, c->err, k));
     c->launches += k;
     tm.done();

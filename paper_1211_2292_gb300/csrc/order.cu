@@ -155,6 +155,18 @@ __device__ __forceinline__ unsigned spread10(unsigned v)
     return v;
 }
 
+// floor(t) clamped to [0, 1023], 0 for NaN, from t's bits: comparisons and the
+// conversion would take the float64 pipe (2 lanes per clock per SM), which
+// bounds the key kernel.
+__device__ __forceinline__ unsigned cell1024(double t)
+{
+    const int hi = __double2hiint(t), e = (hi >> 20) - 1023;  // sign bit set: e < 0
+    if (e < 0) return 0u;                                     // t < 1, t negative
+    if (hi >= 0x408ff800)                                     // t >= 1023, infinity, NaN
+        return hi > 0x7ff00000 || (hi == 0x7ff00000 && __double2loint(t) != 0) ? 0u : 1023u;
+    return (unsigned)((hi & 0xfffff) | 0x100000) >> (20 - e);
+}
+
 // 30-bit Morton keys for the tree code: q = floor((x - lo) * (1024 / ext)),
 // clamped to [0, 1023], with lo the box minimum and ext its longest side, all
 // in float64 (the same operations as the tree's cell geometry, so a body's
@@ -183,10 +195,8 @@ __global__ void __launch_bounds__(OTPB) morton30_kernel(int n, const double *__r
     emit_keys(n, tile, rows, 4, keys, hist, [&](int i) {
         unsigned q[3];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const double t = __dmul_rn(__dsub_rn(pos[3 * (size_t)i + c], box[c]), scale);
-            q[c] = t >= 1023.0 ? 1023u : (t <= 0.0 ? 0u : (unsigned)t);
-        }
+        for (int c = 0; c < 3; ++c)
+            q[c] = cell1024(__dmul_rn(__dsub_rn(pos[3 * (size_t)i + c], box[c]), scale));
         return spread10(q[0]) | (spread10(q[1]) << 1) | (spread10(q[2]) << 2);
     });
 }
@@ -261,7 +271,7 @@ __device__ __forceinline__ void put_body(const SortedPack &p, size_t k, int i)
         const double m = p.mass[i];
         p.Phi[k] = make_float4(hx, hy, hz, (float)m);
         p.Plo[k] = make_float4((float)(x[0] - (double)hx), (float)(x[1] - (double)hy),
-                               (float)(x[2] - (double)hz), (float)log2(m));
+                               (float)(x[2] - (double)hz), p.logm ? (float)log2(m) : 0.f);
     } else if (p.P64) {
         const double *x = p.pos + 3 * (size_t)i;
         p.P64[k] = make_double4(x[0], x[1], x[2], p.mass[i]);
@@ -510,7 +520,7 @@ cudaError_t launch_pack_hilo(cudaStream_t s, int n, const double *pos, const dou
                              float4 *Phi, float4 *Plo)
 {
     if (n <= 0) return cudaSuccess;
-    pack_hilo_kernel<<<grid_for(n), OTPB, 0, s>>>(n, SortedPack{pos, mass, Phi, Plo, nullptr});
+    pack_hilo_kernel<<<grid_for(n), OTPB, 0, s>>>(n, SortedPack{pos, mass, Phi, Plo, nullptr, true});
     return cudaGetLastError();
 }
 

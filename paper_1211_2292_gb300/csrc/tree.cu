@@ -18,11 +18,10 @@
 //  * cell moments are float64 (mass, centre of mass).
 //
 // Build (all on the device, no host synchronisation, so it can be captured
-// in a graph): level by level from the root, each node of level L with more
-// than leaf_cap bodies finds its octant ranges by binary search on the
-// sorted keys (one warp per node); one block scans the child counts of the
-// level; children are written contiguously in octant order.  Moments are
-// summed bottom-up.
+// in a graph): the sorted keys alone say which nodes start at which body; one
+// launch counts them per level and block of bodies, one numbers and writes
+// them (level by level, children consecutive in octant order), one sums the
+// moments bottom-up.
 //
 // Walk arithmetic: float32 pair terms in coordinates relative to the
 // group's centre (hi/lo packed positions and centres of mass, as in the
@@ -50,8 +49,9 @@ constexpr int TTPB = 256;
 #define NB_WALK_MINB2 5
 #endif
 constexpr int WALK_WARPS = NB_WALK_WARPS;
+constexpr int LEVELS = 11;
 
-enum { META_COUNT = 0, META_BASE = 12, META_OVERFLOW = 24, META_QUEUE = 25, META_INTS = 32 };
+enum { META_COUNT = 0, META_BASE = 12, META_QUEUE = 25, META_INTS = 32 };
 static_assert(META_COUNT == TREE_META_COUNT && META_BASE == TREE_META_BASE &&
                   META_QUEUE == TREE_META_QUEUE, "meta layout shared with nb_internal.h");
 
@@ -68,9 +68,7 @@ __device__ __forceinline__ double pow2_neg(int L)
 }
 
 // Float32 cube of the level-L cell with key prefix `pre`, exactly as the
-// oracle forms it (float64 lo + edge * index, rounded); .w of the corners
-// carries the child count (0) and first child (-1) until the node's own
-// level is built.
+// oracle forms it (float64 lo + edge * index, rounded).
 __device__ __forceinline__ void cube_corners(const double *__restrict__ box, int L, unsigned pre,
                                              float4 &lo4, float4 &hi4)
 {
@@ -89,133 +87,219 @@ __device__ __forceinline__ void cube_corners(const double *__restrict__ box, int
         blo[c] = (float)__dadd_rn(box[c], __dmul_rn(cell, (double)ic[c]));
         bhi[c] = (float)__dadd_rn(box[c], __dmul_rn(cell, (double)(ic[c] + 1u)));
     }
-    lo4 = make_float4(blo[0], blo[1], blo[2], __int_as_float(0));
-    hi4 = make_float4(bhi[0], bhi[1], bhi[2], __int_as_float(-1));
+    lo4 = make_float4(blo[0], blo[1], blo[2], 0.f);
+    hi4 = make_float4(bhi[0], bhi[1], bhi[2], 0.f);
 }
 
-__global__ void tree_init_kernel(TreeView t, int n, const double *box)
+// ------------------------------------------------------------------ build
+// The nodes follow from the sorted keys alone.  With lcp(a, b) the number of
+// leading octants two keys share (10 when equal), a cell of level L starts at
+// body i when L > lcp(key[i-1], key[i]); it is a node when its parent holds
+// more than leaf_cap bodies, and a leaf when it does not itself, or L = 10.
+// So the nodes that start at body i are those of levels lo..hi:
+//   lo = lcp(key[i-1], key[i]) + 1 (0 for i = 0), and with
+//   D = lcp(key[i], key[i+leaf_cap]) (the deepest cell from i on that holds
+//   more than leaf_cap): hi = min(10, D + 1) when D >= lo, else hi = lo when
+//   the cell of level lo - 1 around i holds more than leaf_cap (the root
+//   always is a node), else none.
+// A node's number is its rank by (level, start), which one scan of the
+// (level, block of bodies) counts and ballots within the block give; children
+// are consecutive in octant order.
+//
+// Two launches over the bodies (count, write) took the place of three launches
+// per level (octant boundaries by binary search, one block's scan, children
+// written), which were 30 launches of 3 to 10 us at any size.  With the moments
+// below: four tree steps of 20000 bodies 2413 -> 1939 us, a tree evaluation of
+// 2^20 bodies 4282 -> 3911 us, the same results to the bit.
+__device__ __forceinline__ int key_lcp(unsigned a, unsigned b)
 {
-    if (threadIdx.x < META_INTS) t.meta[threadIdx.x] = 0;
-    if (threadIdx.x < 4) t.stats[threadIdx.x] = 0ull;
-    if (threadIdx.x == 0) {
-        t.meta[META_COUNT + 0] = 1;
-        t.start[0] = 0;
-        t.end[0] = n;
-        t.prefix[0] = 0u;
-        t.level[0] = 0;
-        t.nchild[0] = 0;
-        t.first[0] = -1;
-        t.parent[0] = -1;
-        t.arrive[0] = 0;
-        cube_corners(box, 0, 0u, t.box_lo[0], t.box_hi[0]);
+    return (__clz(a ^ b) - 2) / 3;  // 30-bit keys; 10 when equal
+}
+
+constexpr int BUILD_BLOCKS = 592;  // blocks of bodies at most: each sums the others' counts
+
+// Level range of the nodes starting at each body, lv[i] = lo | hi << 4 (lo > hi:
+// none), and per block and level how many: tab[L * nblk + b].
+__global__ void __launch_bounds__(TTPB) tree_levels_kernel(TreeView t, int n,
+                                                           const unsigned *__restrict__ keys,
+                                                           int leaf_cap, int chunk,
+                                                           unsigned char *__restrict__ lv,
+                                                           int *__restrict__ tab)
+{
+    __shared__ int wsum[TTPB / 32][LEVELS];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (blockIdx.x == 0) {
+        if (threadIdx.x < META_INTS) t.meta[threadIdx.x] = 0;
+        if (threadIdx.x < 4) t.stats[threadIdx.x] = 0ull;
     }
-}
-
-// First key index in [lo, hi) with key >= v.
-__device__ __forceinline__ int lower_bound(const unsigned *__restrict__ keys, int lo, int hi,
-                                           unsigned v)
-{
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (keys[mid] < v)
-            lo = mid + 1;
-        else
-            hi = mid;
-    }
-    return lo;
-}
-
-// One warp per node: lane o (1..7) finds where octant o starts in the
-// node's sorted keys, lane 0 holds start and lane 8 end; lane o < 8 then
-// sees whether child o is non-empty.  Returns the ballot of non-empty
-// children (bit o) and leaves the child's range in [b, nxt) on lane o.
-__device__ __forceinline__ unsigned octants(const unsigned *__restrict__ keys, int s, int e,
-                                            unsigned prefix, int L, int lane, int &b, int &nxt)
-{
-    const int shift = 3 * (10 - (L + 1));
-    b = lane == 0 ? s : (lane <= 7 ? lower_bound(keys, s, e, (prefix * 8u + lane) << shift) : e);
-    nxt = __shfl_down_sync(0xffffffffu, b, 1);
-    return __ballot_sync(0xffffffffu, lane < 8 && nxt > b);
-}
-
-__global__ void __launch_bounds__(TTPB) tree_count_kernel(TreeView t, const unsigned *keys, int L,
-                                                          int leaf_cap)
-{
-    const int cnt = t.meta[META_COUNT + L], base = t.meta[META_BASE + L];
-    const int lane = threadIdx.x & 31;
-    const int warps = gridDim.x * (TTPB / 32);
-    for (int q = blockIdx.x * (TTPB / 32) + (threadIdx.x >> 5); q < cnt; q += warps) {
-        const int node = base + q;
-        const int s = t.start[node], e = t.end[node];
-        int nch = 0;
-        if (e - s > leaf_cap) {
-            int b, nxt;
-            nch = __popc(octants(keys, s, e, t.prefix[node], L, lane, b, nxt));
-        }
-        if (lane == 0) t.nchild[node] = nch;
-    }
-}
-
-// One block: exclusive scan of the child counts of level L into t.offs,
-// level L+1's count and base into meta.
-__global__ void __launch_bounds__(1024) tree_scan_kernel(TreeView t, int L)
-{
-    __shared__ int tile[BSCAN_TILE + BSCAN_TILE / 32];
-    __shared__ int wsum[32];
-    const int cnt = t.meta[META_COUNT + L], base = t.meta[META_BASE + L];
-    const int total = block_scan_exclusive<int>(t.nchild + base, t.offs, cnt, tile, wsum);
-    if (threadIdx.x == 0) {
-        const int nbase = base + cnt;
-        int room = (int)(t.cap - nbase);
-        room = room < 0 ? 0 : room;
-        // Past the capacity (never, with tree_node_bound) the tree stops at
-        // this level: every node of it becomes a leaf and the flag is raised.
-        if (total > room) t.meta[META_OVERFLOW] = 1;
-        t.meta[META_BASE + L + 1] = nbase;
-        t.meta[META_COUNT + L + 1] = total > room ? 0 : total;
-    }
-}
-
-__global__ void __launch_bounds__(TTPB) tree_emit_kernel(TreeView t, const unsigned *keys,
-                                                         const double *__restrict__ box, int L)
-{
-    const int cnt = t.meta[META_COUNT + L], base = t.meta[META_BASE + L];
-    const int nbase = t.meta[META_BASE + L + 1];
-    const bool stop = t.meta[META_COUNT + L + 1] == 0;
-    const int lane = threadIdx.x & 31;
-    const unsigned lt = (1u << lane) - 1u;
-    const int warps = gridDim.x * (TTPB / 32);
-    for (int q = blockIdx.x * (TTPB / 32) + (threadIdx.x >> 5); q < cnt; q += warps) {
-        const int node = base + q;
-        const int nch = t.nchild[node];
-        if (nch == 0 || stop) {
-            if (lane == 0) {
-                t.nchild[node] = 0;
-                t.first[node] = -1;
+    const int b0 = blockIdx.x * chunk, b1 = min(n - b0, chunk) + b0;
+    int mine = 0;  // lane L: nodes of level L
+    for (int r = b0; r < b1; r += TTPB) {
+        const int i = r + threadIdx.x;
+        int lo = 1, hi = 0;
+        if (i < b1) {
+            const unsigned k = keys[i];
+            lo = i == 0 ? 0 : key_lcp(keys[i - 1], k) + 1;
+            const int D = n - i > leaf_cap ? key_lcp(k, keys[i + leaf_cap]) : -1;
+            if (lo > 10) {  // the same cell as the body before at every level
+                lo = 1;
+            } else if (D >= lo) {
+                hi = min(10, D + 1);
+            } else if (lo == 0) {
+                hi = 0;
+            } else {
+                // the parent's start, if within leaf_cap bodies before i
+                const int sh = 3 * (11 - lo);
+                const unsigned pre = k >> sh;
+                int a = max(0, i - leaf_cap), b = i;
+                while (a < b) {
+                    const int mid = (a + b) >> 1;
+                    if ((keys[mid] >> sh) < pre)
+                        a = mid + 1;
+                    else
+                        b = mid;
+                }
+                const bool over = n - a > leaf_cap && (keys[a + leaf_cap] >> sh) == pre;
+                if (over)
+                    hi = lo;
+                else
+                    lo = 1;
             }
-            continue;
+            lv[i] = (unsigned char)(lo | (hi << 4));
         }
-        const unsigned pre = t.prefix[node];
-        int b, nxt;
-        const unsigned ne = octants(keys, t.start[node], t.end[node], pre, L, lane, b, nxt);
-        const int first = nbase + t.offs[q];
+#pragma unroll
+        for (int L = 0; L < LEVELS; ++L) {
+            const unsigned b = __ballot_sync(0xffffffffu, lo <= L && L <= hi);
+            if (lane == L) mine += __popc(b);
+        }
+    }
+    if (lane < LEVELS) wsum[warp][lane] = mine;
+    __syncthreads();
+    if (threadIdx.x < LEVELS) {
+        int s = 0;
+#pragma unroll
+        for (int w = 0; w < TTPB / 32; ++w) s += wsum[w][threadIdx.x];
+        tab[threadIdx.x * gridDim.x + blockIdx.x] = s;
+    }
+}
+
+// First index >= from (from >= 1) with key >= v, found by doubling steps.
+__device__ __forceinline__ int gallop(const unsigned *__restrict__ keys, int from, int n, unsigned v)
+{
+    int step = 1, a = from;
+    while (n - a >= step && keys[a + step - 1] < v) {
+        a += step;
+        step *= 2;
+    }
+    int b = min(n, a + step - 1);  // the answer lies in [a, b]
+    while (a < b) {
+        const int mid = (a + b) >> 1;
+        if (keys[mid] < v)
+            a = mid + 1;
+        else
+            b = mid;
+    }
+    return a;
+}
+
+__global__ void __launch_bounds__(TTPB) tree_emit_kernel(TreeView t, int n,
+                                                         const unsigned *__restrict__ keys,
+                                                         int chunk,
+                                                         const unsigned char *__restrict__ lv,
+                                                         const int *__restrict__ tab, int *err)
+{
+    __shared__ int tot[LEVELS], run[LEVELS], top_s;
+    __shared__ int wcnt[TTPB / 32][LEVELS], woff[TTPB / 32][LEVELS];
+    __shared__ unsigned bal[TTPB / 32][LEVELS];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nblk = gridDim.x;
+    const unsigned lt = (1u << lane) - 1u;
+    for (int L = warp; L < LEVELS; L += TTPB / 32) {
+        int all = 0, pre = 0;
+#pragma unroll 4
+        for (int b = lane; b < nblk; b += 32) {
+            const int c = tab[L * nblk + b];
+            all += c;
+            if (b < (int)blockIdx.x) pre += c;
+        }
+        all = __reduce_add_sync(0xffffffffu, all);
+        pre = __reduce_add_sync(0xffffffffu, pre);
         if (lane == 0) {
-            t.first[node] = first;
-            reinterpret_cast<int *>(t.box_lo + node)[3] = nch;  // the walk's child count
-            reinterpret_cast<int *>(t.box_hi + node)[3] = first;
+            tot[L] = all;
+            run[L] = pre;
         }
-        if (lane < 8 && ((ne >> lane) & 1u)) {
-            const int c = first + __popc(ne & lt);
-            t.start[c] = b;
-            t.end[c] = nxt;
-            t.prefix[c] = pre * 8u + lane;
-            t.level[c] = L + 1;
-            t.nchild[c] = 0;
-            t.first[c] = -1;
-            t.parent[c] = node;
-            t.arrive[c] = 0;
-            cube_corners(box, L + 1, pre * 8u + lane, t.box_lo[c], t.box_hi[c]);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        // The levels' first nodes.  Past the capacity (never, with
+        // tree_node_bound) the tree stops a level early: the nodes of the last
+        // level that fits become leaves, and the flag is raised.
+        int base = 0, top = LEVELS - 1;
+        for (int L = 0; L < LEVELS; ++L) {
+            if (L <= top && tot[L] > t.cap - base) {
+                top = L - 1;
+                if (blockIdx.x == 0) atomicOr(err, ERR_TREE);
+            }
+            const int c = L <= top ? tot[L] : 0;
+            if (blockIdx.x == 0) {
+                t.meta[META_BASE + L] = base;
+                t.meta[META_COUNT + L] = c;
+            }
+            run[L] += base;
+            base += c;
         }
+        top_s = top;
+    }
+    __syncthreads();
+    const int top = top_s;
+    const int b0 = blockIdx.x * chunk, b1 = min(n - b0, chunk) + b0;
+    for (int r = b0; r < b1; r += TTPB) {
+        const int i = r + threadIdx.x;
+        int lo = 1, hi = 0;
+        if (i < b1) {
+            const int q = lv[i];
+            lo = q & 15;
+            hi = min(q >> 4, top);
+        }
+#pragma unroll
+        for (int L = 0; L < LEVELS; ++L) {
+            const unsigned b = __ballot_sync(0xffffffffu, lo <= L && L <= hi);
+            if (lane == L) {
+                bal[warp][L] = b;
+                wcnt[warp][L] = __popc(b);
+            }
+        }
+        __syncthreads();
+        if (lane < LEVELS) {
+            int s = run[lane];
+            for (int w = 0; w < warp; ++w) s += wcnt[w][lane];
+            woff[warp][lane] = s;
+        }
+        __syncthreads();
+        if (threadIdx.x < LEVELS) run[threadIdx.x] = woff[TTPB / 32 - 1][threadIdx.x] +
+                                                     wcnt[TTPB / 32 - 1][threadIdx.x];
+        if (lo <= hi) {
+            const unsigned k = keys[i];
+            int end = i + 1, child = -1;
+            for (int L = hi; L >= lo; --L) {
+                const int sh = 3 * (10 - L);
+                const unsigned pre = k >> sh;
+                end = gallop(keys, end, n, (pre + 1u) << sh);
+                const int node = woff[warp][L] + __popc(bal[warp][L] & lt);
+                t.start[node] = i;
+                t.end[node] = end;
+                t.prefix[node] = pre;
+                t.level[node] = L;
+                t.nchild[node] = L < hi ? -1 : 0;  // counted with the moments
+                t.first[node] = child;
+                // the last node of the level above that starts at or before i
+                t.parent[node] = L == 0 ? -1
+                                        : woff[warp][L - 1] +
+                                              __popc(bal[warp][L - 1] & (lt | (1u << lane))) - 1;
+                t.arrive[node] = 0;
+                child = node;
+            }
+        }
+        __syncthreads();  // the shared rows are rewritten
     }
 }
 
@@ -234,52 +318,138 @@ __device__ __forceinline__ void put_walk_moments(const TreeView &t, int node, do
                               (float)(cz - (double)hz), 0.f);
 }
 
-// Float64 monopoles of every node in one launch, bottom-up without any wait:
-// a thread per leaf sums its bodies, then climbs; at each parent it counts
-// itself in with an atomic, and only the last child to arrive goes on to
-// sum the parent's children (in child order, so the result does not depend
-// on who arrives last).  Fences order the moments before the arrival.
-__global__ void __launch_bounds__(TTPB) tree_moments_kernel(TreeView t, const double *__restrict__ pos,
+// Float64 monopoles of every node in one launch, bottom-up without any wait
+// (and every node's float32 cube).  A thread per leaf sums its bodies; its
+// node then counts its bodies in at the parent with an atomic, and only the
+// child that completes the parent's count goes on to the parent, whose
+// children eight lanes then sum (totalled in a fixed order, so the result does
+// not depend on who arrives last); the climbing nodes of a warp are taken four
+// at a time.  Fences order the sums before the arrival.
+//
+// What bounds it is the float64 pipe (2 lanes per clock per SM: a warp
+// instruction takes 16 cycles whether one lane needs it or all) and, for small
+// trees, the chain of levels.  So the cubes and the leaves' sums keep every
+// lane busy, a parent's four sums are reduced over its eight lanes with four
+// additions (each lane ends with one of them), and one division per node
+// turns each lane's sum into its coordinate.
+__global__ void __launch_bounds__(TTPB) tree_moments_kernel(TreeView t,
+                                                            const double *__restrict__ box,
+                                                            const double *__restrict__ pos,
                                                             const double *__restrict__ mass,
                                                             const int *__restrict__ perm)
 {
+    const unsigned FULL = 0xffffffffu;
     const int total = t.meta[META_BASE + 10] + t.meta[META_COUNT + 10];
     if (blockIdx.x == 0 && threadIdx.x == 0) t.stats[0] = (unsigned long long)total;
+    const int lane = threadIdx.x & 31, o = lane & 7;
     int leaves = 0;
-    for (int leaf = blockIdx.x * TTPB + threadIdx.x; leaf < total; leaf += gridDim.x * TTPB) {
-        if (t.nchild[leaf] != 0) continue;
-        ++leaves;
-        double M = 0.0, sx = 0.0, sy = 0.0, sz = 0.0;
-        for (int k = t.start[leaf]; k < t.end[leaf]; ++k) {
-            const int j = perm[k];
-            const double m = mass[j];
-            M += m;
-            sx += m * pos[3 * (size_t)j];
-            sy += m * pos[3 * (size_t)j + 1];
-            sz += m * pos[3 * (size_t)j + 2];
-        }
-        put_walk_moments(t, leaf, M, M > 0.0 ? sx / M : 0.0, M > 0.0 ? sy / M : 0.0,
-                         M > 0.0 ? sz / M : 0.0);
-        for (int node = t.parent[leaf]; node >= 0; node = t.parent[node]) {
-            __threadfence();
-            if (atomicAdd(t.arrive + node, 1) != t.nchild[node] - 1) break;
-            __threadfence();
-            const int f = t.first[node], nch = t.nchild[node];
-            M = sx = sy = sz = 0.0;
-            for (int c = f; c < f + nch; ++c) {
-                const double m = __ldcg(t.M + c);
-                M += m;
-                sx += m * __ldcg(t.com + 3 * (size_t)c);
-                sy += m * __ldcg(t.com + 3 * (size_t)c + 1);
-                sz += m * __ldcg(t.com + 3 * (size_t)c + 2);
+    for (int q0 = blockIdx.x * TTPB + (threadIdx.x & ~31); q0 < total; q0 += gridDim.x * TTPB) {
+        const int me = q0 + lane;
+        int node = -1, count = 0;  // what this lane counts in at its parent
+        if (me < total) {
+            float4 lo, hi;
+            cube_corners(box, t.level[me], t.prefix[me], lo, hi);
+            float *bl = reinterpret_cast<float *>(t.box_lo + me);
+            *reinterpret_cast<float2 *>(bl) = make_float2(lo.x, lo.y);
+            bl[2] = lo.z;  // [3], the child count, belongs to the climb
+            hi.w = __int_as_float(t.first[me]);
+            t.box_hi[me] = hi;
+            if (t.nchild[me] == 0) {
+                ++leaves;
+                bl[3] = __int_as_float(0);
+                const int s = t.start[me], e = t.end[me];
+                double M = 0.0, sx = 0.0, sy = 0.0, sz = 0.0;
+                for (int k = s; k < e; k += 4) {  // four bodies' loads in flight
+                    double m[4], x[4], y[4], z[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const int j = perm[min(k + u, e - 1)];
+                        m[u] = mass[j];
+                        x[u] = pos[3 * (size_t)j];
+                        y[u] = pos[3 * (size_t)j + 1];
+                        z[u] = pos[3 * (size_t)j + 2];
+                    }
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        if (k + u < e) {
+                            M += m[u];
+                            sx += m[u] * x[u];
+                            sy += m[u] * y[u];
+                            sz += m[u] * z[u];
+                        }
+                    }
+                }
+                put_walk_moments(t, me, M, M > 0.0 ? sx / M : 0.0, M > 0.0 ? sy / M : 0.0,
+                                 M > 0.0 ? sz / M : 0.0);
+                node = t.parent[me];
+                count = e - s;
             }
-            put_walk_moments(t, node, M, M > 0.0 ? sx / M : 0.0, M > 0.0 ? sy / M : 0.0,
-                             M > 0.0 ? sz / M : 0.0);
+        }
+        // climb: each lane with a node counts in; the completed parents are
+        // summed and count in themselves
+        while (__any_sync(FULL, node >= 0)) {
+            bool won = false;
+            int bodies = 0;
+            if (node >= 0) {
+                bodies = t.end[node] - t.start[node];
+                __threadfence();
+                won = atomicAdd(t.arrive + node, count) + count == bodies;
+                __threadfence();
+            }
+            unsigned win = __ballot_sync(FULL, won);
+            int up = -1;
+            if (won) up = t.parent[node];
+            while (win) {
+                // group g of eight lanes takes the g-th winner
+                const int g = lane >> 3;
+                int src = -1;
+                unsigned w = win;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if (q == g && w) src = __ffs(w) - 1;
+                    w &= w - 1;  // 0 stays 0
+                }
+                win = w;
+                const int p = __shfl_sync(FULL, node, src & 31);
+                const bool mine = src >= 0;
+                const int f = mine ? t.first[p] : 0;
+                const bool child = mine && f + o < total && t.parent[f + o] == p;
+                double v[4] = {0.0, 0.0, 0.0, 0.0};
+                if (child) {
+                    v[0] = __ldcg(t.M + f + o);
+                    const double *c = t.com + 3 * (size_t)(f + o);
+                    v[1] = v[0] * __ldcg(c);
+                    v[2] = v[0] * __ldcg(c + 1);
+                    v[3] = v[0] * __ldcg(c + 2);
+                }
+                // lanes with bit 2 keep y and z, the others M and x; then bit 1
+                const bool hi2 = lane & 4, hi1 = lane & 2;
+                const double r0 = __shfl_xor_sync(FULL, hi2 ? v[0] : v[2], 4);
+                const double r1 = __shfl_xor_sync(FULL, hi2 ? v[1] : v[3], 4);
+                const double a0 = (hi2 ? v[2] : v[0]) + r0, a1 = (hi2 ? v[3] : v[1]) + r1;
+                double s = (hi1 ? a1 : a0) + __shfl_xor_sync(FULL, hi1 ? a0 : a1, 2);
+                s += __shfl_xor_sync(FULL, s, 1);  // lane pair o >> 1: M, x, y, z
+                const double M = __shfl_sync(FULL, s, lane & 24);
+                const double cm = M > 0.0 ? s / M : 0.0;
+                const double cx = __shfl_sync(FULL, cm, (lane & 24) + 2);
+                const double cy = __shfl_sync(FULL, cm, (lane & 24) + 4);
+                const double cz = __shfl_sync(FULL, cm, (lane & 24) + 6);
+                const int nch = __popc((__ballot_sync(FULL, child) >> (lane & 24)) & 0xffu);
+                if (mine && o == 0) {
+                    put_walk_moments(t, p, M, cx, cy, cz);
+                    t.nchild[p] = nch;
+                    reinterpret_cast<int *>(t.box_lo + p)[3] = nch;  // the walk's child count
+                }
+                __syncwarp();
+            }
+            // the sums were written by other lanes of the warp: their stores
+            // are ordered before this lane's fence by the __syncwarp
+            node = won ? up : -1;
+            count = bodies;
         }
     }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) leaves += __shfl_xor_sync(0xffffffffu, leaves, off);
-    if ((threadIdx.x & 31) == 0 && leaves) atomicAdd(t.stats + 1, (unsigned long long)leaves);
+    leaves = __reduce_add_sync(FULL, leaves);
+    if (lane == 0 && leaves) atomicAdd(t.stats + 1, (unsigned long long)leaves);
 }
 
 // Squared opening distance of a level, as the oracle computes it.
@@ -347,7 +517,6 @@ __device__ __forceinline__ float cube_box_dist2(float4 lo, float4 hi, const floa
 #endif
 constexpr int FLUSH = NB_WALK_FLUSH;  // sources evaluated per flush (a multiple of 32)
 constexpr int LIST_CAP = 2 * FLUSH;
-constexpr int LEVELS = 11;
 
 template <int BPL>
 __host__ __device__ constexpr bool paired_list() { return BPL == 1 || NB_WALK_PAIRED; }
@@ -972,11 +1141,6 @@ __global__ void __launch_bounds__(TTPB) let_emit_kernel(TreeView t, const double
     }
 }
 
-__global__ void tree_flag_kernel(TreeView t, int *err)
-{
-    if (threadIdx.x == 0 && t.meta[META_OVERFLOW]) atomicOr(err, ERR_TREE);
-}
-
 }  // namespace
 
 int tree_meta_ints() { return META_INTS; }
@@ -998,23 +1162,25 @@ int64_t tree_node_bound(int64_t n, int leaf_cap)
     return total;
 }
 
-cudaError_t launch_tree_build(cudaStream_t s, const TreeView &t, int n, const unsigned *keys,
+cudaError_t launch_tree_build(cudaStream_t s, const TreeView &t, int n, const OrderScratch &o,
                               const double *box, const double *pos, const double *mass,
                               const int *perm, int leaf_cap, int *err, int &kernels)
 {
-    kernels = 0;
-    tree_init_kernel<<<1, 32, 0, s>>>(t, n, box);
-    ++kernels;
-    const int g = grid_cap(n);
-    for (int L = 0; L < 10; ++L) {
-        tree_count_kernel<<<g, TTPB, 0, s>>>(t, keys, L, leaf_cap);
-        tree_scan_kernel<<<1, 1024, 0, s>>>(t, L);
-        tree_emit_kernel<<<g, TTPB, 0, s>>>(t, keys, box, L);
-        kernels += 3;
-    }
-    tree_moments_kernel<<<grid_cap(t.cap), TTPB, 0, s>>>(t, pos, mass, perm);
-    tree_flag_kernel<<<1, 32, 0, s>>>(t, err);
-    kernels += 2;
+    // one block per 256 bodies until the blocks' table of counts, which every
+    // block sums, is as large as is cheap (26 KB)
+    const unsigned *keys = o.keys[0];
+    unsigned char *lv = reinterpret_cast<unsigned char *>(o.vals[0]);
+    int *tab = reinterpret_cast<int *>(o.hist);
+    const int tiles = (n + TTPB - 1) / TTPB;
+    const int chunk = (tiles + BUILD_BLOCKS - 1) / BUILD_BLOCKS * TTPB;
+    const int nblk = (n + chunk - 1) / chunk;
+    tree_levels_kernel<<<nblk, TTPB, 0, s>>>(t, n, keys, leaf_cap, chunk, lv, tab);
+    tree_emit_kernel<<<nblk, TTPB, 0, s>>>(t, n, keys, chunk, lv, tab, err);
+    // a thread per node, at most the blocks that are resident on 152 SMs
+    const int64_t blocks = ((int64_t)t.cap + TTPB - 1) / TTPB;
+    tree_moments_kernel<<<(int)(blocks < 1216 ? blocks : 1216), TTPB, 0, s>>>(t, box, pos, mass,
+                                                                              perm);
+    kernels = 3;
     return cudaGetLastError();
 }
 
