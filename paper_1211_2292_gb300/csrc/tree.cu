@@ -605,8 +605,8 @@ __device__ __forceinline__ int warp_span_of(int incl, int pos)
     return lo;
 }
 
-// One warp per group of 32 * BPL consecutive bodies in key order (BPL per
-// lane: bodies base + lane and base + 32 + lane).  The warp walks the tree
+// One warp (or W, below) per group of 32 * BPL consecutive bodies in key order
+// (BPL per lane: bodies base + lane and base + 32 + lane).  The warp walks the tree
 // level by level, deepest level first, 32 nodes per round (one per lane).
 // The opening test against every body of the group decides, per node,
 // between the interaction list (accepted cell: its monopole; leaf: its
@@ -617,19 +617,33 @@ __device__ __forceinline__ int warp_span_of(int incl, int pos)
 // body.  Each level's stack holds at most 32 ranges, the children of one
 // round's nodes, since a level is refilled only once every deeper level is
 // empty.  Whenever FLUSH sources are listed, every lane adds them to its bodies.
-template <int BPL, bool MULTI>
+//
+// W > 1: W warps walk one group together, level by level: the nodes of a level
+// (the shared frontier) are dealt to the warps round robin, each warp appends
+// the children it opens to its own segment of the next frontier (one that is
+// full leaves the rest to its warp's own stacks, which are emptied before the
+// next nodes are dealt), and the block meets once per level.  Who tests what
+// depends on the tree only, so each warp's sums, and their total in warp
+// order, do not depend on timing.
+constexpr int FRONT_CAP = 2048;  // nodes of a frontier, over its segments
+constexpr int walk_warps(int W) { return W > 1 ? W : WALK_WARPS; }  // per block
+
+template <int BPL, bool MULTI, int W>
 struct WalkShared {
-    float4 list[WALK_WARPS][list_f4<BPL>()];  // float4 slots of the lists
-    int2 ranges[WALK_WARPS][LEVELS][32];
-    int lslot[MULTI ? 1 : WALK_WARPS][32];  // a chunk's leaf starts: body index minus position
+    float4 list[walk_warps(W)][list_f4<BPL>()];  // float4 slots of the lists
+    int2 ranges[walk_warps(W)][LEVELS][32];
+    int lslot[MULTI ? 1 : walk_warps(W)][32];  // a chunk's leaf starts: body index minus position
     float crit2[MULTI ? 1 + WALK_MAX_MORE : 1][LEVELS];  // per walked tree
+    int front[W > 1 ? 2 : 1][W > 1 ? W : 1][W > 1 ? FRONT_CAP / W : 1];
+    int seg[2][walk_warps(W)];  // nodes per segment; cells and bodies listed per warp at the end
+    int task;
 };
 
 // The walk of group g (bodies [g * 32 * BPL, ...) in key order) by one warp:
 // over the one tree (tq_only = -1), or (MULTI) over span tq_only of the trees
 // in p.more, the group's last span then writing the sums of all of them.
-template <bool ZEPS, int BPL, bool MULTI>
-__device__ __forceinline__ void walk_group(const TreeWalkParams &p, WalkShared<BPL, MULTI> &sh,
+template <bool ZEPS, int BPL, bool MULTI, int W>
+__device__ __forceinline__ void walk_group(const TreeWalkParams &p, WalkShared<BPL, MULTI, W> &sh,
                                            int g, int tq_only)
 {
     constexpr int GROUP = 32 * BPL;
@@ -770,13 +784,49 @@ __device__ __forceinline__ void walk_group(const TreeWalkParams &p, WalkShared<B
         __syncwarp();
     };
 
-    int lsize = lane == 0 ? 1 : 0;  // lane L holds the size of level L's stack
-    if (lane == 0) rs[0][0] = make_int2(0, 1);
-    __syncwarp();
+    int lsize = 0;  // lane L holds the size of level L's stack
+    // the frontier: ftot nodes of level fl, at first the root; its next round;
+    // the children this warp appended to the next one
+    int fl = 0, ftot = 1, fr = 0, cur = 0, found = 0;
+    if (W > 1) {
+        if (threadIdx.x < W) sh.seg[0][threadIdx.x] = threadIdx.x == 0;
+        if (threadIdx.x == 0) sh.front[0][0][0] = 0;
+        __syncthreads();
+    }
     for (;;) {
+        int node = -1, Lv = fl;
         const unsigned nonempty = __ballot_sync(FULL, lane < LEVELS && lsize > 0);
-        if (!nonempty) break;
-        const int Lv = 31 - __clz(nonempty);
+        const bool shared_round = W > 1 && !nonempty;
+        if (shared_round) {
+            if (32 * W * fr >= ftot) {  // every warp is done with the level
+                if (lane == 0) sh.seg[cur ^ 1][warp] = found;
+                __syncthreads();
+                cur ^= 1;
+                found = fr = ftot = 0;
+#pragma unroll
+                for (int w = 0; w < W; ++w) ftot += sh.seg[cur][w];
+                if (ftot == 0) break;
+                Lv = ++fl;
+            }
+            int at = 32 * W * fr + W * lane + warp, w = 0;
+            ++fr;
+            if (at < ftot) {
+#pragma unroll
+                for (int q = 0; q < W - 1; ++q) {
+                    const int c = sh.seg[cur][q];
+                    if (w == q && at >= c) {
+                        at -= c;
+                        ++w;
+                    }
+                }
+                node = sh.front[cur][w][at];
+            }
+        } else if (!nonempty) {
+            if (fr > 0) break;
+            if (lane == 0) node = 0;
+            ++fr;
+        } else {
+        Lv = 31 - __clz(nonempty);
         const int size = __shfl_sync(FULL, lsize, Lv);
         // take up to 32 nodes from the top ranges of level Lv
         const int R = min(size, 32);
@@ -789,12 +839,13 @@ __device__ __forceinline__ void walk_group(const TreeWalkParams &p, WalkShared<B
         const unsigned starts = __reduce_or_sync(FULL, lane < R && excl < 32 ? 1u << excl : 0u);
         const int src = __popc(starts & (0xffffffffu >> (31 - lane))) - 1;
         const int first_src = __shfl_sync(FULL, r.x, src), excl_src = __shfl_sync(FULL, excl, src);
-        const int node = lane < take ? first_src + (lane - excl_src) : -1;
+        node = lane < take ? first_src + (lane - excl_src) : -1;
         const unsigned done = __ballot_sync(FULL, lane < R && incl <= 32);
         if (lane < R && excl < 32 && incl > 32)
             rs[Lv][size - 1 - lane] = make_int2(r.x + (32 - excl), incl - 32);
         if (lane == Lv) lsize -= __popc(done);
         __syncwarp();
+        }
 
         // opening test
         const bool has = node >= 0;
@@ -830,12 +881,26 @@ __device__ __forceinline__ void walk_group(const TreeWalkParams &p, WalkShared<B
         const bool open = has && !accept && nch > 0;
         const bool leaf = has && !accept && nch == 0;
 
-        // children ranges onto the next level (Lv < 10 whenever a node opens)
-        const unsigned om = __ballot_sync(FULL, open);
+        // children: of a shared node onto the next frontier while this warp's
+        // segment has room
+        bool own = open;
+        if (shared_round) {
+            const int c = open ? nch : 0;
+            const int incl = warp_incl_scan(c, lane);
+            const int at = found + incl - c;
+            own = open && at + c > FRONT_CAP / W;  // then the later lanes' do not fit either
+            if (!own)
+                for (int q = 0; q < c; ++q) sh.front[cur ^ 1][warp][at + q] = __float_as_int(bhi.w) + q;
+            const unsigned full = __ballot_sync(FULL, own);
+            found = full ? __shfl_sync(FULL, at, __ffs(full) - 1)
+                         : found + __shfl_sync(FULL, incl, 31);
+        }
+        // else their ranges onto the next level (Lv < 10 whenever a node opens)
+        const unsigned om = __ballot_sync(FULL, own);
         if (om) {
             const int size1 = __shfl_sync(FULL, lsize, Lv + 1);
             const int slot1 = size1 + __popc(om & lt);
-            if (open && slot1 < 32) rs[Lv + 1][slot1] = make_int2(__float_as_int(bhi.w), nch);
+            if (own && slot1 < 32) rs[Lv + 1][slot1] = make_int2(__float_as_int(bhi.w), nch);
             if (lane == Lv + 1) lsize = min(size1 + __popc(om), 32);
             if (lane == 0 && size1 + __popc(om) > 32) atomicOr(p.err, ERR_TREE);  // never: see above
         }
@@ -916,6 +981,33 @@ __device__ __forceinline__ void walk_group(const TreeWalkParams &p, WalkShared<B
     }
     }  // trees
     bool stats_done = false;
+    if (W > 1) {  // the warps' sums and counts, added in warp order by the first
+        __syncthreads();  // every warp has read the last level's segments
+        double *mine = reinterpret_cast<double *>(list_s[warp]);
+        static_assert(sizeof(float4) * LIST_F4 >= sizeof(double) * 3 * GROUP, "sums fit the list");
+#pragma unroll
+        for (int b = 0; b < BPL; ++b)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) mine[(3 * b + c) * 32 + lane] = tg[b][c];
+        if (lane == 0) {
+            sh.seg[0][warp] = nc;
+            sh.seg[1][warp] = nb;
+        }
+        __syncthreads();
+        if (warp == 0) {
+            for (int w = 1; w < W; ++w) {
+                const double *o = reinterpret_cast<const double *>(list_s[w]);
+#pragma unroll
+                for (int b = 0; b < BPL; ++b)
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) tg[b][c] += o[(3 * b + c) * 32 + lane];
+                nc += sh.seg[0][w];
+                nb += sh.seg[1][w];
+            }
+        }
+        __syncthreads();
+        if (warp != 0) return;
+    }
     if (MULTI && tq_only >= 0) {
         // this task's sums and counts; the group's last task adds all tasks'
         // in tree order (with one tree per task, as the walk over every tree
@@ -1000,41 +1092,53 @@ __device__ __forceinline__ void walk_group(const TreeWalkParams &p, WalkShared<B
 // grid covering all groups; dynamic, a grid of resident warps taking `chunk`
 // groups at a time from an atomic counter; guided, the same with chunks of
 // max(chunk, remaining / (2 x warps)).
-template <bool ZEPS, int BPL, bool MULTI>
-__global__ void __launch_bounds__(32 * WALK_WARPS, BPL == 1 ? NB_WALK_MINB1 : NB_WALK_MINB2)
+// (In units of blocks and groups when a block's W warps walk one group.)
+template <bool ZEPS, int BPL, bool MULTI, int W>
+__global__ void __launch_bounds__(32 * walk_warps(W),
+                                  BPL == 1 ? NB_WALK_MINB1 * WALK_WARPS / walk_warps(W)
+                                           : NB_WALK_MINB2 * WALK_WARPS / walk_warps(W))
     tree_walk_kernel(const TreeWalkParams p)
 {
-    __shared__ WalkShared<BPL, MULTI> sh;
+    extern __shared__ __align__(16) unsigned char walk_smem[];
+    WalkShared<BPL, MULTI, W> &sh = *reinterpret_cast<WalkShared<BPL, MULTI, W> *>(walk_smem);
     for (int q = threadIdx.x; q < (MULTI ? 1 + p.nmore : 1) * LEVELS; q += blockDim.x) {
         const int tq = q / LEVELS, L = q % LEVELS;
         sh.crit2[tq][L] = open_dist2(MULTI ? p.more[tq].box[3] : p.box[3], L, p.theta);
     }
     __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int gw = blockIdx.x * WALK_WARPS + warp;
+    // workers: the warps, or the blocks
+    const int gw = W > 1 ? blockIdx.x : blockIdx.x * WALK_WARPS + warp;
     const int ngroups = (p.n + 32 * BPL - 1) / (32 * BPL);
     // tasks: the groups, or with further trees (split mode) the (group,
     // tree) pairs, tree-major
     const int ntasks = MULTI ? ngroups * ((1 + p.nmore + p.tspan - 1) / p.tspan) : ngroups;
     auto task = [&](int t) {
         if constexpr (MULTI)
-            walk_group<ZEPS, BPL, MULTI>(p, sh, t % ngroups, t / ngroups);
+            walk_group<ZEPS, BPL, MULTI, W>(p, sh, t % ngroups, t / ngroups);
         else
-            walk_group<ZEPS, BPL, MULTI>(p, sh, t, -1);
+            walk_group<ZEPS, BPL, MULTI, W>(p, sh, t, -1);
     };
     if (p.sched == 0) {
         if (gw < ntasks) task(gw);
         return;
     }
-    const int nwarps = gridDim.x * WALK_WARPS;
+    const int nworkers = W > 1 ? gridDim.x : gridDim.x * WALK_WARPS;
     int *queue = p.queue;
     int seen = 0;
     for (;;) {
         int c = p.chunk;
-        if (p.sched == 2) c = max(c, (ntasks - seen) / (2 * nwarps));
+        if (p.sched == 2) c = max(c, (ntasks - seen) / (2 * nworkers));
         int g0 = 0;
-        if (lane == 0) g0 = atomicAdd(queue, c);
-        g0 = __shfl_sync(0xffffffffu, g0, 0);
+        if (W > 1) {
+            if (threadIdx.x == 0) sh.task = atomicAdd(queue, c);
+            __syncthreads();
+            g0 = sh.task;
+            __syncthreads();
+        } else {
+            if (lane == 0) g0 = atomicAdd(queue, c);
+            g0 = __shfl_sync(0xffffffffu, g0, 0);
+        }
         if (g0 >= ntasks) break;
         seen = g0 + c;
         const int g1 = min(g0 + c, ntasks);
@@ -1208,33 +1312,78 @@ cudaError_t launch_let_emit(cudaStream_t s, const TreeView &t, const double *box
     return cudaGetLastError();
 }
 
+namespace {
+
+// Warps that walk one group together.  One warp per group is the most work per
+// instruction, but a launch then lasts as long as its slowest groups' walks,
+// and below a few groups per resident warp SMs idle.  Measured (walk alone, us,
+// Plummer spheres, theta 0.5, leaves of 16; 1 / 4 / 8 warps per group):
+//   groups of 64: 2000 bodies 108 / 58 / 39, 20000 389 / 163 / 101,
+//     60000 516 / 314 / 280, 100000 627 / 442 / 463, 200000 893 / 774 / 870,
+//     400000 1496 / 1497 / 1737, 800000 2746 / 3003 / 3570;
+//   groups of 32: 20000 318 / 146 / 112, 60000 430 / 313 / 306,
+//     100000 538 / 527 / 513, 200000 870 / 971 / 991.
+// (2 warps per group were slower than 4 up to 400000 bodies, 16 than 8 from
+// 20000 on.)  So 8 warps up to 8 groups per SM (20 of the smaller ones), 4 up
+// to 40, then one.
+int walk_split(int groups, int bodies_per_lane, int num_sms)
+{
+    if (bodies_per_lane == 1) return groups < 20 * num_sms ? 8 : 1;
+    return groups < 8 * num_sms ? 8 : (groups < 40 * num_sms ? 4 : 1);
+}
+
+template <int BPL, bool MULTI, int W>
+cudaError_t walk_launch(cudaStream_t s, const TreeWalkParams &p, bool zeps, int tasks, int &kernels)
+{
+    void (*fn)(const TreeWalkParams) = zeps ? tree_walk_kernel<true, BPL, MULTI, W>
+                                            : tree_walk_kernel<false, BPL, MULTI, W>;
+    constexpr int threads = 32 * walk_warps(W);
+    constexpr int smem = (int)sizeof(WalkShared<BPL, MULTI, W>);
+    if (smem > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+    }
+    int blocks = W > 1 ? tasks : (tasks + WALK_WARPS - 1) / WALK_WARPS;
+    if (p.sched != 0) {  // resident blocks only
+        int per_sm = 0;
+        const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem);
+        if (e != cudaSuccess) return e;
+        blocks = min(blocks, max(per_sm, 1) * p.num_sms);
+    }
+    fn<<<blocks, threads, smem, s>>>(p);
+    kernels = 1;
+    return cudaGetLastError();
+}
+
+template <int BPL, bool MULTI>
+cudaError_t walk_launch_split(cudaStream_t s, const TreeWalkParams &p, bool zeps, int W, int tasks,
+                              int &kernels)
+{
+    if (W == 8) return walk_launch<BPL, MULTI, 8>(s, p, zeps, tasks, kernels);
+    if constexpr (BPL == 2)
+        if (W == 4) return walk_launch<BPL, MULTI, 4>(s, p, zeps, tasks, kernels);
+    return walk_launch<BPL, MULTI, 1>(s, p, zeps, tasks, kernels);
+}
+
+}  // namespace
+
 cudaError_t launch_tree_walk(cudaStream_t s, const TreeWalkParams &p, bool zeps, int &kernels)
 {
     kernels = 0;
     if (p.n <= 0) return cudaSuccess;
-    const int G = p.group;
     if (p.nmore > 0 && (!p.tpart || !p.tcnt || !p.tctr || p.tspan < 1))
         return cudaErrorInvalidValue;
-    const int groups =  // tasks
-        (p.n + G - 1) / G * (p.nmore > 0 ? (1 + p.nmore + p.tspan - 1) / p.tspan : 1);
-    // (a separate instance walks further trees: the single-tree walk keeps
-    // its own registers and shared memory)
-    void (*fn)(const TreeWalkParams) =
-        p.nmore > 0
-            ? (G == 32 ? (zeps ? tree_walk_kernel<true, 1, true> : tree_walk_kernel<false, 1, true>)
-                       : (zeps ? tree_walk_kernel<true, 2, true> : tree_walk_kernel<false, 2, true>))
-            : (G == 32 ? (zeps ? tree_walk_kernel<true, 1, false> : tree_walk_kernel<false, 1, false>)
-                       : (zeps ? tree_walk_kernel<true, 2, false> : tree_walk_kernel<false, 2, false>));
-    int blocks = (groups + WALK_WARPS - 1) / WALK_WARPS;
-    if (p.sched != 0) {  // resident blocks only
-        int per_sm = 0;
-        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 32 * WALK_WARPS, 0);
-        if (e != cudaSuccess) return e;
-        blocks = min(blocks, max(per_sm, 1) * p.num_sms);
-    }
-    fn<<<blocks, 32 * WALK_WARPS, 0, s>>>(p);
-    kernels = 1;
-    return cudaGetLastError();
+    const int bpl = p.group / 32;
+    const int groups = (p.n + p.group - 1) / p.group;
+    const int tasks = groups * (p.nmore > 0 ? (1 + p.nmore + p.tspan - 1) / p.tspan : 1);
+    // by the groups alone, so that a tree's sums are the same whether further
+    // trees are walked or not (a task of several trees is one warp's)
+    const int W = p.nmore > 0 && p.tspan > 1 ? 1 : walk_split(groups, bpl, p.num_sms);
+    if (p.nmore > 0)  // a separate instance: the single-tree walk keeps its own registers
+        return bpl == 1 ? walk_launch_split<1, true>(s, p, zeps, W, tasks, kernels)
+                        : walk_launch_split<2, true>(s, p, zeps, W, tasks, kernels);
+    return bpl == 1 ? walk_launch_split<1, false>(s, p, zeps, W, tasks, kernels)
+                    : walk_launch_split<2, false>(s, p, zeps, W, tasks, kernels);
 }
 
 }  // namespace nb
