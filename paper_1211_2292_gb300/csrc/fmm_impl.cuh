@@ -55,6 +55,8 @@ constexpr unsigned FULL = 0xffffffffu;
 constexpr int LEVELS = 11;
 constexpr int WARPS = 4;  // warps per block of the downward and near-field kernels
 constexpr int FLUSH = 256;  // directly summed sources per flush (128 pairs)
+constexpr int LIST_ROUNDS = 2;  // rounds of 32 sources listed at a time
+static_assert(32 * LIST_ROUNDS <= FLUSH, "new sources stay out of the half being evaluated");
 
 // ------------------------------------------------------------ multi-indices
 // Slots in graded order: orders below k first, then a descending, b descending.
@@ -278,13 +280,44 @@ __device__ __forceinline__ void store_exp(float *dst, const float (&v)[nterms(P)
     });
 }
 
+template <int P>
+__device__ __forceinline__ void load_exp(float (&v)[nterms(P)], const float *src)
+{
+    constexpr int N = nterms(P), NP = padded(P);
+    const float4 *s4 = reinterpret_cast<const float4 *>(src);
+    sfor<0, NP / 4>([&](auto iI) {
+        constexpr int i = decltype(iI)::value;
+        const float4 e = s4[i];
+        const float x[4] = {e.x, e.y, e.z, e.w};
+        sfor<0, 4>([&](auto jI) {
+            constexpr int j = decltype(jI)::value;
+            if constexpr (4 * i + j < N) v[4 * i + j] = x[j];
+        });
+    });
+}
+
 // ------------------------------------------------------------ upward pass
 // P2M: a thread per leaf forms its moments from its bodies (the next body's
-// position loaded while this one's monomials are added).  M2M: one launch
-// per level from the deepest up, a warp per cell with children: a child per
-// lane translates the child's moments, and the lanes' terms are totalled in
-// a fixed order.
+// position loaded while this one's monomials are added).  The scaled offsets
+// come from the packed hi/lo pairs in double-float arithmetic: ten float64
+// operations per body held the launch to the float64 pipe (76 us at 2^20
+// bodies).  M2M: one launch
+// per level from the deepest up, eight lanes per cell with children: a child
+// per lane translates the child's moments, and the lanes' terms are totalled
+// in a fixed order.
 constexpr int UP_WARPS = 4;
+
+// ((zh + zl) - (xh + xl)) (ih + il), rounded once (to within a few 2^-45 before
+// the last rounding): the difference of the high parts with its exact error
+// (two-sum), the rest in float32.
+__device__ __forceinline__ float scaled_offset(float zh, float zl, float xh, float xl, float ih,
+                                               float il)
+{
+    const float d = zh - xh;
+    const float b = d - zh;
+    const float e = (zh - (d - b)) - (xh + b) + (zl - xl);
+    return fmaf(d, ih, fmaf(d, il, e * ih));
+}
 
 template <int P>
 __global__ void __launch_bounds__(32 * UP_WARPS) fmm_p2m_kernel(const FmmParams p)
@@ -304,29 +337,31 @@ __global__ void __launch_bounds__(32 * UP_WARPS) fmm_p2m_kernel(const FmmParams 
         f.nd[leaf] = make_int4(0, t.first[leaf], k0, k1);
         double z[3];
         centre_of(p.box, ci, z);
+        float zh[3], zl[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            zh[c] = (float)z[c];
+            zl[c] = (float)(z[c] - (double)zh[c]);
+        }
         const double inv_e = (double)(1 << L) / ext;
+        const float ih = (float)inv_e, il = (float)(inv_e - (double)ih);
         float Mc[N];
 #pragma unroll
         for (int q = 0; q < N; ++q) Mc[q] = 0.0f;
-        double x[3] = {0.0, 0.0, 0.0}, mj = 0.0;
+        float4 h = make_float4(0.f, 0.f, 0.f, 0.f), l = h;
         if (k0 < k1) {
-            const int j = p.perm[k0];
-            x[0] = p.pos[3 * (size_t)j];
-            x[1] = p.pos[3 * (size_t)j + 1];
-            x[2] = p.pos[3 * (size_t)j + 2];
-            mj = p.mass[j];
+            h = __ldg(p.P + k0);
+            l = __ldg(p.Plo + k0);
         }
         for (int k = k0; k < k1; ++k) {
-            const float m = (float)mj;
+            const float m = h.w;
+            const float hx[3] = {h.x, h.y, h.z}, lx[3] = {l.x, l.y, l.z};
             float pw[3][P + 1];
 #pragma unroll
-            for (int c = 0; c < 3; ++c) scaled_powers<P>((float)((z[c] - x[c]) * inv_e), pw[c]);
+            for (int c = 0; c < 3; ++c) scaled_powers<P>(scaled_offset(zh[c], zl[c], hx[c], lx[c], ih, il), pw[c]);
             if (k + 1 < k1) {
-                const int j = p.perm[k + 1];
-                x[0] = p.pos[3 * (size_t)j];
-                x[1] = p.pos[3 * (size_t)j + 1];
-                x[2] = p.pos[3 * (size_t)j + 2];
-                mj = p.mass[j];
+                h = __ldg(p.P + k + 1);
+                l = __ldg(p.Plo + k + 1);
             }
             sfor<0, N>([&](auto qI) {
                 constexpr int q = decltype(qI)::value;
@@ -343,29 +378,30 @@ __global__ void __launch_bounds__(32 * UP_WARPS) fmm_m2m_kernel(const FmmParams 
     constexpr int N = nterms(P), NP = padded(P);
     const TreeView &t = p.tree;
     const FmmView &f = p.f;
-    const int lane = threadIdx.x & 31;
+    const int o = threadIdx.x & 7;
     const int cnt = t.meta[TREE_META_COUNT + L], base = t.meta[TREE_META_BASE + L];
-    for (int q0 = blockIdx.x * UP_WARPS + (threadIdx.x >> 5); q0 < cnt; q0 += gridDim.x * UP_WARPS) {
+    // eight lanes per cell, whole warps in step for the shuffles
+    const int step = gridDim.x * UP_WARPS * 4;
+    for (int w0 = (blockIdx.x * UP_WARPS + (threadIdx.x >> 5)) * 4; w0 < cnt; w0 += step) {
+        const int q0 = w0 + ((threadIdx.x & 31) >> 3);
         const int node = base + q0;
-        const int nch = t.nchild[node];
-        if (nch == 0) continue;
-        const int c0 = t.first[node];
+        const int nch = q0 < cnt ? t.nchild[node] : 0;
+        if (!__any_sync(FULL, nch > 0)) continue;
+        const int c0 = nch > 0 ? t.first[node] : 0;
         float Mc[N];
 #pragma unroll
         for (int q = 0; q < N; ++q) Mc[q] = 0.0f;
-        if (lane < nch) {
+        if (o < nch) {
             float xc[N];
-            const float *src = f.M + (size_t)(c0 + lane) * NP;
-#pragma unroll
-            for (int q = 0; q < N; ++q) xc[q] = src[q];
-            translate_add<P, true>(Mc, xc, (int)(t.prefix[c0 + lane] & 7u));
+            load_exp<P>(xc, f.M + (size_t)(c0 + o) * NP);
+            translate_add<P, true>(Mc, xc, (int)(t.prefix[c0 + o] & 7u));
         }
 #pragma unroll
         for (int q = 0; q < N; ++q) {
 #pragma unroll
-            for (int o = 4; o > 0; o >>= 1) Mc[q] += __shfl_down_sync(FULL, Mc[q], o);
+            for (int off = 4; off > 0; off >>= 1) Mc[q] += __shfl_down_sync(FULL, Mc[q], off, 8);
         }
-        if (lane == 0) {
+        if (o == 0 && nch > 0) {
             f.ci[node] = icentre(t.prefix[node], L);
             f.nd[node] = make_int4(nch, c0, t.start[node], t.end[node]);
             store_exp<P>(f.M + (size_t)node * NP, Mc);
@@ -376,10 +412,10 @@ __global__ void __launch_bounds__(32 * UP_WARPS) fmm_m2m_kernel(const FmmParams 
 // ------------------------------------------------------------ the walks
 // Per warp: stacks of child ranges per level (each holds at most 32 ranges:
 // a level is refilled only from the level above once every deeper level is
-// empty, or from the handed-down list once all are empty).
+// empty, or from the handed-down list once all are empty).  Lane L holds the
+// size of level L's stack.
 struct WalkSh {
     int2 rs[LEVELS][32];
-    int lsz[LEVELS];
 };
 
 __device__ __forceinline__ int warp_incl_scan(int v, int lane)
@@ -412,58 +448,64 @@ __device__ __forceinline__ int warp_sum(int v)
 }
 
 // Next round of up to 32 candidates (one per lane, -1 for none) of a leaf
-// target's walk: from the deepest non-empty level stack, else the next 32
-// handed-down candidates.  False when the walk is over.
-__device__ __forceinline__ bool next_round(WalkSh &w, const int *inh, int ninh, int &cursor,
-                                           int lane, int &node)
+// target's walk: from the deepest non-empty level stack (Lv then is that
+// level), else the next 32 handed-down candidates (of any level: Lv = -1).
+// False when the walk is over.
+__device__ __forceinline__ bool next_round(WalkSh &w, int &lsize, const int *inh, int ninh,
+                                           int &cursor, int lane, int &node, int &Lv)
 {
-    const int sz = lane < LEVELS ? w.lsz[lane] : 0;
-    const unsigned nonempty = __ballot_sync(FULL, sz > 0);
+    const unsigned nonempty = __ballot_sync(FULL, lane < LEVELS && lsize > 0);
     if (!nonempty) {
         if (cursor >= ninh) return false;
         const int k = cursor + lane;
         node = k < ninh ? __ldg(inh + k) : -1;
         cursor += 32;
+        Lv = -1;
         return true;
     }
-    const int Lv = 31 - __clz(nonempty);
-    const int size = __shfl_sync(FULL, sz, Lv);
+    Lv = 31 - __clz(nonempty);
+    const int size = __shfl_sync(FULL, lsize, Lv);
     const int R = min(size, 32);
     const int2 r = lane < R ? w.rs[Lv][size - 1 - lane] : make_int2(0, 0);
     const int incl = warp_incl_scan(r.y, lane);
     const int excl = incl - r.y;
     const int take = min(__shfl_sync(FULL, incl, 31), 32);
-    const int src = warp_span_of(incl, lane) & 31;
+    // the range holding this lane's node: the last one starting at or before
+    // it (ranges 0..R-1 are non-empty, so their starts increase)
+    const unsigned starts = __reduce_or_sync(FULL, lane < R && excl < 32 ? 1u << excl : 0u);
+    const int src = __popc(starts & (0xffffffffu >> (31 - lane))) - 1;
     const int first_src = __shfl_sync(FULL, r.x, src), excl_src = __shfl_sync(FULL, excl, src);
     node = lane < take ? first_src + (lane - excl_src) : -1;
     const unsigned done = __ballot_sync(FULL, lane < R && incl <= 32);
-    __syncwarp();
     if (lane < R && excl < 32 && incl > 32)
         w.rs[Lv][size - 1 - lane] = make_int2(r.x + (32 - excl), incl - 32);
-    if (lane == 0) w.lsz[Lv] = size - __popc(done);
+    if (lane == Lv) lsize -= __popc(done);
     __syncwarp();
     return true;
 }
 
 // Push the child range (first, nch) of every opening lane onto the stack of
-// its node's level + 1.
-__device__ __forceinline__ void push_children(WalkSh &w, bool open, int tgt, int first, int nch,
-                                              int lane, int *err)
+// its node's level + 1 (tgt).
+__device__ __forceinline__ void push_children(WalkSh &w, int &lsize, bool open, int tgt, int first,
+                                              int nch, int lane, int *err)
 {
-    if (!__ballot_sync(FULL, open)) return;
+    unsigned om = __ballot_sync(FULL, open);
     const unsigned lt = (1u << lane) - 1u;
-    const unsigned grp = __match_any_sync(FULL, open ? tgt : -1);
-    int slot = 0;
-    if (open) slot = w.lsz[tgt] + __popc(grp & lt);
-    __syncwarp();
-    if (open) {
-        if (slot < 32)
-            w.rs[tgt][slot] = make_int2(first, nch);
-        else
-            atomicOr(err, ERR_TREE);  // never: at most 32 pushes onto an empty level
+    while (om) {  // once per level among the opening lanes
+        const int lv = __shfl_sync(FULL, tgt, __ffs(om) - 1);
+        const bool mine = open && tgt == lv;
+        const unsigned grp = __ballot_sync(FULL, mine);
+        const int size = __shfl_sync(FULL, lsize, lv);
+        const int slot = size + __popc(grp & lt);
+        if (mine) {
+            if (slot < 32)
+                w.rs[lv][slot] = make_int2(first, nch);
+            else
+                atomicOr(err, ERR_TREE);  // never: at most 32 pushes onto an empty level
+        }
+        if (lane == lv) lsize = min(size + __popc(grp), 32);
+        om &= ~grp;
     }
-    __syncwarp();
-    if (open && (grp & lt) == 0) w.lsz[tgt] = min(w.lsz[tgt] + __popc(grp), 32);
     __syncwarp();
 }
 
@@ -599,23 +641,162 @@ __device__ __forceinline__ void flush_chunk(T *q, int &qcnt, int k, T pad, T *st
 }
 
 // ------------------------------------------------------------ downward pass
-// Three parts.  (1) Per level L, a warp per cell (dynamic) classifies the
-// candidates its parent handed down: a non-leaf hands the unseparated ones
-// (or their children) to its own children, a leaf walks their subtrees; the
-// separated cells go into the cell's expansion list, in chunks of 32 source
-// ids (one per lane of the later evaluation, -1 past the end) linked from
-// chunk_head.  (2) One launch over all cells sums each cell's list (M2L, a
-// source per lane, the lanes' sums totalled in a fixed order) into L.
-// (3) Per level from the top, L2L adds the parent's translated
-// coefficients.  The chunks hold the sources in the order the
+// Three parts.  (1) Per level L, a block per non-leaf cell (dynamic) classifies
+// the candidates its parent handed down and hands the unseparated ones (or
+// their children) to the cell's own children; then a warp per leaf walks its
+// candidates' subtrees.  The separated cells go into the cell's expansion
+// list, in chunks of 32 source ids (one per lane of the later evaluation, -1
+// past the end) linked from chunk_head.  (2) One launch over all cells sums
+// each cell's list (M2L, a source per lane, the lanes' sums totalled in a
+// fixed order) into L.  (3) Per level from the top, L2L adds the parent's
+// translated coefficients.  The chunks hold the sources in the order the
 // classification meets them and each goes to the lane of its position, so
 // every lane's sum, and the result, does not depend on scheduling.
-template <int P, bool LEAVES>
-__global__ void __launch_bounds__(32 * WARPS) fmm_lists_kernel(const FmmParams p, int L)
+
+// The non-leaf cells of level L.  A cell's list may hold a thousand candidates
+// where a level has a handful of cells, so what bounds these launches is the
+// rounds of dependent loads: the block's warps take a segment of the list
+// each, once to count, once to write in list order (a warp per cell took 35 to
+// 53 us per level where 8 warps take 10, 260 us for the levels of a 2^20-body
+// tree).
+constexpr int DOWN_WARPS = 8;
+template <int P>
+__global__ void __launch_bounds__(32 * DOWN_WARPS) fmm_down_kernel(const FmmParams p, int L)
+{
+    __shared__ CritSh crit;
+    __shared__ int wout[DOWN_WARPS], wsep[DOWN_WARPS], wfar[DOWN_WARPS];
+    __shared__ int cell_s, off_s, ch_s;  // off_s, ch_s: -1 when the store is full
+    crit_table(crit, p.f.crit);
+    const TreeView &t = p.tree;
+    const FmmView &f = p.f;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    const int cnt = t.meta[TREE_META_COUNT + L], base = t.meta[TREE_META_BASE + L];
+    for (;;) {
+        __syncthreads();  // the table is there; the last cell's shared words are free
+        if (threadIdx.x == 0) cell_s = atomicAdd(f.meta + FMM_META_LEVEL + L, 1);
+        __syncthreads();
+        if (cell_s >= cnt) break;
+        const int A = base + cell_s;
+        if (t.nchild[A] == 0) continue;
+        const int4 cA = f.ci[A];
+        const int par = t.parent[A];
+        const int2 d = par >= 0 ? f.down[par] : make_int2(0, 1);  // the root's list: pool[0] = 0
+        const int *inh = f.pool + d.x;
+        const int per = ((d.y + DOWN_WARPS - 1) / DOWN_WARPS + 31) & ~31;
+        const int k0 = min(d.y, warp * per), k1 = min(d.y, k0 + per);
+        // the candidate's fate: separated, or how many cells go down for it
+        auto classify = [&](int B, bool &sep, bool &self, int &outc, int &first, int &bodies) {
+            sep = self = false;
+            outc = first = bodies = 0;
+            if (B < 0) return;
+            const int4 cB = __ldg(f.ci + B), nB = __ldg(f.nd + B);
+            sep = separated(cA, cB, crit);
+            bodies = nB.w - nB.z;
+            if (sep) return;
+            self = nB.x == 0 || cB.w > cA.w;
+            outc = self ? 1 : nB.x;
+            first = nB.y;
+            if (!self && cB.w < cA.w) atomicOr(p.err, ERR_TREE);  // never
+        };
+        bool sep, self;
+        int outc, first, bodies, nout = 0, nsep = 0, far = 0;
+#pragma unroll 2
+        for (int k = k0; k < k1; k += 32) {
+            classify(k + lane < k1 ? __ldg(inh + k + lane) : -1, sep, self, outc, first, bodies);
+            nout += outc;
+            nsep += sep;
+            if (sep) far += bodies;
+        }
+        nout = __reduce_add_sync(FULL, nout);
+        nsep = __reduce_add_sync(FULL, nsep);
+        far = __reduce_add_sync(FULL, far);
+        if (lane == 0) {
+            wout[warp] = nout;
+            wsep[warp] = nsep;
+            wfar[warp] = far;
+        }
+        __syncthreads();
+        int out0 = 0, sep0 = 0, outs = 0, seps = 0;  // before this warp, in all
+#pragma unroll
+        for (int w = 0; w < DOWN_WARPS; ++w) {
+            if (w == warp) {
+                out0 = outs;
+                sep0 = seps;
+            }
+            outs += wout[w];
+            seps += wsep[w];
+        }
+        const int nch = (seps + 31) >> 5;
+        if (threadIdx.x == 0) {
+            const long long off = (unsigned)atomicAdd(f.meta + FMM_META_POOL, outs);
+            const bool fits = off + outs <= f.pool_cap;
+            f.down[A] = make_int2(fits ? (int)off : 0, fits ? outs : 0);
+            off_s = fits ? (int)off : -1;
+            const long long ch = nch ? (unsigned)atomicAdd(f.meta + FMM_META_CHUNKS, nch) : 0;
+            const bool room = nch > 0 && ch + nch <= f.chunk_cap;
+            f.chunk_head[A] = room ? (int)ch : -1;
+            ch_s = room ? (int)ch : -1;
+            if (!fits || (nch > 0 && !room))
+                atomicOr(f.meta + FMM_META_OVERFLOW, (fits ? 0 : 1) | (nch > 0 && !room ? 2 : 0));
+            int2 cum = par >= 0 ? f.cum[par] : make_int2(0, 0);
+            cum.x += seps;
+#pragma unroll
+            for (int w = 0; w < DOWN_WARPS; ++w) cum.y += wfar[w];
+            f.cum[A] = cum;
+            if (seps) atomicAdd(f.stats + 2, (unsigned long long)seps);
+        }
+        __syncthreads();
+        const int off = off_s, ch = ch_s;
+#pragma unroll 2
+        for (int k = k0; k < k1; k += 32) {
+            const int B = k + lane < k1 ? __ldg(inh + k + lane) : -1;
+            classify(B, sep, self, outc, first, bodies);
+            const int incl = warp_incl_scan(outc, lane);
+            if (off >= 0 && outc) {
+                int *dst = f.pool + off + out0 + (incl - outc);
+                if (self)
+                    dst[0] = B;
+                else
+                    for (int j = 0; j < outc; ++j) dst[j] = first + j;
+            }
+            out0 += __shfl_sync(FULL, incl, 31);
+            const unsigned sm = __ballot_sync(FULL, sep);
+            if (sep && ch >= 0) f.chunk_src[32 * (size_t)ch + sep0 + __popc(sm & lt)] = B;
+            sep0 += __popc(sm);
+        }
+        if (ch >= 0) {  // the chunks' links, and the last one's end
+            for (int i = threadIdx.x; i < nch; i += 32 * DOWN_WARPS)
+                f.chunk_next[ch + i] = i + 1 < nch ? ch + i + 1 : -1;
+            const int i = seps + threadIdx.x;
+            if (i < 32 * nch) f.chunk_src[32 * (size_t)ch + i] = -1;
+        }
+    }
+}
+
+// Work items of the near field: a leaf's bodies 64 at a time (a level-10 leaf
+// may hold more), times its directly met sources in up to 64 slices of about
+// `slice` (FMM_META_SLICE), so that no warp is left alone with a large leaf's
+// sum.  slice is a share of all the leaves' sources such that the items are
+// some four per resident warp, between 512 (each item looks its leaf up and
+// runs past the sources before its slice) and 8192 (the slices' sums are
+// stored and added by another launch).  With 8192 throughout, the near field of
+// 30001 bodies in leaves of 32 took 202 us, its longest item alone most of it;
+// now 83 us.
+constexpr int SLICE_MIN = 512, SLICE_MAX = 8192, MAX_SLICES = 64;
+__device__ __forceinline__ int body_chunks(int nb) { return (nb + 63) >> 6; }
+__device__ __forceinline__ int src_slices(int nearc, int slice)
+{
+    return min(MAX_SLICES, max(1, (nearc + slice - 1) / slice));
+}
+
+// The leaves, a warp each.
+template <int P>
+__global__ void __launch_bounds__(32 * WARPS) fmm_leaves_kernel(const FmmParams p)
 {
     __shared__ WalkSh wsh[WARPS];
     __shared__ int mq[WARPS][64];
-    __shared__ int2 dq[WARPS][LEAVES ? 64 : 1];  // a leaf's directly summed cells: body ranges
+    __shared__ int2 dq[WARPS][64];  // a leaf's directly summed cells: body ranges
     __shared__ CritSh crit;
     crit_table(crit, p.f.crit);
     __syncthreads();
@@ -623,20 +804,14 @@ __global__ void __launch_bounds__(32 * WARPS) fmm_lists_kernel(const FmmParams p
     const FmmView &f = p.f;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
-    // the non-leaves of level L, or all leaves (coarsest first: their walks
-    // are the longest)
-    const int cnt = LEAVES ? t.meta[TREE_META_BASE + 10] + t.meta[TREE_META_COUNT + 10]
-                           : t.meta[TREE_META_COUNT + L];
-    const int base = LEAVES ? 0 : t.meta[TREE_META_BASE + L];
-    int *queue = f.meta + (LEAVES ? FMM_META_LEAVES_Q : FMM_META_LEVEL + L);
+    // coarsest leaves first: their walks are the longest
+    const int cnt = t.meta[TREE_META_BASE + 10] + t.meta[TREE_META_COUNT + 10];
+    int *queue = f.meta + FMM_META_LEAVES_Q;
     WalkSh &w = wsh[warp];
     int cnext = 0, cend = 0;    // this warp's reserved expansion-list chunks
     int rcnext = 0, rcend = 0;  // and direct-range chunks
-    // one cell: its list (and, for a non-leaf, its hand-down list)
-    auto visit = [&](int qi) {
-        const int A = base + qi;
-        const int nchA = t.nchild[A];
-        if ((nchA == 0) != LEAVES) return;  // the other kernel's cell
+    auto visit = [&](int A) {
+        if (t.nchild[A] != 0) return;
         const int4 cA = f.ci[A];
         const int par = t.parent[A];
         int inh_off = 0, inh_cnt = 1;  // the root's list: pool[0] = 0
@@ -649,107 +824,50 @@ __global__ void __launch_bounds__(32 * WARPS) fmm_lists_kernel(const FmmParams p
         int mcnt = 0, own = 0, farb = 0, nearc = 0, prev = -1, dcnt = 0, dprev = -1;
         if (lane == 0) {
             f.chunk_head[A] = -1;
-            if (LEAVES) f.rhead[A] = -1;
+            f.rhead[A] = -1;
         }
-        // a non-leaf: how many candidates go down (pass 1), and where
-        long long off = 0;
-        bool fits = true;
-        if constexpr (!LEAVES) {
-            int total = 0;
-            for (int c0 = 0; c0 < inh_cnt; c0 += 32) {
-                const int k = c0 + lane;
-                const int B = k < inh_cnt ? __ldg(inh + k) : -1;
-                int outc = 0;
-                if (B >= 0) {
-                    const int4 cB = __ldg(f.ci + B), nB = __ldg(f.nd + B);
-                    if (!separated(cA, cB, crit)) outc = (nB.x == 0 || cB.w > cA.w) ? 1 : nB.x;
-                }
-                total += warp_sum(outc);
-            }
-            if (lane == 0) off = atomicAdd(f.meta + FMM_META_POOL, total);
-            off = __shfl_sync(FULL, off, 0);
-            fits = off + total <= f.pool_cap;
-            if (lane == 0) {
-                f.down[A] = make_int2(fits ? (int)off : 0, fits ? total : 0);
-                if (!fits) atomicOr(f.meta + FMM_META_OVERFLOW, 1);
-            }
-        } else {
-            if (lane < LEVELS) w.lsz[lane] = 0;
-            __syncwarp();
-        }
+        int lsize = 0;
         // Rounds of 32 candidates fill the queue of separated cells; each
         // time it holds 32 (or the candidates are done) the first 32 become
-        // a chunk.  A non-leaf classifies its handed-down candidates and
-        // writes the others down (pass 2); a leaf walks their subtrees.
-        int c0 = 0, cur = 0, cursor = 0;
+        // a chunk.
+        int cursor = 0;
         bool more = true;
         while (more || mcnt > 0) {
             while (more && mcnt < 32) {
                 bool sep = false;
                 int B = -1, bodies = 0;
-                if constexpr (!LEAVES) {
-                    if (c0 >= inh_cnt) {
-                        more = false;
-                        break;
-                    }
-                    const int k = c0 + lane;
-                    B = k < inh_cnt ? __ldg(inh + k) : -1;
-                    c0 += 32;
-                    bool self = false;
-                    int outc = 0, firstB = 0;
-                    if (B >= 0) {
-                        const int4 cB = __ldg(f.ci + B), nB = __ldg(f.nd + B);
-                        sep = separated(cA, cB, crit);
-                        bodies = nB.w - nB.z;
-                        if (!sep) {
-                            self = nB.x == 0 || cB.w > cA.w;
-                            outc = self ? 1 : nB.x;
-                            firstB = nB.y;
-                            if (!self && cB.w < cA.w) atomicOr(p.err, ERR_TREE);  // never
-                        }
-                    }
-                    const int incl = warp_incl_scan(outc, lane);
-                    if (fits && outc) {
-                        int *dst = f.pool + off + cur + (incl - outc);
-                        if (self)
-                            dst[0] = B;
-                        else
-                            for (int j = 0; j < outc; ++j) dst[j] = firstB + j;
-                    }
-                    cur += __shfl_sync(FULL, incl, 31);
-                } else {
-                    if (!next_round(w, inh, inh_cnt, cursor, lane, B)) {
-                        more = false;
-                        break;
-                    }
-                    bool open = false, direct = false;
-                    int nchB = 0, firstB = 0, lvB = 0;
-                    int2 rng = make_int2(0, 0);
-                    if (B >= 0) {
-                        const int4 cB = __ldg(f.ci + B), nB = __ldg(f.nd + B);
-                        sep = separated(cA, cB, crit);
-                        nchB = nB.x;
-                        bodies = nB.w - nB.z;
-                        if (!sep) {
-                            open = nchB > 0 && !all_direct(cA, cB, crit);
-                            direct = !open;
-                            rng = make_int2(nB.z, nB.w);
-                            if (direct) nearc += bodies;
-                        }
-                        firstB = nB.y;
-                        lvB = cB.w;
-                    }
-                    push_children(w, open, lvB + 1, firstB, nchB, lane, p.err);
-                    // the directly summed cells, in walk order, for the near field
-                    const unsigned dm = __ballot_sync(FULL, direct);
-                    if (direct) dq[warp][dcnt + __popc(dm & lt)] = rng;
-                    dcnt += __popc(dm);
-                    __syncwarp();
-                    if (dcnt >= 32)
-                        flush_chunk(dq[warp], dcnt, 32, make_int2(0, 0), f.rchunk, f.rnext,
-                                    f.rhead + A, f.rchunk_cap, f.meta + FMM_META_RCHUNKS,
-                                    f.meta + FMM_META_OVERFLOW, 4, dprev, rcnext, rcend, lane);
+                int Lv;
+                if (!next_round(w, lsize, inh, inh_cnt, cursor, lane, B, Lv)) {
+                    more = false;
+                    break;
                 }
+                bool open = false, direct = false;
+                int nchB = 0, firstB = 0, lvB = 0;
+                int2 rng = make_int2(0, 0);
+                if (B >= 0) {
+                    const int4 cB = __ldg(f.ci + B), nB = __ldg(f.nd + B);
+                    sep = separated(cA, cB, crit);
+                    nchB = nB.x;
+                    bodies = nB.w - nB.z;
+                    if (!sep) {
+                        open = nchB > 0 && !all_direct(cA, cB, crit);
+                        direct = !open;
+                        rng = make_int2(nB.z, nB.w);
+                        if (direct) nearc += bodies;
+                    }
+                    firstB = nB.y;
+                    lvB = cB.w;
+                }
+                push_children(w, lsize, open, lvB + 1, firstB, nchB, lane, p.err);
+                // the directly summed cells, in walk order, for the near field
+                const unsigned dm = __ballot_sync(FULL, direct);
+                if (direct) dq[warp][dcnt + __popc(dm & lt)] = rng;
+                dcnt += __popc(dm);
+                __syncwarp();
+                if (dcnt >= 32)
+                    flush_chunk(dq[warp], dcnt, 32, make_int2(0, 0), f.rchunk, f.rnext,
+                                f.rhead + A, f.rchunk_cap, f.meta + FMM_META_RCHUNKS,
+                                f.meta + FMM_META_OVERFLOW, 4, dprev, rcnext, rcend, lane);
                 const unsigned sm = __ballot_sync(FULL, sep);
                 if (sep) {
                     mq[warp][mcnt + __popc(sm & lt)] = B;
@@ -765,16 +883,19 @@ __global__ void __launch_bounds__(32 * WARPS) fmm_lists_kernel(const FmmParams p
                             f.chunk_cap, f.meta + FMM_META_CHUNKS, f.meta + FMM_META_OVERFLOW, 2,
                             prev, cnext, cend, lane);
         }
-        if constexpr (LEAVES) {
-            if (dcnt > 0)
-                flush_chunk(dq[warp], dcnt, dcnt, make_int2(0, 0), f.rchunk, f.rnext, f.rhead + A,
-                            f.rchunk_cap, f.meta + FMM_META_RCHUNKS, f.meta + FMM_META_OVERFLOW,
-                            4, dprev, rcnext, rcend, lane);
-            nearc = warp_sum(nearc);
-            if (lane == 0) {
-                f.nearc[A] = nearc;
-                f.leaves[atomicAdd(f.meta + FMM_META_NLEAVES, 1)] = A;
-            }
+        if (dcnt > 0)
+            flush_chunk(dq[warp], dcnt, dcnt, make_int2(0, 0), f.rchunk, f.rnext, f.rhead + A,
+                        f.rchunk_cap, f.meta + FMM_META_RCHUNKS, f.meta + FMM_META_OVERFLOW, 4,
+                        dprev, rcnext, rcend, lane);
+        nearc = warp_sum(nearc);
+        if (lane == 0) {
+            f.nearc[A] = nearc;
+            const int q = atomicAdd(f.meta + FMM_META_NLEAVES, 1);
+            f.leaves[q] = A;
+            f.item_off[q] = t.end[A] - t.start[A];  // for fmm_items_kernel
+            f.part_off[q] = nearc;
+            atomicAdd(reinterpret_cast<unsigned long long *>(f.meta + FMM_META_LISTED),
+                      (unsigned long long)body_chunks(t.end[A] - t.start[A]) * (unsigned)nearc);
         }
         farb = warp_sum(farb);
         if (lane == 0) {
@@ -867,12 +988,8 @@ __global__ void __launch_bounds__(128) fmm_l2l_kernel(const FmmParams p, int L)
     for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < cnt; q += gridDim.x * blockDim.x) {
         const int A = base + q, par = t.parent[A];
         float acc[N], xp[N];
-        const float *dst = f.L + (size_t)A * NP, *src = f.L + (size_t)par * NP;
-#pragma unroll
-        for (int k = 0; k < N; ++k) {
-            acc[k] = dst[k];
-            xp[k] = src[k];
-        }
+        load_exp<P>(acc, f.L + (size_t)A * NP);
+        load_exp<P>(xp, f.L + (size_t)par * NP);
         translate_add<P, false>(acc, xp, (int)(t.prefix[A] & 7u));
         store_exp<P>(f.L + (size_t)A * NP, acc);
     }
@@ -907,40 +1024,84 @@ __device__ __forceinline__ void list_put(float *Lf, int q, float x, float y, flo
     b[6] = m;
 }
 
-// Work items of the near field: a leaf's bodies 64 at a time (a level-10 leaf
-// may hold more), times its directly met sources in up to 64 slices of about
-// CHUNK, so that no warp is left alone with a large leaf's sum.
-constexpr int CHUNK = 8192, MAX_SLICES = 64;
-__device__ __forceinline__ int body_chunks(int nb) { return (nb + 63) >> 6; }
-__device__ __forceinline__ int src_slices(int nearc)
-{
-    return min(MAX_SLICES, max(1, (nearc + CHUNK - 1) / CHUNK));
-}
-
-// One block: work items and partial-sum slots per leaf, scanned.
+// One block: work items and partial-sum slots per leaf, scanned (as the two
+// halves of a 64-bit word).  The leaves' pass left their bodies and sources in
+// item_off and part_off and the sum of what the warps will list in meta.
 template <int P>
-__global__ void __launch_bounds__(1024) fmm_items_kernel(FmmParams p)
+__global__ void __launch_bounds__(1024) fmm_items_kernel(FmmParams p, int target)
 {
-    __shared__ int tile[BSCAN_TILE + BSCAN_TILE / 32];
-    __shared__ int wsum[32];
-    const TreeView &t = p.tree;
+    constexpr int PER = 8;
+    __shared__ unsigned long long wsum[32];
     const FmmView &f = p.f;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nl = f.meta[FMM_META_NLEAVES];
-    for (int q = threadIdx.x; q < nl; q += blockDim.x) {
-        const int A = f.leaves[q];
-        const int nb = t.end[A] - t.start[A], ns = src_slices(f.nearc[A]);
-        f.item_off[q] = body_chunks(nb) * ns;
-        f.part_off[q] = ns > 1 ? nb * ns : 0;
+    const unsigned long long share =
+        *reinterpret_cast<const unsigned long long *>(f.meta + FMM_META_LISTED) / (unsigned)target;
+    const int slice = (int)min((unsigned long long)SLICE_MAX,
+                               max((unsigned long long)SLICE_MIN, (share + 255ull) & ~255ull));
+    unsigned long long carry = 0ull;
+    for (int base = 0; base < nl; base += 1024 * PER) {
+        // thread t: entries base + 8 t ... (two 16-byte loads of each array)
+        const int q0 = base + PER * threadIdx.x;
+        unsigned long long v[PER], sum = 0ull;
+        int nb[PER], nc[PER];
+#pragma unroll
+        for (int h = 0; h < PER; h += 4) {
+            int4 a = make_int4(0, 0, 0, 0), b = a;
+            if (q0 + h < nl) {  // the arrays hold cap + 1 entries rounded up to four
+                a = *reinterpret_cast<const int4 *>(f.item_off + q0 + h);
+                b = *reinterpret_cast<const int4 *>(f.part_off + q0 + h);
+            }
+            nb[h] = a.x; nb[h + 1] = a.y; nb[h + 2] = a.z; nb[h + 3] = a.w;
+            nc[h] = b.x; nc[h + 1] = b.y; nc[h + 2] = b.z; nc[h + 3] = b.w;
+        }
+#pragma unroll
+        for (int j = 0; j < PER; ++j) {
+            v[j] = 0ull;
+            if (q0 + j < nl) {
+                const int ns = src_slices(nc[j], slice);
+                v[j] = ((unsigned long long)(unsigned)(body_chunks(nb[j]) * ns) << 32) |
+                       (unsigned)(ns > 1 ? nb[j] * ns : 0);
+            }
+            sum += v[j];
+        }
+        unsigned long long incl = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long u = __shfl_up_sync(FULL, incl, o);
+            if (lane >= o) incl += u;
+        }
+        if (lane == 31) wsum[warp] = incl;
+        __syncthreads();
+        if (warp == 0) {
+            unsigned long long x = wsum[lane];
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned long long u = __shfl_up_sync(FULL, x, o);
+                if (lane >= o) x += u;
+            }
+            wsum[lane] = x;
+        }
+        __syncthreads();
+        unsigned long long run = carry + (warp ? wsum[warp - 1] : 0ull) + incl - sum;
+#pragma unroll
+        for (int j = 0; j < PER; ++j) {
+            if (q0 + j < nl) {
+                f.item_off[q0 + j] = (int)(run >> 32);
+                f.part_off[q0 + j] = (int)(unsigned)run;
+            }
+            run += v[j];
+        }
+        carry += wsum[31];
+        __syncthreads();  // wsum is rewritten
     }
-    __syncthreads();
-    const int items = block_scan_exclusive<int>(f.item_off, f.item_off, nl, tile, wsum);
-    __syncthreads();
-    const int slots = block_scan_exclusive<int>(f.part_off, f.part_off, nl, tile, wsum);
     if (threadIdx.x == 0) {
+        const int items = (int)(carry >> 32), slots = (int)(unsigned)carry;
         f.item_off[nl] = items;
         f.part_off[nl] = slots;
         f.meta[FMM_META_ITEMS] = items;
         f.meta[FMM_META_PSLOTS] = slots;
+        f.meta[FMM_META_SLICE] = slice;
     }
 }
 
@@ -1063,14 +1224,23 @@ __device__ __forceinline__ void write_body_kahan(const FmmParams &p, int A, cons
 // source pairs.  The slices' sums are combined in a fixed
 // order; a leaf in one item gets its result written, a split one its
 // partial sums stored for fmm_combine_kernel.
+//
+// Resident blocks per SM (the register cap) and rounds of 32 sources whose
+// loads are in flight together, measured at 2^20 bodies (order 6, leaves of
+// 64 / order 4, leaves of 32): 4 blocks 1 round 1826 / 1429 us, 2 rounds 1706 /
+// 1281; 5: 1706 / 1315 and 1698 / 1363; 6: 1671 / 1256 and 1660 / 1124 us.
+// Before the ring (its half copied down at each flush, one round at a time,
+// the item's leaf found by bisection): 1746 / 1329 us.
+constexpr int NEAR_BLOCKS = 6;
 template <int P, bool ZEPS>
-__global__ void __launch_bounds__(32 * WARPS) fmm_near_kernel(const FmmParams p)
+__global__ void __launch_bounds__(32 * WARPS, NEAR_BLOCKS) fmm_near_kernel(const FmmParams p)
 {
     __shared__ __align__(16) float4 lists[WARPS][2 * FLUSH];  // 2 * FLUSH sources as pairs
     const TreeView &t = p.tree;
     const FmmView &f = p.f;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nleaves = f.meta[FMM_META_NLEAVES], nitems = f.meta[FMM_META_ITEMS];
+    const int slice_len = f.meta[FMM_META_SLICE];
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         f.stats[0] = (unsigned long long)(t.meta[TREE_META_BASE + 10] + t.meta[TREE_META_COUNT + 10]);
         f.stats[1] = (unsigned long long)nleaves;
@@ -1083,18 +1253,19 @@ __global__ void __launch_bounds__(32 * WARPS) fmm_near_kernel(const FmmParams p)
         if (lane == 0) it = atomicAdd(f.meta + FMM_META_NEAR, 1);
         it = __shfl_sync(FULL, it, 0);
         if (it >= nitems) break;
-        // the leaf holding item `it`: the last qi with item_off[qi] <= it
-        int lo = 0, hi = nleaves;
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (f.item_off[mid] <= it)
-                lo = mid;
-            else
-                hi = mid;
+        // the leaf holding item `it`: the last qi with item_off[qi] <= it, the
+        // lanes probing 32 places at a time
+        int qi = 0;
+        for (int m = nleaves; m > 1;) {
+            const int step = (m + 31) >> 5;
+            const bool le = lane * step < m && f.item_off[qi + lane * step] <= it;
+            const int k = __popc(__ballot_sync(FULL, le)) - 1;
+            qi += k * step;
+            m = min(step, m - k * step);
         }
-        const int qi = lo, A = f.leaves[qi];
+        const int A = f.leaves[qi];
         const int4 cA = f.ci[A];
-        const int nearc = f.nearc[A], ns = src_slices(nearc);
+        const int nearc = f.nearc[A], ns = src_slices(nearc, slice_len);
         const int j = it - f.item_off[qi], bc = j / ns, sc = j % ns;
         const int nbt = t.end[A] - t.start[A];
         const int s0 = t.start[A] + 64 * bc, nb = min(64, t.end[A] - s0);
@@ -1143,22 +1314,24 @@ __global__ void __launch_bounds__(32 * WARPS) fmm_near_kernel(const FmmParams p)
             kahan_add(ks[1][2], kc[1][2], az1.y);
             ax0 = ay0 = az0 = ax1 = ay1 = az1 = make_float2(0.f, 0.f);
         };
-        auto eval = [&](int npairs) {
+        auto eval = [&](const float4 *src, int npairs) {
             for (int q = slice; q < npairs; q += S) {
-                const float4 a = L4[2 * q], bq = L4[2 * q + 1];
+                const float4 a = src[2 * q], bq = src[2 * q + 1];
                 const float2 sx = make_float2(a.x, a.y), sy = make_float2(a.z, a.w);
                 const float2 sz = make_float2(bq.x, bq.y), sm = make_float2(bq.z, bq.w);
                 pair_terms<ZEPS>(add2(sx, nx0), add2(sy, ny0), add2(sz, nz0), sm, e2, ax0, ay0, az0);
                 pair_terms<ZEPS>(add2(sx, nx1), add2(sy, ny1), add2(sz, nz1), sm, e2, ax1, ay1, az1);
             }
         };
+        // the list is a ring of two halves of FLUSH sources: a flush evaluates
+        // the half at the head and moves the head to the other
         int cnt = 0, seen = 0;  // listed sources; direct sources met so far in walk order
+        int head = 0;
         auto flush = [&]() {
             __syncwarp();
-            eval(FLUSH / 2);
+            eval(L4 + head, FLUSH / 2);
             fold();
-            __syncwarp();
-            for (int c = lane; c < FLUSH; c += 32) lists[warp][c] = lists[warp][FLUSH + c];
+            head ^= FLUSH;
             cnt -= FLUSH;
             __syncwarp();
         };
@@ -1171,25 +1344,36 @@ __global__ void __launch_bounds__(32 * WARPS) fmm_near_kernel(const FmmParams p)
             const int tot = __shfl_sync(FULL, linc, 31);
             // this chunk's direct sources are [seen, seen + tot) in walk order
             const int a0 = max(src_lo - seen, 0), a1 = min(src_hi - seen, tot);
-            for (int c0 = a0; c0 < a1; c0 += 32) {
-                const int pos = c0 + lane;
-                const int jj = warp_span_of(linc, pos) & 31;
-                const int body = __shfl_sync(FULL, ls, jj) + (pos - __shfl_sync(FULL, lexc, jj));
-                const int kk = min(32, a1 - c0);
-                if (lane < kk) {
-                    const float4 bh = __ldg(p.P + body), bl = __ldg(p.Plo + body);
-                    list_put(Lf, cnt + lane, rel(bh.x, bl.x, cx), rel(bh.y, bl.y, cy),
-                             rel(bh.z, bl.z, cz), bh.w);
+            // LIST_ROUNDS x 32 sources' loads in flight at a time
+            for (int c0 = a0; c0 < a1; c0 += 32 * LIST_ROUNDS) {
+                float4 bh[LIST_ROUNDS], bl[LIST_ROUNDS];
+#pragma unroll
+                for (int u = 0; u < LIST_ROUNDS; ++u) {
+                    const int pos = c0 + 32 * u + lane;
+                    const int jj = warp_span_of(linc, pos) & 31;
+                    const int body =
+                        __shfl_sync(FULL, ls, jj) + (pos - __shfl_sync(FULL, lexc, jj));
+                    if (pos < a1) {
+                        bh[u] = __ldg(p.P + body);
+                        bl[u] = __ldg(p.Plo + body);
+                    }
                 }
-                cnt += kk;
+#pragma unroll
+                for (int u = 0; u < LIST_ROUNDS; ++u) {
+                    if (c0 + 32 * u + lane < a1)
+                        list_put(Lf, (head + cnt + 32 * u + lane) & (2 * FLUSH - 1),
+                                 rel(bh[u].x, bl[u].x, cx), rel(bh[u].y, bl[u].y, cy),
+                                 rel(bh[u].z, bl[u].z, cz), bh[u].w);
+                }
+                cnt += min(32 * LIST_ROUNDS, a1 - c0);
                 if (cnt >= FLUSH) flush();
             }
             seen += tot;
         }
         if (cnt > 0) {
-            if (lane == 0 && (cnt & 1)) list_put(Lf, cnt, 0.f, 0.f, 0.f, 0.f);
+            if (lane == 0 && (cnt & 1)) list_put(Lf, head + cnt, 0.f, 0.f, 0.f, 0.f);
             __syncwarp();
-            eval((cnt + 1) >> 1);
+            eval(L4 + head, (cnt + 1) >> 1);
             fold();
         }
         // combine the slices' Kahan pairs in float32 (lane b0 of slice 0 ends
@@ -1239,12 +1423,12 @@ __global__ void __launch_bounds__(256) fmm_combine_kernel(const FmmParams p)
 {
     const TreeView &t = p.tree;
     const FmmView &f = p.f;
-    const int nleaves = f.meta[FMM_META_NLEAVES];
+    const int nleaves = f.meta[FMM_META_NLEAVES], slice_len = f.meta[FMM_META_SLICE];
     const int lane = threadIdx.x & 31;
     const int warps = gridDim.x * (blockDim.x >> 5);
     for (int qi = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); qi < nleaves; qi += warps) {
         const int A = f.leaves[qi];
-        const int nearc = f.nearc[A], ns = src_slices(nearc);
+        const int nearc = f.nearc[A], ns = src_slices(nearc, slice_len);
         if (ns == 1) continue;
         const int4 cA = f.ci[A];
         const int nbt = t.end[A] - t.start[A];
@@ -1298,17 +1482,25 @@ cudaError_t launch_fmm_order(cudaStream_t s, const FmmParams &p, bool near, int 
             8 * p.num_sms, ((long long)p.tree.cap + 32 * UP_WARPS - 1) / (32 * UP_WARPS));
         fmm_p2m_kernel<P><<<p2m_grid, 32 * UP_WARPS, 0, s>>>(p);
         for (int L = LEVELS - 2; L >= 0; --L)
-            fmm_m2m_kernel<P><<<8 * p.num_sms, 32 * UP_WARPS, 0, s>>>(p, L);
-        const int lists_grid = resident_grid(fmm_lists_kernel<P, true>, 32 * WARPS, p.num_sms, e);
+            fmm_m2m_kernel<P><<<4 * p.num_sms, 32 * UP_WARPS, 0, s>>>(p, L);
+        const int down_grid = resident_grid(fmm_down_kernel<P>, 32 * DOWN_WARPS, p.num_sms, e);
+        if (e != cudaSuccess) return e;
+        const int leaves_grid = resident_grid(fmm_leaves_kernel<P>, 32 * WARPS, p.num_sms, e);
+        if (e != cudaSuccess) return e;
+        // (the near field's kernel is the same size for either eps)
+        const int near_resident =
+            resident_grid(fmm_near_kernel<P, false>, 32 * WARPS, p.num_sms, e);
         if (e != cudaSuccess) return e;
         const int m2l_grid = resident_grid(fmm_m2l_kernel<P>, 32 * WARPS, p.num_sms, e);
         if (e != cudaSuccess) return e;
-        for (int L = 0; L < LEVELS; ++L)
-            fmm_lists_kernel<P, false><<<lists_grid, 32 * WARPS, 0, s>>>(p, L);
-        fmm_lists_kernel<P, true><<<lists_grid, 32 * WARPS, 0, s>>>(p, 0);
+        for (int L = 0; L < LEVELS; ++L) {  // level L has at most 8^L cells
+            const int g = L < 6 ? std::min(down_grid, 1 << (3 * L)) : down_grid;
+            fmm_down_kernel<P><<<g, 32 * DOWN_WARPS, 0, s>>>(p, L);
+        }
+        fmm_leaves_kernel<P><<<leaves_grid, 32 * WARPS, 0, s>>>(p);
         fmm_m2l_kernel<P><<<m2l_grid, 32 * WARPS, 0, s>>>(p);
         for (int L = 1; L < LEVELS; ++L) fmm_l2l_kernel<P><<<2 * p.num_sms, 128, 0, s>>>(p, L);
-        fmm_items_kernel<P><<<1, 1024, 0, s>>>(p);
+        fmm_items_kernel<P><<<1, 1024, 0, s>>>(p, 4 * WARPS * near_resident);
         kernels = 5 + 3 * LEVELS - 2;
         return cudaGetLastError();
     }

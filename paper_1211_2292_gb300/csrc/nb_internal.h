@@ -282,7 +282,8 @@ constexpr int FMM_MIN_ORDER = 2, FMM_MAX_ORDER = 6, FMM_MAX_LEAF = 64;
 int fmm_floats(int order);
 enum : int { FMM_META_LEVEL = 0, FMM_META_NEAR = 11, FMM_META_POOL = 12, FMM_META_OVERFLOW = 13,
              FMM_META_NLEAVES = 14, FMM_META_ITEMS = 15, FMM_META_PSLOTS = 16,
-             FMM_META_CHUNKS = 17, FMM_META_M2L = 18, FMM_META_LEAVES_Q = 19, FMM_META_RCHUNKS = 20,
+             FMM_META_CHUNKS = 17, FMM_META_M2L = 18, FMM_META_LEAVES_Q = 19, FMM_META_RCHUNKS = 20, FMM_META_SLICE = 21,
+             FMM_META_LISTED = 22 /* 64 bits */,
              FMM_META_INTS = 24 };
 // FMM_META_OVERFLOW bits: the candidate pool (1), the expansion-list chunks
 // (2), the direct-range chunks (4).

@@ -704,8 +704,8 @@ nb_status ensure_fmm(nb_ctx *c, int order, long long pool_need, long long chunk_
         if (st == NB_OK) f.cum = dev_alloc<int2>(c, m, st);
         if (st == NB_OK) f.leaves = dev_alloc<int>(c, m, st);
         if (st == NB_OK) f.nearc = dev_alloc<int>(c, m, st);
-        if (st == NB_OK) f.item_off = dev_alloc<int>(c, m + 1, st);
-        if (st == NB_OK) f.part_off = dev_alloc<int>(c, m + 1, st);
+        if (st == NB_OK) f.item_off = dev_alloc<int>(c, m + 4, st);
+        if (st == NB_OK) f.part_off = dev_alloc<int>(c, m + 4, st);
         if (st == NB_OK) f.chunk_head = dev_alloc<int>(c, m, st);
         if (st == NB_OK) f.rhead = dev_alloc<int>(c, m, st);
         if (st != NB_OK) {
