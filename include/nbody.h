@@ -470,7 +470,7 @@ nb_status nb_let_forces(nb_ctx *ctx, double G, double eps, double theta, int gro
  * counterpart; this is a service of the library.
  *
  * It allocates nothing: no context, no cudaMalloc/cudaFree.  Its scratch
- * (packed bodies, split partials, counters; about 8 MiB) is one fixed
+ * (packed bodies, split partials; about 8 MiB) is one fixed
  * __device__ array that every GPU loading the library holds until the
  * process exits, which bounds n to NB_NOALLOC_MAX_BODIES.  Work runs in the
  * calling thread's current CUDA context and device, enqueued on
@@ -482,8 +482,8 @@ nb_status nb_let_forces(nb_ctx *ctx, double G, double eps, double theta, int gro
  * the scratch array's device address in that context (cudaGetSymbolAddress)
  * and keeps it, keyed by the context; make that first call before any stream
  * capture.  Every call in a context shares the one scratch array and it keeps
- * the last call's contents: each call clears the counters and the error word
- * it uses before its kernels run, and calls whose work overlaps on the GPU
+ * the last call's contents: each call clears the error word it uses before
+ * its kernels run, and calls whose work overlaps on the GPU
  * (different streams without ordering, several threads) race and give wrong
  * results; order them on one stream.
  *

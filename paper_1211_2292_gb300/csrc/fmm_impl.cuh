@@ -1152,17 +1152,6 @@ __device__ __forceinline__ void write_body(const FmmParams &p, int A, const doub
     if (!finite3(gx, gy, gz)) atomicOr(p.err, ERR_NONFINITE);
 }
 
-// (s, c) += (so, co) for Kahan pairs holding s - c: the sums' rounding
-// error goes into the carry (the two-sum of s and so).
-__device__ __forceinline__ void kahan_merge(float &s, float &c, float so, float co)
-{
-    const float t = s + so;
-    const float bp = t - s;
-    const float e = (s - (t - bp)) + (so - bp);
-    s = t;
-    c = (c + co) - e;
-}
-
 // write_body for a near field held as float32 Kahan pairs (s - c): the L2P
 // in float32 from the body's hi/lo position relative to the centre's hi/lo
 // pair (zh, zl) times 1/e, the far field added into the pair, one float64

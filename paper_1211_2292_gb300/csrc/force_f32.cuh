@@ -25,9 +25,11 @@
 //    Kahan (sum, carry) pair, so rounding grows with the tile count, not
 //    with N.  NB_FP32: one running float32 sum.
 //  * j-split: the grid is (i-tiles x nsplit).  With nsplit > 1, each CTA
-//    stores its float64 partial; the last CTA of an i-tile (arrival counter)
-//    adds the partials in split order (deterministic) and runs the epilogue.
-//    No CTA ever waits for another.
+//    stores its sums as float32 (sum, carry) pairs, and an O(n) launch
+//    (integrate.cu: merge_kernel, or the next step's kick and drift) merges
+//    them in split order (deterministic) and runs the epilogue.  The pairs are
+//    merged with float32 two-sums (kahan_merge, relative error about 2^-48):
+//    this part's float64 pipe takes 2 lanes per clock per SM.
 //  * Epilogue: acc = G*sum in float64, optional fused half-kick
 //    vel += dt/2 * acc, non-finite outputs flagged in the error word.
 #pragma once
@@ -222,31 +224,36 @@ struct Acc {
             }
         }
     }
-    // Value of body k's sum in float64.
-    __device__ __forceinline__ void get(int k, double &x, double &y, double &z) const
+    // Coordinate d (0..2) of body k's sum as (sum, carry): the sum is x - y.
+    __device__ __forceinline__ float2 get(int d, int k) const
     {
         if (REG) {
-            x = (double)sx[k] - (double)cx[k];
-            y = (double)sy[k] - (double)cy[k];
-            z = (double)sz[k] - (double)cz[k];
-        } else if (COMP && KSM) {
-            x = (double)ksm(0, k) - (double)ksm(3, k);
-            y = (double)ksm(1, k) - (double)ksm(4, k);
-            z = (double)ksm(2, k) - (double)ksm(5, k);
-        } else {
-            const int p = k >> 1;
-            x = (k & 1) ? ax[p].y : ax[p].x;
-            y = (k & 1) ? ay[p].y : ay[p].x;
-            z = (k & 1) ? az[p].y : az[p].x;
+            const float *s = d == 0 ? sx : (d == 1 ? sy : sz), *c = d == 0 ? cx : (d == 1 ? cy : cz);
+            return make_float2(s[k], c[k]);
         }
+        if (COMP && KSM) return make_float2(ksm(d, k), ksm(d + 3, k));
+        const float2 a = d == 0 ? ax[k >> 1] : (d == 1 ? ay[k >> 1] : az[k >> 1]);
+        return make_float2((k & 1) ? a.y : a.x, 0.f);
     }
 };
+
+// A pair stored as two words: one 64-bit store would tie the sum's and the
+// carry's registers together through the whole sweep.
+__device__ __forceinline__ void put_pair(float2 *q, float2 a)
+{
+    asm volatile("st.global.f32 [%0], %1;" ::"l"(&q->x), "f"(a.x) : "memory");
+    asm volatile("st.global.f32 [%0], %1;" ::"l"(&q->y), "f"(a.y) : "memory");
+}
+
+// The float64 value of a (sum, carry) pair.
+__device__ __forceinline__ double pair_value(float2 a) { return (double)a.x - (double)a.y; }
 
 // Sweep the j-tiles [t0, t1) of bodies [jlo, jhi) (tile t starts at
 // jlo + t*J) for this thread's bodies.  Threads split each tile's j loop in
 // `lanes` interleaved parts (lanes == 1 for the solo kernel).  Body pairs
 // p < LP use the log-domain pair factor, the others rsqrt.
-template <int T, int I, int J, bool COMP, bool ZEPS, int LP, bool LANES, bool KSM, int UNR>
+template <int T, int I, int J, bool COMP, bool ZEPS, int LP, bool LANES, bool KSM, int UNR,
+          bool EVEN = false>
 __device__ __forceinline__ void sweep(const float4 *__restrict__ P, const float4 *__restrict__ Plo,
                                       float3 c, int jlo, int jhi, int t0, int t1, int lane,
                                       int lanes, float2 e2, const float2 (&nx)[I / 2],
@@ -287,8 +294,11 @@ __device__ __forceinline__ void sweep(const float4 *__restrict__ P, const float4
                 }
             }
         } else {
+            // EVEN: a last, partial tile stops at the next multiple of UNR
+            // bodies (massless ones, which add nothing)
+            const int jn = EVEN ? (min(J, jhi - (jlo + t * J)) + UNR - 1) / UNR * UNR : J;
 #pragma unroll UNR
-            for (int jj = 0; jj < J; ++jj) {
+            for (int jj = 0; jj < jn; ++jj) {
                 const float4 q0 = s[W * jj], q1 = s[W * jj + 1];
                 const float2 xj = make_float2(q0.x, q0.y), yj = make_float2(q0.z, q0.w);
                 const float2 zj = make_float2(q1.x, q1.y), mj = make_float2(q1.z, q1.w);
@@ -351,7 +361,7 @@ __device__ __forceinline__ float3 load_i(const float4 *__restrict__ P, const flo
 // -------------------------------------------------------------- solo kernel
 // MINB > 0 caps registers so that MINB CTAs fit per SM; 0 leaves the choice
 // to the compiler.
-template <int T, int I, int J, bool COMP, bool ZEPS, int LP, bool KSM, int MINB, int UNR>
+template <int T, int I, int J, bool COMP, bool ZEPS, int LP, bool KSM, int MINB, int UNR, bool EVEN>
 __global__ void __launch_bounds__(T, MINB) force_f32_kernel(const ForceParams p)
 {
     static_assert(I % 2 == 0 && J % T == 0 && LP <= I / 2, "bad tile shape");
@@ -359,7 +369,6 @@ __global__ void __launch_bounds__(T, MINB) force_f32_kernel(const ForceParams p)
     __shared__ __align__(16) float4 tile[2][Slots<LP>::W * J];
     __shared__ float red[6][T / 32];
     __shared__ float ks[(COMP && KSM) ? 6 * I * T : 1];
-    __shared__ int s_last;
 
     const float4 *P = static_cast<const float4 *>(p.P);
     const int n = p.n;
@@ -367,63 +376,46 @@ __global__ void __launch_bounds__(T, MINB) force_f32_kernel(const ForceParams p)
     const int it = blockIdx.x % n_itiles;
     const int js = blockIdx.x / n_itiles;
     const int i0 = it * TILE_I;
-    int t0, t1;
-    split_range((n + J - 1) / J, p.nsplit, js, t0, t1);
-
+    // this split's j-bodies: whole tiles, or (EVEN) an equal share of the bodies
+    int jlo = 0, jhi = n, t0, t1;
+    if constexpr (EVEN) {
+        jlo = (int)((long long)n * js / p.nsplit);
+        jhi = (int)((long long)n * (js + 1) / p.nsplit);
+        t0 = 0;
+        t1 = (jhi - jlo + J - 1) / J;
+    } else {
+        split_range((n + J - 1) / J, p.nsplit, js, t0, t1);
+    }
     float2 nx[I / 2], ny[I / 2], nz[I / 2];
     const float3 c = load_i<T, I>(P, p.Plo, i0 + threadIdx.x, T, n, nx, ny, nz, red);
     Acc<T, I, COMP, KSM> acc;
     acc.init(ks);
     const float2 e2 = make_float2(p.eps2f, p.eps2f);
-    sweep<T, I, J, COMP, ZEPS, LP, false, KSM, UNR>(
-        P, p.Plo, c, 0, n, t0, t1, 0, 1, e2, nx, ny, nz, acc, tile);
+    sweep<T, I, J, COMP, ZEPS, LP, false, KSM, UNR, EVEN>(
+        P, p.Plo, c, jlo, jhi, t0, t1, 0, 1, e2, nx, ny, nz, acc, tile);
 
+    const int tid = threadIdx.x;
     if (p.nsplit == 1) {
 #pragma unroll
         for (int k = 0; k < I; ++k) {
-            const int i = i0 + threadIdx.x + k * T;
-            if (i < n) {
-                double x, y, z;
-                acc.get(k, x, y, z);
-                write_acc(p, p.perm ? p.perm[i] : i, p.G * x, p.G * y, p.G * z);
-            }
+            const int i = i0 + tid + k * T;
+            if (i < n)
+                write_acc(p, p.perm ? p.perm[i] : i, p.G * pair_value(acc.get(0, k)),
+                          p.G * pair_value(acc.get(1, k)), p.G * pair_value(acc.get(2, k)));
         }
         return;
     }
-    // Split: publish this CTA's partial, the last arriving CTA combines.
+    // Split: this CTA's sums, for the merging launch.
+    float2 *part = reinterpret_cast<float2 *>(p.partial);
 #pragma unroll
     for (int k = 0; k < I; ++k) {
-        const int i = i0 + threadIdx.x + k * T;
+        const int i = i0 + tid + k * T;
         if (i < n) {
-            double x, y, z;
-            acc.get(k, x, y, z);
-            double *q = p.partial + ((size_t)js * n + i) * 3;
-            q[0] = x;
-            q[1] = y;
-            q[2] = z;
-        }
-    }
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) s_last = (atomicAdd(p.counters + it, 1u) == (unsigned)(p.nsplit - 1));
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
+            float2 *q = part + ((size_t)js * n + i) * 3;
 #pragma unroll
-    for (int k = 0; k < I; ++k) {
-        const int i = i0 + threadIdx.x + k * T;
-        if (i < n) {
-            double x = 0.0, y = 0.0, z = 0.0;
-            for (int q = 0; q < p.nsplit; ++q) {
-                const double *r = p.partial + ((size_t)q * n + i) * 3;
-                x += __ldcg(r);
-                y += __ldcg(r + 1);
-                z += __ldcg(r + 2);
-            }
-            write_acc(p, p.perm ? p.perm[i] : i, p.G * x, p.G * y, p.G * z);
+            for (int d = 0; d < 3; ++d) put_pair(q + d, acc.get(d, k));
         }
     }
-    if (threadIdx.x == 0) p.counters[it] = 0u;
 }
 
 // ----------------------------------------------------------- batched kernel
@@ -448,8 +440,8 @@ __device__ __forceinline__ void batch_write(const BatchParams &p, int i, double 
 // Persistent: each CTA pops items (largest cost first) from an atomic
 // counter until the queue is empty, the GPU analogue of the paper's dynamic
 // loop schedule (Sec. V-C, Table VI).  An item whose piece is split over
-// j-chunks stores its float64 partial sums; the last chunk of the piece to
-// arrive (arrival counter) adds the chunks in order and writes the result.
+// j-chunks stores its sums as (sum, carry) pairs; the last chunk of the piece
+// to arrive (arrival counter) merges the chunks in order and writes the result.
 // The last CTA to finish resets the queue counters for the next launch;
 // nothing waits.
 template <int T, int I, int J, bool COMP, bool ZEPS, int LP>
@@ -489,26 +481,29 @@ __global__ void __launch_bounds__(T) force_f32_batched_kernel(const BatchParams 
             sweep<T, I, J, COMP, ZEPS, LP, true, false, UNROLL_F32>(
                 p.P, p.Plo, c, it.j0, it.j1, 0, ntiles, lane, lanes, e2, nx, ny, nz, acc, tile);
         const bool split = it.nchunks > 1;
-        double *slot = split ? p.partial + (size_t)(it.pbase + it.chunk) * TILE_I * 3 : nullptr;
+        float2 *part = reinterpret_cast<float2 *>(p.partial);
+        float2 *slot = split ? part + (size_t)(it.pbase + it.chunk) * TILE_I * 3 : nullptr;
 #pragma unroll
         for (int k = 0; k < I; ++k) {
-            double x, y, z;
-            acc.get(k, x, y, z);
-            // lanes of a group are adjacent in one warp: butterfly sum
-            for (int off = lanes >> 1; off > 0; off >>= 1) {
-                x += __shfl_xor_sync(0xffffffffu, x, off);
-                y += __shfl_xor_sync(0xffffffffu, y, off);
-                z += __shfl_xor_sync(0xffffffffu, z, off);
+            float2 a[3];
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                a[d] = acc.get(d, k);
+                // lanes of a group are adjacent in one warp: butterfly of pair merges
+                for (int off = lanes >> 1; off > 0; off >>= 1) {
+                    const float so = __shfl_xor_sync(0xffffffffu, a[d].x, off);
+                    const float co = __shfl_xor_sync(0xffffffffu, a[d].y, off);
+                    kahan_merge(a[d].x, a[d].y, so, co);
+                }
             }
             const int i = it.i0 + group + k * groups;
             if (lane == 0 && i < it.i_end) {
                 if (split) {
-                    double *q = slot + 3 * (size_t)(i - it.i0);
-                    q[0] = x;
-                    q[1] = y;
-                    q[2] = z;
+                    float2 *q = slot + 3 * (size_t)(i - it.i0);
+#pragma unroll
+                    for (int d = 0; d < 3; ++d) put_pair(q + d, a[d]);
                 } else {
-                    batch_write(p, i, x, y, z);
+                    batch_write(p, i, pair_value(a[0]), pair_value(a[1]), pair_value(a[2]));
                 }
             }
         }
@@ -520,16 +515,11 @@ __global__ void __launch_bounds__(T) force_f32_batched_kernel(const BatchParams 
             __syncthreads();
             if (s_last) {
                 __threadfence();
-                const double *base = p.partial + (size_t)it.pbase * TILE_I * 3;
+                const float2 *base = part + (size_t)it.pbase * TILE_I * 3;
                 for (int q = threadIdx.x; q < it.i_end - it.i0; q += T) {
-                    double x = 0.0, y = 0.0, z = 0.0;
-                    for (int ch = 0; ch < it.nchunks; ++ch) {
-                        const double *r = base + ((size_t)ch * TILE_I + q) * 3;
-                        x += __ldcg(r);
-                        y += __ldcg(r + 1);
-                        z += __ldcg(r + 2);
-                    }
-                    batch_write(p, it.i0 + q, x, y, z);
+                    float2 a[3];
+                    merge_slots(base + (size_t)q * 3, (size_t)TILE_I * 3, it.nchunks, a);
+                    batch_write(p, it.i0 + q, pair_value(a[0]), pair_value(a[1]), pair_value(a[2]));
                 }
                 if (threadIdx.x == 0) p.counters[it.ctr] = 0u;
             }
@@ -545,19 +535,23 @@ __global__ void __launch_bounds__(T) force_f32_batched_kernel(const BatchParams 
     }
 }
 
-#define NB_F32_KERNEL(T, I, J, C, Z, L, K, M, U) \
-    {T, I, J, (const void *)force_f32_kernel<T, I, J, C, Z, L, K, M, U>, (L) > 0}
+#define NB_F32_KERNEL(T, I, J, C, Z, L, K, M, U, E) \
+    {T, I, J, (const void *)force_f32_kernel<T, I, J, C, Z, L, K, M, U, (E) != 0>, (L) > 0, E}
 // [comp][zero_eps]; L = body pairs per thread in the log-domain form;
 // K (Kahan state in shared memory) and M (register cap for M CTAs/SM) only
-// change the compensated kernels; U = unroll depth of the j loop.
-#define NB_F32_ENTRY_XU(T, I, J, L, K, M, U)                                               \
-    {{NB_F32_KERNEL(T, I, J, false, false, L, false, 0, U),                                \
-      NB_F32_KERNEL(T, I, J, false, true, L, false, 0, U)},                                \
-     {NB_F32_KERNEL(T, I, J, true, false, L, K, M, U),                                     \
-      NB_F32_KERNEL(T, I, J, true, true, L, K, M, U)}}
+// change the compensated kernels; U = unroll depth of the j loop; E, EC:
+// j-splits of equal body counts when not 0, and the plain and the compensated
+// kernel's time per pair (KernelEntry::even).
+#define NB_F32_ENTRY_XU(T, I, J, L, K, M, U, E, EC)                                        \
+    {{NB_F32_KERNEL(T, I, J, false, false, L, false, 0, U, E),                             \
+      NB_F32_KERNEL(T, I, J, false, true, L, false, 0, U, E)},                             \
+     {NB_F32_KERNEL(T, I, J, true, false, L, K, M, U, EC),                                 \
+      NB_F32_KERNEL(T, I, J, true, true, L, K, M, U, EC)}}
 #define NB_F32_ENTRY_X(T, I, J, L, K, M) \
-    NB_F32_ENTRY_XU(T, I, J, L, K, M, ((M) >= 4 ? 4 : UNROLL_F32))
+    NB_F32_ENTRY_XU(T, I, J, L, K, M, ((M) >= 4 ? 4 : UNROLL_F32), 0, 0)
 #define NB_F32_ENTRY(T, I, J, L) NB_F32_ENTRY_X(T, I, J, L, false, 0)
+#define NB_F32_ENTRY_EVEN(T, I, J, L, E, EC) \
+    NB_F32_ENTRY_XU(T, I, J, L, false, 0, UNROLL_F32, E, EC)
 
 #define NB_F32B_KERNEL(T, I, J, C, Z, L) \
     {T, I, J, (const void *)force_f32_batched_kernel<T, I, J, C, Z, L>, (L) > 0}

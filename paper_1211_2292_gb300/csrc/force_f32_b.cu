@@ -20,6 +20,14 @@ const Quad kForceB[] = {
     NB_F32_ENTRY_X(128, 6, 256, 2, false, 3),
     NB_F32_ENTRY_X(128, 6, 256, 2, true, 3),
     NB_F32_ENTRY_X(128, 6, 128, 2, true, 3),
+    // j-splits of equal body counts, for systems whose whole tiles would leave
+    // the SMs unevenly loaded (21..24), with their times per pair, plain and
+    // compensated, per mille of the first's (16411 bodies, best split: 129 / 132
+    // / 128 / 119 us and 131 / 126 / 123 / 132 us)
+    NB_F32_ENTRY_EVEN(256, 8, 256, 2, 985, 1000),
+    NB_F32_ENTRY_EVEN(128, 8, 128, 3, 1050, 1000),
+    NB_F32_ENTRY_EVEN(64, 8, 128, 2, 1045, 1000),
+    NB_F32_ENTRY_EVEN(128, 6, 128, 2, 1000, 1170),
 };
 
 }  // namespace

@@ -23,11 +23,16 @@ const Quad kBatched[] = {
 
 }  // namespace
 
-int f32_force_variants() { return f32_force_variants_a() + f32_force_variants_b(); }
+int f32_force_variants()
+{
+    return f32_force_variants_a() + f32_force_variants_b() + f32_team_variants();
+}
 const KernelEntry &f32_force_kernel(int v, bool comp, bool zeps)
 {
-    const int na = f32_force_variants_a();
-    return v < na ? f32_force_kernel_a(v, comp, zeps) : f32_force_kernel_b(v - na, comp, zeps);
+    const int na = f32_force_variants_a(), nab = na + f32_force_variants_b();
+    return v < na    ? f32_force_kernel_a(v, comp, zeps)
+           : v < nab ? f32_force_kernel_b(v - na, comp, zeps)
+                     : f32_team_kernel(v - nab, comp, zeps);
 }
 int f32_batched_variants() { return (int)(sizeof(kBatched) / sizeof(kBatched[0])); }
 const KernelEntry &f32_batched_kernel(int v, bool comp, bool zeps)

@@ -1,0 +1,199 @@
+// The float32 pair sum (force_f32.cuh: the same pair terms, tile-local hi/lo
+// coordinates and compensated sums) for systems too small to fill the chip
+// with one thread per body or two.
+//
+// What bounds such a call is not arithmetic (4096 bodies are 1.7e7 pairs, 6 us
+// of the FP32 pipe; 1000 bodies 0.4 us) but how many warps share it and the
+// steps around it.  So a block's eight warps all keep the same 32 I bodies (I
+// per lane) and take an eighth of the block's j range each, alone: a warp
+// stages 32 j-bodies at a time in its own shared memory, with no block barrier
+// in the loop.  Up to eight blocks of a thread-block cluster share one i-tile
+// and split the j range further; their sums meet in distributed shared memory
+// (added in rank order) instead of global partials, a fence and an arrival
+// counter.  For the smallest systems the bodies are read straight from the
+// caller's float64 arrays (RAW), packed the same way in registers, which saves
+// the packing launch.
+#include <cooperative_groups.h>
+
+#include "force_f32.cuh"
+
+namespace nb {
+namespace {
+
+namespace cg = cooperative_groups;
+
+constexpr int TEAM_T = 256, TEAM_W = TEAM_T / 32;
+constexpr int TEAM_FOLD = 128;  // j-bodies per compensated fold
+
+// Body j as hi/lo pairs, from the packed arrays or (the same values) from float64.
+template <bool RAW>
+__device__ __forceinline__ void team_load(const ForceParams &p, int j, bool ok, float4 &h, float4 &l)
+{
+    if (!ok) {
+        h = l = make_float4(0.f, 0.f, 0.f, 0.f);
+    } else if (RAW) {
+        const double *x = p.pos + 3 * (size_t)j;
+        const double a = __ldg(x), b = __ldg(x + 1), c = __ldg(x + 2);
+        h = make_float4((float)a, (float)b, (float)c, (float)__ldg(p.mass + j));
+        l = make_float4((float)(a - (double)h.x), (float)(b - (double)h.y),
+                        (float)(c - (double)h.z), 0.f);
+    } else {
+        h = __ldg(static_cast<const float4 *>(p.P) + j);
+        l = __ldg(p.Plo + j);
+    }
+}
+
+template <int I, bool COMP, bool ZEPS, bool RAW>
+__global__ void __launch_bounds__(TEAM_T) force_f32_team_kernel(const ForceParams p)
+{
+    constexpr int NP = I / 2, TI = 32 * I, NV = 3 * TI;
+    __shared__ __align__(16) float4 tile[TEAM_W][2 * 32];
+    __shared__ float2 sums[TEAM_W][NV];  // (sum, carry) pairs
+    __shared__ float2 total[NV];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int cs = p.nsplit;  // blocks of the cluster
+    const int rank = blockIdx.x % cs, i0 = blockIdx.x / cs * TI;
+    const int n = p.n;
+    const int part = rank * TEAM_W + warp, parts = cs * TEAM_W;
+    const int j0 = (int)((long long)n * part / parts), j1 = (int)((long long)n * (part + 1) / parts);
+
+    // the first j-bodies' loads overlap the i-bodies'
+    float4 bh, bl;
+    team_load<RAW>(p, j0 + lane, j0 + lane < j1, bh, bl);
+    float4 h[I], l[I];
+    float sum[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+    for (int k = 0; k < I; ++k) {
+        const int i = i0 + lane + 32 * k;
+        team_load<RAW>(p, i, i < n, h[k], l[k]);
+        sum[0] += h[k].x;
+        sum[1] += h[k].y;
+        sum[2] += h[k].z;
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1)
+#pragma unroll
+        for (int d = 0; d < 3; ++d) sum[d] += __shfl_xor_sync(0xffffffffu, sum[d], off);
+    // The tile's origin: the mean of its bodies.  They are in the caller's
+    // order, so 64 of them span the system; the centre of their bounding box
+    // (the larger kernels' origin) is then thrown about by the outermost
+    // bodies, and 1000 bodies of a Plummer sphere came out at 1.6e-6 of |a|
+    // where they are 1.0e-6 with 256-body tiles.
+    const float inv = 1.0f / (float)min(TI, n - i0);
+    const float3 c = make_float3(sum[0] * inv, sum[1] * inv, sum[2] * inv);
+    float2 nx[NP], ny[NP], nz[NP], ax[NP], ay[NP], az[NP];
+#pragma unroll
+    for (int q = 0; q < NP; ++q) {
+        const float4 a = h[2 * q], b = h[2 * q + 1], al = l[2 * q], b2 = l[2 * q + 1];
+        nx[q] = make_float2(-rel(a.x, al.x, c.x), -rel(b.x, b2.x, c.x));
+        ny[q] = make_float2(-rel(a.y, al.y, c.y), -rel(b.y, b2.y, c.y));
+        nz[q] = make_float2(-rel(a.z, al.z, c.z), -rel(b.z, b2.z, c.z));
+        ax[q] = ay[q] = az[q] = make_float2(0.f, 0.f);
+    }
+    float s[3][I], e[3][I];
+#pragma unroll
+    for (int k = 0; k < I; ++k)
+#pragma unroll
+        for (int d = 0; d < 3; ++d) s[d][k] = e[d][k] = 0.f;
+    auto fold = [&]() {
+#pragma unroll
+        for (int q = 0; q < NP; ++q) {
+            kahan_add(s[0][2 * q], e[0][2 * q], ax[q].x);
+            kahan_add(s[0][2 * q + 1], e[0][2 * q + 1], ax[q].y);
+            kahan_add(s[1][2 * q], e[1][2 * q], ay[q].x);
+            kahan_add(s[1][2 * q + 1], e[1][2 * q + 1], ay[q].y);
+            kahan_add(s[2][2 * q], e[2][2 * q], az[q].x);
+            kahan_add(s[2][2 * q + 1], e[2][2 * q + 1], az[q].y);
+            ax[q] = ay[q] = az[q] = make_float2(0.f, 0.f);
+        }
+    };
+    const float2 e2 = make_float2(p.eps2f, p.eps2f);
+    float4 *t = tile[warp];
+    constexpr int UNR = 8;
+    int since = 0;  // j-bodies since the last fold
+    for (int jb = j0; jb < j1; jb += 32) {
+        const float x = rel(bh.x, bl.x, c.x), y = rel(bh.y, bl.y, c.y), z = rel(bh.z, bl.z, c.z);
+        __syncwarp();  // the last tile has been read
+        t[2 * lane] = make_float4(x, x, y, y);
+        t[2 * lane + 1] = make_float4(z, z, bh.w, bh.w);  // past the end: massless
+        __syncwarp();
+        const int jn = jb + 32 + lane;
+        team_load<RAW>(p, jn, jn < j1, bh, bl);
+        const int cnt = min(32, j1 - jb);
+        for (int q = 0; q < cnt; q += UNR) {
+#pragma unroll
+            for (int u = 0; u < UNR; ++u) {
+                const float4 q0 = t[2 * (q + u)], q1 = t[2 * (q + u) + 1];
+                const float2 xj = make_float2(q0.x, q0.y), yj = make_float2(q0.z, q0.w);
+                const float2 zj = make_float2(q1.x, q1.y), mj = make_float2(q1.z, q1.w);
+#pragma unroll
+                for (int r = 0; r < NP; ++r)
+                    interact2<ZEPS, false>(xj, yj, zj, mj, e2, nx[r], ny[r], nz[r], ax[r], ay[r],
+                                           az[r]);
+            }
+        }
+        if (COMP && (since += 32) == TEAM_FOLD) {
+            fold();
+            since = 0;
+        }
+    }
+    if (COMP) fold();
+#pragma unroll
+    for (int k = 0; k < I; ++k) {
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            const float2 a = d == 0 ? ax[k >> 1] : (d == 1 ? ay[k >> 1] : az[k >> 1]);
+            sums[warp][d * TI + 32 * k + lane] =
+                COMP ? make_float2(s[d][k], e[d][k]) : make_float2((k & 1) ? a.y : a.x, 0.f);
+        }
+    }
+    __syncthreads();
+    // the warps' sums in warp order, then the blocks' in rank order (float32
+    // two-sums: eight float64 sums per value held the float64 pipe 3000 cycles)
+    for (int v = threadIdx.x; v < NV; v += TEAM_T) {
+        float2 a = sums[0][v];
+#pragma unroll
+        for (int w = 1; w < TEAM_W; ++w) kahan_merge(a.x, a.y, sums[w][v].x, sums[w][v].y);
+        total[v] = a;
+    }
+    cg::cluster_group cluster = cg::this_cluster();
+    if (cs > 1)
+        cluster.sync();
+    else
+        __syncthreads();
+    const int v0 = NV * rank / cs, v1 = NV * (rank + 1) / cs;
+    for (int v = v0 + threadIdx.x; v < v1; v += TEAM_T) {
+        float2 b[8];
+#pragma unroll
+        for (int r = 0; r < 8; ++r)
+            if (r < cs) b[r] = cs > 1 ? *cluster.map_shared_rank(total + v, r) : total[v];
+#pragma unroll
+        for (int r = 1; r < 8; ++r)
+            if (r < cs) kahan_merge(b[0].x, b[0].y, b[r].x, b[r].y);
+        const int d = v / TI, k = i0 + v % TI;
+        if (k < n) {
+            const int i = p.perm ? p.perm[k] : k;
+            const double a = p.G * pair_value(b[0]);
+            p.acc[3 * (size_t)i + d] = a;
+            if (p.vel) p.vel[3 * (size_t)i + d] += p.half_dt * a;
+            if (!isfinite(a)) atomicOr(p.err, ERR_NONFINITE);
+        }
+    }
+    if (cs > 1) cluster.sync();  // no block leaves while its sums are being read
+}
+
+#define NB_TEAM_KERNEL(I, C, Z)                                                            \
+    {TEAM_T, I, 32, (const void *)force_f32_team_kernel<I, C, Z, false>, false, 0,         \
+     (const void *)force_f32_team_kernel<I, C, Z, true>}
+#define NB_TEAM_ENTRY(I)                                                                   \
+    {{NB_TEAM_KERNEL(I, false, false), NB_TEAM_KERNEL(I, false, true)},                     \
+     {NB_TEAM_KERNEL(I, true, false), NB_TEAM_KERNEL(I, true, true)}}
+
+const Quad kTeam[] = {NB_TEAM_ENTRY(2), NB_TEAM_ENTRY(4)};
+
+}  // namespace
+
+int f32_team_variants() { return (int)(sizeof(kTeam) / sizeof(kTeam[0])); }
+const KernelEntry &f32_team_kernel(int v, bool comp, bool zeps) { return kTeam[v][comp][zeps]; }
+
+}  // namespace nb

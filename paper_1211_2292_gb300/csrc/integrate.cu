@@ -29,14 +29,14 @@ __device__ __forceinline__ void put(double4 *P, int i, double x, double y, doubl
     P[i] = make_double4(x, y, z, m);
 }
 // float32 hi/lo pair: x = hi + lo with hi = fl(x), lo = fl(x - hi); the lo
-// slot's w carries log2 m for the log-domain pair factor.
+// slot's w carries log2 m for the log-domain pair factor (logm), else 0.
 __device__ __forceinline__ void put_hilo(float4 *P, float4 *Plo, int i, double x, double y,
-                                         double z, double m)
+                                         double z, double m, bool logm)
 {
     const float hx = (float)x, hy = (float)y, hz = (float)z;
     P[i] = make_float4(hx, hy, hz, (float)m);
     Plo[i] = make_float4((float)(x - (double)hx), (float)(y - (double)hy), (float)(z - (double)hz),
-                         (float)log2(m));
+                         logm ? log2_packed(m) : 0.f);
 }
 
 __global__ void pack_kernel(int n, const double *__restrict__ pos, const double *__restrict__ mass,
@@ -48,21 +48,66 @@ __global__ void pack_kernel(int n, const double *__restrict__ pos, const double 
     }
 }
 
+// One body's force from the j-split slots of a float32 force kernel:
+// G * (slots merged in order), into acc.
+__device__ __forceinline__ void merged_force(const MergeParams &g, int i, double (&a)[3])
+{
+    float2 s[3];
+    merge_slots(g.slots + (size_t)i * 3, (size_t)g.n * 3, g.nslots, s);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) a[c] = g.G * ((double)s[c].x - (double)s[c].y);
+    const int b = g.perm ? g.perm[i] : i;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) g.acc[3 * (size_t)b + c] = a[c];
+    if (!finite3(a[0], a[1], a[2])) atomicOr(g.err, 1 /* ERR_NONFINITE */);
+}
+
+// The end of a split force evaluation: a thread per body merges the slots,
+// writes acc and applies the closing half-kick.  A launch of its own rather
+// than the last CTA of each i-tile: that CTA's 128 threads went through
+// nslots x 6 bodies alone at the end of the launch (7 us of 133 at 16384
+// bodies with 7 splits, more with the splits that balance the SMs).
+__global__ void __launch_bounds__(128) merge_kernel(const MergeParams g, double *__restrict__ vel,
+                                                    double half_dt)
+{
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < g.n; i += gridDim.x * blockDim.x) {
+        double a[3];
+        merged_force(g, i, a);
+        if (vel) {
+            const int b = g.perm ? g.perm[i] : i;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) vel[3 * (size_t)b + c] += half_dt * a[c];
+        }
+    }
+}
+
 // Opening half-kick and drift of one leapfrog step, then repack:
 //   v += half_dt * a;  x += dt * v.
-// (x, v) before the update are copied to rec_pos/rec_vel when given.
-template <typename V>
-__global__ void kdp_kernel(int n, double *__restrict__ pos, double *__restrict__ vel,
-                           const double *__restrict__ acc, const double *__restrict__ mass,
-                           double half_dt, double dt, V *__restrict__ P, float4 *__restrict__ Plo,
-                           double *__restrict__ rec_pos, double *__restrict__ rec_vel)
+// (x, v) before the update are copied to rec_pos/rec_vel when given.  MERGE:
+// first the end of the step before, whose force is still in its slots:
+// a = G (slots merged), v += half_dt * a.
+template <typename V, bool MERGE>
+__global__ void __launch_bounds__(MERGE ? 128 : TPB)
+    kdp_kernel(int n, double *__restrict__ pos, double *__restrict__ vel,
+               const double *__restrict__ acc, const double *__restrict__ mass, double half_dt,
+               double dt, V *__restrict__ P, float4 *__restrict__ Plo, bool logm,
+               double *__restrict__ rec_pos, double *__restrict__ rec_vel, const MergeParams g)
 {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         double *x = pos + 3 * (size_t)i;
         double *v = vel + 3 * (size_t)i;
-        const double *a = acc + 3 * (size_t)i;
         double xx = x[0], xy = x[1], xz = x[2];
         double vx = v[0], vy = v[1], vz = v[2];
+        double a[3];
+        if constexpr (MERGE) {
+            merged_force(g, i, a);
+            vx += half_dt * a[0];
+            vy += half_dt * a[1];
+            vz += half_dt * a[2];
+        } else {
+#pragma unroll
+            for (int c = 0; c < 3; ++c) a[c] = acc[3 * (size_t)i + c];
+        }
         if (rec_pos) {
             double *r = rec_pos + 3 * (size_t)i;
             r[0] = xx; r[1] = xy; r[2] = xz;
@@ -80,7 +125,7 @@ __global__ void kdp_kernel(int n, double *__restrict__ pos, double *__restrict__
         v[0] = vx; v[1] = vy; v[2] = vz;
         x[0] = xx; x[1] = xy; x[2] = xz;
         if (Plo)
-            put_hilo((float4 *)P, Plo, i, xx, xy, xz, mass[i]);
+            put_hilo((float4 *)P, Plo, i, xx, xy, xz, mass[i], logm);
         else if (P)
             put(P, i, xx, xy, xz, mass[i]);
     }
@@ -118,7 +163,7 @@ __global__ void pack_vjp_kernel(int n, const double *__restrict__ pos,
             put(PV, 2 * i + 1, coef * l0, coef * l1, coef * l2, 0.0);
         } else {
             float4 *F = reinterpret_cast<float4 *>(PV);
-            put_hilo(F, F + stride, i, x[0], x[1], x[2], mass[i]);
+            put_hilo(F, F + stride, i, x[0], x[1], x[2], mass[i], false);
             put(F + 2 * stride, i, coef * l0, coef * l1, coef * l2, 0.0);
         }
     }
@@ -172,15 +217,27 @@ cudaError_t launch_pack_f64(cudaStream_t s, int n, const double *pos, const doub
 
 cudaError_t launch_kdp(cudaStream_t s, bool f64, int n, double *pos, double *vel,
                        const double *acc, const double *mass, double half_dt, double dt, void *P,
-                       float4 *Plo, double *rec_pos, double *rec_vel)
+                       float4 *Plo, bool logm, double *rec_pos, double *rec_vel,
+                       const MergeParams *merge)
 {
-    if (f64)
-        kdp_kernel<double4><<<grid_for(n), TPB, 0, s>>>(n, pos, vel, acc, mass, half_dt, dt,
-                                                         (double4 *)P, nullptr, rec_pos, rec_vel);
+    if (merge)
+        kdp_kernel<float4, true><<<(n + 127) / 128, 128, 0, s>>>(
+            n, pos, vel, acc, mass, half_dt, dt, (float4 *)P, P ? Plo : nullptr, logm, rec_pos,
+            rec_vel, *merge);
+    else if (f64)
+        kdp_kernel<double4, false><<<grid_for(n), TPB, 0, s>>>(n, pos, vel, acc, mass, half_dt, dt,
+                                                               (double4 *)P, nullptr, false,
+                                                               rec_pos, rec_vel, MergeParams{});
     else
-        kdp_kernel<float4><<<grid_for(n), TPB, 0, s>>>(n, pos, vel, acc, mass, half_dt, dt,
-                                                        (float4 *)P, P ? Plo : nullptr, rec_pos,
-                                                        rec_vel);
+        kdp_kernel<float4, false><<<grid_for(n), TPB, 0, s>>>(
+            n, pos, vel, acc, mass, half_dt, dt, (float4 *)P, P ? Plo : nullptr, logm, rec_pos,
+            rec_vel, MergeParams{});
+    return cudaGetLastError();
+}
+
+cudaError_t launch_merge(cudaStream_t s, const MergeParams &g, double *vel, double half_dt)
+{
+    merge_kernel<<<(g.n + 127) / 128, 128, 0, s>>>(g, vel, half_dt);
     return cudaGetLastError();
 }
 

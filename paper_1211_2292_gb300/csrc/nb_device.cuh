@@ -43,6 +43,65 @@ __device__ __forceinline__ float ex2_mufu(float x)
     return y;
 }
 
+// log2(m) of a float64 mass as float32: m = 2^e f, 1 <= f < 2; with r about 1/f
+// (nine bits, from the top five bits of f) log2 m = e - log2 r + log2(1 + z),
+// z = f r - 1 exact, |z| < 1/60.  -log2 r is tabulated as hi (a multiple of
+// 2^-12, so that e + hi is exact) and lo, log2(1 + z) a polynomial: the result
+// is within half an ulp plus about 2^-29.  Two float64 operations in place of
+// the library's logarithm's dozens: on this part (2 float64 lanes per clock per
+// SM) those took the packing of 2^20 bodies 75 us.
+struct Log2Row {
+    double r;
+    float hi, lo;
+};
+static __device__ const Log2Row LOG2_ROWS[32] = {
+    {0.984375, 0.02270507812f, 1.49983751e-05f},
+    {0.955078125, 0.06640625f, -9.69049522e-05f},
+    {0.927734375, 0.1081542969f, 6.19999067e-05f},
+    {0.90234375, 0.1481933594f, 5.75992089e-05f},
+    {0.876953125, 0.189453125f, -2.47597411e-05f},
+    {0.853515625, 0.228515625f, -5.0945006e-06f},
+    {0.83203125, 0.2653808594f, -9.04796008e-05f},
+    {0.810546875, 0.3029785156f, 5.39581407e-05f},
+    {0.791015625, 0.3381347656f, 8.7136603e-05f},
+    {0.771484375, 0.3742675781f, 2.35788105e-05f},
+    {0.75390625, 0.4074707031f, 7.22596069e-05f},
+    {0.736328125, 0.4416503906f, -7.11038937e-05f},
+    {0.71875, 0.4763183594f, 0.000119684568f},
+    {0.703125, 0.5080566406f, 9.02630453e-05f},
+    {0.6875, 0.5405273438f, 4.10376127e-05f},
+    {0.673828125, 0.5695800781f, -3.26297905e-05f},
+    {0.66015625, 0.5991210938f, -5.30032184e-07f},
+    {0.646484375, 0.6293945312f, -8.19380572e-05f},
+    {0.6328125, 0.66015625f, -6.25288462e-06f},
+    {0.62109375, 0.6870117188f, 0.000105325966f},
+    {0.609375, 0.7145996094f, -1.82823725e-06f},
+    {0.59765625, 0.7426757812f, -6.36239427e-05f},
+    {0.587890625, 0.7663574219f, 2.29013653e-05f},
+    {0.576171875, 0.7954101562f, 1.86995008e-05f},
+    {0.56640625, 0.8200683594f, 2.25506101e-05f},
+    {0.556640625, 0.8452148438f, -3.29528021e-05f},
+    {0.546875, 0.8706054688f, 0.000111514305f},
+    {0.537109375, 0.8967285156f, -1.6324037e-05f},
+    {0.529296875, 0.91796875f, -0.000117791354f},
+    {0.51953125, 0.9448242188f, -0.000106654251f},
+    {0.51171875, 0.9665527344f, 2.42640875e-05f},
+    {0.50390625, 0.9887695312f, 3.21332675e-06f}};
+__device__ __forceinline__ float log2_packed(double m)
+{
+    const int h = __double2hiint(m);
+    if ((unsigned)(h >> 20) - 1u >= 2046u) return (float)log2(m);  // 0, < 0, subnormal, inf, NaN
+    const Log2Row w = LOG2_ROWS[(h >> 15) & 31];
+    const double f = __hiloint2double((h & 0xfffff) | 0x3ff00000, __double2loint(m));
+    const float z = (float)fma(f, w.r, -1.0);
+    // log2(1 + z) = z (c1 + z (c2 + z (c3 + z (c4 + z c5)))), c_k = (-1)^(k+1) / (k ln 2)
+    float q = fmaf(z, 0.288539008f, -0.360673760f);
+    q = fmaf(z, q, 0.480898347f);
+    q = fmaf(z, q, -0.721347520f);
+    q = fmaf(z, q, 1.442695041f);
+    return ((float)((h >> 20) - 1023) + w.hi) + fmaf(z, q, w.lo);
+}
+
 // float64 reciprocal square root: a float32 MUFU seed y0 (relative error
 // e0 < 2^-22) refined by one second-order Householder step for
 // f(y) = 1/y^2 - x.  With e = 1 - x*y0^2 the exact answer is
@@ -133,6 +192,43 @@ __device__ __forceinline__ void kahan_add(float &s, float &c, float p)
     float t = s + y;
     c = (t - s) - y;
     s = t;
+}
+
+// (s, c) += (so, co) for Kahan pairs holding s - c: the sums' rounding
+// error goes into the carry (the two-sum of s and so).
+__device__ __forceinline__ void kahan_merge(float &s, float &c, float so, float co)
+{
+    const float t = s + so;
+    const float bp = t - s;
+    const float e = (s - (t - bp)) + (so - bp);
+    s = t;
+    c = (c + co) - e;
+}
+
+// The three coordinates' pairs of one body over n slots `stride` apart, merged
+// in slot order, eight slots' loads in flight.
+__device__ __forceinline__ void merge_slots(const float2 *slot, size_t stride, int n, float2 (&a)[3])
+{
+#pragma unroll
+    for (int d = 0; d < 3; ++d) a[d] = __ldcg(slot + d);
+    int q = 1;
+    for (; q + 8 <= n; q += 8) {
+        float2 b[8][3];
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+#pragma unroll
+            for (int d = 0; d < 3; ++d) b[u][d] = __ldcg(slot + (q + u) * stride + d);
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+#pragma unroll
+            for (int d = 0; d < 3; ++d) kahan_merge(a[d].x, a[d].y, b[u][d].x, b[u][d].y);
+    }
+    for (; q < n; ++q)
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            const float2 b = __ldcg(slot + q * stride + d);
+            kahan_merge(a[d].x, a[d].y, b.x, b.y);
+        }
 }
 
 // Range of j-tiles [t0, t1) handled by split `js` of `nsplit`.

@@ -29,11 +29,22 @@ struct KernelEntry {
     int J;   // j-bodies per shared-memory tile
     const void *fn;
     bool logm = false;  // float32 kernels with log-domain pairs (read log2 m from P_lo.w)
+    // float32 kernels whose j-splits are equal body counts, not whole j-tiles:
+    // their time per pair, per mille (adjacent to the first compensated one); 0 for the others.
+    int even = 0;
+    // Kernels whose blocks share an i-tile of 32 I bodies in clusters of
+    // nsplit blocks (force_f32_team.cu); `raw` is the form that reads the
+    // caller's float64 arrays.  NULL: T I bodies per block, splits through
+    // `partial`.
+    const void *raw = nullptr;
+    bool team() const { return raw != nullptr; }
+    int64_t tile() const { return team() ? 32 * (int64_t)I : (int64_t)T * I; }
 };
 
 // -------------------------------------------------------------- parameters
 struct ForceParams {
     const void *P;        // packed bodies: float4 (x_hi,y_hi,z_hi,m) or double4 (x,y,z,m)
+    const double *pos, *mass;  // the caller's arrays (kernels that read those instead)
     const float4 *Plo;    // float32 modes: (x_lo,y_lo,z_lo,0), x = x_hi + x_lo
     const int *perm;      // float32 modes: body stored at packed slot k (NULL = identity)
     int n;                // bodies
@@ -44,9 +55,19 @@ struct ForceParams {
     double *acc;          // out [n][3]
     double *vel;          // optional fused half-kick: vel += half_dt * acc
     double half_dt;
-    double *partial;      // [nsplit][n][3] split partial sums (nsplit > 1)
-    unsigned *counters;   // per-i-tile arrival counters, zero between launches
+    double *partial;      // [nsplit][n][3] split partial sums (nsplit > 1): float64, or the
+                          // float32 kernels' (sum, carry) pairs
+    unsigned *counters;   // per-i-tile arrival counters, zero between launches (float64 forms)
     int *err;             // error word
+};
+// The sums a split float32 force launch left in ForceParams::partial.
+struct MergeParams {
+    const float2 *slots;  // [nslots][n][3] (sum, carry)
+    int n, nslots;
+    const int *perm;      // body of packed slot k (NULL = identity)
+    double G;
+    double *acc;
+    int *err;
 };
 
 // One work item of the batched kernel: bodies [i0, i_end) of one system,
@@ -70,7 +91,7 @@ struct BatchParams {
     const BatchItem *items;
     int n_items;
     unsigned *queue;      // [0] next item, [1] CTAs done; both zero between launches
-    double *partial;      // [slots][threads * bodies_per_thread][3] chunk partial sums
+    double *partial;      // [slots][threads * bodies_per_thread][3] chunk sums as (sum, carry) float2
     unsigned *counters;   // per split piece, zero between launches
     float eps2f;
     double G;
@@ -114,6 +135,8 @@ int f32_force_variants_a();
 const KernelEntry &f32_force_kernel_a(int variant, bool comp, bool zeps);
 int f32_force_variants_b();
 const KernelEntry &f32_force_kernel_b(int variant, bool comp, bool zeps);
+int f32_team_variants();
+const KernelEntry &f32_team_kernel(int variant, bool comp, bool zeps);
 int f32_force_variants();
 const KernelEntry &f32_force_kernel(int variant, bool comp, bool zeps);
 int f32_batched_variants();
@@ -157,8 +180,9 @@ cudaError_t launch_tree_sort(cudaStream_t s, int n, const double *pos, OrderScra
 cudaError_t launch_key_sort(cudaStream_t s, int n, const int *k32, const long long *k64,
                             int passes, OrderScratch &o, int *perm_out, int &kernels);
 // Phi[k], Plo[k] = float32 hi/lo packing of body k; Phi.w = m, Plo.w = log2(m).
+// (Plo.w = 0 unless logm)
 cudaError_t launch_pack_hilo(cudaStream_t s, int n, const double *pos, const double *mass,
-                             float4 *Phi, float4 *Plo);
+                             float4 *Phi, float4 *Plo, bool logm);
 
 // ------------------------------------------------------ tree code (tree.cu)
 // Octree over bodies in 30-bit Morton order.  Node arrays hold `cap` entries;
@@ -375,11 +399,16 @@ cudaError_t launch_hi_box(cudaStream_t s, int n, const float4 *P, float *box);
 // P[k] = (x, y, z, m) of body k.
 cudaError_t launch_pack_f64(cudaStream_t s, int n, const double *pos, const double *mass, double4 *P);
 // v += half_dt a; x += dt v; then repack into P (double4) when f64, into the
-// float32 hi/lo pair (P, Plo) otherwise; P == NULL skips the packing.  Records
-// (x, v) before the update when rec_* is set.
+// float32 hi/lo pair (P, Plo) otherwise (Plo.w = log2 m when logm); P == NULL
+// skips the packing.  Records (x, v) before the update when rec_* is set.
+// merge: first ends the step before, whose force is in merge's slots:
+// acc = G (merged slots), v += half_dt a (float32 contexts, input order).
 cudaError_t launch_kdp(cudaStream_t s, bool f64, int n, double *pos, double *vel, const double *acc,
                        const double *mass, double half_dt, double dt, void *P, float4 *Plo,
-                       double *rec_pos, double *rec_vel);
+                       bool logm, double *rec_pos, double *rec_vel,
+                       const MergeParams *merge = nullptr);
+// acc = G (merged slots); vel += half_dt acc when vel.
+cudaError_t launch_merge(cudaStream_t s, const MergeParams &g, double *vel, double half_dt);
 // Adjoint packing: lam_v += drift * lam_x (if lam_x), mu = coef * lam_v, pack (x, m, mu):
 // float64 as double4 pairs at PV[2i], PV[2i+1]; float32 as three float4 arrays
 // PV[i] = (x_hi,y_hi,z_hi,m), PV[stride + i] = (x_lo,..,0), PV[2 stride + i] = (mu,0).

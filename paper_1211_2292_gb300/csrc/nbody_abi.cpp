@@ -165,6 +165,10 @@ int default_variant(int kind, nb_precision p, int64_t n)
 {
     // double-float: 128-body tiles (more CTAs, more compact tiles) below 4096 bodies
     if (kind == nb::KIND_FORCE && p == NB_DF64) return n < 4096 ? 2 : 0;
+    // float32: the team kernels (the table's last two) while blocks of one
+    // thread per body or two leave SMs idle
+    if (kind == nb::KIND_FORCE && !f64_like(p) && n < 8192)
+        return nb::f32_force_variants() - (n < 3000 ? 2 : 1);
     return 0;
 }
 
@@ -208,15 +212,22 @@ cudaEvent_t pooled_event(nb_ctx *c)
     return e;
 }
 
+// Whether launches on s are timed (nb_profile; not inside captures).
+bool timed_now(nb_ctx *c, cudaStream_t s)
+{
+    if (!c->prof_on) return false;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    cudaStreamIsCapturing(s, &cs);
+    return cs == cudaStreamCaptureStatusNone;
+}
 // Launch a pair kernel; `kind` tags its event timing (nb_profile).
+// cluster > 1: in thread-block clusters of that many blocks.
 nb_status launch(nb_ctx *c, const KernelEntry &k, int64_t grid, void *params, cudaStream_t s,
-                 int kind)
+                 int kind, const void *fn = nullptr, int cluster = 1)
 {
     if (grid <= 0) return NB_OK;
     if (grid > 0x7fffffffLL) return failf(c, NB_EINVAL, "grid of %lld CTAs too large", (long long)grid);
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    cudaStreamIsCapturing(s, &cs);
-    const bool timed = c->prof_on && cs == cudaStreamCaptureStatusNone;
+    const bool timed = timed_now(c, s);
     cudaEvent_t ea = nullptr, eb = nullptr;
     if (timed) {
         ea = pooled_event(c);
@@ -224,7 +235,17 @@ nb_status launch(nb_ctx *c, const KernelEntry &k, int64_t grid, void *params, cu
         if (ea && eb) NB_CUDA(c, cudaEventRecord(ea, s));
     }
     void *args[] = {params};
-    NB_CUDA(c, cudaLaunchKernel(k.fn, dim3((unsigned)grid), dim3(k.T), args, 0, s));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(k.T);
+    cfg.stream = s;
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = (unsigned)cluster;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = cluster > 1 ? 1 : 0;
+    NB_CUDA(c, cudaLaunchKernelExC(&cfg, fn ? fn : k.fn, args));
     c->launches++;
     if (timed && ea && eb) {
         NB_CUDA(c, cudaEventRecord(eb, s));
@@ -238,6 +259,29 @@ nb_status launch(nb_ctx *c, const KernelEntry &k, int64_t grid, void *params, cu
         NB_CUDA(ctx, (expr));      \
         (ctx)->launches++;         \
     } while (0)
+
+// Blocks per cluster (1, 2, 4 or 8) of a team kernel over n bodies: the least
+// time of the busiest SM.  Its k blocks' warps go through j j-bodies each in
+// about j max(100, 14 I k) cycles (one block per SM waits on its own latency;
+// 13 I cycles of issue per j-body and block of 8 warps on 4 schedulers).
+// `forced` > 0 is rounded down to a power of two.
+int team_cluster(const nb_ctx *c, const KernelEntry &k, int64_t n, int forced)
+{
+    if (forced > 0) return forced >= 8 ? 8 : (forced >= 4 ? 4 : (forced >= 2 ? 2 : 1));
+    const int64_t tiles = (n + k.tile() - 1) / k.tile(), warps = k.T / 32;
+    int best = 1;
+    int64_t cost = -1;
+    for (int cs = 1; cs <= 8; cs *= 2) {
+        const int64_t blocks = (tiles * cs + c->num_sms - 1) / c->num_sms;
+        const int64_t j = ((n + warps * cs - 1) / (warps * cs) + 31) & ~(int64_t)7;
+        const int64_t w = j * std::max<int64_t>(100, 14 * k.I * blocks) + 200 * cs;
+        if (cost < 0 || w < cost) {
+            cost = w;
+            best = cs;
+        }
+    }
+    return best;
+}
 
 // Number of j-splits for a pair kernel over n bodies (see nb_choose_split).
 int splits_for(nb_ctx *c, const KernelEntry &k, int64_t n, int forced, int64_t per_split_doubles)
@@ -256,6 +300,38 @@ int splits_for(nb_ctx *c, const KernelEntry &k, int64_t n, int forced, int64_t p
     return s < 1 ? 1 : s;
 }
 
+// j-splits of equal body counts for a float32 force kernel (KernelEntry::even)
+// over n bodies, and the cycles they should take.  A launch lasts as long as
+// the scheduler that receives the most warps: the CTAs of the busiest SM, at
+// most ceil(tiles s / SMs), give each of its four schedulers ceil(CTAs T / 128)
+// warps of n / s j-bodies.  Per j-body a warp takes 27.75 cycles per body pair,
+// 31.5 when it is its scheduler's only one; a CTA costs some 60 j-bodies
+// besides, a split launch its merge (its gap, 24 bytes per body-split).  Fitted
+// to every split from 3 to 63 of the four kernels at 11000, 16411 and 24000
+// bodies (within 10 %).  At 16384 bodies that gives 19 splits where whole tiles
+// gave 7, and 111 us for the call instead of 137.
+int even_splits(const nb_ctx *c, const KernelEntry &k, int64_t n, double &cycles)
+{
+    const int64_t tiles = (n + k.tile() - 1) / k.tile();
+    const int64_t cap = c->partial_bodies * 4 / 3;  // body-splits that fit
+    const double rate = k.even * 1e-3 * (k.I / 2);
+    int best = 1;
+    cycles = -1;
+    const int64_t smax = std::min<int64_t>(std::max<int64_t>(n / 64, 1), 256);
+    for (int64_t s = 1; s <= smax && (s == 1 || s * n <= cap); ++s) {
+        const int64_t ctas = (tiles * s + c->num_sms - 1) / c->num_sms;
+        const int64_t warps = (ctas * k.T + 127) / 128;
+        const double w = ((double)((n + s - 1) / s) + 67) * rate *
+                             (warps == 1 ? 31.5 : 27.75 * (double)warps) +
+                         (s > 1 ? 16000 + 0.0025 * (double)(s * n) : 0.0);
+        if (cycles < 0 || w < cycles) {
+            cycles = w;
+            best = (int)s;
+        }
+    }
+    return best;
+}
+
 // float4 slots between the arrays of the float32 pack (hi, lo, cotangent).
 size_t pack_stride(const nb_ctx *c) { return (size_t)std::max<int64_t>(c->n_max, 1); }
 
@@ -263,19 +339,67 @@ size_t pack_stride(const nb_ctx *c) { return (size_t)std::max<int64_t>(c->n_max,
 float4 *lo_half(nb_ctx *c) { return (float4 *)c->pack + pack_stride(c); }
 
 // ------------------------------------------------------------- force paths
-// Force on the already packed bodies; optional fused half-kick of vel.
-nb_status force_packed(nb_ctx *c, cudaStream_t s, int64_t n, double G, double eps, double *acc,
-                       double *vel, double half_dt)
+// Largest system whose team kernel reads the caller's arrays: packing is a
+// launch of its own (3 us with its gap), reading float64 in every block costs
+// the float64 pipe about n / 1000 us.
+constexpr int64_t RAW_MAX = 2048;
+
+bool use_order(const nb_ctx *c, int64_t n);
+
+// The force kernel for n bodies in this context.  The kernels with even splits
+// are one family: where the table names one of them (without a split) and the
+// bodies are in the caller's order, the one that should take the fewest cycles
+// is taken, since 2048-body tiles waste an eighth of 16411 bodies and 1024-body
+// ones a fourteenth.  (In Morton order the tile's size also sets its extent,
+// and with it the rounding of the tile-local coordinates: the table decides.)
+const KernelEntry &force_kernel(nb_ctx *c, int64_t n, double eps, int &forced)
 {
-    if (n == 0) return NB_OK;
-    const bool zeps = eps == 0.0;
-    int v, forced;
+    int v;
     pick(c, nb::KIND_FORCE, n, v, forced);
-    const KernelEntry &k = kernel_for(nb::KIND_FORCE, c->prec, v, zeps);
-    const int S = splits_for(c, k, n, forced, 3);
+    const KernelEntry *k = &kernel_for(nb::KIND_FORCE, c->prec, v, eps == 0.0);
+    if (k->even && forced == 0 && !use_order(c, n)) {
+        double best, w;
+        even_splits(c, *k, n, best);
+        for (int u = 0; u < variant_count(nb::KIND_FORCE, c->prec); ++u) {
+            const KernelEntry &q = kernel_for(nb::KIND_FORCE, c->prec, u, eps == 0.0);
+            if (!q.even) continue;
+            even_splits(c, q, n, w);
+            if (w < best) {
+                best = w;
+                k = &q;
+            }
+        }
+    }
+    return *k;
+}
+bool force_logm(nb_ctx *c, int64_t n, double eps)
+{
+    int forced;
+    return force_kernel(c, n, eps, forced).logm;
+}
+
+// Force on the already packed bodies; optional fused half-kick of vel.  With
+// pos and mass (team kernels only) the bodies are read from those instead.
+// later != NULL: where a split launch's sums are left unmerged (later->nslots
+// > 0) for the caller's next kick and drift to merge.
+nb_status force_packed(nb_ctx *c, cudaStream_t s, int64_t n, double G, double eps, double *acc,
+                       double *vel, double half_dt, const double *pos = nullptr,
+                       const double *mass = nullptr, nb::MergeParams *later = nullptr)
+{
+    if (later) later->nslots = 0;
+    if (n == 0) return NB_OK;
+    int forced;
+    const KernelEntry &k = force_kernel(c, n, eps, forced);
+    const bool f32 = !is_f64(c);
+    double cycles;
+    const int S = k.team()              ? team_cluster(c, k, n, forced)
+                  : k.even && forced == 0 ? even_splits(c, k, n, cycles)
+                                          : splits_for(c, k, n, forced, 3);
     nb::ForceParams p;
     p.P = c->pack;
-    p.Plo = is_f64(c) ? nullptr : lo_half(c);
+    p.pos = pos;
+    p.mass = mass;
+    p.Plo = f32 ? lo_half(c) : nullptr;
     p.perm = c->perm_active ? c->perm : nullptr;
     p.n = (int)n;
     p.nsplit = S;
@@ -288,8 +412,21 @@ nb_status force_packed(nb_ctx *c, cudaStream_t s, int64_t n, double G, double ep
     p.partial = c->partial;
     p.counters = c->counters;
     p.err = c->err;
-    const int64_t tile = (int64_t)k.T * k.I;
-    return launch(c, k, (n + tile - 1) / tile * S, &p, s, 0);
+    const int64_t tile = k.tile();
+    NB_TRY(launch(c, k, (n + tile - 1) / tile * S, &p, s, 0, pos ? k.raw : k.fn,
+                  k.team() ? S : 1));
+    if (f32 && !k.team() && S > 1) {
+        const nb::MergeParams g{reinterpret_cast<const float2 *>(c->partial), (int)n, S, p.perm, G,
+                                acc, c->err};
+        if (later && !p.perm)
+            *later = g;
+        else {
+            NB_LAUNCHED(c, nb::launch_merge(s, g, vel, half_dt));
+            // the merge belongs to the launch's timing
+            if (timed_now(c, s) && !c->prof.empty()) NB_CUDA(c, cudaEventRecord(c->prof.back().b, s));
+        }
+    }
+    return NB_OK;
 }
 
 // Whether force calls with n bodies process them in Morton order: float32
@@ -304,13 +441,14 @@ bool use_order(const nb_ctx *c, int64_t n)
 
 // Pack bodies for a force call: float64 (x,y,z,m) in FP64 mode; float32
 // hi/lo pairs otherwise, in Morton order when use_order() holds (never for
-// the batched kernel, allow_order = false).
+// the batched kernel, allow_order = false).  logm: with log2 m for the
+// log-domain pair kernels.
 nb_status pack(nb_ctx *c, cudaStream_t s, int64_t n, const double *pos, const double *mass,
-               bool allow_order = true)
+               bool logm, bool allow_order = true)
 {
     if (n == 0) return NB_OK;
     c->perm_active = allow_order && use_order(c, n);
-    nb::SortedPack pk{pos, mass, nullptr, nullptr, nullptr, true};
+    nb::SortedPack pk{pos, mass, nullptr, nullptr, nullptr, logm};
     if (is_f64(c))
         pk.P64 = (double4 *)c->pack;
     else
@@ -322,9 +460,26 @@ nb_status pack(nb_ctx *c, cudaStream_t s, int64_t n, const double *pos, const do
     } else if (is_f64(c)) {
         NB_LAUNCHED(c, nb::launch_pack_f64(s, (int)n, pos, mass, pk.P64));
     } else {
-        NB_LAUNCHED(c, nb::launch_pack_hilo(s, (int)n, pos, mass, pk.Phi, pk.Plo));
+        NB_LAUNCHED(c, nb::launch_pack_hilo(s, (int)n, pos, mass, pk.Phi, pk.Plo, logm));
     }
     return NB_OK;
+}
+
+// Force at the caller's positions: pack and sum.
+nb_status force_at(nb_ctx *c, cudaStream_t s, int64_t n, const double *pos, const double *mass,
+                   double G, double eps, double *acc)
+{
+    // (acc may overlap the inputs only when they are packed before it is written)
+    const bool apart = (acc + 3 * n <= pos || pos + 3 * n <= acc) &&
+                       (acc + 3 * n <= mass || mass + n <= acc);
+    int forced;
+    const KernelEntry &k = force_kernel(c, n, eps, forced);
+    if (n <= RAW_MAX && apart && k.team() && !use_order(c, n)) {
+        c->perm_active = false;
+        return force_packed(c, s, n, G, eps, acc, nullptr, 0.0, pos, mass);
+    }
+    NB_TRY(pack(c, s, n, pos, mass, k.logm));
+    return force_packed(c, s, n, G, eps, acc, nullptr, 0.0);
 }
 
 // Forward leapfrog loop (shared by nb_step, nb_rollout and the graph body).
@@ -334,27 +489,28 @@ nb_status rollout_enqueue(nb_ctx *c, cudaStream_t s, int64_t n, double *pos, dou
                           double *rec_vel)
 {
     if (n == 0) return NB_OK;
-    if (!(flags & NB_ACC_VALID)) {
-        NB_TRY(pack(c, s, n, pos, mass));
-        NB_TRY(force_packed(c, s, n, G, eps, acc, nullptr, 0.0));
-    }
+    if (!(flags & NB_ACC_VALID)) NB_TRY(force_at(c, s, n, pos, mass, G, eps, acc));
     const size_t rec = (size_t)n * 3;
-    const bool order = use_order(c, n);
+    const bool order = use_order(c, n), logm = force_logm(c, n, eps);
+    nb::MergeParams left{};  // a step's force still in its splits' slots
     for (int64_t st = 0; st < nsteps; ++st) {
         double *rp = nullptr, *rv = nullptr;
         if (every > 0 && st % every == 0) {
             rp = rec_pos + rec * (size_t)(st / every);
             rv = rec_vel ? rec_vel + rec * (size_t)(st / every) : nullptr;
         }
-        // kick + drift; it also repacks unless the bodies are re-ordered first
+        // (the step before's closing half-kick if it was left,) kick + drift;
+        // it also repacks unless the bodies are re-ordered first
         NB_LAUNCHED(c, nb::launch_kdp(s, is_f64(c), (int)n, pos, vel, acc, mass, 0.5 * dt, dt,
-                                      order ? nullptr : c->pack, lo_half(c), rp, rv));
+                                      order ? nullptr : c->pack, lo_half(c), logm, rp, rv,
+                                      left.nslots ? &left : nullptr));
         if (order) {
-            NB_TRY(pack(c, s, n, pos, mass));
+            NB_TRY(pack(c, s, n, pos, mass, logm));
         } else {
             c->perm_active = false;
         }
-        NB_TRY(force_packed(c, s, n, G, eps, acc, vel, 0.5 * dt));
+        NB_TRY(force_packed(c, s, n, G, eps, acc, vel, 0.5 * dt, nullptr, nullptr,
+                            st + 1 < nsteps ? &left : nullptr));
     }
     if (every > 0 && nsteps % every == 0) {
         const size_t r = (size_t)(nsteps / every);
@@ -426,13 +582,14 @@ nb_status batched_enqueue(nb_ctx *c, cudaStream_t s, double *pos, double *vel, c
 {
     const int64_t n = c->batch_n;
     if (n == 0) return NB_OK;
+    const bool logm = kernel_for(nb::KIND_BATCHED, c->prec, c->batch_variant, eps == 0.0).logm;
     if (!(flags & NB_ACC_VALID)) {
-        NB_TRY(pack(c, s, n, pos, mass, false));
+        NB_TRY(pack(c, s, n, pos, mass, logm, false));
         NB_TRY(batched_force(c, s, G, eps, acc, nullptr, 0.0));
     }
     for (int64_t st = 0; st < nsteps; ++st) {
         NB_LAUNCHED(c, nb::launch_kdp(s, false, (int)n, pos, vel, acc, mass, 0.5 * dt, dt, c->pack,
-                                      lo_half(c), nullptr, nullptr));
+                                      lo_half(c), logm, nullptr, nullptr));
         NB_TRY(batched_force(c, s, G, eps, acc, vel, 0.5 * dt));
     }
     return NB_OK;
@@ -925,7 +1082,7 @@ nb_status tree_step_enqueue(nb_ctx *c, cudaStream_t s, int64_t n, double *pos, d
                                    nullptr, 0.0, nullptr));
     for (int64_t st = 0; st < nsteps; ++st) {
         NB_LAUNCHED(c, nb::launch_kdp(s, is_f64(c), (int)n, pos, vel, acc, mass, 0.5 * dt, dt,
-                                      nullptr, nullptr, nullptr, nullptr));
+                                      nullptr, nullptr, false, nullptr, nullptr));
         NB_TRY(tree_forces_enqueue(c, s, n, pos, mass, G, eps, theta, leaf_cap, group, acc, vel,
                                    0.5 * dt, nullptr));
     }
@@ -1212,8 +1369,7 @@ nb_status nb_forces(nb_ctx *c, int64_t n, const double *pos, const double *mass,
     NB_TRY(check_dev(c, mass, v1, "mass"));
     NB_TRY(check_dev(c, acc, v3, "acc"));
     if (n == 0) return NB_OK;
-    NB_TRY(pack(c, c->stream, n, pos, mass));
-    return force_packed(c, c->stream, n, G, eps, acc, nullptr, 0.0);
+    return force_at(c, c->stream, n, pos, mass, G, eps, acc);
 }
 
 nb_status nb_rollout(nb_ctx *c, int64_t n, double *pos, double *vel, const double *mass, double G,
@@ -1440,7 +1596,8 @@ nb_status nb_forces_batched(nb_ctx *c, const double *pos, const double *mass, do
     NB_TRY(check_dev(c, mass, v1, "mass"));
     NB_TRY(check_dev(c, acc, v3, "acc"));
     if (n == 0) return NB_OK;
-    NB_TRY(pack(c, c->stream, n, pos, mass, false));
+    const bool logm = kernel_for(nb::KIND_BATCHED, c->prec, c->batch_variant, eps == 0.0).logm;
+    NB_TRY(pack(c, c->stream, n, pos, mass, logm, false));
     return batched_force(c, c->stream, G, eps, acc, nullptr, 0.0);
 }
 
@@ -1658,7 +1815,7 @@ nb_status nb_fmm_step(nb_ctx *c, int64_t n, double *pos, double *vel, const doub
         NB_TRY(fmm_forces_run(c, n, pos, mass, G, eps, theta, order, leaf_cap, acc, nullptr));
     for (int64_t st = 0; st < nsteps; ++st) {
         NB_LAUNCHED(c, nb::launch_kdp(c->stream, is_f64(c), (int)n, pos, vel, acc, mass, 0.5 * dt,
-                                      dt, nullptr, nullptr, nullptr, nullptr));
+                                      dt, nullptr, nullptr, false, nullptr, nullptr));
         NB_TRY(fmm_forces_run(c, n, pos, mass, G, eps, theta, order, leaf_cap, acc, nullptr, vel,
                               0.5 * dt));
     }

@@ -8,7 +8,7 @@
 // them, because creating a context allocates its scratch.
 //
 // How: the scratch the kernel needs (packed hi/lo bodies, j-split partial
-// sums, arrival counters, an error word) lives in one file-scope
+// sums, an error word) lives in one file-scope
 // __device__ array of fixed size, which every GPU that loads the library
 // holds until the process exits.  Host code cannot use the array's name as a
 // device address.  The first call made in a CUDA context (with that context
@@ -32,15 +32,13 @@ namespace {
 
 constexpr int64_t kMaxBodies = NB_NOALLOC_MAX_BODIES;
 constexpr int64_t kMaxSplitBodies = 4 * kMaxBodies;  // sum over splits of partial rows
-constexpr int kMaxCounters = 1024;
 constexpr int kVariant = 2;  // (128 threads, 8 bodies/thread, j-tile 128)
 
 // Byte layout of the static scratch.
 constexpr size_t kPackBytes = (size_t)kMaxBodies * 2 * sizeof(float4);  // hi + lo
 constexpr size_t kPartialOff = kPackBytes;
 constexpr size_t kPartialBytes = (size_t)kMaxSplitBodies * 3 * sizeof(double);
-constexpr size_t kCountersOff = kPartialOff + kPartialBytes;
-constexpr size_t kErrOff = kCountersOff + kMaxCounters * sizeof(unsigned);
+constexpr size_t kErrOff = kPartialOff + kPartialBytes;
 constexpr size_t kScratchBytes = kErrOff + 256;
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
@@ -173,7 +171,6 @@ extern "C" nb_status nb_forces_noalloc(int64_t n, const double *pos, const doubl
     float4 *Phi = (float4 *)base;
     float4 *Plo = Phi + kMaxBodies;
     double *partial = (double *)(base + kPartialOff);
-    unsigned *counters = (unsigned *)(base + kCountersOff);
     int *err = (int *)(base + kErrOff);
 
     const nb::KernelEntry &k = nb::f32_force_kernel(kVariant, true, eps == 0.0);
@@ -190,11 +187,10 @@ extern "C" nb_status nb_forces_noalloc(int64_t n, const double *pos, const doubl
     while (S > 1 && (int64_t)S * n > kMaxSplitBodies) --S;
     if (S < 1) S = 1;
 
-    // The counters and the error word must start at zero; clear them here
-    // rather than trusting the previous call's contents.
-    cudaError_t e = cudaMemsetAsync(counters, 0, (size_t)n_itiles * sizeof(unsigned), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(err, 0, sizeof(int), s);
-    if (e == cudaSuccess) e = nb::launch_pack_hilo(s, (int)n, pos, mass, Phi, Plo);
+    // The error word must start at zero; clear it here rather than trusting
+    // the previous call's contents.
+    cudaError_t e = cudaMemsetAsync(err, 0, sizeof(int), s);
+    if (e == cudaSuccess) e = nb::launch_pack_hilo(s, (int)n, pos, mass, Phi, Plo, k.logm);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return fail(NB_ECUDA, "memset or pack launch failed");
@@ -203,6 +199,7 @@ extern "C" nb_status nb_forces_noalloc(int64_t n, const double *pos, const doubl
     nb::ForceParams p;
     p.P = Phi;
     p.Plo = Plo;
+    p.pos = p.mass = nullptr;
     p.perm = nullptr;
     p.n = (int)n;
     p.nsplit = S;
@@ -213,7 +210,7 @@ extern "C" nb_status nb_forces_noalloc(int64_t n, const double *pos, const doubl
     p.vel = nullptr;
     p.half_dt = 0.0;
     p.partial = partial;
-    p.counters = counters;
+    p.counters = nullptr;
     p.err = err;
     void *args[] = {&p};
     e = cudaLaunchKernel(k.fn, dim3((unsigned)(n_itiles * S)), dim3(k.T), args, 0, s);
@@ -221,7 +218,15 @@ extern "C" nb_status nb_forces_noalloc(int64_t n, const double *pos, const doubl
         cudaGetLastError();
         return fail(NB_ECUDA, "force kernel launch failed");
     }
+    if (S > 1) {
+        const nb::MergeParams g{reinterpret_cast<const float2 *>(partial), (int)n, S, nullptr, G, acc,
+                                err};
+        e = nb::launch_merge(s, g, nullptr, 0.0);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            return fail(NB_ECUDA, "merge launch failed");
+        }
+    }
     return NB_OK;
 }
 
-static_assert(kMaxBodies / 256 + 1 <= kMaxCounters, "counter scratch too small");

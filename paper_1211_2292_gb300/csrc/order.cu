@@ -271,7 +271,7 @@ __device__ __forceinline__ void put_body(const SortedPack &p, size_t k, int i)
         const double m = p.mass[i];
         p.Phi[k] = make_float4(hx, hy, hz, (float)m);
         p.Plo[k] = make_float4((float)(x[0] - (double)hx), (float)(x[1] - (double)hy),
-                               (float)(x[2] - (double)hz), p.logm ? (float)log2(m) : 0.f);
+                               (float)(x[2] - (double)hz), p.logm ? log2_packed(m) : 0.f);
     } else if (p.P64) {
         const double *x = p.pos + 3 * (size_t)i;
         p.P64[k] = make_double4(x[0], x[1], x[2], p.mass[i]);
@@ -517,10 +517,10 @@ cudaError_t launch_key_sort(cudaStream_t s, int n, const int *k32, const long lo
 }
 
 cudaError_t launch_pack_hilo(cudaStream_t s, int n, const double *pos, const double *mass,
-                             float4 *Phi, float4 *Plo)
+                             float4 *Phi, float4 *Plo, bool logm)
 {
     if (n <= 0) return cudaSuccess;
-    pack_hilo_kernel<<<grid_for(n), OTPB, 0, s>>>(n, SortedPack{pos, mass, Phi, Plo, nullptr, true});
+    pack_hilo_kernel<<<grid_for(n), OTPB, 0, s>>>(n, SortedPack{pos, mass, Phi, Plo, nullptr, logm});
     return cudaGetLastError();
 }
 

@@ -1,0 +1,87 @@
+"""Direct sums of small systems: the team kernels, and j-splits of equal body counts."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_1211_2292_gb300 import inputs, nbody
+from helpers import host, relerr_per_body, to_dev
+
+pytestmark = pytest.mark.gpu
+
+# float32 pair terms, compensated sums: the mode's bounds, rms 1e-5 and max 1e-4
+BOUND = (1e-5, 1e-4)
+
+
+def _check(a, b, eps):
+    err = relerr_per_body(host(a), oracle.accel(b.pos, b.mass, 1.0, eps))
+    assert np.sqrt(np.mean(err ** 2)) <= BOUND[0] and err.max() <= BOUND[1]
+
+
+@pytest.mark.parametrize("variant", [-2, -1])  # the table's last two: 64 and 128 bodies per block
+@pytest.mark.parametrize("n", [1, 7, 63, 64, 65, 129, 2047, 2048, 2049, 5003])
+def test_team_kernels_at_tile_and_cluster_edges(cuda, variant, n):
+    # 2048 bodies is the largest system read straight from float64
+    b = inputs.random_system(n, seed=n)
+    v = len(nbody.variants(nbody.KIND_FORCE, "fp32_comp")) + variant
+    x, m = to_dev(b.pos, cuda), to_dev(b.mass, cuda)
+    with nbody.NBody(n, "fp32_comp") as nb:
+        for eps, split in ((0.02, 0), (0.02, 1), (0.0, 2), (0.02, 8)):
+            nb.tune_set(nbody.KIND_FORCE, 0, 1 << 40, v, split)
+            a = nb.forces(x, m, 1.0, eps)
+            again = nb.forces(x, m, 1.0, eps)
+            nb.sync()
+            assert np.array_equal(host(a), host(again))
+            if n > 1:
+                _check(a, b, eps)
+            else:
+                assert np.array_equal(host(a), np.zeros((1, 3)))
+
+
+def test_output_may_overlap_the_positions(cuda):
+    # acc written over pos: the bodies are packed before anything is written
+    b = inputs.plummer(700, seed=3)
+    x, m = to_dev(b.pos, cuda), to_dev(b.mass, cuda)
+    with nbody.NBody(b.n, "fp32_comp") as nb:
+        want = host(nb.forces(x, m, 1.0, 0.01))
+        got = host(nb.forces(x, m, 1.0, 0.01, out=x))
+    assert np.array_equal(got, want)
+
+
+@pytest.mark.parametrize("variant", [5, 21, 22, 23, 24])  # 21..24 split by bodies, 5 by tiles
+@pytest.mark.parametrize("n", [65, 4097, 9001, 16411])
+def test_even_splits_and_their_merge(cuda, variant, n):
+    b = inputs.plummer(n, seed=n)
+    x, m = to_dev(b.pos, cuda), to_dev(b.mass, cuda)
+    with nbody.NBody(n, "fp32_comp") as nb:
+        nb.tune_set(nbody.KIND_FORCE, 0, 1 << 40, variant, 0)
+        a = nb.forces(x, m, 1.0, 0.01)
+        _check(a, b, 0.01)
+        # three steps (merges fused with the next kick) against three calls of
+        # one step (merges of their own): the same operations
+        run = []
+        for calls in ([3], [1, 1, 1]):
+            p, v, acc = to_dev(b.pos, cuda), to_dev(b.vel, cuda), a.clone()
+            for k in calls:
+                nb.step(p, v, m, 1.0, 0.01, 1e-3, k, acc, acc_valid=True)
+            run.append((host(p), host(v), host(acc)))
+        nb.sync()
+    for p, q in zip(*run):
+        assert np.array_equal(p, q)
+
+
+def test_masses_in_the_log_domain(cuda):
+    # variant 8 takes every pair as 2^(log2 m - 1.5 log2 r^2): masses over many
+    # binades, zero and subnormal ones among them
+    n = 600
+    b = inputs.random_system(n, seed=4)
+    rng = np.random.default_rng(5)
+    mass = rng.uniform(1.0, 2.0, n) * 2.0 ** rng.integers(-30, 30, n)
+    mass[:3] = [0.0, 5e-310, 1.0]
+    ref = oracle.accel(b.pos, mass, 1.0, 0.05)
+    with nbody.NBody(n, "fp32_comp") as nb:
+        nb.tune_set(nbody.KIND_FORCE, 0, 1 << 40, 8, 0)
+        a = nb.forces(to_dev(b.pos, cuda), torch.as_tensor(mass, device=cuda), 1.0, 0.05)
+        nb.sync()
+    err = relerr_per_body(host(a), ref)
+    assert np.sqrt(np.mean(err ** 2)) <= BOUND[0] and err.max() <= BOUND[1]
