@@ -518,7 +518,9 @@ __global__ void __launch_bounds__(T) force_f32_batched_kernel(const BatchParams 
                 const float2 *base = part + (size_t)it.pbase * TILE_I * 3;
                 for (int q = threadIdx.x; q < it.i_end - it.i0; q += T) {
                     float2 a[3];
-                    merge_slots(base + (size_t)q * 3, (size_t)TILE_I * 3, it.nchunks, a);
+#pragma unroll
+                    for (int d = 0; d < 3; ++d)
+                        a[d] = merge_slots(base + (size_t)q * 3 + d, (size_t)TILE_I * 3, it.nchunks);
                     batch_write(p, it.i0 + q, pair_value(a[0]), pair_value(a[1]), pair_value(a[2]));
                 }
                 if (threadIdx.x == 0) p.counters[it.ctr] = 0u;

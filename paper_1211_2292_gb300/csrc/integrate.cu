@@ -48,37 +48,30 @@ __global__ void pack_kernel(int n, const double *__restrict__ pos, const double 
     }
 }
 
-// One body's force from the j-split slots of a float32 force kernel:
-// G * (slots merged in order), into acc.
-__device__ __forceinline__ void merged_force(const MergeParams &g, int i, double (&a)[3])
+// One coordinate (index i = 3 body + axis, in packed order) of the force from a
+// float32 force kernel's j-split slots: G * (slots merged in order).
+__device__ __forceinline__ double merged_force(const MergeParams &g, size_t i)
 {
-    float2 s[3];
-    merge_slots(g.slots + (size_t)i * 3, (size_t)g.n * 3, g.nslots, s);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) a[c] = g.G * ((double)s[c].x - (double)s[c].y);
-    const int b = g.perm ? g.perm[i] : i;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) g.acc[3 * (size_t)b + c] = a[c];
-    if (!finite3(a[0], a[1], a[2])) atomicOr(g.err, 1 /* ERR_NONFINITE */);
+    const float2 s = merge_slots(g.slots + i, (size_t)g.n * 3, g.nslots);
+    const double a = g.G * ((double)s.x - (double)s.y);
+    if (!isfinite(a)) atomicOr(g.err, (int)ERR_NONFINITE);
+    return a;
 }
 
-// The end of a split force evaluation: a thread per body merges the slots,
-// writes acc and applies the closing half-kick.  A launch of its own rather
-// than the last CTA of each i-tile: that CTA's 128 threads went through
-// nslots x 6 bodies alone at the end of the launch (7 us of 133 at 16384
-// bodies with 7 splits, more with the splits that balance the SMs).
+// The end of a split force evaluation: a thread per coordinate merges the
+// slots, writes acc and applies the closing half-kick.  A launch of its own
+// rather than the last CTA of each i-tile, whose 128 threads went through
+// nslots x 6 bodies alone at the end of the launch; a thread per body took
+// 9.2 us at 16384 bodies and 19 slots (dependent batches of loads).
 __global__ void __launch_bounds__(128) merge_kernel(const MergeParams g, double *__restrict__ vel,
                                                     double half_dt)
 {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < g.n; i += gridDim.x * blockDim.x) {
-        double a[3];
-        merged_force(g, i, a);
-        if (vel) {
-            const int b = g.perm ? g.perm[i] : i;
-#pragma unroll
-            for (int c = 0; c < 3; ++c) vel[3 * (size_t)b + c] += half_dt * a[c];
-        }
-    }
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= 3ll * g.n) return;
+    const double a = merged_force(g, (size_t)i);
+    const size_t b = g.perm ? 3 * (size_t)g.perm[i / 3] + (size_t)(i % 3) : (size_t)i;
+    g.acc[b] = a;
+    if (vel) vel[b] += half_dt * a;
 }
 
 // Opening half-kick and drift of one leapfrog step, then repack:
@@ -86,28 +79,50 @@ __global__ void __launch_bounds__(128) merge_kernel(const MergeParams g, double 
 // (x, v) before the update are copied to rec_pos/rec_vel when given.  MERGE:
 // first the end of the step before, whose force is still in its slots:
 // a = G (slots merged), v += half_dt * a.
-template <typename V, bool MERGE>
-__global__ void __launch_bounds__(MERGE ? 128 : TPB)
-    kdp_kernel(int n, double *__restrict__ pos, double *__restrict__ vel,
-               const double *__restrict__ acc, const double *__restrict__ mass, double half_dt,
-               double dt, V *__restrict__ P, float4 *__restrict__ Plo, bool logm,
-               double *__restrict__ rec_pos, double *__restrict__ rec_vel, const MergeParams g)
+// MERGE takes 96 threads (32 bodies) a block, a thread per coordinate, whose
+// new positions meet in shared memory for the packing.
+constexpr int KM_T = 96;
+__global__ void __launch_bounds__(KM_T)
+    kdp_merge_kernel(int n, double *__restrict__ pos, double *__restrict__ vel,
+                     const double *__restrict__ mass, double half_dt, double dt,
+                     float4 *__restrict__ P, float4 *__restrict__ Plo, bool logm,
+                     double *__restrict__ rec_pos, double *__restrict__ rec_vel,
+                     const MergeParams g)
+{
+    __shared__ double xs[KM_T];
+    const size_t i = (size_t)blockIdx.x * KM_T + threadIdx.x;
+    if (i < 3 * (size_t)n) {
+        double x = pos[i], v = vel[i];
+        const double a = merged_force(g, i);
+        g.acc[i] = a;
+        v += half_dt * a;
+        if (rec_pos) rec_pos[i] = x;
+        if (rec_vel) rec_vel[i] = v;
+        v += half_dt * a;
+        x += dt * v;
+        vel[i] = v;
+        pos[i] = x;
+        xs[threadIdx.x] = x;
+    }
+    __syncthreads();
+    const int b = blockIdx.x * (KM_T / 3) + threadIdx.x;
+    if (threadIdx.x < KM_T / 3 && b < n && P)
+        put_hilo(P, Plo, b, xs[3 * threadIdx.x], xs[3 * threadIdx.x + 1], xs[3 * threadIdx.x + 2],
+                 mass[b], logm);
+}
+
+template <typename V>
+__global__ void kdp_kernel(int n, double *__restrict__ pos, double *__restrict__ vel,
+                           const double *__restrict__ acc, const double *__restrict__ mass,
+                           double half_dt, double dt, V *__restrict__ P, float4 *__restrict__ Plo,
+                           bool logm, double *__restrict__ rec_pos, double *__restrict__ rec_vel)
 {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         double *x = pos + 3 * (size_t)i;
         double *v = vel + 3 * (size_t)i;
+        const double *a = acc + 3 * (size_t)i;
         double xx = x[0], xy = x[1], xz = x[2];
         double vx = v[0], vy = v[1], vz = v[2];
-        double a[3];
-        if constexpr (MERGE) {
-            merged_force(g, i, a);
-            vx += half_dt * a[0];
-            vy += half_dt * a[1];
-            vz += half_dt * a[2];
-        } else {
-#pragma unroll
-            for (int c = 0; c < 3; ++c) a[c] = acc[3 * (size_t)i + c];
-        }
         if (rec_pos) {
             double *r = rec_pos + 3 * (size_t)i;
             r[0] = xx; r[1] = xy; r[2] = xz;
@@ -221,23 +236,22 @@ cudaError_t launch_kdp(cudaStream_t s, bool f64, int n, double *pos, double *vel
                        const MergeParams *merge)
 {
     if (merge)
-        kdp_kernel<float4, true><<<(n + 127) / 128, 128, 0, s>>>(
-            n, pos, vel, acc, mass, half_dt, dt, (float4 *)P, P ? Plo : nullptr, logm, rec_pos,
-            rec_vel, *merge);
+        kdp_merge_kernel<<<(unsigned)((3 * (int64_t)n + KM_T - 1) / KM_T), KM_T, 0, s>>>(
+            n, pos, vel, mass, half_dt, dt, (float4 *)P, Plo, logm, rec_pos, rec_vel, *merge);
     else if (f64)
-        kdp_kernel<double4, false><<<grid_for(n), TPB, 0, s>>>(n, pos, vel, acc, mass, half_dt, dt,
-                                                               (double4 *)P, nullptr, false,
-                                                               rec_pos, rec_vel, MergeParams{});
+        kdp_kernel<double4><<<grid_for(n), TPB, 0, s>>>(n, pos, vel, acc, mass, half_dt, dt,
+                                                         (double4 *)P, nullptr, false, rec_pos,
+                                                         rec_vel);
     else
-        kdp_kernel<float4, false><<<grid_for(n), TPB, 0, s>>>(
-            n, pos, vel, acc, mass, half_dt, dt, (float4 *)P, P ? Plo : nullptr, logm, rec_pos,
-            rec_vel, MergeParams{});
+        kdp_kernel<float4><<<grid_for(n), TPB, 0, s>>>(n, pos, vel, acc, mass, half_dt, dt,
+                                                        (float4 *)P, P ? Plo : nullptr, logm,
+                                                        rec_pos, rec_vel);
     return cudaGetLastError();
 }
 
 cudaError_t launch_merge(cudaStream_t s, const MergeParams &g, double *vel, double half_dt)
 {
-    merge_kernel<<<(g.n + 127) / 128, 128, 0, s>>>(g, vel, half_dt);
+    merge_kernel<<<(unsigned)((3 * (int64_t)g.n + 127) / 128), 128, 0, s>>>(g, vel, half_dt);
     return cudaGetLastError();
 }
 

@@ -205,30 +205,21 @@ __device__ __forceinline__ void kahan_merge(float &s, float &c, float so, float 
     c = (c + co) - e;
 }
 
-// The three coordinates' pairs of one body over n slots `stride` apart, merged
-// in slot order, eight slots' loads in flight.
-__device__ __forceinline__ void merge_slots(const float2 *slot, size_t stride, int n, float2 (&a)[3])
+// One (sum, carry) pair over n slots `stride` apart, merged in slot order, 16
+// slots' loads in flight.
+__device__ __forceinline__ float2 merge_slots(const float2 *slot, size_t stride, int n)
 {
+    float2 a = __ldcg(slot);
+    for (int q = 1; q < n; q += 16) {
+        float2 b[16];
 #pragma unroll
-    for (int d = 0; d < 3; ++d) a[d] = __ldcg(slot + d);
-    int q = 1;
-    for (; q + 8 <= n; q += 8) {
-        float2 b[8][3];
+        for (int u = 0; u < 16; ++u)
+            b[u] = q + u < n ? __ldcg(slot + (size_t)(q + u) * stride) : make_float2(0.f, 0.f);
 #pragma unroll
-        for (int u = 0; u < 8; ++u)
-#pragma unroll
-            for (int d = 0; d < 3; ++d) b[u][d] = __ldcg(slot + (q + u) * stride + d);
-#pragma unroll
-        for (int u = 0; u < 8; ++u)
-#pragma unroll
-            for (int d = 0; d < 3; ++d) kahan_merge(a[d].x, a[d].y, b[u][d].x, b[u][d].y);
+        for (int u = 0; u < 16; ++u)
+            if (q + u < n) kahan_merge(a.x, a.y, b[u].x, b[u].y);
     }
-    for (; q < n; ++q)
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            const float2 b = __ldcg(slot + q * stride + d);
-            kahan_merge(a[d].x, a[d].y, b.x, b.y);
-        }
+    return a;
 }
 
 // Range of j-tiles [t0, t1) handled by split `js` of `nsplit`.

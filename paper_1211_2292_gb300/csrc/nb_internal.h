@@ -153,7 +153,7 @@ const KernelEntry &f64_vjp_kernel(int variant, bool zeps);
 
 // -------------------------------------------------- spatial order (order.cu)
 struct OrderScratch {
-    double *box;        // [1024][6]: bounding-box partials
+    long long *box;     // [1024][6]: bounding-box partials (order-preserving integer images)
     unsigned *keys[2];  // [n] Morton keys (ping-pong)
     int *vals[2];       // [n] body indices (ping-pong)
     unsigned *hist;     // sort_hist_entries: per pass [tiles][256] digit counts, then digit totals

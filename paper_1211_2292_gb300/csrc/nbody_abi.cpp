@@ -743,7 +743,7 @@ nb_status ensure_order(nb_ctx *c)
     if (c->order.hist) return NB_OK;
     nb_status st = NB_OK;
     const size_t nc = (size_t)std::max<int64_t>(c->n_max, 1);
-    if (!c->order.box) c->order.box = dev_alloc<double>(c, 1024 * 6, st);
+    if (!c->order.box) c->order.box = dev_alloc<long long>(c, 1024 * 6, st);
     for (int q = 0; q < 2 && st == NB_OK; ++q) {
         if (!c->order.keys[q]) c->order.keys[q] = dev_alloc<unsigned>(c, nc, st);
         if (st == NB_OK && !c->order.vals[q]) c->order.vals[q] = dev_alloc<int>(c, nc, st);
@@ -1299,7 +1299,7 @@ nb_status nb_create(nb_ctx **out, int64_t n_max, nb_precision p, int device, voi
     if (p != NB_FP64) {  // Morton-order scratch for the float32 kernels
         const size_t nc = (size_t)ncap;
         if (st == NB_OK) c->perm = dev_alloc<int>(c, nc, st);
-        if (st == NB_OK) c->order.box = dev_alloc<double>(c, 1024 * 6, st);
+        if (st == NB_OK) c->order.box = dev_alloc<long long>(c, 1024 * 6, st);
         for (int q = 0; q < 2 && st == NB_OK; ++q) {
             c->order.keys[q] = dev_alloc<unsigned>(c, nc, st);
             if (st == NB_OK) c->order.vals[q] = dev_alloc<int>(c, nc, st);

@@ -38,61 +38,98 @@ __device__ __forceinline__ unsigned spread8(unsigned v)
     return v;
 }
 
-// Per-block min/max of the positions: parts[b] = {minx,miny,minz,maxx,maxy,maxz}.
-__global__ void __launch_bounds__(OTPB) bbox_kernel(int n, const double *__restrict__ pos,
-                                                     double *__restrict__ parts)
+// Order-preserving 64-bit integer image of a float64 (and back): the boxes'
+// minima and maxima are taken on the integer pipe (the float64 pipe has 2
+// lanes per clock per SM).
+__device__ __forceinline__ long long order_image(double v)
 {
-    __shared__ double sh[6][OTPB];
-    double mn[3] = {DBL_MAX, DBL_MAX, DBL_MAX}, mx[3] = {-DBL_MAX, -DBL_MAX, -DBL_MAX};
+    const long long b = __double_as_longlong(v);
+    return b ^ ((b >> 63) & 0x7fffffffffffffffLL);
+}
+__device__ __forceinline__ double from_image(long long b)
+{
+    return __longlong_as_double(b ^ ((b >> 63) & 0x7fffffffffffffffLL));
+}
+constexpr long long IMAGE_INF = 0x7ff0000000000000LL;  // of +infinity; NaNs lie beyond +-it
+constexpr long long IMAGE_MAX = 0x7fefffffffffffffLL;  // of DBL_MAX; ~ gives -DBL_MAX's
+
+// Box of the warp's lanes in every lane: mn, mx of each component.
+__device__ __forceinline__ void warp_box(long long (&mn)[3], long long (&mx)[3])
+{
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            mn[c] = min(mn[c], __shfl_xor_sync(0xffffffffu, mn[c], off));
+            mx[c] = max(mx[c], __shfl_xor_sync(0xffffffffu, mx[c], off));
+        }
+    }
+}
+
+// Per-block min/max of the positions (NaNs left out), as images:
+// parts[b] = {minx,miny,minz,maxx,maxy,maxz}.
+__global__ void __launch_bounds__(OTPB) bbox_kernel(int n, const double *__restrict__ pos,
+                                                     long long *__restrict__ parts)
+{
+    __shared__ long long sh[OTPB / 32][6];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    long long mn[3], mx[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        mn[c] = IMAGE_MAX;
+        mx[c] = ~IMAGE_MAX;
+    }
+#pragma unroll 2
     for (int i = blockIdx.x * OTPB + threadIdx.x; i < n; i += gridDim.x * OTPB) {
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            const double v = pos[3 * (size_t)i + c];
-            mn[c] = fmin(mn[c], v);
-            mx[c] = fmax(mx[c], v);
-        }
-    }
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        sh[c][threadIdx.x] = mn[c];
-        sh[3 + c][threadIdx.x] = mx[c];
-    }
-    __syncthreads();
-    for (int w = OTPB / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) {
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                sh[c][threadIdx.x] = fmin(sh[c][threadIdx.x], sh[c][threadIdx.x + w]);
-                sh[3 + c][threadIdx.x] = fmax(sh[3 + c][threadIdx.x], sh[3 + c][threadIdx.x + w]);
+            const long long v = order_image(pos[3 * (size_t)i + c]);
+            if (v <= IMAGE_INF && v >= ~IMAGE_INF) {
+                mn[c] = min(mn[c], v);
+                mx[c] = max(mx[c], v);
             }
         }
-        __syncthreads();
     }
-    if (threadIdx.x < 6) parts[6 * (size_t)blockIdx.x + threadIdx.x] = sh[threadIdx.x][0];
+    warp_box(mn, mx);
+    if (lane == 0) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            sh[warp][c] = mn[c];
+            sh[warp][3 + c] = mx[c];
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < 6) {
+        long long v = sh[0][threadIdx.x];
+#pragma unroll
+        for (int w = 1; w < OTPB / 32; ++w)
+            v = threadIdx.x < 3 ? min(v, sh[w][threadIdx.x]) : max(v, sh[w][threadIdx.x]);
+        parts[6 * (size_t)blockIdx.x + threadIdx.x] = v;
+    }
 }
 
 // The box {min x,y,z, max x,y,z} of the partials, folded by every block for
 // itself (at most MAX_BOX_PARTS x 48 bytes from L2, ~1 us; a launch of its own
 // took as long and its gap more).
-__device__ __forceinline__ void fold_box(const double *__restrict__ parts, int nparts,
+__device__ __forceinline__ void fold_box(const long long *__restrict__ parts, int nparts,
                                          double (&box)[6])
 {
     __shared__ double sh[6];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (warp < 6) {
         const bool is_min = warp < 3;
-        double v = is_min ? DBL_MAX : -DBL_MAX;
+        long long v = is_min ? IMAGE_MAX : ~IMAGE_MAX;
 #pragma unroll 4
         for (int b = lane; b < nparts; b += 32) {
-            const double p = parts[6 * (size_t)b + warp];
-            v = is_min ? fmin(v, p) : fmax(v, p);
+            const long long p = parts[6 * (size_t)b + warp];
+            v = is_min ? min(v, p) : max(v, p);
         }
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) {
-            const double o = __shfl_xor_sync(0xffffffffu, v, off);
-            v = is_min ? fmin(v, o) : fmax(v, o);
+            const long long o = __shfl_xor_sync(0xffffffffu, v, off);
+            v = is_min ? min(v, o) : max(v, o);
         }
-        if (lane == 0) sh[warp] = v;
+        if (lane == 0) sh[warp] = from_image(v);
     }
     __syncthreads();
 #pragma unroll
@@ -124,8 +161,8 @@ __device__ __forceinline__ void emit_keys(int n, int tile, int rows, int passes,
 
 // Morton keys (8 bits per axis) in the folded box.
 __global__ void __launch_bounds__(OTPB) morton_kernel(int n, const double *__restrict__ pos,
-                                                       const double *__restrict__ parts, int nparts,
-                                                       int tile, int rows,
+                                                       const long long *__restrict__ parts,
+                                                       int nparts, int tile, int rows,
                                                        unsigned *__restrict__ keys,
                                                        unsigned *__restrict__ hist)
 {
@@ -173,7 +210,7 @@ __device__ __forceinline__ unsigned cell1024(double t)
 // key and its cells agree exactly).  Block 0 also stores {lo_x, lo_y, lo_z,
 // ext} for the tree kernels.
 __global__ void __launch_bounds__(OTPB) morton30_kernel(int n, const double *__restrict__ pos,
-                                                         const double *__restrict__ parts,
+                                                         const long long *__restrict__ parts,
                                                          int nparts, int tile, int rows,
                                                          unsigned *__restrict__ keys,
                                                          unsigned *__restrict__ hist,

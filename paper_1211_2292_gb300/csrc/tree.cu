@@ -104,7 +104,10 @@ __device__ __forceinline__ void cube_corners(const double *__restrict__ box, int
 //   always is a node), else none.
 // A node's number is its rank by (level, start), which one scan of the
 // (level, block of bodies) counts and ballots within the block give; children
-// are consecutive in octant order.
+// are consecutive in octant order.  It ends where the next cell of its level
+// starts: in the warp's ballot, else at the first one of a later warp, or of a
+// later block (searching the keys for it, by doubling steps, was 14 of the
+// build's 85 us at 20000 bodies and 64 us at 2^20).
 //
 // Two launches over the bodies (count, write) took the place of three launches
 // per level (octant boundaries by binary search, one block's scan, children
@@ -118,31 +121,33 @@ __device__ __forceinline__ int key_lcp(unsigned a, unsigned b)
 
 constexpr int BUILD_BLOCKS = 592;  // blocks of bodies at most: each sums the others' counts
 
-// Level range of the nodes starting at each body, lv[i] = lo | hi << 4 (lo > hi:
-// none), and per block and level how many: tab[L * nblk + b].
+// Per body, lv[i] = lo | hi << 4 (hi < lo: no node starts there; lo is the
+// shallowest level whose cell starts at i, 11 for none), and per block and
+// level how many nodes start, tab[L * nblk + b], and the first body a cell
+// starts at, tab[(LEVELS + L) * nblk + b] (n for none).
 __global__ void __launch_bounds__(TTPB) tree_levels_kernel(TreeView t, int n,
                                                            const unsigned *__restrict__ keys,
                                                            int leaf_cap, int chunk,
                                                            unsigned char *__restrict__ lv,
                                                            int *__restrict__ tab)
 {
-    __shared__ int wsum[TTPB / 32][LEVELS];
+    __shared__ int wsum[TTPB / 32][LEVELS], wfirst[TTPB / 32][LEVELS];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (blockIdx.x == 0) {
         if (threadIdx.x < META_INTS) t.meta[threadIdx.x] = 0;
         if (threadIdx.x < 4) t.stats[threadIdx.x] = 0ull;
     }
     const int b0 = blockIdx.x * chunk, b1 = min(n - b0, chunk) + b0;
-    int mine = 0;  // lane L: nodes of level L
+    int mine = 0, first = n;  // lane L: nodes of level L, the first cell start
     for (int r = b0; r < b1; r += TTPB) {
         const int i = r + threadIdx.x;
-        int lo = 1, hi = 0;
+        int lo = 11, hi = 0;
         if (i < b1) {
             const unsigned k = keys[i];
             lo = i == 0 ? 0 : key_lcp(keys[i - 1], k) + 1;
             const int D = n - i > leaf_cap ? key_lcp(k, keys[i + leaf_cap]) : -1;
-            if (lo > 10) {  // the same cell as the body before at every level
-                lo = 1;
+            if (lo > 10) {
+                hi = 0;  // the same cell as the body before at every level
             } else if (D >= lo) {
                 hi = min(10, D + 1);
             } else if (lo == 0) {
@@ -160,46 +165,35 @@ __global__ void __launch_bounds__(TTPB) tree_levels_kernel(TreeView t, int n,
                         b = mid;
                 }
                 const bool over = n - a > leaf_cap && (keys[a + leaf_cap] >> sh) == pre;
-                if (over)
-                    hi = lo;
-                else
-                    lo = 1;
+                hi = over ? lo : lo - 1;
             }
             lv[i] = (unsigned char)(lo | (hi << 4));
         }
 #pragma unroll
         for (int L = 0; L < LEVELS; ++L) {
             const unsigned b = __ballot_sync(0xffffffffu, lo <= L && L <= hi);
-            if (lane == L) mine += __popc(b);
+            const unsigned st = __ballot_sync(0xffffffffu, lo <= L);
+            if (lane == L) {
+                mine += __popc(b);
+                if (st) first = min(first, r + 32 * warp + __ffs(st) - 1);
+            }
         }
     }
-    if (lane < LEVELS) wsum[warp][lane] = mine;
+    if (lane < LEVELS) {
+        wsum[warp][lane] = mine;
+        wfirst[warp][lane] = first;
+    }
     __syncthreads();
     if (threadIdx.x < LEVELS) {
-        int s = 0;
+        int s = 0, f = n;
 #pragma unroll
-        for (int w = 0; w < TTPB / 32; ++w) s += wsum[w][threadIdx.x];
+        for (int w = 0; w < TTPB / 32; ++w) {
+            s += wsum[w][threadIdx.x];
+            f = min(f, wfirst[w][threadIdx.x]);
+        }
         tab[threadIdx.x * gridDim.x + blockIdx.x] = s;
+        tab[(LEVELS + threadIdx.x) * gridDim.x + blockIdx.x] = f;
     }
-}
-
-// First index >= from (from >= 1) with key >= v, found by doubling steps.
-__device__ __forceinline__ int gallop(const unsigned *__restrict__ keys, int from, int n, unsigned v)
-{
-    int step = 1, a = from;
-    while (n - a >= step && keys[a + step - 1] < v) {
-        a += step;
-        step *= 2;
-    }
-    int b = min(n, a + step - 1);  // the answer lies in [a, b]
-    while (a < b) {
-        const int mid = (a + b) >> 1;
-        if (keys[mid] < v)
-            a = mid + 1;
-        else
-            b = mid;
-    }
-    return a;
 }
 
 __global__ void __launch_bounds__(TTPB) tree_emit_kernel(TreeView t, int n,
@@ -208,24 +202,29 @@ __global__ void __launch_bounds__(TTPB) tree_emit_kernel(TreeView t, int n,
                                                          const unsigned char *__restrict__ lv,
                                                          const int *__restrict__ tab, int *err)
 {
-    __shared__ int tot[LEVELS], run[LEVELS], top_s;
-    __shared__ int wcnt[TTPB / 32][LEVELS], woff[TTPB / 32][LEVELS];
-    __shared__ unsigned bal[TTPB / 32][LEVELS];
+    __shared__ int tot[LEVELS], run[LEVELS], nxt[LEVELS], top_s;
+    __shared__ int wcnt[TTPB / 32][LEVELS], woff[TTPB / 32][LEVELS], wnext[TTPB / 32][LEVELS];
+    __shared__ unsigned bal[TTPB / 32][LEVELS], stt[TTPB / 32][LEVELS];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nblk = gridDim.x;
     const unsigned lt = (1u << lane) - 1u;
     for (int L = warp; L < LEVELS; L += TTPB / 32) {
-        int all = 0, pre = 0;
+        int all = 0, pre = 0, next = n;  // in all blocks, up to this one's end; the next cell start
 #pragma unroll 4
         for (int b = lane; b < nblk; b += 32) {
-            const int c = tab[L * nblk + b];
+            const int c = tab[L * nblk + b], f = tab[(LEVELS + L) * nblk + b];
             all += c;
-            if (b < (int)blockIdx.x) pre += c;
+            if (b <= (int)blockIdx.x)
+                pre += c;
+            else
+                next = min(next, f);
         }
         all = __reduce_add_sync(0xffffffffu, all);
         pre = __reduce_add_sync(0xffffffffu, pre);
+        next = __reduce_min_sync(0xffffffffu, next);
         if (lane == 0) {
             tot[L] = all;
             run[L] = pre;
+            nxt[L] = next;
         }
     }
     __syncthreads();
@@ -252,9 +251,11 @@ __global__ void __launch_bounds__(TTPB) tree_emit_kernel(TreeView t, int n,
     __syncthreads();
     const int top = top_s;
     const int b0 = blockIdx.x * chunk, b1 = min(n - b0, chunk) + b0;
-    for (int r = b0; r < b1; r += TTPB) {
+    // from the block's end: run holds the numbers past its nodes, nxt the cell
+    // starts past them
+    for (int r = b0 + (b1 - b0 - 1) / TTPB * TTPB; r >= b0; r -= TTPB) {
         const int i = r + threadIdx.x;
-        int lo = 1, hi = 0;
+        int lo = 11, hi = 0;
         if (i < b1) {
             const int q = lv[i];
             lo = q & 15;
@@ -263,31 +264,37 @@ __global__ void __launch_bounds__(TTPB) tree_emit_kernel(TreeView t, int n,
 #pragma unroll
         for (int L = 0; L < LEVELS; ++L) {
             const unsigned b = __ballot_sync(0xffffffffu, lo <= L && L <= hi);
+            const unsigned st = __ballot_sync(0xffffffffu, lo <= L);
             if (lane == L) {
                 bal[warp][L] = b;
                 wcnt[warp][L] = __popc(b);
+                stt[warp][L] = st;
             }
         }
         __syncthreads();
         if (lane < LEVELS) {
-            int s = run[lane];
-            for (int w = 0; w < warp; ++w) s += wcnt[w][lane];
+            int s = run[lane], next = nxt[lane];
+            for (int w = warp; w < TTPB / 32; ++w) s -= wcnt[w][lane];
+            for (int w = TTPB / 32 - 1; w > warp; --w)
+                if (stt[w][lane]) next = r + 32 * w + __ffs(stt[w][lane]) - 1;
             woff[warp][lane] = s;
+            wnext[warp][lane] = next;
         }
         __syncthreads();
-        if (threadIdx.x < LEVELS) run[threadIdx.x] = woff[TTPB / 32 - 1][threadIdx.x] +
-                                                     wcnt[TTPB / 32 - 1][threadIdx.x];
+        if (threadIdx.x < LEVELS) {
+            run[threadIdx.x] = woff[0][threadIdx.x];
+            nxt[threadIdx.x] = stt[0][threadIdx.x] ? r + __ffs(stt[0][threadIdx.x]) - 1
+                                                   : wnext[0][threadIdx.x];
+        }
         if (lo <= hi) {
             const unsigned k = keys[i];
-            int end = i + 1, child = -1;
+            int child = -1;
             for (int L = hi; L >= lo; --L) {
-                const int sh = 3 * (10 - L);
-                const unsigned pre = k >> sh;
-                end = gallop(keys, end, n, (pre + 1u) << sh);
+                const unsigned later = stt[warp][L] & ~(lt | (1u << lane));
                 const int node = woff[warp][L] + __popc(bal[warp][L] & lt);
                 t.start[node] = i;
-                t.end[node] = end;
-                t.prefix[node] = pre;
+                t.end[node] = later ? r + 32 * warp + __ffs(later) - 1 : wnext[warp][L];
+                t.prefix[node] = k >> (3 * (10 - L));
                 t.level[node] = L;
                 t.nchild[node] = L < hi ? -1 : 0;  // counted with the moments
                 t.first[node] = child;
@@ -318,6 +325,19 @@ __device__ __forceinline__ void put_walk_moments(const TreeView &t, int node, do
                               (float)(cz - (double)hz), 0.f);
 }
 
+// Counts v in at p, releasing this thread's writes (and those it has observed)
+// to whoever counts in later, and acquiring those of all who did before (one
+// instruction, lighter than two sequentially consistent __threadfence()).
+__device__ __forceinline__ int arrive_add(int *p, int v)
+{
+    int old;
+    asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], %2;"
+                 : "=r"(old)
+                 : "l"(p), "r"(v)
+                 : "memory");
+    return old;
+}
+
 // Float64 monopoles of every node in one launch, bottom-up without any wait
 // (and every node's float32 cube).  A thread per leaf sums its bodies; its
 // node then counts its bodies in at the parent with an atomic, and only the
@@ -331,8 +351,13 @@ __device__ __forceinline__ void put_walk_moments(const TreeView &t, int node, do
 // trees, the chain of levels.  So the cubes and the leaves' sums keep every
 // lane busy, a parent's four sums are reduced over its eight lanes with four
 // additions (each lane ends with one of them), and one division per node
-// turns each lane's sum into its coordinate.
-__global__ void __launch_bounds__(TTPB) tree_moments_kernel(TreeView t,
+// turns each lane's sum into its coordinate.  Blocks of two warps, so that the
+// nodes of a small tree spread over the SMs' float64 pipes.  20000 bodies: 42 ->
+// 34 us with the parent's tree data loaded beside the arrival and eight bodies'
+// loads in flight per leaf; what is left is the chain of levels (arrival,
+// children's sums, division).
+constexpr int MTPB = 64;
+__global__ void __launch_bounds__(MTPB) tree_moments_kernel(TreeView t,
                                                             const double *__restrict__ box,
                                                             const double *__restrict__ pos,
                                                             const double *__restrict__ mass,
@@ -343,7 +368,7 @@ __global__ void __launch_bounds__(TTPB) tree_moments_kernel(TreeView t,
     if (blockIdx.x == 0 && threadIdx.x == 0) t.stats[0] = (unsigned long long)total;
     const int lane = threadIdx.x & 31, o = lane & 7;
     int leaves = 0;
-    for (int q0 = blockIdx.x * TTPB + (threadIdx.x & ~31); q0 < total; q0 += gridDim.x * TTPB) {
+    for (int q0 = blockIdx.x * MTPB + (threadIdx.x & ~31); q0 < total; q0 += gridDim.x * MTPB) {
         const int me = q0 + lane;
         int node = -1, count = 0;  // what this lane counts in at its parent
         if (me < total) {
@@ -359,10 +384,10 @@ __global__ void __launch_bounds__(TTPB) tree_moments_kernel(TreeView t,
                 bl[3] = __int_as_float(0);
                 const int s = t.start[me], e = t.end[me];
                 double M = 0.0, sx = 0.0, sy = 0.0, sz = 0.0;
-                for (int k = s; k < e; k += 4) {  // four bodies' loads in flight
-                    double m[4], x[4], y[4], z[4];
+                for (int k = s; k < e; k += 8) {  // eight bodies' loads in flight
+                    double m[8], x[8], y[8], z[8];
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
+                    for (int u = 0; u < 8; ++u) {
                         const int j = perm[min(k + u, e - 1)];
                         m[u] = mass[j];
                         x[u] = pos[3 * (size_t)j];
@@ -370,7 +395,7 @@ __global__ void __launch_bounds__(TTPB) tree_moments_kernel(TreeView t,
                         z[u] = pos[3 * (size_t)j + 2];
                     }
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
+                    for (int u = 0; u < 8; ++u) {
                         if (k + u < e) {
                             M += m[u];
                             sx += m[u] * x[u];
@@ -379,8 +404,8 @@ __global__ void __launch_bounds__(TTPB) tree_moments_kernel(TreeView t,
                         }
                     }
                 }
-                put_walk_moments(t, me, M, M > 0.0 ? sx / M : 0.0, M > 0.0 ? sy / M : 0.0,
-                                 M > 0.0 ? sz / M : 0.0);
+                const double inv = M > 0.0 ? 1.0 / M : 0.0;
+                put_walk_moments(t, me, M, sx * inv, sy * inv, sz * inv);
                 node = t.parent[me];
                 count = e - s;
             }
@@ -388,17 +413,19 @@ __global__ void __launch_bounds__(TTPB) tree_moments_kernel(TreeView t,
         // climb: each lane with a node counts in; the completed parents are
         // summed and count in themselves
         while (__any_sync(FULL, node >= 0)) {
+            // (what the parent's sum will need of the tree is loaded beside
+            // the arrival, whose fence and atomic are the longest link)
             bool won = false;
-            int bodies = 0;
+            int bodies = 0, up = -1, f0 = 0, nch = 0;
             if (node >= 0) {
                 bodies = t.end[node] - t.start[node];
-                __threadfence();
-                won = atomicAdd(t.arrive + node, count) + count == bodies;
-                __threadfence();
+                up = t.parent[node];
+                f0 = t.first[node];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) nch += f0 + q < total && t.parent[f0 + q] == node;
+                won = arrive_add(t.arrive + node, count) + count == bodies;
             }
             unsigned win = __ballot_sync(FULL, won);
-            int up = -1;
-            if (won) up = t.parent[node];
             while (win) {
                 // group g of eight lanes takes the g-th winner
                 const int g = lane >> 3;
@@ -411,9 +438,9 @@ __global__ void __launch_bounds__(TTPB) tree_moments_kernel(TreeView t,
                 }
                 win = w;
                 const int p = __shfl_sync(FULL, node, src & 31);
+                const int f = __shfl_sync(FULL, f0, src & 31), nc = __shfl_sync(FULL, nch, src & 31);
                 const bool mine = src >= 0;
-                const int f = mine ? t.first[p] : 0;
-                const bool child = mine && f + o < total && t.parent[f + o] == p;
+                const bool child = mine && o < nc;
                 double v[4] = {0.0, 0.0, 0.0, 0.0};
                 if (child) {
                     v[0] = __ldcg(t.M + f + o);
@@ -434,11 +461,10 @@ __global__ void __launch_bounds__(TTPB) tree_moments_kernel(TreeView t,
                 const double cx = __shfl_sync(FULL, cm, (lane & 24) + 2);
                 const double cy = __shfl_sync(FULL, cm, (lane & 24) + 4);
                 const double cz = __shfl_sync(FULL, cm, (lane & 24) + 6);
-                const int nch = __popc((__ballot_sync(FULL, child) >> (lane & 24)) & 0xffu);
                 if (mine && o == 0) {
                     put_walk_moments(t, p, M, cx, cy, cz);
-                    t.nchild[p] = nch;
-                    reinterpret_cast<int *>(t.box_lo + p)[3] = nch;  // the walk's child count
+                    t.nchild[p] = nc;
+                    reinterpret_cast<int *>(t.box_lo + p)[3] = nc;  // the walk's child count
                 }
                 __syncwarp();
             }
@@ -1281,8 +1307,8 @@ cudaError_t launch_tree_build(cudaStream_t s, const TreeView &t, int n, const Or
     tree_levels_kernel<<<nblk, TTPB, 0, s>>>(t, n, keys, leaf_cap, chunk, lv, tab);
     tree_emit_kernel<<<nblk, TTPB, 0, s>>>(t, n, keys, chunk, lv, tab, err);
     // a thread per node, at most the blocks that are resident on 152 SMs
-    const int64_t blocks = ((int64_t)t.cap + TTPB - 1) / TTPB;
-    tree_moments_kernel<<<(int)(blocks < 1216 ? blocks : 1216), TTPB, 0, s>>>(t, box, pos, mass,
+    const int64_t blocks = ((int64_t)t.cap + MTPB - 1) / MTPB;
+    tree_moments_kernel<<<(int)(blocks < 3040 ? blocks : 3040), MTPB, 0, s>>>(t, box, pos, mass,
                                                                               perm);
     kernels = 3;
     return cudaGetLastError();
