@@ -1,12 +1,13 @@
 // float64 force and energy kernels (paper Sec. IV-A/IV-B force calculation
 // as the exact all-pairs sum, every operation in float64).
 //
-// Same schedule as the float32 kernels: an i-tile of T*I bodies per CTA in
-// registers, j-bodies streamed through a double-buffered shared tile of J
-// double4 (x,y,z,m), the grid split over j with the last arriving CTA adding
-// the float64 partials in split order.  The reciprocal square root is a
-// float32 MUFU seed refined by one second-order Householder step (see
-// nb_device.cuh), since float64 has no MUFU path.
+// An i-tile of T*I bodies per CTA in registers, j-bodies streamed through a
+// double-buffered shared tile of J double4 (x,y,z,m), the grid split over j in
+// equal body counts with the last arriving CTA adding the float64 partials in
+// split order.  The force kernel's pair factor is formed on the integer pipe
+// (f64_pair.cuh); the energy kernel, which also needs the potential, refines a
+// float32 MUFU seed of the reciprocal root by one second-order Householder
+// step (nb_device.cuh).
 //
 // The energy kernel also accumulates the softened potential
 // phi_i = sum_{j != i} m_j / s_ij (self pair skipped by index) and reduces,
@@ -15,12 +16,13 @@
 #include <cuda_runtime.h>
 
 #include "nb_device.cuh"
+#include "f64_pair.cuh"
 #include "nb_internal.h"
 
 namespace nb {
 namespace {
 
-constexpr int UNROLL_F64 = 4;
+constexpr int UNROLL_F64 = 2;
 
 template <int T, int J>
 __device__ __forceinline__ void stage_load64(double4 (&buf)[J / T], const double4 *__restrict__ P,
@@ -49,41 +51,82 @@ __device__ __forceinline__ double pair_rinv(double r2)
 }
 
 template <int T, int I, int J, bool ZEPS, bool ENERGY>
-__device__ __forceinline__ void sweep64(const double4 *__restrict__ P, int n, int t0, int t1,
+__device__ __forceinline__ void sweep64(const double4 *__restrict__ P, int jlo, int jhi,
                                         double eps2, const double (&xi)[I], const double (&yi)[I],
                                         const double (&zi)[I], const int (&ii)[I], double (&ax)[I],
                                         double (&ay)[I], double (&az)[I], double (&ph)[I],
                                         double4 (*tile)[J])
 {
+    const EpsFixed ef = eps_fixed(eps2);
+    // j-bodies [jlo, jhi) in tiles of J from jlo on; the last tile stops at the
+    // next multiple of the unrolling (massless bodies, which add nothing)
     double4 buf[J / T];
-    if (t0 < t1) {
-        stage_load64<T, J>(buf, P, t0 * J, n);
+    if (jlo < jhi) {
+        stage_load64<T, J>(buf, P, jlo, jhi);
         stage_store64<T, J>(tile[0], buf);
     }
     __syncthreads();
-    for (int t = t0; t < t1; ++t) {
-        const int b = (t - t0) & 1;
-        if (t + 1 < t1) stage_load64<T, J>(buf, P, (t + 1) * J, n);
+    int b = 0;
+    for (int j0 = jlo; j0 < jhi; j0 += J, b ^= 1) {
+        if (j0 + J < jhi) stage_load64<T, J>(buf, P, j0 + J, jhi);
         const double4 *s = tile[b];
-#pragma unroll UNROLL_F64
-        for (int jj = 0; jj < J; ++jj) {
-            const double4 q = s[jj];
+        const int jn = min(J, jhi - j0);
+        for (int jj = 0; jj < jn; jj += UNROLL_F64) {
+            if (ENERGY) {
 #pragma unroll
-            for (int k = 0; k < I; ++k) {
-                const double dx = q.x - xi[k], dy = q.y - yi[k], dz = q.z - zi[k];
-                double r2 = fma(dx, dx, eps2);
-                r2 = fma(dy, dy, r2);
-                r2 = fma(dz, dz, r2);
-                const double ri = pair_rinv<ZEPS>(r2);
-                const double mri = q.w * ri;
-                const double sc = mri * (ri * ri);
-                ax[k] = fma(dx, sc, ax[k]);
-                ay[k] = fma(dy, sc, ay[k]);
-                az[k] = fma(dz, sc, az[k]);
-                if (ENERGY) ph[k] += (t * J + jj == ii[k]) ? 0.0 : mri;
+                for (int u = 0; u < UNROLL_F64; ++u) {
+                    const double4 q = s[jj + u];
+#pragma unroll
+                    for (int k = 0; k < I; ++k) {
+                        const double dx = q.x - xi[k], dy = q.y - yi[k], dz = q.z - zi[k];
+                        const double ri = pair_rinv<ZEPS>(fma(dz, dz, fma(dy, dy, fma(dx, dx, eps2))));
+                        const double mri = q.w * ri;
+                        const double sc = mri * (ri * ri);
+                        ax[k] = fma(dx, sc, ax[k]);
+                        ay[k] = fma(dy, sc, ay[k]);
+                        az[k] = fma(dz, sc, az[k]);
+                        ph[k] += (j0 + jj + u == ii[k]) ? 0.0 : mri;
+                    }
+                }
+            } else {
+                // all of a step's factors first (independent chains), then the
+                // rare ones that need the general form in one branch
+                double dx[UNROLL_F64][I], dy[UNROLL_F64][I], dz[UNROLL_F64][I], sc[UNROLL_F64][I];
+                unsigned general = 0;
+#pragma unroll
+                for (int u = 0; u < UNROLL_F64; ++u) {
+                    const double4 q = s[jj + u];
+#pragma unroll
+                    for (int k = 0; k < I; ++k) {
+                        dx[u][k] = q.x - xi[k];
+                        dy[u][k] = q.y - yi[k];
+                        dz[u][k] = q.z - zi[k];
+                        double r;
+                        if (!pair_inv_cube<ZEPS>(dx[u][k], dy[u][k], dz[u][k], ef, r))
+                            general |= 1u << (u * I + k);
+                        sc[u][k] = q.w * r;
+                    }
+                }
+                if (general) {
+#pragma unroll
+                    for (int u = 0; u < UNROLL_F64; ++u)
+#pragma unroll
+                        for (int k = 0; k < I; ++k)
+                            if (general >> (u * I + k) & 1)
+                                sc[u][k] = pair_factor_general<ZEPS>(dx[u][k], dy[u][k], dz[u][k],
+                                                                     s[jj + u].w, eps2);
+                }
+#pragma unroll
+                for (int u = 0; u < UNROLL_F64; ++u)
+#pragma unroll
+                    for (int k = 0; k < I; ++k) {
+                        ax[k] = fma(dx[u][k], sc[u][k], ax[k]);
+                        ay[k] = fma(dy[u][k], sc[u][k], ay[k]);
+                        az[k] = fma(dz[u][k], sc[u][k], az[k]);
+                    }
             }
         }
-        if (t + 1 < t1) stage_store64<T, J>(tile[b ^ 1], buf);
+        if (j0 + J < jhi) stage_store64<T, J>(tile[b ^ 1], buf);
         __syncthreads();
     }
 }
@@ -100,8 +143,8 @@ __global__ void __launch_bounds__(T) force_f64_kernel(const ForceParams p)
     const int it = blockIdx.x % n_itiles;
     const int js = blockIdx.x / n_itiles;
     const int i0 = it * TILE_I;
-    int t0, t1;
-    split_range((n + J - 1) / J, p.nsplit, js, t0, t1);
+    const int jlo = (int)((long long)n * js / p.nsplit);  // an equal share of the bodies
+    const int jhi = (int)((long long)n * (js + 1) / p.nsplit);
 
     double xi[I], yi[I], zi[I], ax[I], ay[I], az[I], ph[I];
     int ii[I];
@@ -115,7 +158,7 @@ __global__ void __launch_bounds__(T) force_f64_kernel(const ForceParams p)
         ii[k] = i;
         ax[k] = ay[k] = az[k] = ph[k] = 0.0;
     }
-    sweep64<T, I, J, ZEPS, false>(P, n, t0, t1, p.eps2, xi, yi, zi, ii, ax, ay, az, ph, tile);
+    sweep64<T, I, J, ZEPS, false>(P, jlo, jhi, p.eps2, xi, yi, zi, ii, ax, ay, az, ph, tile);
 
     if (p.nsplit == 1) {
 #pragma unroll
@@ -158,15 +201,10 @@ __global__ void __launch_bounds__(T) force_f64_kernel(const ForceParams p)
     for (int k = 0; k < I; ++k) {
         const int i = i0 + threadIdx.x + k * T;
         if (i < n) {
-            double x = 0.0, y = 0.0, z = 0.0;
-            for (int q = 0; q < p.nsplit; ++q) {
-                const double *r = p.partial + ((size_t)q * n + i) * 3;
-                x += __ldcg(r);
-                y += __ldcg(r + 1);
-                z += __ldcg(r + 2);
-            }
+            double t[3];
+            sum_slots(p.partial + (size_t)i * 3, (size_t)n * 3, p.nsplit, t);
             double *a = p.acc + 3 * (size_t)i;
-            const double gx = p.G * x, gy = p.G * y, gz = p.G * z;
+            const double gx = p.G * t[0], gy = p.G * t[1], gz = p.G * t[2];
             a[0] = gx;
             a[1] = gy;
             a[2] = gz;
@@ -231,7 +269,7 @@ __global__ void __launch_bounds__(T) energy_f64_kernel(const EnergyParams p)
         ii[k] = i;
         ax[k] = ay[k] = az[k] = ph[k] = 0.0;
     }
-    sweep64<T, I, J, ZEPS, true>(P, n, t0, t1, p.eps2, xi, yi, zi, ii, ax, ay, az, ph, tile);
+    sweep64<T, I, J, ZEPS, true>(P, t0 * J, min(t1 * J, n), p.eps2, xi, yi, zi, ii, ax, ay, az, ph, tile);
 
     double v[8] = {0, 0, 0, 0, 0, 0, 0, 0};
 #pragma unroll

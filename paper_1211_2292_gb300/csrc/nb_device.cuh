@@ -102,24 +102,32 @@ __device__ __forceinline__ float log2_packed(double m)
     return ((float)((h >> 20) - 1023) + w.hi) + fmaf(z, q, w.lo);
 }
 
-// float64 reciprocal square root: a float32 MUFU seed y0 (relative error
-// e0 < 2^-22) refined by one second-order Householder step for
-// f(y) = 1/y^2 - x.  With e = 1 - x*y0^2 the exact answer is
-// y0*(1-e)^(-1/2) = y0*(1 + e/2 + 3e^2/8 + ...); keeping two terms leaves a
-// relative error of about (5/16)e^3 ~ 1e-20, below float64 rounding.
-// The seed is taken at x' = x 2^-2k in [1, 4) (2k the even part of x's
-// exponent) and scaled back by 2^-k, both exact edits of the exponent field
-// on the integer pipe, so every positive normal float64 x gets a normal seed
-// (a float32 seed of x itself would overflow or flush to zero outside
-// 1.2e-38 .. 3.4e38, e.g. for r^2 = 1e-40 at eps = 0).  Valid for positive
-// normal x; x = 0 gives a large finite value (callers mask the self pair).
-__device__ __forceinline__ double rsqrt_f64(double x)
+// Seed of the float64 reciprocal square root: y0 = x^(-1/2) (1 + e0), |e0| <
+// 2^-22, with a 24-bit significand, for any positive normal x.  x is scaled by
+// an even power of two into [1, 4), cut to float32 and sent through the MUFU,
+// and the result scaled back, all on the integer pipe: a conversion between
+// float64 and float32 takes the float64 pipe (2 lanes per clock per SM) as an
+// operation would.  (A float32 seed of x itself would overflow or flush to
+// zero outside 1.2e-38 .. 3.4e38, e.g. for r^2 = 1e-40 at eps = 0.)
+__device__ __forceinline__ double rsqrt_seed(double x)
 {
     const int hi = __double2hiint(x), lo = __double2loint(x);
-    const int k2 = ((int)(((unsigned)hi >> 20) & 0x7ffu) - 1023) & ~1;  // even part of the exponent
-    const double xs = __hiloint2double(hi - k2 * (1 << 20), lo);   // x 2^-k2, in [1, 4)
-    const double ys = (double)rsqrt_mufu((float)xs);
-    const double y = __hiloint2double(__double2hiint(ys) - (k2 / 2) * (1 << 20), __double2loint(ys));
+    const int ex = (int)(((unsigned)hi >> 20) & 0x7ffu) - 1023;  // x = f 2^ex, 1 <= f < 2
+    const unsigned xf = ((unsigned)(127 + (ex & 1)) << 23) | (((unsigned)hi & 0xfffffu) << 3) |
+                        ((unsigned)lo >> 29);
+    const unsigned yf = __float_as_uint(rsqrt_mufu(__uint_as_float(xf)));  // in (1/2, 1]
+    return __hiloint2double((int)(yf >> 3) + (1023 - 127 - (ex >> 1)) * (1 << 20), (int)(yf << 29));
+}
+
+// float64 reciprocal square root: the seed y0 refined by one second-order
+// Householder step for f(y) = 1/y^2 - x.  With e = 1 - x*y0^2 the exact answer
+// is y0*(1-e)^(-1/2) = y0*(1 + e/2 + 3e^2/8 + ...); keeping two terms leaves a
+// relative error of about (5/16)e^3 ~ 1e-20, below float64 rounding.  Valid
+// for positive normal x; x = 0 gives a large finite value (callers mask the
+// self pair).
+__device__ __forceinline__ double rsqrt_f64(double x)
+{
+    const double y = rsqrt_seed(x);
     double h = x * y;
     double e = fma(-h, y, 1.0);
     double p = fma(e, 0.375, 0.5);
@@ -220,6 +228,26 @@ __device__ __forceinline__ float2 merge_slots(const float2 *slot, size_t stride,
             if (q + u < n) kahan_merge(a.x, a.y, b[u].x, b[u].y);
     }
     return a;
+}
+
+// Sum of n float64 triples `stride` doubles apart in slot order, 24 loads in
+// flight.
+__device__ __forceinline__ void sum_slots(const double *slot, size_t stride, int n, double (&a)[3])
+{
+    a[0] = a[1] = a[2] = 0.0;
+    for (int q = 0; q < n; q += 8) {
+        double b[8][3];
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+#pragma unroll
+            for (int d = 0; d < 3; ++d)
+                b[u][d] = q + u < n ? __ldcg(slot + (size_t)(q + u) * stride + d) : 0.0;
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (q + u < n)
+#pragma unroll
+                for (int d = 0; d < 3; ++d) a[d] += b[u][d];
+    }
 }
 
 // Range of j-tiles [t0, t1) handled by split `js` of `nsplit`.

@@ -1,0 +1,59 @@
+"""float64 forces: the integer pair factor at the edges of its ranges, j-splits of equal body counts."""
+import numpy as np
+import pytest
+
+from paper_1211_2292_gb300 import inputs, nbody
+from helpers import host, to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+def _exact(pos, mass, eps):
+    """Extended-precision sums and, per body, the sum of the terms' magnitudes."""
+    p, m, e = pos.astype(np.longdouble), mass.astype(np.longdouble), np.longdouble(eps)
+    d = p[None, :, :] - p[:, None, :]
+    r2 = (d * d).sum(2) + e * e
+    own = r2 == e * e if eps == 0.0 else np.zeros_like(r2, dtype=bool)
+    s2 = np.where(own, np.longdouble(1), r2)
+    t = np.where(own, 0, m[None, :] / (s2 * np.sqrt(s2)))[:, :, None] * d
+    return t.sum(1), np.abs(t).sum(1)
+
+
+def _check(cuda, pos, mass, eps, split=0, variant=0):
+    n = len(mass)
+    x, m = to_dev(pos, cuda), to_dev(mass, cuda)
+    with nbody.NBody(n, "fp64") as nb:
+        nb.tune_set(nbody.KIND_FORCE, 0, 1 << 40, variant, split)
+        a = host(nb.forces(x, m, 1.0, eps))
+        nb.sync()
+    ref, size = _exact(pos, mass, eps)
+    # a pair's term: differences and r^2 3 x 2^-53 (1.5 fold for the power), the
+    # factor and its two products below 5 x 2^-53; n additions of 2^-53 each
+    assert (np.abs(a - ref) <= (n + 10) * 2.0 ** -53 * size).all()
+
+
+@pytest.mark.parametrize("variant", range(4))
+@pytest.mark.parametrize("n", [1, 2, 15, 17, 127, 129, 257, 400])
+def test_even_splits_and_tile_edges(cuda, n, variant):
+    b = inputs.random_system(n, seed=n)
+    for eps, split in ((0.01, 0), (0.0, 0), (0.01, 1), (0.0, 3)):
+        _check(cuda, b.pos, b.mass, eps, split, variant)
+
+
+@pytest.mark.parametrize("scale", [0, -329, -331, 328, 331])
+@pytest.mark.parametrize("rel", [0.0, 1e-6, 1.0, 1e5])
+def test_exponents_of_differences_and_softening(cuda, scale, rel):
+    # separations over 80 octaves, equal and zero coordinates, massless and
+    # negative masses, around the exponents at which the general form takes over
+    rng = np.random.default_rng(5)
+    n = 70
+    pos = rng.uniform(-1, 1, (n, 3)) * np.ldexp(1.0, -rng.integers(0, 80, (n, 3)))
+    pos[:10, 1] = 0.0
+    pos[10:20, 2] = pos[5, 2]
+    pos[20] = pos[21]
+    mass = rng.uniform(0.1, 1.0, n)
+    mass[::7] = 0.0
+    mass[3] = -mass[3]
+    # |a| ~ m 2^(-2 scale): scaled so that the sums stay in range
+    mass = np.ldexp(mass, scale)
+    _check(cuda, np.ldexp(pos, scale), mass, float(np.ldexp(rel, scale)))
