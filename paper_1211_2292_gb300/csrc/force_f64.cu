@@ -4,7 +4,7 @@
 // An i-tile of T*I bodies per CTA in registers, j-bodies streamed through a
 // double-buffered shared tile of J double4 (x,y,z,m), the grid split over j in
 // equal body counts with the last arriving CTA adding the float64 partials in
-// split order.  The force kernel's pair factor is formed on the integer pipe
+// split order.  The force kernel's pair terms and sums are integers
 // (f64_pair.cuh); the energy kernel, which also needs the potential, refines a
 // float32 MUFU seed of the reciprocal root by one second-order Householder
 // step (nb_device.cuh).
@@ -22,7 +22,7 @@
 namespace nb {
 namespace {
 
-constexpr int UNROLL_F64 = 2;
+constexpr int UNROLL_F64 = 2;  // pairs in flight: 2.27 ms at 16384 bodies (1: 2.34, 4: 2.45)
 
 template <int T, int J>
 __device__ __forceinline__ void stage_load64(double4 (&buf)[J / T], const double4 *__restrict__ P,
@@ -50,16 +50,14 @@ __device__ __forceinline__ double pair_rinv(double r2)
     return ri;
 }
 
-template <int T, int I, int J, bool ZEPS, bool ENERGY>
-__device__ __forceinline__ void sweep64(const double4 *__restrict__ P, int jlo, int jhi,
-                                        double eps2, const double (&xi)[I], const double (&yi)[I],
-                                        const double (&zi)[I], const int (&ii)[I], double (&ax)[I],
-                                        double (&ay)[I], double (&az)[I], double (&ph)[I],
-                                        double4 (*tile)[J])
+// Sums over the j-bodies [jlo, jhi) for the energy kernel.
+template <int T, int I, int J, bool ZEPS>
+__device__ __forceinline__ void energy_sweep(const double4 *__restrict__ P, int jlo, int jhi,
+                                             double eps2, const double (&xi)[I],
+                                             const double (&yi)[I], const double (&zi)[I],
+                                             const int (&ii)[I], double (&ax)[I], double (&ay)[I],
+                                             double (&az)[I], double (&ph)[I], double4 (*tile)[J])
 {
-    const EpsFixed ef = eps_fixed(eps2);
-    // j-bodies [jlo, jhi) in tiles of J from jlo on; the last tile stops at the
-    // next multiple of the unrolling (massless bodies, which add nothing)
     double4 buf[J / T];
     if (jlo < jhi) {
         stage_load64<T, J>(buf, P, jlo, jhi);
@@ -70,63 +68,116 @@ __device__ __forceinline__ void sweep64(const double4 *__restrict__ P, int jlo, 
     for (int j0 = jlo; j0 < jhi; j0 += J, b ^= 1) {
         if (j0 + J < jhi) stage_load64<T, J>(buf, P, j0 + J, jhi);
         const double4 *s = tile[b];
+#pragma unroll 4
+        for (int jj = 0; jj < J; ++jj) {
+            const double4 q = s[jj];
+#pragma unroll
+            for (int k = 0; k < I; ++k) {
+                const double dx = q.x - xi[k], dy = q.y - yi[k], dz = q.z - zi[k];
+                const double ri = pair_rinv<ZEPS>(fma(dz, dz, fma(dy, dy, fma(dx, dx, eps2))));
+                const double mri = q.w * ri;
+                const double sc = mri * (ri * ri);
+                ax[k] = fma(dx, sc, ax[k]);
+                ay[k] = fma(dy, sc, ay[k]);
+                az[k] = fma(dz, sc, az[k]);
+                ph[k] += (j0 + jj == ii[k]) ? 0.0 : mri;
+            }
+        }
+        if (j0 + J < jhi) stage_store64<T, J>(tile[b ^ 1], buf);
+        __syncthreads();
+    }
+}
+
+// Sums over the j-bodies [jlo, jhi), in tiles of J from jlo on; the last tile
+// stops at the next multiple of the step (massless bodies, which add nothing).
+// Masses are brought into their integer form once per tile.
+template <int T, int I, int J, bool ZEPS>
+__device__ __forceinline__ void force_sweep(const double4 *__restrict__ P, int jlo, int jhi,
+                                            double eps2, const double (&xi)[I],
+                                            const double (&yi)[I], const double (&zi)[I],
+                                            double (&a)[I][3], double4 (*tile)[J],
+                                            MassFixed (*mtile)[J])
+{
+    const EpsFixed ef = eps_fixed(eps2);
+    double4 buf[J / T];
+    auto store = [&](int b) {
+        stage_store64<T, J>(tile[b], buf);
+#pragma unroll
+        for (int l = 0; l < J / T; ++l) mtile[b][l * T + threadIdx.x] = mass_fixed(buf[l].w);
+    };
+    FixedSum<J> sum[I][3];
+#pragma unroll
+    for (int k = 0; k < I; ++k)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            sum[k][c].acc = 0;
+            sum[k][c].E = 2 * F64_NO_TERM;
+        }
+    if (jlo < jhi) {
+        stage_load64<T, J>(buf, P, jlo, jhi);
+        store(0);
+    }
+    __syncthreads();
+    int b = 0;
+    for (int j0 = jlo; j0 < jhi; j0 += J, b ^= 1) {
+        if (j0 + J < jhi) stage_load64<T, J>(buf, P, j0 + J, jhi);
+        const double4 *s = tile[b];
+        const MassFixed *ms = mtile[b];
         const int jn = min(J, jhi - j0);
         for (int jj = 0; jj < jn; jj += UNROLL_F64) {
-            if (ENERGY) {
+#pragma unroll
+            for (int k = 0; k < I; ++k) {
+                // a step's terms first (independent chains), then in one branch
+                // the rare pairs of the general form
+                PairTerm t[UNROLL_F64];
+                int sign[UNROLL_F64][3];
+                bool general = false;
 #pragma unroll
                 for (int u = 0; u < UNROLL_F64; ++u) {
                     const double4 q = s[jj + u];
-#pragma unroll
-                    for (int k = 0; k < I; ++k) {
-                        const double dx = q.x - xi[k], dy = q.y - yi[k], dz = q.z - zi[k];
-                        const double ri = pair_rinv<ZEPS>(fma(dz, dz, fma(dy, dy, fma(dx, dx, eps2))));
-                        const double mri = q.w * ri;
-                        const double sc = mri * (ri * ri);
-                        ax[k] = fma(dx, sc, ax[k]);
-                        ay[k] = fma(dy, sc, ay[k]);
-                        az[k] = fma(dz, sc, az[k]);
-                        ph[k] += (j0 + jj + u == ii[k]) ? 0.0 : mri;
-                    }
-                }
-            } else {
-                // all of a step's factors first (independent chains), then the
-                // rare ones that need the general form in one branch
-                double dx[UNROLL_F64][I], dy[UNROLL_F64][I], dz[UNROLL_F64][I], sc[UNROLL_F64][I];
-                unsigned general = 0;
-#pragma unroll
-                for (int u = 0; u < UNROLL_F64; ++u) {
-                    const double4 q = s[jj + u];
-#pragma unroll
-                    for (int k = 0; k < I; ++k) {
-                        dx[u][k] = q.x - xi[k];
-                        dy[u][k] = q.y - yi[k];
-                        dz[u][k] = q.z - zi[k];
-                        double r;
-                        if (!pair_inv_cube<ZEPS>(dx[u][k], dy[u][k], dz[u][k], ef, r))
-                            general |= 1u << (u * I + k);
-                        sc[u][k] = q.w * r;
-                    }
+                    const MassFixed m = ms[jj + u];
+                    const double dx = q.x - xi[k], dy = q.y - yi[k], dz = q.z - zi[k];
+                    general |= !pair_term<ZEPS>(dx, dy, dz, m, ef, t[u]);
+                    sign[u][0] = (__double2hiint(dx) ^ (m.e2 << 31)) >> 31;
+                    sign[u][1] = (__double2hiint(dy) ^ (m.e2 << 31)) >> 31;
+                    sign[u][2] = (__double2hiint(dz) ^ (m.e2 << 31)) >> 31;
                 }
                 if (general) {
 #pragma unroll
-                    for (int u = 0; u < UNROLL_F64; ++u)
+                    for (int u = 0; u < UNROLL_F64; ++u) {
+                        const double4 q = s[jj + u];
+                        const MassFixed m = ms[jj + u];
+                        const double dx = q.x - xi[k], dy = q.y - yi[k], dz = q.z - zi[k];
+                        // a body and itself: no force, unless its factor overflows
+                        if (in_integer_form(dx, dy, dz, m) ||
+                            (dx == 0.0 && dy == 0.0 && dz == 0.0 && m.lim && m.e2 < 1000 &&
+                             (ZEPS || ef.e > 863)))
+                            continue;
+                        const double sc = pair_factor_general<ZEPS>(dx, dy, dz, q.w, eps2);
+                        a[k][0] = fma(dx, sc, a[k][0]);
+                        a[k][1] = fma(dy, sc, a[k][1]);
+                        a[k][2] = fma(dz, sc, a[k][2]);
+                    }
+                }
 #pragma unroll
-                        for (int k = 0; k < I; ++k)
-                            if (general >> (u * I + k) & 1)
-                                sc[u][k] = pair_factor_general<ZEPS>(dx[u][k], dy[u][k], dz[u][k],
-                                                                     s[jj + u].w, eps2);
+                for (int c = 0; c < 3; ++c) {
+                    int e = sum[k][c].E;
+#pragma unroll
+                    for (int u = 0; u < UNROLL_F64; ++u) e = max(e, t[u].e[c]);
+                    sum[k][c].raise(e);
                 }
 #pragma unroll
                 for (int u = 0; u < UNROLL_F64; ++u)
 #pragma unroll
-                    for (int k = 0; k < I; ++k) {
-                        ax[k] = fma(dx[u][k], sc[u][k], ax[k]);
-                        ay[k] = fma(dy[u][k], sc[u][k], ay[k]);
-                        az[k] = fma(dz[u][k], sc[u][k], az[k]);
-                    }
+                    for (int c = 0; c < 3; ++c)
+                        sum[k][c].add(t[u].A[c], t[u].S, t[u].e[c], sign[u][c]);
             }
         }
-        if (j0 + J < jhi) stage_store64<T, J>(tile[b ^ 1], buf);
+#pragma unroll
+        for (int k = 0; k < I; ++k)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) a[k][c] += sum[k][c].take();
+        if (j0 + J < jhi) store(b ^ 1);
         __syncthreads();
     }
 }
@@ -136,6 +187,7 @@ __global__ void __launch_bounds__(T) force_f64_kernel(const ForceParams p)
 {
     constexpr int TILE_I = T * I;
     __shared__ __align__(16) double4 tile[2][J];
+    __shared__ __align__(16) MassFixed mtile[2][J];
     __shared__ int s_last;
     const double4 *P = static_cast<const double4 *>(p.P);
     const int n = p.n;
@@ -146,8 +198,7 @@ __global__ void __launch_bounds__(T) force_f64_kernel(const ForceParams p)
     const int jlo = (int)((long long)n * js / p.nsplit);  // an equal share of the bodies
     const int jhi = (int)((long long)n * (js + 1) / p.nsplit);
 
-    double xi[I], yi[I], zi[I], ax[I], ay[I], az[I], ph[I];
-    int ii[I];
+    double xi[I], yi[I], zi[I], a[I][3];
 #pragma unroll
     for (int k = 0; k < I; ++k) {
         const int i = i0 + threadIdx.x + k * T;
@@ -155,21 +206,20 @@ __global__ void __launch_bounds__(T) force_f64_kernel(const ForceParams p)
         xi[k] = b.x;
         yi[k] = b.y;
         zi[k] = b.z;
-        ii[k] = i;
-        ax[k] = ay[k] = az[k] = ph[k] = 0.0;
+        a[k][0] = a[k][1] = a[k][2] = 0.0;
     }
-    sweep64<T, I, J, ZEPS, false>(P, jlo, jhi, p.eps2, xi, yi, zi, ii, ax, ay, az, ph, tile);
+    force_sweep<T, I, J, ZEPS>(P, jlo, jhi, p.eps2, xi, yi, zi, a, tile, mtile);
 
     if (p.nsplit == 1) {
 #pragma unroll
         for (int k = 0; k < I; ++k) {
             const int i = i0 + threadIdx.x + k * T;
             if (i < n) {
-                double *a = p.acc + 3 * (size_t)i;
-                const double gx = p.G * ax[k], gy = p.G * ay[k], gz = p.G * az[k];
-                a[0] = gx;
-                a[1] = gy;
-                a[2] = gz;
+                double *o = p.acc + 3 * (size_t)i;
+                const double gx = p.G * a[k][0], gy = p.G * a[k][1], gz = p.G * a[k][2];
+                o[0] = gx;
+                o[1] = gy;
+                o[2] = gz;
                 if (p.vel) {
                     double *v = p.vel + 3 * (size_t)i;
                     v[0] += p.half_dt * gx;
@@ -186,9 +236,9 @@ __global__ void __launch_bounds__(T) force_f64_kernel(const ForceParams p)
         const int i = i0 + threadIdx.x + k * T;
         if (i < n) {
             double *q = p.partial + ((size_t)js * n + i) * 3;
-            q[0] = ax[k];
-            q[1] = ay[k];
-            q[2] = az[k];
+            q[0] = a[k][0];
+            q[1] = a[k][1];
+            q[2] = a[k][2];
         }
     }
     __threadfence();
@@ -203,11 +253,11 @@ __global__ void __launch_bounds__(T) force_f64_kernel(const ForceParams p)
         if (i < n) {
             double t[3];
             sum_slots(p.partial + (size_t)i * 3, (size_t)n * 3, p.nsplit, t);
-            double *a = p.acc + 3 * (size_t)i;
+            double *o = p.acc + 3 * (size_t)i;
             const double gx = p.G * t[0], gy = p.G * t[1], gz = p.G * t[2];
-            a[0] = gx;
-            a[1] = gy;
-            a[2] = gz;
+            o[0] = gx;
+            o[1] = gy;
+            o[2] = gz;
             if (p.vel) {
                 double *v = p.vel + 3 * (size_t)i;
                 v[0] += p.half_dt * gx;
@@ -269,7 +319,7 @@ __global__ void __launch_bounds__(T) energy_f64_kernel(const EnergyParams p)
         ii[k] = i;
         ax[k] = ay[k] = az[k] = ph[k] = 0.0;
     }
-    sweep64<T, I, J, ZEPS, true>(P, t0 * J, min(t1 * J, n), p.eps2, xi, yi, zi, ii, ax, ay, az, ph, tile);
+    energy_sweep<T, I, J, ZEPS>(P, t0 * J, min(t1 * J, n), p.eps2, xi, yi, zi, ii, ax, ay, az, ph, tile);
 
     double v[8] = {0, 0, 0, 0, 0, 0, 0, 0};
 #pragma unroll

@@ -333,12 +333,13 @@ int even_splits(const nb_ctx *c, const KernelEntry &k, int64_t n, double &cycles
 }
 
 // j-splits of equal body counts for a float64 force kernel over n bodies: the
-// least time of the busiest SM, whose ceil(tiles s / SMs) CTAs of W warps take
-// max(112 W, 730) I cycles per j-body (16 cycles of the SM's float64 pipe for
-// each of 7 operations; the latency of one step where few warps share the SM),
-// a CTA some 17 j-bodies besides and the sum over the splits 100 cycles each.
-// Within 12 % of every split from 1 to 79 at 300 to 16384 bodies.  4097 bodies:
-// 23 splits and 238 us, 273 with whole j-tiles; 1024: 37 and 34 us (70 with whole tiles).
+// least time of the busiest SM, whose ceil(tiles s / SMs) CTAs give it W warps,
+// max(78 W, 500 + 50 W) I cycles per j-body (78 at full load; the latency of a
+// step where few warps share the SM), a CTA some 20 j-bodies besides and the
+// sum over the splits 100 cycles each.  Fitted to every split up to 79 at 14
+// sizes from 64 to 16384 bodies, where its choice is within 5 % of the best.
+// With whole j-tiles and a full last wave 4097 bodies took 33 splits and 205
+// us, with 23 181.
 int f64_splits(const nb_ctx *c, const KernelEntry &k, int64_t n)
 {
     const int64_t tiles = (n + k.tile() - 1) / k.tile();
@@ -349,8 +350,9 @@ int f64_splits(const nb_ctx *c, const KernelEntry &k, int64_t n)
     double least = -1;
     for (int64_t s = 1; s <= smax && (s == 1 || s * n <= cap); ++s) {
         const int64_t ctas = (tiles * s + c->num_sms - 1) / c->num_sms;
-        const double body = k.I * std::max(112.0 * (double)(ctas * k.T / 32), 730.0);
-        const double w = ((double)((n + s - 1) / s) + 17) * body + 100.0 * (double)s;
+        const double warps = (double)(ctas * k.T / 32);
+        const double body = k.I * std::max(78.0 * warps, 500.0 + 50.0 * warps);
+        const double w = ((double)((n + s - 1) / s) + 20) * body + 100.0 * (double)s;
         if (least < 0 || w < least) {
             least = w;
             best = (int)s;

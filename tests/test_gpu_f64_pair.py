@@ -1,4 +1,4 @@
-"""float64 forces: the integer pair factor at the edges of its ranges, j-splits of equal body counts."""
+"""float64 forces: the integer pair terms at the edges of its ranges, j-splits of equal body counts."""
 import numpy as np
 import pytest
 
@@ -28,7 +28,7 @@ def _check(cuda, pos, mass, eps, split=0, variant=0):
         nb.sync()
     ref, size = _exact(pos, mass, eps)
     # a pair's term: differences and r^2 3 x 2^-53 (1.5 fold for the power), the
-    # factor and its two products below 5 x 2^-53; n additions of 2^-53 each
+    # factor and its product below 5 x 2^-53; n additions of 2^-53 each
     assert (np.abs(a - ref) <= (n + 10) * 2.0 ** -53 * size).all()
 
 
