@@ -13,8 +13,8 @@
 //
 // Layout and schedule follow the float64 kernel: an i-tile of T*I bodies per
 // CTA, j-bodies streamed through a double-buffered shared tile, the grid
-// split over j with the last arriving CTA adding the float64 partials in split
-// order.  Positions are float64 (double4 x,y,z,m) in Morton order; each CTA
+// split over j in equal body counts with the last arriving CTA adding the
+// float64 partials in split order.  Positions are float64 (double4 x,y,z,m) in Morton order; each CTA
 // takes the centre of its i-tile's bounding box as origin c and forms, in
 // float64, x - c for its i-bodies and c - x for the j-bodies before splitting
 // them into hi/lo float32 pairs, so that close pairs (whose differences need
@@ -194,8 +194,8 @@ __global__ void __launch_bounds__(T) force_df_kernel(const ForceParams p)
     const int it = blockIdx.x % n_itiles;
     const int js = blockIdx.x / n_itiles;
     const int i0 = it * TILE_I;
-    int t0, t1;
-    split_range((n + J - 1) / J, p.nsplit, js, t0, t1);
+    const int jlo = (int)((long long)n * js / p.nsplit);  // an equal share of the bodies
+    const int jhi = (int)((long long)n * (js + 1) / p.nsplit);
 
     // origin: the centre of the i-tile's bounding box (float64)
     __shared__ double red[6][T / 32];
@@ -260,25 +260,28 @@ __global__ void __launch_bounds__(T) force_df_kernel(const ForceParams p)
     const float2 e2h = make_float2(e2hs, e2hs), e2l = make_float2(e2ls, e2ls);
 
     double4 buf[J / T];
-    if (t0 < t1) {
-        df_stage_load<T, J>(buf, P, t0 * J, n);
+    if (jlo < jhi) {
+        df_stage_load<T, J>(buf, P, jlo, jhi);
         df_stage_store<T, J>(tile[0], buf, c);
     }
     __syncthreads();
-    for (int t = t0; t < t1; ++t) {
-        const int bsel = (t - t0) & 1;
-        if (t + 1 < t1) df_stage_load<T, J>(buf, P, (t + 1) * J, n);
+    int bsel = 0;
+    for (int j0 = jlo; j0 < jhi; j0 += J, bsel ^= 1) {
+        if (j0 + J < jhi) df_stage_load<T, J>(buf, P, j0 + J, jhi);
         DF2 acc[NP][3];
 #pragma unroll
         for (int q = 0; q < NP; ++q)
 #pragma unroll
             for (int k = 0; k < 3; ++k) acc[q][k].h = acc[q][k].l = make_float2(0.f, 0.f);
         const float4(*s)[4] = tile[bsel];
-#pragma unroll 2
-        for (int jj = 0; jj < J; ++jj) {
-            const float4 A = s[jj][0], B = s[jj][1], C = s[jj][2], D = s[jj][3];
+        const int jn = min(J, jhi - j0);  // odd: a massless body more
+        for (int j2 = 0; j2 < jn; j2 += 2) {
 #pragma unroll
-            for (int q = 0; q < NP; ++q) df_pair<ZEPS>(A, B, C, D, xi[q], e2h, e2l, acc[q]);
+            for (int jj = j2; jj < j2 + 2; ++jj) {
+                const float4 A = s[jj][0], B = s[jj][1], C = s[jj][2], D = s[jj][3];
+#pragma unroll
+                for (int q = 0; q < NP; ++q) df_pair<ZEPS>(A, B, C, D, xi[q], e2h, e2l, acc[q]);
+            }
         }
         // fold the tile's double-float sums (of -a) into float64
 #pragma unroll
@@ -290,7 +293,7 @@ __global__ void __launch_bounds__(T) force_df_kernel(const ForceParams p)
             ay[2 * q + 1] -= (double)acc[q][1].h.y + (double)acc[q][1].l.y;
             az[2 * q + 1] -= (double)acc[q][2].h.y + (double)acc[q][2].l.y;
         }
-        if (t + 1 < t1) df_stage_store<T, J>(tile[bsel ^ 1], buf, c);
+        if (j0 + J < jhi) df_stage_store<T, J>(tile[bsel ^ 1], buf, c);
         __syncthreads();
     }
 
@@ -336,14 +339,9 @@ __global__ void __launch_bounds__(T) force_df_kernel(const ForceParams p)
     for (int k = 0; k < I; ++k) {
         const int i = i0 + threadIdx.x + k * T;
         if (i < n) {
-            double x = 0.0, y = 0.0, z = 0.0;
-            for (int q = 0; q < p.nsplit; ++q) {
-                const double *r = p.partial + ((size_t)q * n + i) * 3;
-                x += __ldcg(r);
-                y += __ldcg(r + 1);
-                z += __ldcg(r + 2);
-            }
-            emit(k, x, y, z);
+            double t[3];
+            sum_slots(p.partial + (size_t)i * 3, (size_t)n * 3, p.nsplit, t);
+            emit(k, t[0], t[1], t[2]);
         }
     }
     if (threadIdx.x == 0) p.counters[it] = 0u;

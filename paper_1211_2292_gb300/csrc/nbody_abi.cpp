@@ -163,8 +163,8 @@ const KernelEntry &kernel_for(int kind, nb_precision p, int v, bool zeps)
 // Untuned defaults.
 int default_variant(int kind, nb_precision p, int64_t n)
 {
-    // double-float: 128-body tiles (more CTAs, more compact tiles) below 4096 bodies
-    if (kind == nb::KIND_FORCE && p == NB_DF64) return n < 4096 ? 2 : 0;
+    // double-float: 128-body tiles (more compact, and as fast as 256-body ones)
+    if (kind == nb::KIND_FORCE && p == NB_DF64) return 2;
     // float32: the team kernels (the table's last two) while blocks of one
     // thread per body or two leave SMs idle
     if (kind == nb::KIND_FORCE && !f64_like(p) && n < 8192)
@@ -332,27 +332,35 @@ int even_splits(const nb_ctx *c, const KernelEntry &k, int64_t n, double &cycles
     return best;
 }
 
-// j-splits of equal body counts for a float64 force kernel over n bodies: the
-// least time of the busiest SM, whose ceil(tiles s / SMs) CTAs give it W warps,
-// max(78 W, 500 + 50 W) I cycles per j-body (78 at full load; the latency of a
-// step where few warps share the SM), a CTA some 20 j-bodies besides and the
-// sum over the splits 100 cycles each.  Fitted to every split up to 79 at 14
-// sizes from 64 to 16384 bodies, where its choice is within 5 % of the best.
-// With whole j-tiles and a full last wave 4097 bodies took 33 splits and 205
-// us, with 23 181.
+// j-splits of equal body counts for a float64 or double-float force kernel over
+// n bodies: the least time of the busiest SM, whose ceil(tiles s / SMs) CTAs
+// give it W warps.  A j-body takes them max(78 W, 500 + 50 W) I cycles in the
+// float64 kernel, max(136 ceil(W / 4) + 30, 110 + 20 W) I in the double-float
+// one, whose pipes are each scheduler's own (full load; the latency of a step
+// where few warps share the SM), a CTA some 20 or 50 j-bodies besides (the
+// double-float one splits its bodies in float64), the sum over the splits 100
+// or 200 cycles each.  Fitted to every split up to 79 at 14 sizes
+// from 64 to 33000 bodies, where the choice is within 5 % of the best.  Whole
+// j-tiles and a full last wave gave 4097 float64 bodies 33 splits and 205 us,
+// 23 take 181; 16384 double-float bodies 1136 us, 19 splits 1077.
 int f64_splits(const nb_ctx *c, const KernelEntry &k, int64_t n)
 {
     const int64_t tiles = (n + k.tile() - 1) / k.tile();
     if (tiles > c->n_counters) return 1;
+    const bool df = c->prec == NB_DF64;
     const int64_t cap = c->partial_bodies * 4 / 3;  // body-splits that fit
     const int64_t smax = std::min<int64_t>(std::max<int64_t>(n / 8, 1), 256);
     int best = 1;
     double least = -1;
     for (int64_t s = 1; s <= smax && (s == 1 || s * n <= cap); ++s) {
         const int64_t ctas = (tiles * s + c->num_sms - 1) / c->num_sms;
-        const double warps = (double)(ctas * k.T / 32);
-        const double body = k.I * std::max(78.0 * warps, 500.0 + 50.0 * warps);
-        const double w = ((double)((n + s - 1) / s) + 20) * body + 100.0 * (double)s;
+        const double W = (double)(ctas * k.T / 32);
+        const double w =
+            df ? ((double)((n + s - 1) / s) + 50) * k.I *
+                         std::max(136.0 * std::ceil(W / 4) + 30, 110 + 20 * W) +
+                     200.0 * (double)s
+               : ((double)((n + s - 1) / s) + 20) * k.I * std::max(78 * W, 500 + 50 * W) +
+                     100.0 * (double)s;
         if (least < 0 || w < least) {
             least = w;
             best = (int)s;
@@ -423,7 +431,7 @@ nb_status force_packed(nb_ctx *c, cudaStream_t s, int64_t n, double G, double ep
     double cycles;
     const int S = k.team()              ? team_cluster(c, k, n, forced)
                   : k.even && forced == 0 ? even_splits(c, k, n, cycles)
-                  : c->prec == NB_FP64 && forced == 0 ? f64_splits(c, k, n)
+                  : is_f64(c) && forced == 0 ? f64_splits(c, k, n)
                                           : splits_for(c, k, n, forced, 3);
     nb::ForceParams p;
     p.P = c->pack;

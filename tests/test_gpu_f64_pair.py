@@ -1,9 +1,10 @@
-"""float64 forces: the integer pair terms at the edges of its ranges, j-splits of equal body counts."""
+"""float64 forces: the integer pair terms at the edges of their ranges; j-splits of equal body counts."""
 import numpy as np
 import pytest
 
+import oracle
 from paper_1211_2292_gb300 import inputs, nbody
-from helpers import host, to_dev
+from helpers import host, relerr_per_body, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -57,3 +58,17 @@ def test_exponents_of_differences_and_softening(cuda, scale, rel):
     # |a| ~ m 2^(-2 scale): scaled so that the sums stay in range
     mass = np.ldexp(mass, scale)
     _check(cuda, np.ldexp(pos, scale), mass, float(np.ldexp(rel, scale)))
+
+
+@pytest.mark.parametrize("variant", range(3))
+@pytest.mark.parametrize("n", [2, 15, 127, 129, 257, 3001])
+def test_double_float_even_splits(cuda, n, variant):
+    # the mode's bound, 1e-12 per body
+    b = inputs.random_system(n, seed=n)
+    x, m = to_dev(b.pos, cuda), to_dev(b.mass, cuda)
+    for eps, split in ((0.05, 0), (0.05, 1), (0.05, 3)):
+        with nbody.NBody(n, "df64") as nb:
+            nb.tune_set(nbody.KIND_FORCE, 0, 1 << 40, variant, split)
+            a = host(nb.forces(x, m, 1.0, eps))
+            nb.sync()
+        assert relerr_per_body(a, oracle.accel(b.pos, b.mass, 1.0, eps)).max() <= 1e-12
