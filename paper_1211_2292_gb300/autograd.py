@@ -7,13 +7,13 @@ autograd can differentiate with respect to x0, v0 and m.
 
 Forward: one ``nb_rollout`` call that records the state every ``every``
 steps (segment checkpoints).  Backward, segment by segment from the last:
-restore the checkpoint, recompute the segment's positions with
-``nb_rollout(record_every=1)``, then run ``nb_step_backward`` (the reverse
-sweep with the force VJP kernel).  Memory: (nsteps/every + 1) checkpoints of
-(x, v) plus one segment of positions; compute: one extra forward pass.
-
-This module only allocates tensors and orders library calls; all arithmetic
-runs in the CUDA kernels.
+restore the checkpoint, recompute the positions up to the next checkpoint with
+``nb_rollout(record_every=1)`` and one more kick and drift, then run
+``nb_step_backward`` (the reverse sweep with the force VJP kernel).  Memory:
+(nsteps/every + 1) checkpoints of (x, v) plus one segment of positions;
+compute: every - 1 force evaluations per segment of `every` steps.  (With the
+segment's end position and the force there computed again too, every + 1:
+2.63 ms for 4 steps of 16384 bodies with every = 2, 2.22 now.)
 """
 from __future__ import annotations
 
@@ -64,10 +64,21 @@ class NBodyRollout(torch.autograd.Function):
         for s in range(nseg - 1, -1, -1):
             start = s * every
             length = min(every, nsteps - start)
-            x.copy_(ckx[s])
-            v.copy_(ckv[s])
-            seg = traj[: length + 1]
-            nb.rollout(x, v, m, G, eps, dt, length, acc, 1, seg)
+            ends_recorded = length == every  # in ckx[s + 1]
+            if ends_recorded and length == 1:
+                seg = ckx[s: s + 2]
+            else:
+                # positions 1..new are computed again: new force evaluations, the
+                # last kick and drift needs none after it
+                seg = traj[: length + 1]
+                new = length - 1 if ends_recorded else length
+                x.copy_(ckx[s])
+                v.copy_(ckv[s])
+                nb.rollout(x, v, m, G, eps, dt, new - 1, acc, 1, seg[:new])
+                v.add_(acc, alpha=0.5 * dt)
+                torch.add(x, v, alpha=dt, out=seg[new])
+                if ends_recorded:
+                    seg[length].copy_(ckx[s + 1])
             nb.step_backward(seg, m, G, eps, dt, length, lam_x, lam_v, lam_m,
                              at_start=(s == 0), at_end=(s == nseg - 1))
         return lam_x, lam_v, lam_m, None, None, None, None, None, None
