@@ -333,8 +333,6 @@ __global__ void __launch_bounds__(32 * UP_WARPS) fmm_p2m_kernel(const FmmParams 
         const int L = t.level[leaf];
         const int4 ci = icentre(t.prefix[leaf], L);
         const int k0 = t.start[leaf], k1 = t.end[leaf];
-        f.ci[leaf] = ci;
-        f.nd[leaf] = make_int4(0, t.first[leaf], k0, k1);
         double z[3];
         centre_of(p.box, ci, z);
         float zh[3], zl[3];
@@ -401,11 +399,7 @@ __global__ void __launch_bounds__(32 * UP_WARPS) fmm_m2m_kernel(const FmmParams 
 #pragma unroll
             for (int off = 4; off > 0; off >>= 1) Mc[q] += __shfl_down_sync(FULL, Mc[q], off, 8);
         }
-        if (o == 0 && nch > 0) {
-            f.ci[node] = icentre(t.prefix[node], L);
-            f.nd[node] = make_int4(nch, c0, t.start[node], t.end[node]);
-            store_exp<P>(f.M + (size_t)node * NP, Mc);
-        }
+        if (o == 0 && nch > 0) store_exp<P>(f.M + (size_t)node * NP, Mc);
     }
 }
 
@@ -1232,7 +1226,7 @@ __global__ void __launch_bounds__(32 * WARPS, NEAR_BLOCKS) fmm_near_kernel(const
     const int slice_len = f.meta[FMM_META_SLICE];
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         f.stats[0] = (unsigned long long)(t.meta[TREE_META_BASE + 10] + t.meta[TREE_META_COUNT + 10]);
-        f.stats[1] = (unsigned long long)nleaves;
+        f.stats[1] = t.stats[1] = (unsigned long long)nleaves;
     }
     float *Lf = reinterpret_cast<float *>(lists[warp]);
     const float4 *L4 = lists[warp];
@@ -1450,6 +1444,29 @@ __global__ void __launch_bounds__(128) fmm_init_kernel(FmmView f, double theta)
     }
 }
 
+// The cells' centres, ranges and child counts (the children of a cell are a run
+// of the next level's nodes), which the passes read.  They make the upward pass
+// and the lists independent of each other, and of the tree code's moments,
+// which are not formed for an FMM call (36 us at 30001 bodies, 114 at 2^20).
+template <int P>
+__global__ void __launch_bounds__(256) fmm_cells_kernel(const FmmParams p)
+{
+    const TreeView &t = p.tree;
+    const int total = t.meta[TREE_META_BASE + 10] + t.meta[TREE_META_COUNT + 10];
+    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < total; q += gridDim.x * blockDim.x) {
+        const int first = t.first[q];
+        int nch = t.nchild[q];  // 0: a leaf
+        if (nch != 0) {
+            nch = 1;  // eight at most
+            while (first + nch < total && t.parent[first + nch] == q) ++nch;
+            t.nchild[q] = nch;
+        }
+        p.f.ci[q] = icentre(t.prefix[q], t.level[q]);
+        p.f.nd[q] = make_int4(nch, first, t.start[q], t.end[q]);
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) t.stats[0] = (unsigned long long)total;
+}
+
 template <class K>
 int resident_grid(K kernel, int threads, int num_sms, cudaError_t &e)
 {
@@ -1460,18 +1477,24 @@ int resident_grid(K kernel, int threads, int num_sms, cudaError_t &e)
 
 // near = false: upward pass, downward levels and the near-field work items;
 // near = true: the near field and the split leaves' combination.
+//
+// On stream s the lists, the work items and (by the caller) the near field; on
+// fs.side the expansions: the upward pass beside the lists, M2L and L2L once
+// these are there, beside the work items and the host's reading of their
+// number.  On a small tree all of these are chains of short launches: 30001
+// bodies (order 4) 500 -> 434 us, 2^20 bodies (order 6) 4.64 -> 4.46 ms; without
+// the tree code's moments 391 us and 4.38 ms.
 template <int P>
-cudaError_t launch_fmm_order(cudaStream_t s, const FmmParams &p, bool near, int &kernels)
+cudaError_t launch_fmm_order(cudaStream_t s, const FmmStreams &fs, const FmmParams &p, bool near,
+                             int &kernels)
 {
     kernels = 0;
     cudaError_t e = cudaSuccess;
+    auto then = [&](cudaStream_t from, cudaEvent_t ev, cudaStream_t to) {  // `to` waits for `from`
+        if (e == cudaSuccess) e = cudaEventRecord(ev, from);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(to, ev, 0);
+    };
     if (!near) {
-        fmm_init_kernel<P><<<1, 128, 0, s>>>(p.f, p.theta);
-        const int p2m_grid = (int)std::min<long long>(
-            8 * p.num_sms, ((long long)p.tree.cap + 32 * UP_WARPS - 1) / (32 * UP_WARPS));
-        fmm_p2m_kernel<P><<<p2m_grid, 32 * UP_WARPS, 0, s>>>(p);
-        for (int L = LEVELS - 2; L >= 0; --L)
-            fmm_m2m_kernel<P><<<4 * p.num_sms, 32 * UP_WARPS, 0, s>>>(p, L);
         const int down_grid = resident_grid(fmm_down_kernel<P>, 32 * DOWN_WARPS, p.num_sms, e);
         if (e != cudaSuccess) return e;
         const int leaves_grid = resident_grid(fmm_leaves_kernel<P>, 32 * WARPS, p.num_sms, e);
@@ -1482,16 +1505,26 @@ cudaError_t launch_fmm_order(cudaStream_t s, const FmmParams &p, bool near, int 
         if (e != cudaSuccess) return e;
         const int m2l_grid = resident_grid(fmm_m2l_kernel<P>, 32 * WARPS, p.num_sms, e);
         if (e != cudaSuccess) return e;
+        fmm_init_kernel<P><<<1, 128, 0, s>>>(p.f, p.theta);
+        fmm_cells_kernel<P><<<2 * p.num_sms, 256, 0, s>>>(p);
+        then(s, fs.tree, fs.side);
+        const int p2m_grid = (int)std::min<long long>(
+            8 * p.num_sms, ((long long)p.tree.cap + 32 * UP_WARPS - 1) / (32 * UP_WARPS));
+        fmm_p2m_kernel<P><<<p2m_grid, 32 * UP_WARPS, 0, fs.side>>>(p);
+        for (int L = LEVELS - 2; L >= 0; --L)
+            fmm_m2m_kernel<P><<<4 * p.num_sms, 32 * UP_WARPS, 0, fs.side>>>(p, L);
         for (int L = 0; L < LEVELS; ++L) {  // level L has at most 8^L cells
             const int g = L < 6 ? std::min(down_grid, 1 << (3 * L)) : down_grid;
             fmm_down_kernel<P><<<g, 32 * DOWN_WARPS, 0, s>>>(p, L);
         }
         fmm_leaves_kernel<P><<<leaves_grid, 32 * WARPS, 0, s>>>(p);
-        fmm_m2l_kernel<P><<<m2l_grid, 32 * WARPS, 0, s>>>(p);
-        for (int L = 1; L < LEVELS; ++L) fmm_l2l_kernel<P><<<2 * p.num_sms, 128, 0, s>>>(p, L);
+        then(s, fs.lists, fs.side);
         fmm_items_kernel<P><<<1, 1024, 0, s>>>(p, 4 * WARPS * near_resident);
-        kernels = 5 + 3 * LEVELS - 2;
-        return cudaGetLastError();
+        fmm_m2l_kernel<P><<<m2l_grid, 32 * WARPS, 0, fs.side>>>(p);
+        for (int L = 1; L < LEVELS; ++L)
+            fmm_l2l_kernel<P><<<2 * p.num_sms, 128, 0, fs.side>>>(p, L);
+        kernels = 6 + 3 * LEVELS - 2;
+        return e != cudaSuccess ? e : cudaGetLastError();
     }
     const bool zeps = p.eps2f == 0.0f;
     const int near_grid = zeps ? resident_grid(fmm_near_kernel<P, true>, 32 * WARPS, p.num_sms, e)

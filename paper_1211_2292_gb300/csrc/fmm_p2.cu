@@ -3,6 +3,7 @@
 
 namespace nb {
 namespace fmm {
-template cudaError_t launch_fmm_order<2>(cudaStream_t, const FmmParams &, bool, int &);
+template cudaError_t launch_fmm_order<2>(cudaStream_t, const FmmStreams &, const FmmParams &, bool,
+                                         int &);
 }  // namespace fmm
 }  // namespace nb

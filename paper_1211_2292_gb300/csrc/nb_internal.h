@@ -243,11 +243,12 @@ int tree_meta_ints();
 // most leaf_cap bodies (no build can exceed it).
 int64_t tree_node_bound(int64_t n, int leaf_cap);
 // Build over the sorted keys launch_tree_sort left in o.keys[0] (o.vals[0] and
-// o.hist are scratch), float64 moments, float32 walk data.
+// o.hist are scratch); with `moments` the float64 monopoles, the children's
+// counts and the float32 walk data too.
 // box = {lo_x, lo_y, lo_z, ext} from launch_tree_sort.
 cudaError_t launch_tree_build(cudaStream_t s, const TreeView &t, int n, const OrderScratch &o,
                               const double *box, const double *pos, const double *mass,
-                              const int *perm, int leaf_cap, int *err, int &kernels);
+                              const int *perm, int leaf_cap, bool moments, int *err, int &kernels);
 cudaError_t launch_tree_walk(cudaStream_t s, const TreeWalkParams &p, bool zeps, int &kernels);
 // Where tree.cu keeps each level's node count and first node, and the walk's
 // group queue, in TreeView::meta.
@@ -358,9 +359,18 @@ struct FmmParams {
     int *err;
     int num_sms;
 };
+// A second stream of the context's own for the expansions, and the points at
+// which the two wait for one another: the tree is there, the lists are, the
+// expansions are.
+struct FmmStreams {
+    cudaStream_t side = nullptr;
+    cudaEvent_t tree = nullptr, lists = nullptr, far = nullptr;
+};
 // near = false: upward pass, downward levels, near-field work items (the
-// host then reads the meta counters); near = true: the near field.
-cudaError_t launch_fmm(cudaStream_t s, const FmmParams &p, bool near, int &kernels);
+// host then reads the meta counters), the expansions on fs.side, from where the
+// caller joins them; near = true: the near field.
+cudaError_t launch_fmm(cudaStream_t s, const FmmStreams &fs, const FmmParams &p, bool near,
+                       int &kernels);
 
 // ------------------------------------ orthogonal recursive bisection (orb.cu)
 // Group ids are the first processor of a part; `slot` maps a group id to
@@ -431,6 +441,7 @@ struct nb_ctx {
     int64_t n_max = 0;
     cudaStream_t stream = nullptr;      // caller's stream
     cudaStream_t cap_stream = nullptr;  // library stream used for graph capture/launch
+    nb::FmmStreams fmm_streams;
     cudaEvent_t ev_in = nullptr, ev_out = nullptr;
 
     // scratch

@@ -769,6 +769,9 @@ void free_ctx(nb_ctx *c)
     cudaFree(c->let_tctr);
     if (c->host_out) cudaFreeHost(c->host_out);
     if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
+    if (c->fmm_streams.side) cudaStreamDestroy(c->fmm_streams.side);
+    for (cudaEvent_t ev : {c->fmm_streams.tree, c->fmm_streams.lists, c->fmm_streams.far})
+        if (ev) cudaEventDestroy(ev);
     if (c->ev_in) cudaEventDestroy(c->ev_in);
     if (c->ev_out) cudaEventDestroy(c->ev_out);
     delete c;
@@ -972,7 +975,7 @@ struct TreeTimer {
 
 // Sort, pack and build the tree over n bodies (kept in the context).
 nb_status tree_build_enqueue(nb_ctx *c, cudaStream_t s, int64_t n, const double *pos,
-                             const double *mass, int leaf_cap)
+                             const double *mass, int leaf_cap, bool moments = true)
 {
     int k = 0;
     TreeTimer tm(c, nb::PROF_TREE_BUILD, s);
@@ -980,7 +983,7 @@ nb_status tree_build_enqueue(nb_ctx *c, cudaStream_t s, int64_t n, const double 
     NB_CUDA(c, nb::launch_tree_sort(s, (int)n, pos, c->order, c->tree_perm, c->tree_box, pk, k));
     c->launches += k;
     NB_CUDA(c, nb::launch_tree_build(s, c->tree, (int)n, c->order, c->tree_box, pos, mass,
-                                     c->tree_perm, leaf_cap, c->err, k));
+                                     c->tree_perm, leaf_cap, moments, c->err, k));
     c->launches += k;
     tm.done();
     return NB_OK;
@@ -1056,7 +1059,7 @@ nb_status fmm_forces_run(nb_ctx *c, int64_t n, const double *pos, const double *
     cudaStream_t s = c->stream;
     int k = 0;
     c->let_n = 0;  // the local tree of nb_let_build is replaced
-    NB_TRY(tree_build_enqueue(c, s, n, pos, mass, leaf_cap));
+    NB_TRY(tree_build_enqueue(c, s, n, pos, mass, leaf_cap, false));
     for (int attempt = 0;; ++attempt) {
         nb::FmmParams p;
         p.tree = c->tree;
@@ -1081,23 +1084,33 @@ nb_status fmm_forces_run(nb_ctx *c, int64_t n, const double *pos, const double *
         p.err = c->err;
         p.num_sms = c->num_sms;
         TreeTimer tm(c, nb::PROF_FMM_FAR, s);
-        NB_CUDA(c, nb::launch_fmm(s, p, false, k));
+        const nb::FmmStreams &fs = c->fmm_streams;
+        const cudaError_t launched = nb::launch_fmm(s, fs, p, false, k);
         c->launches += k;
-        tm.done();
         int meta[nb::FMM_META_INTS];
-        NB_CUDA(c, cudaMemcpyAsync(meta, c->fmm.meta, sizeof(meta), cudaMemcpyDeviceToHost, s));
-        NB_CUDA(c, cudaStreamSynchronize(s));
+        cudaError_t e = launched;
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(meta, c->fmm.meta, sizeof(meta), cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess) e = cudaEventRecord(c->ev_in, s);  // (a copy to pageable memory)
+        // s takes the expansions in, whatever failed before
+        if (cudaEventRecord(fs.far, fs.side) != cudaSuccess ||
+            cudaStreamWaitEvent(s, fs.far, 0) != cudaSuccess)
+            cudaStreamSynchronize(fs.side);
+        NB_CUDA(c, e);
+        tm.done();
+        NB_CUDA(c, cudaEventSynchronize(c->ev_in));
         if (!meta[nb::FMM_META_OVERFLOW]) {
             NB_TRY(ensure_fmm_part(c, std::max(1, meta[nb::FMM_META_PSLOTS])));
             p.f = c->fmm;
             p.f.order = order;
             p.f.np = nb::fmm_floats(order);
             TreeTimer tn(c, nb::PROF_FMM_NEAR, s);
-            NB_CUDA(c, nb::launch_fmm(s, p, true, k));
+            NB_CUDA(c, nb::launch_fmm(s, fs, p, true, k));
             c->launches += k;
             tn.done();
             return NB_OK;
         }
+        NB_CUDA(c, cudaStreamSynchronize(s));  // the arrays below are replaced
         if (attempt == 8) return failf(c, NB_ENOMEM, "FMM candidate lists keep overflowing");
         // the counters hold what was asked for (past the end too); what the
         // cut-short passes did not reach, the next attempt asks for
@@ -1350,7 +1363,11 @@ nb_status nb_create(nb_ctx **out, int64_t n_max, nb_precision p, int device, voi
         return bail(failf(c, NB_ENOMEM, "cudaMallocHost failed"));
     if (cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&c->ev_in, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&c->ev_out, cudaEventDisableTiming) != cudaSuccess)
+        cudaEventCreateWithFlags(&c->ev_out, cudaEventDisableTiming) != cudaSuccess ||
+        cudaStreamCreateWithFlags(&c->fmm_streams.side, cudaStreamNonBlocking) != cudaSuccess ||
+        cudaEventCreateWithFlags(&c->fmm_streams.tree, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&c->fmm_streams.lists, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&c->fmm_streams.far, cudaEventDisableTiming) != cudaSuccess)
         return bail(failf(c, NB_ECUDA, "stream/event creation failed"));
     if (cudaMemset(c->counters, 0, (size_t)c->n_counters * sizeof(unsigned)) != cudaSuccess ||
         cudaMemset(c->err, 0, 4 * sizeof(int)) != cudaSuccess ||
@@ -1367,6 +1384,7 @@ nb_status nb_destroy(nb_ctx *c)
     DeviceGuard guard(c->device);
     cudaStreamSynchronize(c->stream);
     cudaStreamSynchronize(c->cap_stream);
+    cudaStreamSynchronize(c->fmm_streams.side);
     free_ctx(c);
     return NB_OK;
 }

@@ -1294,7 +1294,7 @@ int64_t tree_node_bound(int64_t n, int leaf_cap)
 
 cudaError_t launch_tree_build(cudaStream_t s, const TreeView &t, int n, const OrderScratch &o,
                               const double *box, const double *pos, const double *mass,
-                              const int *perm, int leaf_cap, int *err, int &kernels)
+                              const int *perm, int leaf_cap, bool moments, int *err, int &kernels)
 {
     // one block per 256 bodies until the blocks' table of counts, which every
     // block sums, is as large as is cheap (26 KB)
@@ -1306,6 +1306,8 @@ cudaError_t launch_tree_build(cudaStream_t s, const TreeView &t, int n, const Or
     const int nblk = (n + chunk - 1) / chunk;
     tree_levels_kernel<<<nblk, TTPB, 0, s>>>(t, n, keys, leaf_cap, chunk, lv, tab);
     tree_emit_kernel<<<nblk, TTPB, 0, s>>>(t, n, keys, chunk, lv, tab, err);
+    kernels = 2;
+    if (!moments) return cudaGetLastError();
     // a thread per node, at most the blocks that are resident on 152 SMs
     const int64_t blocks = ((int64_t)t.cap + MTPB - 1) / MTPB;
     tree_moments_kernel<<<(int)(blocks < 3040 ? blocks : 3040), MTPB, 0, s>>>(t, box, pos, mass,
