@@ -338,7 +338,7 @@ __device__ __forceinline__ int arrive_add(int *p, int v)
     return old;
 }
 
-// Float64 monopoles of every node in one launch, bottom-up without any wait
+// Float64 monopoles of every node in one launch, bottom-up without any block waiting
 // (and every node's float32 cube).  A thread per leaf sums its bodies; its
 // node then counts its bodies in at the parent with an atomic, and only the
 // child that completes the parent's count goes on to the parent, whose
@@ -356,62 +356,32 @@ __device__ __forceinline__ int arrive_add(int *p, int v)
 // 34 us with the parent's tree data loaded beside the arrival and eight bodies'
 // loads in flight per leaf; what is left is the chain of levels (arrival,
 // children's sums, division).
+//
+// In a small tree the cells of at most direct_max bodies do not wait for their
+// children but are summed from their bodies, a warp each, which leaves two or
+// three levels to climb: walk and build of 2000 bodies 123 -> 107 us, 20000
+// 182 -> 173 (this kernel 36 -> 29), 40000 244 -> 239, but 60000 319 -> 318,
+// 200000 714 -> 731 (each body summed once more per such level).  Cells of up to
+// 256, 512, 2048 bodies: 177, 175, 177 us at 20000.
 constexpr int MTPB = 64;
+constexpr int DIRECT_BODIES = 1024, DIRECT_MAX_N = 50000;
 __global__ void __launch_bounds__(MTPB) tree_moments_kernel(TreeView t,
                                                             const double *__restrict__ box,
                                                             const double *__restrict__ pos,
                                                             const double *__restrict__ mass,
-                                                            const int *__restrict__ perm)
+                                                            const int *__restrict__ perm,
+                                                            int direct_max)
 {
     const unsigned FULL = 0xffffffffu;
     const int total = t.meta[META_BASE + 10] + t.meta[META_COUNT + 10];
     if (blockIdx.x == 0 && threadIdx.x == 0) t.stats[0] = (unsigned long long)total;
     const int lane = threadIdx.x & 31, o = lane & 7;
     int leaves = 0;
-    for (int q0 = blockIdx.x * MTPB + (threadIdx.x & ~31); q0 < total; q0 += gridDim.x * MTPB) {
-        const int me = q0 + lane;
-        int node = -1, count = 0;  // what this lane counts in at its parent
-        if (me < total) {
-            float4 lo, hi;
-            cube_corners(box, t.level[me], t.prefix[me], lo, hi);
-            float *bl = reinterpret_cast<float *>(t.box_lo + me);
-            *reinterpret_cast<float2 *>(bl) = make_float2(lo.x, lo.y);
-            bl[2] = lo.z;  // [3], the child count, belongs to the climb
-            hi.w = __int_as_float(t.first[me]);
-            t.box_hi[me] = hi;
-            if (t.nchild[me] == 0) {
-                ++leaves;
-                bl[3] = __int_as_float(0);
-                const int s = t.start[me], e = t.end[me];
-                double M = 0.0, sx = 0.0, sy = 0.0, sz = 0.0;
-                for (int k = s; k < e; k += 8) {  // eight bodies' loads in flight
-                    double m[8], x[8], y[8], z[8];
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) {
-                        const int j = perm[min(k + u, e - 1)];
-                        m[u] = mass[j];
-                        x[u] = pos[3 * (size_t)j];
-                        y[u] = pos[3 * (size_t)j + 1];
-                        z[u] = pos[3 * (size_t)j + 2];
-                    }
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) {
-                        if (k + u < e) {
-                            M += m[u];
-                            sx += m[u] * x[u];
-                            sy += m[u] * y[u];
-                            sz += m[u] * z[u];
-                        }
-                    }
-                }
-                const double inv = M > 0.0 ? 1.0 / M : 0.0;
-                put_walk_moments(t, me, M, sx * inv, sy * inv, sz * inv);
-                node = t.parent[me];
-                count = e - s;
-            }
-        }
-        // climb: each lane with a node counts in; the completed parents are
-        // summed and count in themselves
+    // whether node q's sums come from its children's (else from its bodies)
+    auto climbed = [&](int q) { return q >= 0 && t.end[q] - t.start[q] > direct_max; };
+    // climb: each lane with a node (and the bodies it stands for) counts in; the
+    // completed parents are summed and count in themselves
+    auto climb = [&](int node, int count) {
         while (__any_sync(FULL, node >= 0)) {
             // (what the parent's sum will need of the tree is loaded beside
             // the arrival, whose fence and atomic are the longest link)
@@ -473,6 +443,102 @@ __global__ void __launch_bounds__(MTPB) tree_moments_kernel(TreeView t,
             node = won ? up : -1;
             count = bodies;
         }
+    };
+    for (int q0 = blockIdx.x * MTPB + (threadIdx.x & ~31); q0 < total; q0 += gridDim.x * MTPB) {
+        const int me = q0 + lane;
+        int node = -1, count = 0;  // what this lane counts in at its parent
+        if (me < total) {
+            float4 lo, hi;
+            cube_corners(box, t.level[me], t.prefix[me], lo, hi);
+            float *bl = reinterpret_cast<float *>(t.box_lo + me);
+            *reinterpret_cast<float2 *>(bl) = make_float2(lo.x, lo.y);
+            bl[2] = lo.z;  // [3], the child count, belongs to the climb
+            hi.w = __int_as_float(t.first[me]);
+            t.box_hi[me] = hi;
+            if (t.nchild[me] == 0) {
+                ++leaves;
+                bl[3] = __int_as_float(0);
+                const int s = t.start[me], e = t.end[me];
+                double M = 0.0, sx = 0.0, sy = 0.0, sz = 0.0;
+                for (int k = s; k < e; k += 8) {  // eight bodies' loads in flight
+                    double m[8], x[8], y[8], z[8];
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) {
+                        const int j = perm[min(k + u, e - 1)];
+                        m[u] = mass[j];
+                        x[u] = pos[3 * (size_t)j];
+                        y[u] = pos[3 * (size_t)j + 1];
+                        z[u] = pos[3 * (size_t)j + 2];
+                    }
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) {
+                        if (k + u < e) {
+                            M += m[u];
+                            sx += m[u] * x[u];
+                            sy += m[u] * y[u];
+                            sz += m[u] * z[u];
+                        }
+                    }
+                }
+                const double inv = M > 0.0 ? 1.0 / M : 0.0;
+                put_walk_moments(t, me, M, sx * inv, sy * inv, sz * inv);
+                node = t.parent[me];
+                if (!climbed(node)) node = -1;
+                count = e - s;
+            }
+        }
+        climb(node, count);
+    }
+    // cells of few bodies: a warp each, from the bodies, the first ones by the
+    // warps that had no leaves
+    const int nw = gridDim.x * (MTPB / 32), busy = min(nw, (total + 31) >> 5);
+    const int gw = blockIdx.x * (MTPB / 32) + (threadIdx.x >> 5);
+    for (int q = gw < busy ? nw - busy + gw : gw - busy; direct_max > 0 && q < total; q += nw) {
+        if (t.nchild[q] == 0 || climbed(q)) continue;
+        const int s = t.start[q], e = t.end[q], f = t.first[q];
+        const int nc = __popc(__ballot_sync(FULL, lane < 8 && f + o < total && t.parent[f + o] == q));
+        double v[4] = {0.0, 0.0, 0.0, 0.0};
+        for (int k = s + lane; k < e; k += 128) {
+            double m[4], x[4], y[4], z[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int j = perm[min(k + 32 * u, e - 1)];
+                m[u] = k + 32 * u < e ? mass[j] : 0.0;
+                x[u] = pos[3 * (size_t)j];
+                y[u] = pos[3 * (size_t)j + 1];
+                z[u] = pos[3 * (size_t)j + 2];
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (k + 32 * u < e) {
+                    v[0] += m[u];
+                    v[1] += m[u] * x[u];
+                    v[2] += m[u] * y[u];
+                    v[3] += m[u] * z[u];
+                }
+            }
+        }
+        // lanes with bit 4 keep y and z, the others M and x; then bit 3
+        const bool hi4 = lane & 16, hi3 = lane & 8;
+        const double r0 = __shfl_xor_sync(FULL, hi4 ? v[0] : v[2], 16);
+        const double r1 = __shfl_xor_sync(FULL, hi4 ? v[1] : v[3], 16);
+        const double a0 = (hi4 ? v[2] : v[0]) + r0, a1 = (hi4 ? v[3] : v[1]) + r1;
+        double sum = (hi3 ? a1 : a0) + __shfl_xor_sync(FULL, hi3 ? a0 : a1, 8);
+#pragma unroll
+        for (int off = 4; off > 0; off >>= 1) sum += __shfl_xor_sync(FULL, sum, off);
+        const double M = __shfl_sync(FULL, sum, 0);
+        const double cm = M > 0.0 ? sum / M : 0.0;
+        const double cx = __shfl_sync(FULL, cm, 8), cy = __shfl_sync(FULL, cm, 16),
+                     cz = __shfl_sync(FULL, cm, 24);
+        int node = -1;
+        if (lane == 0) {
+            put_walk_moments(t, q, M, cx, cy, cz);
+            t.nchild[q] = nc;
+            reinterpret_cast<int *>(t.box_lo + q)[3] = nc;
+            node = t.parent[q];
+            if (!climbed(node)) node = -1;
+        }
+        climb(node, e - s);
     }
     leaves = __reduce_add_sync(FULL, leaves);
     if (lane == 0 && leaves) atomicAdd(t.stats + 1, (unsigned long long)leaves);
@@ -1310,8 +1376,9 @@ cudaError_t launch_tree_build(cudaStream_t s, const TreeView &t, int n, const Or
     if (!moments) return cudaGetLastError();
     // a thread per node, at most the blocks that are resident on 152 SMs
     const int64_t blocks = ((int64_t)t.cap + MTPB - 1) / MTPB;
+    const int direct_max = n <= DIRECT_MAX_N ? DIRECT_BODIES : 0;
     tree_moments_kernel<<<(int)(blocks < 3040 ? blocks : 3040), MTPB, 0, s>>>(t, box, pos, mass,
-                                                                              perm);
+                                                                              perm, direct_max);
     kernels = 3;
     return cudaGetLastError();
 }
