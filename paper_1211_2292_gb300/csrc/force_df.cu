@@ -81,12 +81,6 @@ __device__ __forceinline__ void df_stage_load(double4 (&buf)[J / T], const doubl
     }
 }
 
-__device__ __forceinline__ void split_df(double v, float &h, float &l)
-{
-    h = (float)v;
-    l = (float)(v - (double)h);
-}
-
 template <int T, int J>
 __device__ __forceinline__ void df_stage_store(float4 (*tile)[4], const double4 (&buf)[J / T],
                                                double3 c)
@@ -94,10 +88,10 @@ __device__ __forceinline__ void df_stage_store(float4 (*tile)[4], const double4 
 #pragma unroll
     for (int l = 0; l < J / T; ++l) {
         float xh, xl, yh, yl, zh, zl, mh, ml;
-        split_df(c.x - buf[l].x, xh, xl);
-        split_df(c.y - buf[l].y, yh, yl);
-        split_df(c.z - buf[l].z, zh, zl);
-        split_df(buf[l].w, mh, ml);
+        split_f64(c.x - buf[l].x, xh, xl);
+        split_f64(c.y - buf[l].y, yh, yl);
+        split_f64(c.z - buf[l].z, zh, zl);
+        split_f64(buf[l].w, mh, ml);
         float4 *e = tile[l * T + threadIdx.x];
         e[0] = make_float4(xh, xh, yh, yh);
         e[1] = make_float4(zh, zh, mh, mh);
@@ -243,9 +237,9 @@ __global__ void __launch_bounds__(T) force_df_kernel(const ForceParams p)
         for (int b = 0; b < 2; ++b) {
             const int i = i0 + threadIdx.x + (2 * q + b) * T;
             const double4 v = i < n ? P[i] : c4;
-            split_df(v.x - c.x, h[b][0], l[b][0]);
-            split_df(v.y - c.y, h[b][1], l[b][1]);
-            split_df(v.z - c.z, h[b][2], l[b][2]);
+            split_f64(v.x - c.x, h[b][0], l[b][0]);
+            split_f64(v.y - c.y, h[b][1], l[b][1]);
+            split_f64(v.z - c.z, h[b][2], l[b][2]);
         }
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
@@ -256,7 +250,7 @@ __global__ void __launch_bounds__(T) force_df_kernel(const ForceParams p)
 #pragma unroll
     for (int k = 0; k < I; ++k) ax[k] = ay[k] = az[k] = 0.0;
     float e2hs, e2ls;
-    split_df(p.eps2, e2hs, e2ls);
+    split_f64(p.eps2, e2hs, e2ls);
     const float2 e2h = make_float2(e2hs, e2hs), e2l = make_float2(e2ls, e2ls);
 
     double4 buf[J / T];

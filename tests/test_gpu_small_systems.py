@@ -19,9 +19,9 @@ def _check(a, b, eps):
 
 
 @pytest.mark.parametrize("variant", [-2, -1])  # the table's last two: 64 and 128 bodies per block
-@pytest.mark.parametrize("n", [1, 7, 63, 64, 65, 129, 2047, 2048, 2049, 5003])
+@pytest.mark.parametrize("n", [1, 7, 63, 64, 65, 129, 2047, 2048, 2049, 4096, 4097, 5003])
 def test_team_kernels_at_tile_and_cluster_edges(cuda, variant, n):
-    # 2048 bodies is the largest system read straight from float64
+    # 4096 bodies is the largest system read straight from float64
     b = inputs.random_system(n, seed=n)
     v = len(nbody.variants(nbody.KIND_FORCE, "fp32_comp")) + variant
     x, m = to_dev(b.pos, cuda), to_dev(b.mass, cuda)
@@ -85,3 +85,27 @@ def test_masses_in_the_log_domain(cuda):
         nb.sync()
     err = relerr_per_body(host(a), ref)
     assert np.sqrt(np.mean(err ** 2)) <= BOUND[0] and err.max() <= BOUND[1]
+
+
+def test_packed_pairs_at_every_exponent(cuda):
+    # pairs of bodies a 2^-8 of their coordinates apart, coordinates of both
+    # signs with all 53 bits over 110 octaves and some zero: their difference is
+    # only as good as x = h + l, so a wrong bit of either half shows
+    rng = np.random.default_rng(11)
+    npair = 512
+    e = rng.integers(-50, 60, (npair, 1)).astype(float)
+    p = rng.choice([-1.0, 1.0], (npair, 3)) * (1.0 + rng.integers(0, 1 << 52, (npair, 3)) * 2.0 ** -52)
+    p *= 2.0 ** e
+    p[::7, 1] = 0.0
+    q = p + rng.choice([-1.0, 1.0], (npair, 3)) * 2.0 ** (e - 8) * rng.uniform(0.5, 1.0, (npair, 3))
+    pos = np.stack([p, q], 1).reshape(-1, 3)
+    mass = np.repeat(2.0 ** (2 * e[:, 0]), 2)  # accelerations of order 1
+    with nbody.NBody(2 * npair, "fp32_comp") as nb:
+        nb.batch_plan(np.arange(0, 2 * npair + 1, 2))
+        a = host(nb.forces_batched(to_dev(pos, cuda), to_dev(mass, cuda), 1.0, 0.0))
+        nb.sync()
+    d = q - p
+    want = mass[::2, None] * d / ((d * d).sum(1) ** 1.5)[:, None]
+    # coordinates to 2^-48 of themselves, 2^-40 of the difference; the pair in float32
+    for got, w in ((a[::2], want), (a[1::2], -want)):
+        assert (np.abs(got - w).max(1) <= 1e-5 * np.abs(w).max(1)).all()
