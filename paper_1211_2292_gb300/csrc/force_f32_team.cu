@@ -45,6 +45,17 @@ __device__ __forceinline__ void team_load(const ForceParams &p, int j, bool ok, 
     }
 }
 
+// float32 values as integers in the same order, and back.
+__device__ __forceinline__ int ordered(float x)
+{
+    const int b = __float_as_int(x);
+    return b ^ ((b >> 31) & 0x7fffffff);
+}
+__device__ __forceinline__ float from_ordered(int b)
+{
+    return __int_as_float(b ^ ((b >> 31) & 0x7fffffff));
+}
+
 template <int I, bool COMP, bool ZEPS, bool RAW>
 __global__ void __launch_bounds__(TEAM_T) force_f32_team_kernel(const ForceParams p)
 {
@@ -52,6 +63,7 @@ __global__ void __launch_bounds__(TEAM_T) force_f32_team_kernel(const ForceParam
     __shared__ __align__(16) float4 tile[TEAM_W][2 * 32];
     __shared__ float2 sums[TEAM_W][NV];  // (sum, carry) pairs
     __shared__ float2 total[NV];
+    __shared__ int2 box[3][TEAM_W];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int cs = p.nsplit;  // blocks of the cluster
     const int rank = blockIdx.x % cs, i0 = blockIdx.x / cs * TI;
@@ -63,26 +75,48 @@ __global__ void __launch_bounds__(TEAM_T) force_f32_team_kernel(const ForceParam
     float4 bh, bl;
     team_load<RAW>(p, j0 + lane, j0 + lane < j1, bh, bl);
     float4 h[I], l[I];
-    float sum[3] = {0.f, 0.f, 0.f};
 #pragma unroll
     for (int k = 0; k < I; ++k) {
         const int i = i0 + lane + 32 * k;
         team_load<RAW>(p, i, i < n, h[k], l[k]);
-        sum[0] += h[k].x;
-        sum[1] += h[k].y;
-        sum[2] += h[k].z;
+    }
+    // The origin: the centre of the bounding box of the 256 bodies around the
+    // tile (512 from 2048 bodies on with compensated sums), as if they shared a
+    // block of one or two bodies per thread.  A pair's term is then bit for bit
+    // the same in both kinds of kernel and only the order of the sums differs,
+    // so a trajectory does not depend on which of them a size is given.  (The
+    // mean of the tile's own bodies is a better origin, 6.4e-7 of |a| where this
+    // gives 1.0e-6 at 1000 bodies; the box of 64 bodies a worse one, 1.6e-6.)
+    const int around = COMP && n >= 2048 ? 512 : 256;
+    const int o0 = i0 & ~(around - 1);
+    int lo_[3], hi_[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) lo_[d] = 0x7fffffff, hi_[d] = (int)0x80000000;
+    for (int i = o0 + threadIdx.x; i < min(n, o0 + around); i += TEAM_T) {
+        float4 a, b;
+        team_load<RAW>(p, i, true, a, b);
+        const int v[3] = {ordered(a.x), ordered(a.y), ordered(a.z)};
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            lo_[d] = min(lo_[d], v[d]);
+            hi_[d] = max(hi_[d], v[d]);
+        }
     }
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1)
+    for (int d = 0; d < 3; ++d) {
+        lo_[d] = __reduce_min_sync(0xffffffffu, lo_[d]);
+        hi_[d] = __reduce_max_sync(0xffffffffu, hi_[d]);
+        if (lane == 0) box[d][warp] = make_int2(lo_[d], hi_[d]);
+    }
+    __syncthreads();
+    float cc[3];
 #pragma unroll
-        for (int d = 0; d < 3; ++d) sum[d] += __shfl_xor_sync(0xffffffffu, sum[d], off);
-    // The tile's origin: the mean of its bodies.  They are in the caller's
-    // order, so 64 of them span the system; the centre of their bounding box
-    // (the larger kernels' origin) is then thrown about by the outermost
-    // bodies, and 1000 bodies of a Plummer sphere came out at 1.6e-6 of |a|
-    // where they are 1.0e-6 with 256-body tiles.
-    const float inv = 1.0f / (float)min(TI, n - i0);
-    const float3 c = make_float3(sum[0] * inv, sum[1] * inv, sum[2] * inv);
+    for (int d = 0; d < 3; ++d) {
+        const int2 b = box[d][lane % TEAM_W];
+        cc[d] = 0.5f * (from_ordered(__reduce_min_sync(0xffffffffu, b.x)) +
+                        from_ordered(__reduce_max_sync(0xffffffffu, b.y)));
+    }
+    const float3 c = make_float3(cc[0], cc[1], cc[2]);
     float2 nx[NP], ny[NP], nz[NP], ax[NP], ay[NP], az[NP];
 #pragma unroll
     for (int q = 0; q < NP; ++q) {

@@ -30,7 +30,8 @@ struct KernelEntry {
     const void *fn;
     bool logm = false;  // float32 kernels with log-domain pairs (read log2 m from P_lo.w)
     // float32 kernels whose j-splits are equal body counts, not whole j-tiles:
-    // their time per pair, per mille (adjacent to the first compensated one); 0 for the others.
+    // their time per pair relative to the family's first compensated one, per
+    // mille; 0 for the others.
     int even = 0;
     // Kernels whose blocks share an i-tile of 32 I bodies in clusters of
     // nsplit blocks (force_f32_team.cu); `raw` is the form that reads the
