@@ -209,11 +209,8 @@ nb_status nb_step_batched(nb_ctx *ctx, double *pos, double *vel, const double *m
  * nb_variant_info fills threads per CTA, bodies per thread and j-tile size.
  * nb_tune_set makes calls with lo <= n < hi use `variant`, with `split`
  * j-splits across CTAs (0 = chosen by the scheduler); later entries win.
- * The float32 force's variants 25 and 26 share an i-tile among a cluster of
+ * The float32 force's variants 23 and 24 share an i-tile among a cluster of
  * blocks: their split is the blocks per cluster, rounded down to 1, 2, 4 or 8.
- * Its variants 21 to 24 differ in their tiles only: where a table names one of
- * them with split 0 and the bodies are in input order, the call uses the one of
- * the four whose tiles suit n best.
  * For the batched kind, n is the planned bodies and `split` is the item-cap
  * divisor d (0 = 4): when a plan has more items than resident CTAs, a work
  * item holds at most 1/d of an even per-CTA share of the pairs; it takes

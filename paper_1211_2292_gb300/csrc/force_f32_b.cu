@@ -21,11 +21,13 @@ const Quad kForceB[] = {
     NB_F32_ENTRY_X(128, 6, 256, 2, true, 3),
     NB_F32_ENTRY_X(128, 6, 128, 2, true, 3),
     // j-splits of equal body counts, for systems whose whole tiles would leave
-    // the SMs unevenly loaded (21..24), with their times per pair, plain and
-    // compensated, per mille of the first's (16411 bodies, best split: 129 / 132
-    // / 128 / 119 us and 131 / 126 / 123 / 132 us)
-    NB_F32_ENTRY_EVEN(256, 8, 256, 2, 985, 1000),
-    NB_F32_ENTRY_EVEN(128, 8, 128, 3, 1050, 1000),
+    // the SMs unevenly loaded (21..22): the bodies' layout and pair terms of
+    // variant 14 and of 12 and 20, so that results differ only by the order of
+    // the sums; with their times per pair, plain and compensated, per mille.
+    // Whole tiles / equal counts, us per call: 16411 bodies plain (20 / 22) 122 /
+    // 117, 40000 compensated (14 / 21) 603 / 591, 9000 (12 / 22) 58 / 50; but
+    // compensated (12 / 22) 79 / 76 at 12000 and 120 / 136 at 16384, where the
+    // loop of known length counts for more: variant 12 from 11000 bodies on.
     NB_F32_ENTRY_EVEN(64, 8, 128, 2, 1045, 1000),
     NB_F32_ENTRY_EVEN(128, 6, 128, 2, 1000, 1170),
 };

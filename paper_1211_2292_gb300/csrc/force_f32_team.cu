@@ -218,8 +218,10 @@ __global__ void __launch_bounds__(TEAM_T) force_f32_team_kernel(const ForceParam
     if (cs > 1) cluster.sync();  // no block leaves while its sums are being read
 }
 
-#define NB_TEAM_KERNEL(I, C, Z)                                                            \
-    {TEAM_T, I, 32, (const void *)force_f32_team_kernel<I, C, Z, false>, false, 0,         \
+// (the block's warps stage 32 j-bodies each)
+// (j-tile: 32 bodies staged by each warp)
+#define NB_TEAM_KERNEL(I, C, Z)                                                             \
+    {TEAM_T, I, 32 * TEAM_W, (const void *)force_f32_team_kernel<I, C, Z, false>, false, 0, \
      (const void *)force_f32_team_kernel<I, C, Z, true>}
 #define NB_TEAM_ENTRY(I)                                                                   \
     {{NB_TEAM_KERNEL(I, false, false), NB_TEAM_KERNEL(I, false, true)},                     \

@@ -301,22 +301,21 @@ int splits_for(nb_ctx *c, const KernelEntry &k, int64_t n, int forced, int64_t p
 }
 
 // j-splits of equal body counts for a float32 force kernel (KernelEntry::even)
-// over n bodies, and the cycles they should take.  A launch lasts as long as
-// the scheduler that receives the most warps: the CTAs of the busiest SM, at
-// most ceil(tiles s / SMs), give each of its four schedulers ceil(CTAs T / 128)
-// warps of n / s j-bodies.  Per j-body a warp takes 27.75 cycles per body pair,
-// 31.5 when it is its scheduler's only one; a CTA costs some 60 j-bodies
-// besides, a split launch its merge (its gap, 24 bytes per body-split).  Fitted
-// to every split from 3 to 63 of the four kernels at 11000, 16411 and 24000
-// bodies (within 10 %).  At 16384 bodies that gives 19 splits where whole tiles
-// gave 7, and 111 us for the call instead of 137.
-int even_splits(const nb_ctx *c, const KernelEntry &k, int64_t n, double &cycles)
+// over n bodies, the fewest cycles.  A launch lasts as long as the scheduler
+// that receives the most warps: the CTAs of the busiest SM, at most
+// ceil(tiles s / SMs), give each of its four schedulers ceil(CTAs T / 128) warps
+// of n / s j-bodies.  Per j-body a warp takes 27.75 cycles per body pair, 31.5
+// when it is its scheduler's only one; a CTA costs some 60 j-bodies besides, a
+// split launch its merge (its gap, 24 bytes per body-split).  Fitted to every
+// split from 3 to 63 of these kernels at 11000, 16411 and 24000 bodies (within
+// 10 %).
+int even_splits(const nb_ctx *c, const KernelEntry &k, int64_t n)
 {
     const int64_t tiles = (n + k.tile() - 1) / k.tile();
     const int64_t cap = c->partial_bodies * 4 / 3;  // body-splits that fit
     const double rate = k.even * 1e-3 * (k.I / 2);
     int best = 1;
-    cycles = -1;
+    double cycles = -1;
     const int64_t smax = std::min<int64_t>(std::max<int64_t>(n / 64, 1), 256);
     for (int64_t s = 1; s <= smax && (s == 1 || s * n <= cap); ++s) {
         const int64_t ctas = (tiles * s + c->num_sms - 1) / c->num_sms;
@@ -384,31 +383,12 @@ constexpr int64_t RAW_MAX = 4096;
 
 bool use_order(const nb_ctx *c, int64_t n);
 
-// The force kernel for n bodies in this context.  The kernels with even splits
-// are one family: where the table names one of them (without a split) and the
-// bodies are in the caller's order, the one that should take the fewest cycles
-// is taken, since 2048-body tiles waste an eighth of 16411 bodies and 1024-body
-// ones a fourteenth.  (In Morton order the tile's size also sets its extent,
-// and with it the rounding of the tile-local coordinates: the table decides.)
+// The force kernel for n bodies in this context.
 const KernelEntry &force_kernel(nb_ctx *c, int64_t n, double eps, int &forced)
 {
     int v;
     pick(c, nb::KIND_FORCE, n, v, forced);
-    const KernelEntry *k = &kernel_for(nb::KIND_FORCE, c->prec, v, eps == 0.0);
-    if (k->even && forced == 0 && !use_order(c, n)) {
-        double best, w;
-        even_splits(c, *k, n, best);
-        for (int u = 0; u < variant_count(nb::KIND_FORCE, c->prec); ++u) {
-            const KernelEntry &q = kernel_for(nb::KIND_FORCE, c->prec, u, eps == 0.0);
-            if (!q.even) continue;
-            even_splits(c, q, n, w);
-            if (w < best) {
-                best = w;
-                k = &q;
-            }
-        }
-    }
-    return *k;
+    return kernel_for(nb::KIND_FORCE, c->prec, v, eps == 0.0);
 }
 bool force_logm(nb_ctx *c, int64_t n, double eps)
 {
@@ -429,9 +409,8 @@ nb_status force_packed(nb_ctx *c, cudaStream_t s, int64_t n, double G, double ep
     int forced;
     const KernelEntry &k = force_kernel(c, n, eps, forced);
     const bool f32 = !is_f64(c);
-    double cycles;
     const int S = k.team()              ? team_cluster(c, k, n, forced)
-                  : k.even && forced == 0 ? even_splits(c, k, n, cycles)
+                  : k.even && forced == 0 ? even_splits(c, k, n)
                   : is_f64(c) && forced == 0 ? f64_splits(c, k, n)
                                           : splits_for(c, k, n, forced, 3);
     nb::ForceParams p;

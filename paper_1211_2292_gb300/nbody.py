@@ -128,11 +128,21 @@ def load(build_if_missing: bool = True):
         return lib
 
 
+_torch = None  # imported by the first call: an import statement per argument shows in small calls
+
+
+def _load_torch():
+    global _torch
+    import torch
+    _torch = torch
+    return torch
+
+
 def _ptr(t, name, n3=None):
     """Device pointer of a contiguous float64 CUDA tensor (None -> NULL)."""
     if t is None:
         return None
-    import torch
+    torch = _torch or _load_torch()
     if not isinstance(t, torch.Tensor):
         raise TypeError(f"{name} must be a torch.Tensor")
     if not t.is_cuda:
@@ -141,9 +151,10 @@ def _ptr(t, name, n3=None):
         raise ValueError(f"{name} must be float64")
     if not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
-    if n3 is not None and t.numel() < n3:
-        raise ValueError(f"{name} has {t.numel()} elements, needs {n3}")
-    return t.data_ptr() if t.numel() else None
+    numel = t.numel()
+    if n3 is not None and numel < n3:
+        raise ValueError(f"{name} has {numel} elements, needs {n3}")
+    return t.data_ptr() if numel else None
 
 
 def _ptr_i32(t, name, numel):
@@ -221,7 +232,9 @@ class NBody:
         self.close()
 
     def _call(self, name, *args):
-        _check(self.h, name, getattr(self.lib, name)(self.h, *args))
+        status = getattr(self.lib, name)(self.h, *args)
+        if status != 0:
+            _check(self.h, name, status)
 
     # ------------------------------------------------------------------ API
     def set_stream(self, stream=None):
@@ -235,7 +248,7 @@ class NBody:
         return int(self.lib.nb_launch_count(self.h))
 
     def forces(self, pos, mass, G, eps, out=None):
-        import torch
+        torch = _torch or _load_torch()
         n = mass.shape[0]
         if out is None:
             out = torch.empty((n, 3), dtype=torch.float64, device=pos.device)

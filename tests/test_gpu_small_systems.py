@@ -48,7 +48,7 @@ def test_output_may_overlap_the_positions(cuda):
     assert np.array_equal(got, want)
 
 
-@pytest.mark.parametrize("variant", [5, 21, 22, 23, 24])  # 21..24 split by bodies, 5 by tiles
+@pytest.mark.parametrize("variant", [5, 21, 22])  # 21, 22 split by bodies, 5 by tiles
 @pytest.mark.parametrize("n", [65, 4097, 9001, 16411])
 def test_even_splits_and_their_merge(cuda, variant, n):
     b = inputs.plummer(n, seed=n)
