@@ -3,9 +3,9 @@
 // sm_103a has two float64 lanes per SM and clock (a warp operation takes 16
 // cycles) against 64 integer ones.  So only a pair's three differences are left
 // to the float64 pipe; the squares, the -3/2 power, the product with m and the
-// sums are fixed-point, some 215 instructions and 79 cycles a warp, where 19
+// sums are fixed-point, some 225 instructions and 83 cycles a warp, where 19
 // float64 operations and two conversions took 340.  Bound by the integer pipe
-// (66 % busy, issue 64 %, float64 59 %).  16384 bodies: 9.56 ms before, 2.27
+// (66 % busy, issue 64 %, float64 59 %).  16384 bodies: 9.56 ms before, 2.47
 // now; with only the power in integers and a float64 product and sums 3.38.
 // A single term's error against 113 bits is 0.45 x 2^-53 rms and 1.6 x 2^-53 at
 // most (1.8 and 8.4 before).
@@ -174,7 +174,8 @@ __device__ __forceinline__ bool pair_term(double dx, double dy, double dz, const
 // HEAD - 6), E the largest exponent of a term so far.  A term is rounded to
 // 2^-54 of the largest (J = 128), as a float64 addition would round the sum.
 // Each step raises E without asking whether it must: in a branch, some lane of
-// a warp met a new largest term in most steps (181 us at 4097 bodies, 195).
+// a warp met a new largest term in most steps (181 us at 4097 bodies, 195; 186
+// with the rounding below).
 template <int J>
 struct FixedSum {
     static constexpr int HEAD = J <= 128 ? 6 : 7;  // terms below 2^(62 - HEAD), J of them below 2^63
@@ -192,9 +193,12 @@ struct FixedSum {
         const uint64_t s = shr_clamped(S, (unsigned)(E - e + HEAD));
         const uint32_t A1 = (uint32_t)(A >> 32), A0 = (uint32_t)A;
         const uint32_t s1 = (uint32_t)(s >> 32), s0 = (uint32_t)s;
-        // rounded; A0 s0 is left out, on the mean 2^62
-        uint64_t p = (uint64_t)A1 * s0 + 0xc0000000u;
+        // A (s + 1/2) 2^-64, rounded: s lost half a unit on the mean.  (Without
+        // the half, and with A0 s0 taken at its mean, a million terms far below
+        // the largest add up to 1e-12 of it.)
+        uint64_t p = (uint64_t)A1 * s0 + (0x80000000u + (A1 >> 1));
         p += (uint64_t)A0 * s1;
+        p += __umulhi(A0, s0);
         p = (uint64_t)A1 * s1 + (p >> 32);
         acc += (int64_t)(p ^ (uint64_t)(int64_t)sign) - sign;
     }

@@ -340,8 +340,8 @@ int even_splits(const nb_ctx *c, const KernelEntry &k, int64_t n)
 // double-float one splits its bodies in float64), the sum over the splits 100
 // or 200 cycles each.  Fitted to every split up to 79 at 14 sizes
 // from 64 to 33000 bodies, where the choice is within 5 % of the best.  Whole
-// j-tiles and a full last wave gave 4097 float64 bodies 33 splits and 205 us,
-// 23 take 181; 16384 double-float bodies 1136 us, 19 splits 1077.
+// j-tiles and a full last wave gave 4097 float64 bodies 33 splits and 13 % more
+// time than 23; 16384 double-float bodies 1136 us, 19 splits 1077.
 int f64_splits(const nb_ctx *c, const KernelEntry &k, int64_t n)
 {
     const int64_t tiles = (n + k.tile() - 1) / k.tile();
