@@ -72,3 +72,22 @@ def test_double_float_even_splits(cuda, n, variant):
             a = host(nb.forces(x, m, 1.0, eps))
             nb.sync()
         assert relerr_per_body(a, oracle.accel(b.pos, b.mass, 1.0, eps)).max() <= 1e-12
+
+
+def test_many_small_terms_beside_a_large_one(cuda):
+    # 1e5 terms of one sign, 2^-28 of the largest: rounded to 2^-55 of it at most
+    # each (300 units of 2^-54 together by chance, 1.6e-14); a quarter of a unit
+    # in one direction would make 1.4e-12
+    rng = np.random.default_rng(3)
+    n = 100001
+    pos = rng.uniform(-0.2, 0.2, (n, 3)) + np.array([1.0, 1.0, 1.0])
+    pos[0], pos[1] = 0.0, 2.0 ** -14 * np.array([0.6, 0.5, 0.7])
+    mass = rng.uniform(0.5, 1.5, n)
+    x, m = to_dev(pos, cuda), to_dev(mass, cuda)
+    with nbody.NBody(n, "fp64") as nb:
+        a = host(nb.forces(x, m, 1.0, 0.0))[0]
+        nb.sync()
+    d, w = pos[1:].astype(np.longdouble), mass[1:].astype(np.longdouble)
+    r2 = (d * d).sum(1)
+    t = (w / (r2 * np.sqrt(r2)))[:, None] * d
+    assert (np.abs(a - t.sum(0)) <= 1e-13 * np.abs(t).max(0)).all()
