@@ -395,6 +395,10 @@ __global__ void __launch_bounds__(MTPB) tree_moments_kernel(TreeView t,
                 for (int q = 0; q < 8; ++q) nch += f0 + q < total && t.parent[f0 + q] == node;
                 won = arrive_add(t.arrive + node, count) + count == bodies;
             }
+            // The children's sums are read by other lanes than the one that
+            // arrived last: what its arrival acquired becomes theirs here (a
+            // ballot or shuffle orders no memory).
+            __syncwarp();
             unsigned win = __ballot_sync(FULL, won);
             while (win) {
                 // group g of eight lanes takes the g-th winner
@@ -438,8 +442,8 @@ __global__ void __launch_bounds__(MTPB) tree_moments_kernel(TreeView t,
                 }
                 __syncwarp();
             }
-            // the sums were written by other lanes of the warp: their stores
-            // are ordered before this lane's fence by the __syncwarp
+            // and the parents' sums, written by other lanes too, are ordered
+            // before the next round's releasing arrivals by the loop's __syncwarp
             node = won ? up : -1;
             count = bodies;
         }
@@ -455,6 +459,8 @@ __global__ void __launch_bounds__(MTPB) tree_moments_kernel(TreeView t,
             bl[2] = lo.z;  // [3], the child count, belongs to the climb
             hi.w = __int_as_float(t.first[me]);
             t.box_hi[me] = hi;
+            // (a climbing warp may be replacing a parent's -1 by its count
+            // meanwhile: either is not 0, which only a leaf has, from the start)
             if (t.nchild[me] == 0) {
                 ++leaves;
                 bl[3] = __int_as_float(0);
@@ -1125,6 +1131,7 @@ __device__ __forceinline__ void walk_group(const TreeWalkParams &p, WalkShared<B
         unsigned last = 0;
         const int nspans = (ntrees + p.tspan - 1) / p.tspan;
         if (lane == 0) last = atomicAdd(p.tctr + g, 1u) == (unsigned)(nspans - 1);
+        __syncwarp();  // lane 0's arrival before the other lanes' fences
         if (!__shfl_sync(FULL, last, 0)) return;
         __threadfence();
         nc = nb = 0;

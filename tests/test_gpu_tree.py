@@ -236,3 +236,15 @@ def test_shapes_the_tree_can_take(cuda, group):
     # one leaf: the walk is the direct sum for every body
     _, cnt, st, _, _, _ = _both(cuda, cases[1][0], cases[1][1], 1.0, 0.01, 0.5, 1000, group)
     assert st["nodes"] == 1 and np.all(cnt[:, 1] == 500) and np.all(cnt[:, 0] == 0)
+
+
+@pytest.mark.parametrize("n", [20000, 60001])  # some cells summed from their bodies; all climbed
+def test_moments_do_not_depend_on_who_arrives_last(cuda, n):
+    # every evaluation's cells meet their children's sums in another order
+    b = inputs.plummer(n, seed=n)
+    x, m = to_dev(b.pos, cuda), to_dev(b.mass, cuda)
+    with nbody.NBody(n, "fp32_comp") as nb:
+        want = host(nb.tree_forces(x, m, 1.0, 0.01, 1.0, 4))
+        for _ in range(40):
+            assert np.array_equal(host(nb.tree_forces(x, m, 1.0, 0.01, 1.0, 4)), want)
+        nb.sync()
