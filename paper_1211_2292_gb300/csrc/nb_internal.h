@@ -230,6 +230,8 @@ struct TreeWalkParams {
     int *counts;            // optional [n][2]: cells, bodies met per body
     int *err;
     const WalkSource *more;  // device [1 + nmore] when nmore > 0: `tree` (again) and the trees
+    int trees;               // all trees the call walks onto these targets (64 at most counted):
+                             // the warps per group follow them, alike in each of its launches
     int nmore;               // walked after it, their sums added in order (as separate
                              // accumulating walks would); nmore 0..WALK_MAX_MORE
     // Split mode (nmore > 0): one task per group and span of tspan trees; each

@@ -1004,6 +1004,7 @@ nb_status tree_forces_enqueue(nb_ctx *c, cudaStream_t s, int64_t n, const double
     p.err = c->err;
     p.more = nullptr;
     p.nmore = 0;
+    p.trees = 1;
     p.tspan = 1;
     p.tpart = nullptr;
     p.tcnt = nullptr;
@@ -2015,8 +2016,8 @@ nb_status ensure_let_split(nb_ctx *c, cudaStream_t s, int ntrees, int64_t groups
 // received trees, one task per (group, tree).
 nb_status let_walk(nb_ctx *c, cudaStream_t s, const nb::TreeView &t, const float4 *sP,
                    const float4 *sPlo, const double *box, const nb::WalkSource *more,
-                   int nmore, double G, double eps, double theta, int group, double *acc,
-                   int *counts, int accumulate)
+                   int nmore, int trees, double G, double eps, double theta, int group,
+                   double *acc, int *counts, int accumulate)
 {
     NB_CUDA(c, cudaMemsetAsync(c->let_queue, 0, sizeof(int), s));
     nb::TreeWalkParams p;
@@ -2044,6 +2045,7 @@ nb_status let_walk(nb_ctx *c, cudaStream_t s, const nb::TreeView &t, const float
     p.err = c->err;
     p.more = more;
     p.nmore = nmore;
+    p.trees = trees;
     p.tspan = 1;
     p.tpart = nullptr;
     p.tcnt = nullptr;
@@ -2318,12 +2320,12 @@ nb_status nb_let_forces(nb_ctx *c, double G, double eps, double theta, int group
     src.insert(src.begin(), nb::WalkSource{c->tree.box_lo, c->tree.box_hi, c->tree.chi,
                                            c->tree.clo, c->tree.start, c->tree.end, c->tree_P,
                                            c->tree_Plo, c->tree_box});
-    const int first = (int)std::min<int64_t>(nlet, nb::WALK_MAX_MORE);
+    const int first = (int)std::min<int64_t>(nlet, nb::WALK_MAX_MORE), trees = 1 + first;
     if (first > 0)  // from pageable memory: staged before the call returns
         NB_CUDA(c, cudaMemcpyAsync(c->let_src, src.data(), (1 + first) * sizeof(nb::WalkSource),
                                    cudaMemcpyHostToDevice, s));
-    NB_TRY(let_walk(c, s, c->tree, c->tree_P, c->tree_Plo, c->tree_box, c->let_src, first, G, eps,
-                    theta, group, acc, counts, 0));
+    NB_TRY(let_walk(c, s, c->tree, c->tree_P, c->tree_Plo, c->tree_box, c->let_src, first, trees,
+                    G, eps, theta, group, acc, counts, 0));
     for (int64_t q0 = first; q0 < nlet; q0 += 1 + nb::WALK_MAX_MORE) {
         // a further launch: tree q0, then up to WALK_MAX_MORE more, added on
         const int more = (int)std::min<int64_t>(nlet - q0 - 1, nb::WALK_MAX_MORE);
@@ -2341,8 +2343,8 @@ nb_status nb_let_forces(nb_ctx *c, double G, double eps, double theta, int group
         t.start = const_cast<int *>(w.start);
         t.end = const_cast<int *>(w.end);
         t.stats = c->tree.stats;
-        NB_TRY(let_walk(c, s, t, w.sP, w.sPlo, w.box, c->let_src, more, G, eps, theta, group, acc,
-                        counts, 1));
+        NB_TRY(let_walk(c, s, t, w.sP, w.sPlo, w.box, c->let_src, more, trees, G, eps, theta, group,
+                        acc, counts, 1));
     }
     return NB_OK;
 }

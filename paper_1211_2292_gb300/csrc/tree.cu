@@ -1434,6 +1434,26 @@ int walk_split(int groups, int bodies_per_lane, int num_sms)
     return groups < 8 * num_sms ? 8 : (groups < 40 * num_sms ? 4 : 1);
 }
 
+// The same for a walk over `trees` trees (a process's own and the LETs it
+// received) in one launch, whose tasks are the (group, tree) pairs: what fills
+// the SMs is their number.  Measured (walk alone, us, two Plummer spheres over P
+// processes, theta 0.5, leaves of 16; 1 / 4 / 8 warps per task):
+//   groups of 64: 1024 tasks (P = 4) 466 / 189 / 147, 2048 (P = 2) 720 / 388 /
+//     360, (P = 8) 436 / 177 / 187, 4096 (P = 8) 578 / 246 / 348, 8192 (P = 2)
+//     1294 / 1206 / 1436, (P = 8) 652 / 450 / 662, 16384 (P = 8) 779 / 882 / 1297;
+//   groups of 32: 1024 (P = 2) 363 / 155 / 129, 2048 (P = 4) 386 / 172 / 186,
+//     4096 (P = 2) 591 / 457 / 486, 8192 (P = 2) 723 / 884 / 1006, (P = 8) 423 /
+//     362 / 487, 16384 (P = 8) 503 / 693 / 939.
+// (By the groups alone, as for one tree, 8 x 65536 bodies in groups of 32 took
+// 939 us, 8 x 131072 in groups of 64 882.)  Above 16 trees they are counted as
+// 16 for the step from 8 to 4 warps: most are remote and walked in a few rounds.
+int walk_split_trees(int groups, int trees, int bodies_per_lane, int num_sms)
+{
+    if (trees <= 1) return walk_split(groups, bodies_per_lane, num_sms);
+    if (groups * (int64_t)min(trees, 16) < 12 * num_sms) return 8;
+    return groups * (int64_t)trees < (bodies_per_lane == 1 ? 40 : 56) * num_sms ? 4 : 1;
+}
+
 template <int BPL, bool MULTI, int W>
 cudaError_t walk_launch(cudaStream_t s, const TreeWalkParams &p, bool zeps, int tasks, int &kernels)
 {
@@ -1462,7 +1482,7 @@ cudaError_t walk_launch_split(cudaStream_t s, const TreeWalkParams &p, bool zeps
                               int &kernels)
 {
     if (W == 8) return walk_launch<BPL, MULTI, 8>(s, p, zeps, tasks, kernels);
-    if constexpr (BPL == 2)
+    if constexpr (BPL == 2 || MULTI)
         if (W == 4) return walk_launch<BPL, MULTI, 4>(s, p, zeps, tasks, kernels);
     return walk_launch<BPL, MULTI, 1>(s, p, zeps, tasks, kernels);
 }
@@ -1478,9 +1498,8 @@ cudaError_t launch_tree_walk(cudaStream_t s, const TreeWalkParams &p, bool zeps,
     const int bpl = p.group / 32;
     const int groups = (p.n + p.group - 1) / p.group;
     const int tasks = groups * (p.nmore > 0 ? (1 + p.nmore + p.tspan - 1) / p.tspan : 1);
-    // by the groups alone, so that a tree's sums are the same whether further
-    // trees are walked or not (a task of several trees is one warp's)
-    const int W = p.nmore > 0 && p.tspan > 1 ? 1 : walk_split(groups, bpl, p.num_sms);
+    // (a task of several trees is one warp's)
+    const int W = p.nmore > 0 && p.tspan > 1 ? 1 : walk_split_trees(groups, p.trees, bpl, p.num_sms);
     if (p.nmore > 0)  // a separate instance: the single-tree walk keeps its own registers
         return bpl == 1 ? walk_launch_split<1, true>(s, p, zeps, W, tasks, kernels)
                         : walk_launch_split<2, true>(s, p, zeps, W, tasks, kernels);

@@ -171,3 +171,26 @@ def test_more_trees_than_one_launch_takes(cuda):
     assert np.array_equal(c70, c0 + 70 * (c1 - c0))
     d = a1 - a0
     assert np.allclose(a70, a0 + 70 * d, rtol=0, atol=1e-11 * np.abs(a70).max())
+
+
+@pytest.mark.parametrize("group,tasks_per_sm", [(64, 12), (64, 56), (32, 12), (32, 40)])
+@pytest.mark.parametrize("side", [0, 1])
+def test_lists_at_the_edges_of_the_warps_per_group(cuda, group, tasks_per_sm, side):
+    # two processes' walks take (group, tree) tasks with eight, four or one warp
+    # each: 8 below 12 tasks per SM, 1 from 56 (groups of 64) or 40 (of 32) on;
+    # the last number of groups below the edge and the first at it.  Lists are
+    # exact; of the forces the mean error only (in half a million bodies some
+    # close pair takes a body of small |a| past the per-body bound, whatever
+    # number of warps walks it)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    groups = -(-tasks_per_sm * sms // 2) - 1 + side
+    n = groups * group
+    b = inputs.two_plummer(n, seed=groups)
+    res = _run(cuda, b, 2, 0.8, 32, group, 0.002)
+    ref_rank = oracle.orb(b.pos, 2)
+    ref, _, ref_cnt = oracle.bh_sharded(b.pos, b.mass, 1.0, 0.002, 0.8, 32, group, ref_rank, 2)
+    for r, (_, ids, _, acc, cnt) in enumerate(res):
+        mine = np.flatnonzero(ref_rank == r)
+        assert np.array_equal(ids, mine) and len(mine) == n
+        assert np.array_equal(cnt.astype(np.int64), ref_cnt[mine, :2])
+        assert np.sqrt((relerr_per_body(acc, ref[mine]) ** 2).mean()) <= 1e-5
