@@ -10,6 +10,7 @@ context for convenience.
 """
 from __future__ import annotations
 
+import contextlib
 import ctypes
 import os
 import threading
@@ -207,8 +208,9 @@ class NBody:
         self.device = device
         h = ctypes.c_void_p()
         with torch.cuda.device(device):
+            self._stream = _stream_ptr(stream)
             st = self.lib.nb_create(ctypes.byref(h), int(n_max), PRECISIONS[precision], device,
-                                    _stream_ptr(stream))
+                                    self._stream)
         if st != 0:
             raise NBodyError("nb_create", st, self.lib.nb_last_error(None).decode())
         self.h = h.value
@@ -238,7 +240,29 @@ class NBody:
 
     # ------------------------------------------------------------------ API
     def set_stream(self, stream=None):
-        self._call("nb_set_stream", _stream_ptr(stream))
+        ptr = _stream_ptr(stream)
+        self._call("nb_set_stream", ptr)
+        self._stream = ptr
+
+    @contextlib.contextmanager
+    def in_order(self):
+        """Torch operations inside run on the context's stream: after all that
+        torch's current stream of this device holds, and before what it is given
+        next.  So tensors of that stream may be used inside, and ones written
+        inside after it, wherever the context's stream is another."""
+        torch = _torch or _load_torch()
+        here = torch.cuda.current_stream(self.device)
+        if here.cuda_stream == self._stream:
+            yield
+            return
+        there = torch.cuda.ExternalStream(self._stream, device=self.device) if self._stream \
+            else torch.cuda.default_stream(self.device)
+        there.wait_stream(here)
+        try:
+            with torch.cuda.stream(there):
+                yield
+        finally:
+            here.wait_stream(there)
 
     def sync(self):
         self._call("nb_sync")

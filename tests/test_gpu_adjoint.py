@@ -203,3 +203,33 @@ def test_zero_steps_passes_gradients_through(cuda):
         (xT.sum() + 2 * vT.sum()).backward()
     assert np.all(host(x0.grad) == 1) and np.all(host(v0.grad) == 2)
     assert np.all(host(m.grad) == 0)
+
+
+@pytest.mark.parametrize("K,every", [(4, 2), (3, 1), (5, 3)])
+def test_rollout_and_gradients_of_a_context_on_its_own_stream(cuda, K, every):
+    # the caller stays on torch's current stream; a delay on either stream before
+    # each half leaves the other far ahead unless the two wait for one another
+    import torch
+    b = inputs.plummer(3000, seed=48)
+    tgt = to_dev(b.pos * 1.01, cuda)
+    side, delay = torch.cuda.Stream(), 2_000_000  # cycles: about a millisecond
+
+    def grads(stream, here, there):
+        x, v, m = (to_dev(a, cuda).requires_grad_() for a in (b.pos, b.vel, b.mass))
+        torch.cuda.synchronize()
+        with nbody.NBody(b.n, "fp32_comp", stream=stream) as nb:
+            def lag():
+                for lagging, s in ((here, torch.cuda.current_stream()), (there, side)):
+                    if lagging:
+                        with torch.cuda.stream(s):
+                            torch.cuda._sleep(delay)
+            lag()
+            xT, vT = rollout(nb, x * 1.0, v * 1.0, m * 1.0, 1.0, 0.01, 1e-3, K, every)
+            loss = ((xT - tgt) ** 2).sum() + vT.sum()
+            lag()
+            return [host(t) for t in (xT.detach(), vT.detach(), *torch.autograd.grad(loss, (x, v, m)))]
+
+    want = grads(None, False, False)
+    for here, there in ((True, False), (False, True)):
+        for a, w in zip(grads(side, here, there), want):
+            assert np.array_equal(a, w)
