@@ -72,7 +72,7 @@ class NBodyRollout(torch.autograd.Function):
                 length = min(every, nsteps - start)
                 ends_recorded = length == every  # in ckx[s + 1]
                 if ends_recorded and length == 1:
-                    seg = ckx[s: s + 2]
+                    seg = ckx[s: s + 2].to(m).contiguous()  # (as a hook may have unpacked them)
                 else:
                     # positions 1..new are computed again: new force evaluations, the
                     # last kick and drift needs none after it

@@ -233,3 +233,16 @@ def test_rollout_and_gradients_of_a_context_on_its_own_stream(cuda, K, every):
     for here, there in ((True, False), (False, True)):
         for a, w in zip(grads(side, here, there), want):
             assert np.array_equal(a, w)
+
+
+@pytest.mark.parametrize("K,every", [(3, 1), (4, 2)])
+def test_checkpoints_as_saved_tensor_hooks_return_them(cuda, K, every):
+    # hooks may give the saved checkpoints back in another memory layout
+    b = inputs.plummer(200, seed=49)
+    want = _grads(cuda, "fp32_comp", b, 1.0, 0.01, 1e-3, K, every, b.pos * 1.01)
+    with torch.autograd.graph.saved_tensors_hooks(
+            lambda t: t.cpu().movedim(0, -1).contiguous() if t.dim() == 3 else t,
+            lambda t: t.to(cuda).movedim(-1, 0) if t.dim() == 3 else t):
+        got = _grads(cuda, "fp32_comp", b, 1.0, 0.01, 1e-3, K, every, b.pos * 1.01)
+    for g, w in zip(got, want):
+        assert np.array_equal(g, w)
