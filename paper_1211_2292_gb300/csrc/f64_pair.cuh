@@ -171,17 +171,25 @@ __device__ __forceinline__ bool pair_term(double dx, double dy, double dz, const
 }
 
 // One coordinate's fixed-point sum over a tile of J bodies: acc 2^(E - 1075 +
-// HEAD - 6), E the largest exponent of a term so far.  A term is rounded to
-// 2^-54 of the largest (J = 128), as a float64 addition would round the sum.
-// Each step raises E without asking whether it must: in a branch, some lane of
-// a warp met a new largest term in most steps (181 us at 4097 bodies, 195; 186
-// with the rounding below).
+// HEAD - 6), E the largest exponent of a term of this tile so far.  A term is
+// rounded to 2^-54 of the largest (J = 128), as a float64 addition would round
+// the sum.  E starts again with each tile: kept over the tiles, two close
+// bodies on either side, whose terms cancel, left every later term rounded to
+// 2^-54 of theirs (1e6 of them: 6.0e-15 of such a term together, 6.2e-17 so).  Each
+// step raises E without asking whether it must: in a branch, some lane of a warp
+// met a new largest term in most steps (181 us at 4097 bodies, 195; 186 with the
+// rounding below).
 template <int J>
 struct FixedSum {
     static constexpr int HEAD = J <= 128 ? 6 : 7;  // terms below 2^(62 - HEAD), J of them below 2^63
     static_assert(J <= 256, "");
     int64_t acc;
     int E;
+    __device__ __forceinline__ void reset()
+    {
+        acc = 0;
+        E = 2 * F64_NO_TERM;
+    }
     // to a new largest exponent
     __device__ __forceinline__ void raise(int e)
     {
@@ -205,7 +213,7 @@ struct FixedSum {
     __device__ __forceinline__ double take()
     {
         const double v = ldexp((double)acc, E - 1075 + HEAD - 6);
-        acc = 0;
+        reset();
         return v;
     }
 };

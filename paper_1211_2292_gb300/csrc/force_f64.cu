@@ -109,10 +109,7 @@ __device__ __forceinline__ void force_sweep(const double4 *__restrict__ P, int j
 #pragma unroll
     for (int k = 0; k < I; ++k)
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            sum[k][c].acc = 0;
-            sum[k][c].E = 2 * F64_NO_TERM;
-        }
+        for (int c = 0; c < 3; ++c) sum[k][c].reset();
     if (jlo < jhi) {
         stage_load64<T, J>(buf, P, jlo, jhi);
         store(0);

@@ -91,3 +91,31 @@ def test_many_small_terms_beside_a_large_one(cuda):
     r2 = (d * d).sum(1)
     t = (w / (r2 * np.sqrt(r2)))[:, None] * d
     assert (np.abs(a - t.sum(0)) <= 1e-13 * np.abs(t).max(0)).all()
+
+
+def test_large_terms_that_cancel(cuda):
+    # 40 bodies, each between two others at the same distance on either side,
+    # whose terms (2^28 and more) cancel to the bit; then 1e5 others.  Only the
+    # terms of the pairs' own tile (128 bodies) are rounded to 2^-55 of the
+    # largest: 0.29 x 2^-55 rms each, so 128 of them 2^-53.3, six times that
+    # 2^-50.7.  The others' own errors lie far below: 1e5 terms of some 1 each, to
+    # 2^-53 of themselves and, in 800 tiles, of their sum, 2^-11 of a pair's term.
+    rng = np.random.default_rng(9)
+    k, n = 40, 100001
+    mid = rng.integers(1 << 19, 1 << 20, (k, 3)) * 2.0 ** -20
+    d = rng.integers(1 << 11, 1 << 12, (k, 3)) * 2.0 ** -26 * rng.choice([-1.0, 1.0], (k, 3))
+    pos = rng.uniform(-1.5, -0.5, (n, 3))
+    mass = rng.uniform(0.5, 1.5, n)
+    pos[0:3 * k:3], pos[1:3 * k:3], pos[2:3 * k:3] = mid - d, mid, mid + d
+    mass[0:3 * k:3] = mass[2:3 * k:3] = rng.uniform(1.0, 2.0, k)
+    with nbody.NBody(n, "fp64") as nb:
+        a = host(nb.forces(to_dev(pos, cuda), to_dev(mass, cuda), 1.0, 0.0))
+        nb.sync()
+    p, m = pos.astype(np.longdouble), mass.astype(np.longdouble)
+    for i in range(1, 3 * k, 3):
+        s = np.delete(p, i, 0) - p[i]
+        r2 = (s * s).sum(1)
+        t = (np.delete(m, i) / (r2 * np.sqrt(r2)))[:, None] * s
+        big = np.abs(t[i - 1])
+        rest = np.delete(t, [i - 1, i], 0).sum(0)
+        assert (np.abs(a[i] - rest) <= 2.0 ** -50.7 * big).all()
