@@ -56,8 +56,7 @@ __global__ void pack_kernel(int n, const double *__restrict__ pos, const double 
 // float32 force kernel's j-split slots: G * (slots merged in order).
 __device__ __forceinline__ double merged_force(const MergeParams &g, size_t i)
 {
-    const float2 s = merge_slots(g.slots + i, (size_t)g.n * 3, g.nslots);
-    const double a = g.G * ((double)s.x - (double)s.y);
+    const double a = g.G * merge_slots(g.slots + i, (size_t)g.n * 3, g.nslots);
     if (!isfinite(a)) atomicOr(g.err, (int)ERR_NONFINITE);
     return a;
 }

@@ -242,21 +242,53 @@ __device__ __forceinline__ void kahan_merge(float &s, float &c, float so, float 
     c = (c + co) - e;
 }
 
-// One (sum, carry) pair over n slots `stride` apart, merged in slot order, 16
-// slots' loads in flight.
-__device__ __forceinline__ float2 merge_slots(const float2 *slot, size_t stride, int n)
+// a + b = s + e exactly (s the rounded sum).
+__device__ __forceinline__ float two_sum(float a, float b, float &e)
 {
-    float2 a = __ldcg(slot);
+    const float s = a + b;
+    const float bp = s - a;
+    e = (a - (s - bp)) + (b - bp);
+    return s;
+}
+
+// A sum s - (c + d) of float32 (sum, carry) pairs with what the merged carries
+// lost, so that merging rounds no more than float64 additions would: to about
+// 2^-70 of the sum, where a carry alone keeps 2^-48.  Some 20 float32 operations
+// a merge; a float64 addition takes a warp 16 cycles and a conversion as many.
+struct Sum3 {
+    float s, c, d;
+    __device__ __forceinline__ void merge(float so, float co, float dd = 0.f)
+    {
+        float e, e1, e2;
+        s = two_sum(s, so, e);
+        c = two_sum(two_sum(c, co, e1), -e, e2);
+        d += dd + (e1 + e2);
+    }
+    __device__ __forceinline__ double value() const { return (double)s - ((double)c + (double)d); }
+};
+
+// n (sum, carry) slots `stride` apart, merged in slot order, 16 slots' loads in
+// flight (and four merges in the code: unrolled to 16 their instructions took
+// longer to arrive than to run).
+__device__ __forceinline__ double merge_slots(const float2 *slot, size_t stride, int n)
+{
+    const float2 f = __ldcg(slot);
+    Sum3 a = {f.x, f.y, 0.f};
     for (int q = 1; q < n; q += 16) {
         float2 b[16];
 #pragma unroll
         for (int u = 0; u < 16; ++u)
             b[u] = q + u < n ? __ldcg(slot + (size_t)(q + u) * stride) : make_float2(0.f, 0.f);
+        const int m = min(4, (n - q + 3) >> 2);
+#pragma unroll 1
+        for (int r = 0; r < m; ++r) {
 #pragma unroll
-        for (int u = 0; u < 16; ++u)
-            if (q + u < n) kahan_merge(a.x, a.y, b[u].x, b[u].y);
+            for (int u = 0; u < 4; ++u) a.merge(b[u].x, b[u].y);
+#pragma unroll
+            for (int u = 0; u < 12; ++u) b[u] = b[u + 4];
+        }
     }
-    return a;
+    return a.value();
 }
 
 // Sum of n float64 triples `stride` doubles apart in slot order, 24 loads in

@@ -92,7 +92,7 @@ struct BatchParams {
     const BatchItem *items;
     int n_items;
     unsigned *queue;      // [0] next item, [1] CTAs done; both zero between launches
-    double *partial;      // [slots][threads * bodies_per_thread][3] chunk sums as (sum, carry) float2
+    double *partial;      // [slots][threads * bodies_per_thread][3] chunk partial sums
     unsigned *counters;   // per split piece, zero between launches
     float eps2f;
     double G;

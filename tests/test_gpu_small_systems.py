@@ -109,3 +109,32 @@ def test_packed_pairs_at_every_exponent(cuda):
     # coordinates to 2^-48 of themselves, 2^-40 of the difference; the pair in float32
     for got, w in ((a[::2], want), (a[1::2], -want)):
         assert (np.abs(got - w).max(1) <= 1e-5 * np.abs(w).max(1)).all()
+
+
+@pytest.mark.parametrize("variant,split,parts", [
+    (5, 5, 5), (21, 5, 5), (22, 5, 5), (22, 20, 20)])  # splits by tiles and by bodies
+def test_merging_splits_rounds_no_more_than_float64(cuda, variant, split, parts):
+    # one body with mass in each part of the j range, so that every part's sum
+    # is one float32 pair term, which a call with only that body's mass shows:
+    # their sum must be as good as parts - 1 float64 additions (terms over 28
+    # octaves, whose sum takes more bits than two float32 hold)
+    n = 5120
+    rng = np.random.default_rng(variant)
+    b = inputs.random_system(n, seed=7)
+    at = ((np.arange(parts) + 0.5) * n / parts).astype(int)
+    mass = np.zeros(n)
+    mass[at] = 2.0 ** -rng.uniform(0, 28, parts)
+    x = to_dev(b.pos, cuda)
+    with nbody.NBody(n, "fp32_comp") as nb:
+        nb.tune_set(nbody.KIND_FORCE, 0, 1 << 40, variant, split)
+        got = host(nb.forces(x, to_dev(mass, cuda), 1.0, 0.05)).astype(np.longdouble)
+        want, size = np.zeros_like(got), np.zeros_like(got)
+        for k in at:
+            one = np.zeros(n)
+            one[k] = mass[k]
+            t = host(nb.forces(x, to_dev(one, cuda), 1.0, 0.05)).astype(np.longdouble)
+            assert np.array_equal(t, t.astype(np.float32))
+            want += t
+            size += np.abs(t)
+        nb.sync()
+    assert (np.abs(got - want) <= (parts - 1) * 2.0 ** -53 * size).all()
