@@ -456,12 +456,16 @@ __global__ void __launch_bounds__(T) force_f32_batched_kernel(const BatchParams 
     __shared__ int s_idx, s_last;
     const float2 e2 = make_float2(p.eps2f, p.eps2f);
 
+    // A CTA's first item is its own number, the next ones come from the queue.
+    // (Popped like the others, the first and largest items went to CTAs in the
+    // order in which they happened to arrive, two or more of them to one SM: 64
+    // systems of 500 to 8192 bodies 883 us a call, now 537; 100 of 64 to 3000, 332
+    // and 186, or 250 to 310 from one run to the next.)
+    if (threadIdx.x == 0) {
+        s_idx = (int)blockIdx.x;
+        s_item = p.items[blockIdx.x];
+    }
     for (;;) {
-        if (threadIdx.x == 0) {
-            const int q = (int)atomicAdd(p.queue, 1u);
-            s_idx = q;
-            if (q < p.n_items) s_item = p.items[q];
-        }
         __syncthreads();
         if (s_idx >= p.n_items) break;
         const BatchItem it = s_item;
@@ -484,26 +488,48 @@ __global__ void __launch_bounds__(T) force_f32_batched_kernel(const BatchParams 
                 p.P, p.Plo, c, it.j0, it.j1, 0, ntiles, lane, lanes, e2, nx, ny, nz, acc, tile);
         const bool split = it.nchunks > 1;
         double *slot = split ? p.partial + (size_t)(it.pbase + it.chunk) * TILE_I * 3 : nullptr;
-#pragma unroll
-        for (int k = 0; k < I; ++k) {
-            double x = pair_value(acc.get(0, k)), y = pair_value(acc.get(1, k)),
-                   z = pair_value(acc.get(2, k));
-            // lanes of a group are adjacent in one warp: butterfly sum
-            for (int off = lanes >> 1; off > 0; off >>= 1) {
-                x += __shfl_xor_sync(0xffffffffu, x, off);
-                y += __shfl_xor_sync(0xffffffffu, y, off);
-                z += __shfl_xor_sync(0xffffffffu, z, off);
-            }
+        auto put = [&](int k, const double (&v)[3]) {
             const int i = it.i0 + group + k * groups;
-            if (lane == 0 && i < it.i_end) {
-                if (split) {
-                    double *q = slot + 3 * (size_t)(i - it.i0);
-                    q[0] = x;
-                    q[1] = y;
-                    q[2] = z;
-                } else {
-                    batch_write(p, i, x, y, z);
+            if (i >= it.i_end) return;
+            if (split) {
+                double *q = slot + 3 * (size_t)(i - it.i0);
+                q[0] = v[0];
+                q[1] = v[1];
+                q[2] = v[2];
+            } else {
+                batch_write(p, i, v[0], v[1], v[2]);
+            }
+        };
+        if (lanes == 1) {
+#pragma unroll
+            for (int k = 0; k < I; ++k) {
+                const double v[3] = {pair_value(acc.get(0, k)), pair_value(acc.get(1, k)),
+                                     pair_value(acc.get(2, k))};
+                put(k, v);
+            }
+        } else {
+            // The lanes of a group are adjacent in one warp.  In the first step
+            // of their sum each half of them keeps half of the bodies, so that
+            // only half of the values go on to float64 (300 systems of 30 to 300
+            // bodies took 43 us a call when all did, 29 so).
+            const int half = lanes >> 1;
+            const bool up = lane & half;
+#pragma unroll
+            for (int k = 0; k < I / 2; ++k) {
+                double v[3];
+#pragma unroll
+                for (int d = 0; d < 3; ++d) {
+                    const float2 a = acc.get(d, k), b = acc.get(d, k + I / 2);
+                    Sum3 t = {up ? b.x : a.x, up ? b.y : a.y, 0.f};
+                    t.merge(__shfl_xor_sync(0xffffffffu, up ? a.x : b.x, half),
+                            __shfl_xor_sync(0xffffffffu, up ? a.y : b.y, half));
+                    v[d] = t.value();
                 }
+                for (int off = half >> 1; off > 0; off >>= 1) {
+#pragma unroll
+                    for (int d = 0; d < 3; ++d) v[d] += __shfl_xor_sync(0xffffffffu, v[d], off);
+                }
+                if ((lane & (half - 1)) == 0) put(up ? k + I / 2 : k, v);
             }
         }
         if (split) {
@@ -527,6 +553,11 @@ __global__ void __launch_bounds__(T) force_f32_batched_kernel(const BatchParams 
                 }
                 if (threadIdx.x == 0) p.counters[it.ctr] = 0u;
             }
+        }
+        if (threadIdx.x == 0) {
+            const int q = (int)(gridDim.x + atomicAdd(p.queue, 1u));
+            s_idx = q;
+            if (q < p.n_items) s_item = p.items[q];
         }
     }
     if (threadIdx.x == 0) {

@@ -242,6 +242,17 @@ __device__ __forceinline__ void kahan_merge(float &s, float &c, float so, float 
     c = (c + co) - e;
 }
 
+// (double)x on the integer pipe, where a conversion would take the float64 pipe
+// as long as an operation; subnormal and non-finite values go the plain way.
+static __device__ __noinline__ double widen_plain(float x) { return (double)x; }
+__device__ __forceinline__ double widen(float x)
+{
+    const unsigned b = __float_as_uint(x), e = b & 0x7f800000u, a = b & 0x7fffffffu;
+    if (a != 0u && e - 0x00800000u >= 0x7f000000u) return widen_plain(x);
+    const unsigned hi = (a >> 3) + (a ? 0x38000000u : 0u);
+    return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)(b << 29));
+}
+
 // a + b = s + e exactly (s the rounded sum).
 __device__ __forceinline__ float two_sum(float a, float b, float &e)
 {
@@ -264,7 +275,7 @@ struct Sum3 {
         c = two_sum(two_sum(c, co, e1), -e, e2);
         d += dd + (e1 + e2);
     }
-    __device__ __forceinline__ double value() const { return (double)s - ((double)c + (double)d); }
+    __device__ __forceinline__ double value() const { return widen(s) - (widen(c) + widen(d)); }
 };
 
 // n (sum, carry) slots `stride` apart, merged in slot order, 16 slots' loads in
