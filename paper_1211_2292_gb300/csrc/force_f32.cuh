@@ -247,6 +247,8 @@ __device__ __forceinline__ void put_pair(float2 *q, float2 a)
 
 // The float64 value of a (sum, carry) pair.
 __device__ __forceinline__ double pair_value(float2 a) { return (double)a.x - (double)a.y; }
+// (a call: rare, and its instructions are kept out of the batched kernel's loop)
+static __device__ __noinline__ double add_pairs(float2 a, float2 b) { return pair_value(a) + pair_value(b); }
 
 // Sweep the j-tiles [t0, t1) of bodies [jlo, jhi) (tile t starts at
 // jlo + t*J) for this thread's bodies.  Threads split each tile's j loop in
@@ -511,7 +513,7 @@ __global__ void __launch_bounds__(T) force_f32_batched_kernel(const BatchParams 
             // The lanes of a group are adjacent in one warp.  In the first step
             // of their sum each half of them keeps half of the bodies, so that
             // only half of the values go on to float64 (300 systems of 30 to 300
-            // bodies took 43 us a call when all did, 29 so).
+            // bodies took 43 us a call when all did, 31 so).
             const int half = lanes >> 1;
             const bool up = lane & half;
 #pragma unroll
@@ -520,10 +522,13 @@ __global__ void __launch_bounds__(T) force_f32_batched_kernel(const BatchParams 
 #pragma unroll
                 for (int d = 0; d < 3; ++d) {
                     const float2 a = acc.get(d, k), b = acc.get(d, k + I / 2);
-                    Sum3 t = {up ? b.x : a.x, up ? b.y : a.y, 0.f};
-                    t.merge(__shfl_xor_sync(0xffffffffu, up ? a.x : b.x, half),
-                            __shfl_xor_sync(0xffffffffu, up ? a.y : b.y, half));
+                    const float2 mine = up ? b : a, send = up ? a : b;
+                    const float2 other = make_float2(__shfl_xor_sync(0xffffffffu, send.x, half),
+                                                     __shfl_xor_sync(0xffffffffu, send.y, half));
+                    Sum3 t = {mine.x, mine.y, 0.f};
+                    t.merge(other.x, other.y);
                     v[d] = t.value();
+                    if (!isfinite(v[d])) v[d] = add_pairs(mine, other);  // (merge_slots)
                 }
                 for (int off = half >> 1; off > 0; off >>= 1) {
 #pragma unroll

@@ -209,7 +209,14 @@ __global__ void __launch_bounds__(TEAM_T) force_f32_team_kernel(const ForceParam
         const int d = v / TI, k = i0 + v % TI;
         if (k < n) {
             const int i = p.perm ? p.perm[k] : k;
-            const double a = p.G * pair_value(b[0]);
+            double t = pair_value(b[0]);
+            if (!isfinite(t)) {  // as in merge_slots: the warps' own sums in float64
+                t = 0.0;
+                for (int r = 0; r < cs; ++r)
+                    for (int w = 0; w < TEAM_W; ++w)
+                        t += pair_value(cs > 1 ? *cluster.map_shared_rank(&sums[w][v], r) : sums[w][v]);
+            }
+            const double a = p.G * t;
             p.acc[3 * (size_t)i + d] = a;
             if (p.vel) p.vel[3 * (size_t)i + d] += p.half_dt * a;
             if (!isfinite(a)) atomicOr(p.err, ERR_NONFINITE);

@@ -299,7 +299,15 @@ __device__ __forceinline__ double merge_slots(const float2 *slot, size_t stride,
             for (int u = 0; u < 12; ++u) b[u] = b[u + 4];
         }
     }
-    return a.value();
+    double v = a.value();
+    if (!isfinite(v)) {  // past float32's range on the way, or a slot is not finite
+        v = (double)f.x - (double)f.y;
+        for (int q = 1; q < n; ++q) {
+            const float2 b = __ldcg(slot + (size_t)q * stride);
+            v += (double)b.x - (double)b.y;
+        }
+    }
+    return v;
 }
 
 // Sum of n float64 triples `stride` doubles apart in slot order, 24 loads in

@@ -138,3 +138,29 @@ def test_merging_splits_rounds_no_more_than_float64(cuda, variant, split, parts)
             size += np.abs(t)
         nb.sync()
     assert (np.abs(got - want) <= (parts - 1) * 2.0 ** -53 * size).all()
+
+
+@pytest.mark.parametrize("prec", ["fp32_comp", "fp32"])
+@pytest.mark.parametrize("variant,split,n", [(23, 1, 500), (24, 8, 5003), (5, 16, 5003), (21, 9, 5003),
+                                             (22, 20, 9001), ("batch", 0, 61)])
+def test_sums_past_float32_of_parts_within_it(cuda, prec, variant, split, n):
+    # two clouds pull at one another with sums of up to 6e38, above float32's range
+    # (3.4e38), of which each of four parts or more (splits, warps or lanes, the
+    # bodies in random order) adds a fourth or so; G brings them back to 6e8
+    rng = np.random.default_rng(n)
+    pos = rng.uniform(-0.5, 0.5, (n, 3))
+    pos[: n // 2, 0] += 3.0
+    pos = pos[rng.permutation(n)]
+    mass = rng.uniform(0.5, 1.5, n)
+    mass *= 6e38 / np.abs(oracle.accel(pos, mass, 1.0, 1.0)).max()
+    x, m = to_dev(pos, cuda), to_dev(mass, cuda)
+    with nbody.NBody(n, prec) as nb:
+        if variant == "batch":
+            nb.batch_plan([0, n])
+            a = host(nb.forces_batched(x, m, 1e-30, 1.0))
+        else:
+            nb.tune_set(nbody.KIND_FORCE, 0, 1 << 40, variant, split)
+            a = host(nb.forces(x, m, 1e-30, 1.0))
+        nb.sync()  # raises if anything is not finite
+    err = relerr_per_body(a, oracle.accel(pos, mass, 1e-30, 1.0))
+    assert np.sqrt(np.mean(err ** 2)) <= BOUND[0] and err.max() <= BOUND[1]
