@@ -309,15 +309,23 @@ int splits_for(nb_ctx *c, const KernelEntry &k, int64_t n, int forced, int64_t p
 // split launch its merge (its gap, 24 bytes per body-split).  Fitted to every
 // split from 3 to 63 of these kernels at 11000, 16411 and 24000 bodies (within
 // 10 %).
+//
+// A plain sum (NB_FP32) runs over a split's n / s bodies in one float32, and its
+// error grows with that: at least as many splits as whole tiles would take for
+// four CTAs per SM.  (By time alone 262144 bodies took 4 for 16 and the rms error
+// went from 1.4e-6 to 4.4e-6.)
 int even_splits(const nb_ctx *c, const KernelEntry &k, int64_t n)
 {
     const int64_t tiles = (n + k.tile() - 1) / k.tile();
     const int64_t cap = c->partial_bodies * 4 / 3;  // body-splits that fit
     const double rate = k.even * 1e-3 * (k.I / 2);
-    int best = 1;
+    const int64_t smin = c->prec == NB_FP32 ? nb::choose_split(tiles, (n + k.J - 1) / k.J,
+                                                               4 * c->num_sms, cap, k.tile())
+                                            : 1;
+    int best = (int)smin;
     double cycles = -1;
-    const int64_t smax = std::min<int64_t>(std::max<int64_t>(n / 64, 1), 256);
-    for (int64_t s = 1; s <= smax && (s == 1 || s * n <= cap); ++s) {
+    const int64_t smax = std::max(smin, std::min<int64_t>(std::max<int64_t>(n / 64, 1), 256));
+    for (int64_t s = smin; s <= smax && (s == smin || s * n <= cap); ++s) {
         const int64_t ctas = (tiles * s + c->num_sms - 1) / c->num_sms;
         const int64_t warps = (ctas * k.T + 127) / 128;
         const double w = ((double)((n + s - 1) / s) + 67) * rate *

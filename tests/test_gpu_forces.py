@@ -12,7 +12,7 @@ import numpy as np
 import pytest
 
 import oracle
-from paper_1211_2292_gb300 import inputs, nbody
+from paper_1211_2292_gb300 import inputs, nbody, tune
 from helpers import host, relerr_per_body, to_dev
 
 pytestmark = pytest.mark.gpu
@@ -256,3 +256,25 @@ def test_morton_order_in_step_loop(cuda):
 def torch_empty_like(x):
     import torch
     return torch.empty_like(x)
+
+
+def test_plain_sums_of_many_bodies_are_split(cuda):
+    # the plain mode runs over n / s bodies in one float32, so its error falls as
+    # the splits s grow: what the call chooses is no worse than 12 splits (16 are
+    # what whole tiles take on four blocks per SM of 152; the two errors are the
+    # same bodies', a tenth apart at most by chance)
+    b = inputs.two_plummer(1 << 17, seed=6)
+    rows = np.random.default_rng(6).permutation(b.n)[:4000]
+    ref = oracle.accel_rows(b.pos, b.mass, rows, 1.0, 0.01)
+    x, m = to_dev(b.pos, cuda), to_dev(b.mass, cuda)
+    rms = []
+    with nbody.NBody(b.n, "fp32") as nb:
+        tune.apply(nb)
+        v, s = nb.tune_get(nbody.KIND_FORCE, b.n)
+        assert s == 0
+        for split in (0, 12):
+            nb.tune_set(nbody.KIND_FORCE, 0, 1 << 40, v, split)
+            a = host(nb.forces(x, m, 1.0, 0.01))[rows]
+            rms.append(np.sqrt(np.mean(relerr_per_body(a, ref) ** 2)))
+        nb.sync()
+    assert rms[0] <= 1.1 * rms[1]
