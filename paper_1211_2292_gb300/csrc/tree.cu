@@ -486,8 +486,9 @@ __global__ void __launch_bounds__(MTPB) tree_moments_kernel(TreeView t,
                         }
                     }
                 }
-                const double inv = M > 0.0 ? 1.0 / M : 0.0;
-                put_walk_moments(t, me, M, sx * inv, sy * inv, sz * inv);
+                // (three divisions: 1 / M of nearly massless bodies overflows)
+                put_walk_moments(t, me, M, M > 0.0 ? sx / M : 0.0, M > 0.0 ? sy / M : 0.0,
+                                 M > 0.0 ? sz / M : 0.0);
                 node = t.parent[me];
                 if (!climbed(node)) node = -1;
                 count = e - s;

@@ -248,3 +248,18 @@ def test_moments_do_not_depend_on_who_arrives_last(cuda, n):
         for _ in range(40):
             assert np.array_equal(host(nb.tree_forces(x, m, 1.0, 0.01, 1.0, 4)), want)
         nb.sync()
+
+
+@pytest.mark.parametrize("n", [3000, 60000])  # cells summed from their bodies; climbed
+def test_leaves_of_nearly_massless_bodies(cuda, n):
+    # test particles far out, in leaves of their own, whose masses add up to less
+    # than 1 / DBL_MAX
+    b = inputs.plummer(n, seed=4)
+    rng = np.random.default_rng(4)
+    pos = np.concatenate([b.pos, rng.uniform(30.0, 31.0, (500, 3))])
+    mass = np.concatenate([b.mass, np.full(500, 1e-310)])
+    b = inputs.Bodies(pos, np.zeros_like(pos), mass)
+    ref, _, _ = oracle.bh_forces(pos, mass, 1.0, 0.01, 0.5, 16, 64, counts=True)
+    a, _, _ = _gpu_tree(cuda, b, 1.0, 0.01, 0.5, 16)
+    e = relerr_per_body(a, ref)
+    assert np.sqrt(np.mean(e ** 2)) <= RMS_TOL and e.max() <= MAX_TOL
