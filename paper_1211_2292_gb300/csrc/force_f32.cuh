@@ -144,7 +144,11 @@ __device__ __forceinline__ void stage_store(float4 *tile, const float4 (&bh)[J /
     }
 }
 
-// Out-of-range j slots become massless bodies (m = 0, log2 m = -inf).
+// Out-of-range j slots become massless bodies (m = 0, log2 m = -inf) far from any
+// other (r^2 stays in float32's range): next to a body, as at the origin one may
+// be, m / r^3 would be 0 times infinity at eps = 0.
+__device__ __forceinline__ float4 far_body(float w) { return make_float4(1e18f, 1e18f, 1e18f, w); }
+
 template <int T, int J>
 __device__ __forceinline__ void stage_load(float4 (&bh)[J / T], float4 (&bl)[J / T],
                                            const float4 *__restrict__ P,
@@ -154,7 +158,7 @@ __device__ __forceinline__ void stage_load(float4 (&bh)[J / T], float4 (&bl)[J /
     for (int l = 0; l < J / T; ++l) {
         const int j = jbase + l * T + threadIdx.x;
         const bool ok = j < jend;
-        bh[l] = ok ? __ldg(P + j) : make_float4(0.f, 0.f, 0.f, 0.f);
+        bh[l] = ok ? __ldg(P + j) : far_body(0.f);
         bl[l] = ok ? __ldg(Plo + j) : make_float4(0.f, 0.f, 0.f, -INFINITY);
     }
 }

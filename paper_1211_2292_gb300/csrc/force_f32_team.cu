@@ -30,7 +30,8 @@ template <bool RAW>
 __device__ __forceinline__ void team_load(const ForceParams &p, int j, bool ok, float4 &h, float4 &l)
 {
     if (!ok) {
-        h = l = make_float4(0.f, 0.f, 0.f, 0.f);
+        h = far_body(0.f);
+        l = make_float4(0.f, 0.f, 0.f, 0.f);
     } else if (RAW) {
         const double *x = p.pos + 3 * (size_t)j;
         const double a = __ldg(x), b = __ldg(x + 1), c = __ldg(x + 2);

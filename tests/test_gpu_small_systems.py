@@ -164,3 +164,23 @@ def test_sums_past_float32_of_parts_within_it(cuda, prec, variant, split, n):
         nb.sync()  # raises if anything is not finite
     err = relerr_per_body(a, oracle.accel(pos, mass, 1e-30, 1.0))
     assert np.sqrt(np.mean(err ** 2)) <= BOUND[0] and err.max() <= BOUND[1]
+
+
+@pytest.mark.parametrize("prec", ["fp32_comp", "fp32"])
+@pytest.mark.parametrize("variant,split,n", [(23, 8, 1280), (24, 8, 5120), (21, 9, 7680), (22, 7, 7680), (5, 5, 7600)])
+def test_a_body_next_to_the_origin_without_softening(cuda, prec, variant, split, n):
+    # the slots past the end of a part of the j range hold massless bodies, which
+    # must not lie so close to a body that 1 / r^3 overflows: one body 3e-20 from the
+    # origin, its tile's coordinates relative to the origin itself (bodies in
+    # opposite pairs)
+    rng = np.random.default_rng(8)
+    half = rng.uniform(-1.0, 1.0, (n // 2, 3))
+    pos = np.stack([half, -half], 1).reshape(-1, 3)
+    pos[0], pos[1] = (3e-20, 0.0, 0.0), (0.3, -0.2, 0.4)
+    mass = rng.uniform(0.5, 1.5, n) / n
+    with nbody.NBody(n, prec) as nb:
+        nb.tune_set(nbody.KIND_FORCE, 0, 1 << 40, variant, split)
+        a = host(nb.forces(to_dev(pos, cuda), to_dev(mass, cuda), 1.0, 0.0))
+        nb.sync()
+    err = relerr_per_body(a, oracle.accel(pos, mass, 1.0, 0.0))
+    assert np.sqrt(np.mean(err ** 2)) <= BOUND[0] * 10
