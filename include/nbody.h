@@ -246,7 +246,10 @@ int64_t nb_launch_count(const nb_ctx *ctx);
  * (0 force, 1 batched force, 2 force VJP, 3 energy, 4 tree walk, 5 tree
  * build: sort, pack, levels, moments, 6 fast multipole upward and downward
  * passes, 7 fast multipole near field), the launches (sequences, for 5 to 7)
- * recorded and their summed duration in milliseconds.
+ * recorded and their summed duration in milliseconds.  A float32 force's time
+ * includes the merging of its j-splits where that is a launch of its own (the
+ * next step's kick merges all but the last step's), never the packing of the
+ * bodies, which the small kernels that read pos and mass themselves do inside.
  */
 nb_status nb_profile(nb_ctx *ctx, int enable);
 nb_status nb_profile_read(nb_ctx *ctx, int kind, int64_t *launches, double *total_ms);

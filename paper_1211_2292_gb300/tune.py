@@ -2,11 +2,20 @@
 j-split count, per precision and size bucket.
 
 Each candidate (variant, split) is timed through the library itself: the
-variant is forced with ``nb_tune_set`` and its launches are timed with the
-library's CUDA events (``nb_profile``) on synthetic Plummer inputs.  The best
-candidate per size becomes an entry {kind, precision, lo, hi, variant,
-split}; buckets meet at the geometric midpoints between tuned sizes.  The
-table is saved as JSON and applied to a context with :func:`apply`.
+variant is forced with ``nb_tune_set`` and whole calls on synthetic Plummer
+inputs are timed with CUDA events.  (The pair kernel's own events,
+``nb_profile``, would favour kernels that leave the packing or the merging of
+splits to other launches.)  The best candidate per size becomes an entry {kind,
+precision, lo, hi, variant, split}; buckets meet at the geometric midpoints
+between tuned sizes.  The table is saved as JSON and applied to a context with
+:func:`apply`.
+
+The packaged table's float32 force entries are set by hand: their edges (2900,
+8192, 11000, 32768, 131072) are where measured kernels cross, and between 8192
+and 131072 bodies each keeps the pair arithmetic (which body pairs take the log
+form) that its size has always had, so that a trajectory does not change with a
+release by more than the order of sums.  A table written here goes by time
+alone, and trajectories under it differ by some 5e-9 in the velocities.
 
   python -m paper_1211_2292_gb300.tune --out tuning.json [--sizes 4096,65536,...]
 """
@@ -28,18 +37,27 @@ BATCH_DIVISORS = (1, 2, 4, 8)
 DEFAULT_TABLE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "tuning_gb300.json")
 
 
-def _time_call(nb, fn, kind, reps):
-    fn()  # warm-up (and first-use setup)
-    nb.profile(True)
-    for _ in range(reps):
-        fn()
-    cnt, ms = nb.profile_read(kind)
-    nb.profile(False)
-    return ms / max(cnt, 1)
+def _time_call(nb, fn, reps):
+    """Milliseconds per call of fn, the mean of `reps` calls or of as many as take
+    about 2 ms (a small call's launches then wait for the GPU, not for the host)."""
+    import torch
+    ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+
+    def mean(calls):
+        ev[0].record()
+        for _ in range(calls):
+            fn()
+        ev[1].record()
+        ev[1].synchronize()
+        return ev[0].elapsed_time(ev[1]) / calls
+
+    with torch.cuda.device(nb.device):
+        fn()  # warm-up (and first-use setup)
+        return mean(max(reps, min(200, int(2.0 / max(mean(1), 1e-3)))))
 
 
 def time_candidates(kind, precision, n, splits=(0,), reps=3, seed=0, device=0, log=None):
-    """[(ms per launch, variant, split)] for every compiled variant at size n."""
+    """[(ms per call, variant, split)] for every compiled variant at size n."""
     import torch
     dev = torch.device("cuda", device)
     b = inputs.plummer(n, seed=seed)
@@ -59,7 +77,7 @@ def time_candidates(kind, precision, n, splits=(0,), reps=3, seed=0, device=0, l
         for v in range(len(nbody.variants(kind, precision))):
             for s in splits:
                 nb.tune_set(kind, 0, 1 << 40, v, s)
-                ms = _time_call(nb, fn, kind, reps)
+                ms = _time_call(nb, fn, reps)
                 out.append((ms, v, s))
                 if log:
                     log(f"kind={kind} {precision} n={n} variant={v}"
@@ -69,7 +87,7 @@ def time_candidates(kind, precision, n, splits=(0,), reps=3, seed=0, device=0, l
 
 
 def time_batched(precision, offsets, bodies, reps=3, device=0, log=None, divisors=(0,)):
-    """[(ms per launch, variant, divisor)] of the batched kernel on one set of
+    """[(ms per call, variant, divisor)] of the batched kernel on one set of
     systems; the divisor (a tuning entry's split field, 0 = the default 4)
     caps a work item at 1/divisor of an even per-CTA share of the pairs."""
     import torch
@@ -84,7 +102,7 @@ def time_batched(precision, offsets, bodies, reps=3, device=0, log=None, divisor
                 nb.tune_set(nbody.KIND_BATCHED, 0, 1 << 40, v, d)
                 nb.batch_plan(offsets)
                 ms = _time_call(nb, lambda: nb.forces_batched(x, m, 1.0, 0.01, out=acc),
-                                nbody.KIND_BATCHED, reps)
+                                reps)
                 out.append((ms, v, d))
                 if log:
                     log(f"batched {precision} variant={v}"

@@ -58,3 +58,18 @@ def test_packaged_table_covers_every_precision(cuda):
         assert nbody.KIND_FORCE in kinds and nbody.KIND_VJP in kinds, prec
         with nbody.NBody(1024, prec) as nb:
             assert tune.apply(nb, table) > 0
+
+
+def test_candidates_are_timed_by_whole_calls(cuda):
+    # a double-float call of 16384 bodies sorts and packs them first, some 4 % of it
+    ms = dict((v, t) for t, v, _ in tune.time_candidates(nbody.KIND_FORCE, "df64", 16384, reps=3))
+    b = inputs.plummer(16384, seed=0)
+    x, m = to_dev(b.pos, cuda), to_dev(b.mass, cuda)
+    with nbody.NBody(b.n, "df64") as nb:
+        nb.tune_set(nbody.KIND_FORCE, 0, 1 << 40, 2, 0)
+        nb.forces(x, m, 1.0, 0.01)
+        nb.profile(True)
+        for _ in range(10):
+            nb.forces(x, m, 1.0, 0.01)
+        cnt, kernel_ms = nb.profile_read(nbody.KIND_FORCE)
+    assert ms[2] >= 1.01 * kernel_ms / cnt
