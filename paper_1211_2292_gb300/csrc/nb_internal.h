@@ -251,7 +251,8 @@ int64_t tree_node_bound(int64_t n, int leaf_cap);
 // box = {lo_x, lo_y, lo_z, ext} from launch_tree_sort.
 cudaError_t launch_tree_build(cudaStream_t s, const TreeView &t, int n, const OrderScratch &o,
                               const double *box, const double *pos, const double *mass,
-                              const int *perm, int leaf_cap, bool moments, int *err, int &kernels);
+                              const int *perm, int leaf_cap, bool moments, int num_sms, int *err,
+                              int &kernels);
 cudaError_t launch_tree_walk(cudaStream_t s, const TreeWalkParams &p, bool zeps, int &kernels);
 // Where tree.cu keeps each level's node count and first node, and the walk's
 // group queue, in TreeView::meta.

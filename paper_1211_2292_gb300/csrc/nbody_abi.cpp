@@ -971,7 +971,7 @@ nb_status tree_build_enqueue(nb_ctx *c, cudaStream_t s, int64_t n, const double 
     NB_CUDA(c, nb::launch_tree_sort(s, (int)n, pos, c->order, c->tree_perm, c->tree_box, pk, k));
     c->launches += k;
     NB_CUDA(c, nb::launch_tree_build(s, c->tree, (int)n, c->order, c->tree_box, pos, mass,
-                                     c->tree_perm, leaf_cap, moments, c->err, k));
+                                     c->tree_perm, leaf_cap, moments, c->num_sms, c->err, k));
     c->launches += k;
     tm.done();
     return NB_OK;

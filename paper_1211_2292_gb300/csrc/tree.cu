@@ -30,6 +30,8 @@
 #include <cuda_runtime.h>
 #include <float.h>
 
+#include <algorithm>
+
 #include "nb_device.cuh"
 #include "nb_internal.h"
 
@@ -1368,7 +1370,8 @@ int64_t tree_node_bound(int64_t n, int leaf_cap)
 
 cudaError_t launch_tree_build(cudaStream_t s, const TreeView &t, int n, const OrderScratch &o,
                               const double *box, const double *pos, const double *mass,
-                              const int *perm, int leaf_cap, bool moments, int *err, int &kernels)
+                              const int *perm, int leaf_cap, bool moments, int num_sms, int *err,
+                              int &kernels)
 {
     // one block per 256 bodies until the blocks' table of counts, which every
     // block sums, is as large as is cheap (26 KB)
@@ -1382,11 +1385,10 @@ cudaError_t launch_tree_build(cudaStream_t s, const TreeView &t, int n, const Or
     tree_emit_kernel<<<nblk, TTPB, 0, s>>>(t, n, keys, chunk, lv, tab, err);
     kernels = 2;
     if (!moments) return cudaGetLastError();
-    // a thread per node, at most the blocks that are resident on 152 SMs
-    const int64_t blocks = ((int64_t)t.cap + MTPB - 1) / MTPB;
+    // a thread per node, at most 20 blocks of two warps per SM
+    const int64_t blocks = std::min<int64_t>(((int64_t)t.cap + MTPB - 1) / MTPB, 20 * num_sms);
     const int direct_max = n <= DIRECT_MAX_N ? DIRECT_BODIES : 0;
-    tree_moments_kernel<<<(int)(blocks < 3040 ? blocks : 3040), MTPB, 0, s>>>(t, box, pos, mass,
-                                                                              perm, direct_max);
+    tree_moments_kernel<<<(int)blocks, MTPB, 0, s>>>(t, box, pos, mass, perm, direct_max);
     kernels = 3;
     return cudaGetLastError();
 }
