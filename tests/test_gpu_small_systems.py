@@ -184,3 +184,24 @@ def test_a_body_next_to_the_origin_without_softening(cuda, prec, variant, split,
         nb.sync()
     err = relerr_per_body(a, oracle.accel(pos, mass, 1.0, 0.0))
     assert np.sqrt(np.mean(err ** 2)) <= BOUND[0] * 10
+
+
+@pytest.mark.parametrize("prec,variant", [("fp32_comp", 22), ("fp32", 21)])
+def test_records_between_the_two_half_kicks(cuda, prec, variant):
+    # with split forces a launch ends one step and opens the next: what it records
+    # in between is the state that single-step calls return
+    n, dt = 9001, 1e-3
+    b = inputs.plummer(n, seed=12)
+    m = to_dev(b.mass, cuda)
+    with nbody.NBody(n, prec) as nb:
+        nb.tune_set(nbody.KIND_FORCE, 0, 1 << 40, variant, 0)
+        x, v, acc = to_dev(b.pos, cuda), to_dev(b.vel, cuda), torch.empty_like(to_dev(b.pos, cuda))
+        rx, rv = (torch.empty((4, n, 3), dtype=torch.float64, device=cuda) for _ in range(2))
+        nb.rollout(x, v, m, 1.0, 0.01, dt, 3, acc, 1, rx, rv)
+        p, q, a = to_dev(b.pos, cuda), to_dev(b.vel, cuda), torch.empty_like(acc)
+        for k in range(4):
+            assert np.array_equal(host(rx[k]), host(p)) and np.array_equal(host(rv[k]), host(q))
+            if k < 3:
+                nb.step(p, q, m, 1.0, 0.01, dt, 1, a, acc_valid=k > 0)
+        assert np.array_equal(host(x), host(p)) and np.array_equal(host(acc), host(a))
+        nb.sync()
