@@ -316,7 +316,8 @@ nb_status nb_tree_stats(nb_ctx *ctx, int64_t *out);
  * sched 0 static (one warp per group, a grid covering every group), 1
  * dynamic (the default: resident warps take `chunk` consecutive groups at a
  * time from an atomic counter), 2 guided (chunks of max(chunk, remaining /
- * (2 x warps))).  1 <= chunk <= 2^20 (default 1).  Results do not depend on
+ * (2 x warps))).  Where a block's 4 or 8 warps walk one group together (few
+ * groups), the blocks are dealt the groups in the warps' place.  1 <= chunk <= 2^20 (default 1).  Results do not depend on
  * the schedule, only the time does.  Drops the context's captured graphs.
  */
 nb_status nb_tree_schedule(nb_ctx *ctx, int sched, int chunk);

@@ -13,7 +13,7 @@ restore the checkpoint, recompute the positions up to the next checkpoint with
 (nsteps/every + 1) checkpoints of (x, v) plus one segment of positions;
 compute: every - 1 force evaluations per segment of `every` steps.  (With the
 segment's end position and the force there computed again too, every + 1:
-2.63 ms for 4 steps of 16384 bodies with every = 2, 2.22 now.)
+2.63 ms for 4 steps of 16384 bodies with every = 2, 2.30 now.)
 
 Library calls and torch operations meet on the context's stream, whichever
 stream the caller is on (``NBody.in_order``): the tensors are allocated on the

@@ -3,9 +3,9 @@
 // sm_103a has two float64 lanes per SM and clock (a warp operation takes 16
 // cycles) against 64 integer ones.  So only a pair's three differences are left
 // to the float64 pipe; the squares, the -3/2 power, the product with m and the
-// sums are fixed-point, some 225 instructions and 83 cycles a warp, where 19
+// sums are fixed-point, some 230 instructions and 92 cycles a warp, where 19
 // float64 operations and two conversions took 340.  Bound by the integer pipe
-// (66 % busy, issue 64 %, float64 59 %).  16384 bodies: 9.56 ms before, 2.47
+// (ALU 66 % busy at 65536 bodies, issue 65 %, float64 57 %; 63, 63, 55 at 16384).  16384 bodies: 9.56 ms before, 2.47
 // now; with only the power in integers and a float64 product and sums 3.38.
 // A single term's error against 113 bits is 0.45 x 2^-53 rms and 1.6 x 2^-53 at
 // most (1.8 and 8.4 before).

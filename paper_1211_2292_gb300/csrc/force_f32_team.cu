@@ -201,7 +201,10 @@ __global__ void __launch_bounds__(TEAM_T) force_f32_team_kernel(const ForceParam
     }
     __syncthreads();
     // the warps' sums in warp order, then the blocks' in rank order (float32
-    // two-sums: eight float64 sums per value held the float64 pipe 3000 cycles)
+    // two-sums, to 2^-48 of the sum: eight float64 sums per value held the float64
+    // pipe 3000 cycles, and Sum3 made a step of 4096 bodies 0.9 us longer; the
+    // errors against float64, 1e-7 from the pair terms, are 1 to 13 % below those
+    // of the block kernels with float64 merges at 64 to 8191 bodies)
     for (int v = threadIdx.x; v < NV; v += TEAM_T) {
         float2 a = sums[0][v];
 #pragma unroll

@@ -22,7 +22,7 @@
 namespace nb {
 namespace {
 
-constexpr int UNROLL_F64 = 2;  // pairs in flight: 2.27 ms at 16384 bodies (1: 2.34, 4: 2.45)
+constexpr int UNROLL_F64 = 2;  // pairs in flight: 2.47 ms at 16384 bodies (1: 2.54, 4: 2.61)
 
 template <int T, int J>
 __device__ __forceinline__ void stage_load64(double4 (&buf)[J / T], const double4 *__restrict__ P,

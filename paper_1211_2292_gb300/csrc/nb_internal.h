@@ -46,7 +46,8 @@ struct KernelEntry {
 struct ForceParams {
     const void *P;        // packed bodies: float4 (x_hi,y_hi,z_hi,m) or double4 (x,y,z,m)
     const double *pos, *mass;  // the caller's arrays (kernels that read those instead)
-    const float4 *Plo;    // float32 modes: (x_lo,y_lo,z_lo,0), x = x_hi + x_lo
+    const float4 *Plo;    // float32 modes: (x_lo,y_lo,z_lo,w), x = x_hi + x_lo, w = log2 m
+                          // when the kernel is `logm`, else 0
     const int *perm;      // float32 modes: body stored at packed slot k (NULL = identity)
     int n;                // bodies
     int nsplit;           // j-splits across CTAs (grid = i-tiles * nsplit)

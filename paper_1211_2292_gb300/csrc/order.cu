@@ -14,7 +14,8 @@
 //      each pass also counts the next pass's digits per destination tile;
 //   4. packing in sorted order as float32 hi/lo pairs:
 //      P_hi = (fl(x), fl(y), fl(z), fl(m)),
-//      P_lo = (fl(x - fl(x)), ..., fl(log2 m)) (log2 m for the log-domain pairs),
+//      P_lo = (fl(x - fl(x)), ..., fl(log2 m) for kernels with log-domain pairs,
+//      else 0),
 //      or as float64 (x, y, z, m), by the sort's last pass.
 // Every step is deterministic, so the order and the forces are reproducible.
 #include <cuda_runtime.h>
