@@ -506,18 +506,24 @@ __global__ void __launch_bounds__(T) force_f32_batched_kernel(const BatchParams 
                 batch_write(p, i, v[0], v[1], v[2]);
             }
         };
-        if (lanes == 1) {
+        // The lanes of a group are adjacent in one warp.
+        if (lanes == 1 || !COMP) {
 #pragma unroll
             for (int k = 0; k < I; ++k) {
-                const double v[3] = {pair_value(acc.get(0, k)), pair_value(acc.get(1, k)),
-                                     pair_value(acc.get(2, k))};
-                put(k, v);
+                double v[3] = {pair_value(acc.get(0, k)), pair_value(acc.get(1, k)),
+                               pair_value(acc.get(2, k))};
+                for (int off = lanes >> 1; !COMP && off > 0; off >>= 1) {
+#pragma unroll
+                    for (int d = 0; d < 3; ++d) v[d] += __shfl_xor_sync(0xffffffffu, v[d], off);
+                }
+                if (lane == 0) put(k, v);
             }
         } else {
-            // The lanes of a group are adjacent in one warp.  In the first step
-            // of their sum each half of them keeps half of the bodies, so that
-            // only half of the values go on to float64 (300 systems of 30 to 300
-            // bodies took 43 us a call when all did, 31 so).
+            // With carries to convert too, each half of the lanes keeps half of the
+            // bodies in the first step of their sum, so that only half of the values
+            // go on to float64 (300 systems of 30 to 300 bodies took 43 us a call when
+            // all did, 31 so; without carries that was no gain, and 512 systems took
+            // 1148 us for 1122).
             const int half = lanes >> 1;
             const bool up = lane & half;
 #pragma unroll
