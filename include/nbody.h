@@ -73,6 +73,7 @@ typedef enum {
 /* Flags for nb_step / nb_rollout / nb_step_batched. */
 #define NB_ACC_VALID 1u   /* acc already holds F(pos): skip the initial force evaluation */
 #define NB_USE_GRAPH 2u   /* run the step loop as one captured CUDA graph */
+#define NB_END_AT_DRIFT 4u /* nb_step, nb_rollout: the last step ends after x += dt v */
 
 /* Flags for nb_step_backward. */
 #define NB_BWD_AT_END   1u  /* traj[nsteps] is the last state of the run */
@@ -129,6 +130,10 @@ nb_status nb_step(nb_ctx *ctx, int64_t n, double *pos, double *vel, const double
  * and, if rec_vel is not NULL, rec_vel[r][n][3].  The caller sizes them for
  * nsteps / record_every + 1 records.  record_every <= 0 records nothing.
  * Used for adjoint checkpoints and for recomputing a segment's trajectory.
+ * NB_END_AT_DRIFT leaves out the last step's force and closing half-kick: pos
+ * is the final position, vel lacks that half-kick, acc holds the force before
+ * it (nsteps force evaluations, one less with NB_ACC_VALID; nsteps = 0 as
+ * without the flag).  A trajectory's positions need no more.
  */
 nb_status nb_rollout(nb_ctx *ctx, int64_t n, double *pos, double *vel, const double *mass,
                      double G, double eps, double dt, int64_t nsteps, double *acc,

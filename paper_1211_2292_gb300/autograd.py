@@ -8,12 +8,15 @@ autograd can differentiate with respect to x0, v0 and m.
 Forward: one ``nb_rollout`` call that records the state every ``every``
 steps (segment checkpoints).  Backward, segment by segment from the last:
 restore the checkpoint, recompute the positions up to the next checkpoint with
-``nb_rollout(record_every=1)`` and one more kick and drift, then run
-``nb_step_backward`` (the reverse sweep with the force VJP kernel).  Memory:
+``nb_rollout(record_every=1)``, which ends after the last of them is reached
+(``NB_END_AT_DRIFT``), then run ``nb_step_backward`` (the reverse sweep with the
+force VJP kernel).  Memory:
 (nsteps/every + 1) checkpoints of (x, v) plus one segment of positions;
 compute: every - 1 force evaluations per segment of `every` steps.  (With the
 segment's end position and the force there computed again too, every + 1:
-2.63 ms for 4 steps of 16384 bodies with every = 2, 2.30 now.)
+2.63 ms for 4 steps of 16384 bodies with every = 2, 2.30 now.  Three torch operations
+per segment in the place of ``NB_END_AT_DRIFT`` made a small system's backward, which
+is the host's, 12 % longer: 735 us for 4 steps of 300 bodies, 670 now.)
 
 Library calls and torch operations meet on the context's stream, whichever
 stream the caller is on (``NBody.in_order``): the tensors are allocated on the
@@ -62,29 +65,31 @@ class NBodyRollout(torch.autograd.Function):
         if nsteps == 0:
             return lam_x, lam_v, lam_m, None, None, None, None, None, None
         nseg = (nsteps + every - 1) // every
-        traj = torch.empty((every + 1, n, 3), dtype=m.dtype, device=m.device)
-        x = torch.empty((n, 3), dtype=m.dtype, device=m.device)
-        v = torch.empty_like(x)
-        acc = torch.empty_like(x)
+        if every == 1:
+            traj = ckx.to(m).contiguous()  # (as a hook may have unpacked it)
+        else:
+            traj = torch.empty((every + 1, n, 3), dtype=m.dtype, device=m.device)
+            x = torch.empty((n, 3), dtype=m.dtype, device=m.device)
+            v, acc = torch.empty_like(x), torch.empty_like(x)
+            xs, vs, upto, end = ckx.unbind(0), ckv.unbind(0), traj[:every], traj[every]
         with nb.in_order():  # the loop's own torch operations too
             for s in range(nseg - 1, -1, -1):
                 start = s * every
                 length = min(every, nsteps - start)
-                ends_recorded = length == every  # in ckx[s + 1]
-                if ends_recorded and length == 1:
-                    seg = ckx[s: s + 2].to(m).contiguous()  # (as a hook may have unpacked them)
+                if every == 1:
+                    seg = traj[s: s + 2]
                 else:
-                    # positions 1..new are computed again: new force evaluations, the
-                    # last kick and drift needs none after it
-                    seg = traj[: length + 1]
-                    new = length - 1 if ends_recorded else length
-                    x.copy_(ckx[s])
-                    v.copy_(ckv[s])
-                    nb.rollout(x, v, m, G, eps, dt, new - 1, acc, 1, seg[:new])
-                    v.add_(acc, alpha=0.5 * dt)
-                    torch.add(x, v, alpha=dt, out=seg[new])
-                    if ends_recorded:
-                        seg[length].copy_(ckx[s + 1])
+                    # the positions after the first are computed again, but for the
+                    # last of a whole segment: that one is the next checkpoint
+                    x.copy_(xs[s])
+                    v.copy_(vs[s])
+                    if length == every:
+                        seg, rec, new = traj, upto, every - 1
+                        end.copy_(xs[s + 1])
+                    else:
+                        seg = rec = traj[: length + 1]
+                        new = length
+                    nb.rollout(x, v, m, G, eps, dt, new, acc, 1, rec, end_at_drift=True)
                 nb.step_backward(seg, m, G, eps, dt, length, lam_x, lam_v, lam_m,
                                  at_start=(s == 0), at_end=(s == nseg - 1))
         return lam_x, lam_v, lam_m, None, None, None, None, None, None

@@ -527,9 +527,11 @@ nb_status rollout_enqueue(nb_ctx *c, cudaStream_t s, int64_t n, double *pos, dou
         }
         // (the step before's closing half-kick if it was left,) kick + drift;
         // it also repacks unless the bodies are re-ordered first
+        const bool end = (flags & NB_END_AT_DRIFT) && st + 1 == nsteps;
         NB_LAUNCHED(c, nb::launch_kdp(s, is_f64(c), (int)n, pos, vel, acc, mass, 0.5 * dt, dt,
-                                      order ? nullptr : c->pack, lo_half(c), logm, rp, rv,
+                                      order || end ? nullptr : c->pack, lo_half(c), logm, rp, rv,
                                       left.nslots ? &left : nullptr));
+        if (end) break;
         if (order) {
             NB_TRY(pack(c, s, n, pos, mass, logm));
         } else {
@@ -1427,7 +1429,8 @@ nb_status nb_rollout(nb_ctx *c, int64_t n, double *pos, double *vel, const doubl
     NB_TRY(check_scalars(c, G, eps));
     if (!std::isfinite(dt)) return failf(c, NB_EINVAL, "dt is not finite");
     if (nsteps < 0) return failf(c, NB_EINVAL, "nsteps < 0");
-    if (flags & ~(NB_ACC_VALID | NB_USE_GRAPH)) return failf(c, NB_EINVAL, "unknown flags");
+    if (flags & ~(NB_ACC_VALID | NB_USE_GRAPH | NB_END_AT_DRIFT))
+        return failf(c, NB_EINVAL, "unknown flags");
     const size_t v3 = (size_t)n * 3 * sizeof(double), v1 = (size_t)n * sizeof(double);
     NB_TRY(check_dev(c, pos, v3, "pos"));
     NB_TRY(check_dev(c, vel, v3, "vel"));

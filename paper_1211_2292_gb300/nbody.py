@@ -19,7 +19,7 @@ from . import build as _build
 
 NB_FP64, NB_FP32, NB_FP32_COMP, NB_DF64 = 0, 1, 2, 3
 PRECISIONS = {"fp64": NB_FP64, "fp32": NB_FP32, "fp32_comp": NB_FP32_COMP, "df64": NB_DF64}
-NB_ACC_VALID, NB_USE_GRAPH = 1, 2
+NB_ACC_VALID, NB_USE_GRAPH, NB_END_AT_DRIFT = 1, 2, 4
 NB_BWD_AT_END, NB_BWD_AT_START = 1, 2
 KIND_FORCE, KIND_BATCHED, KIND_VJP = 0, 1, 2
 STATUS = {0: "NB_OK", 1: "NB_EINVAL", 2: "NB_ECUDA", 3: "NB_ENOMEM", 4: "NB_ENONFINITE",
@@ -129,6 +129,7 @@ def load(build_if_missing: bool = True):
         return lib
 
 
+_HERE = contextlib.nullcontext()
 _torch = None  # imported by the first call: an import statement per argument shows in small calls
 
 
@@ -244,7 +245,6 @@ class NBody:
         self._call("nb_set_stream", ptr)
         self._stream = ptr
 
-    @contextlib.contextmanager
     def in_order(self):
         """Torch operations inside run on the context's stream: after all that
         torch's current stream of this device holds, and before what it is given
@@ -252,9 +252,10 @@ class NBody:
         inside after it, wherever the context's stream is another."""
         torch = _torch or _load_torch()
         here = torch.cuda.current_stream(self.device)
-        if here.cuda_stream == self._stream:
-            yield
-            return
+        return _HERE if here.cuda_stream == self._stream else self._on_stream(torch, here)
+
+    @contextlib.contextmanager
+    def _on_stream(self, torch, here):
         there = torch.cuda.ExternalStream(self._stream, device=self.device) if self._stream \
             else torch.cuda.default_stream(self.device)
         there.wait_stream(here)
@@ -288,9 +289,10 @@ class NBody:
                    _ptr(acc, "acc", 3 * n), flags)
 
     def rollout(self, pos, vel, mass, G, eps, dt, nsteps, acc, record_every, rec_pos,
-                rec_vel=None, acc_valid=False, graph=False):
+                rec_vel=None, acc_valid=False, graph=False, end_at_drift=False):
         n = mass.shape[0]
-        flags = (NB_ACC_VALID if acc_valid else 0) | (NB_USE_GRAPH if graph else 0)
+        flags = ((NB_ACC_VALID if acc_valid else 0) | (NB_USE_GRAPH if graph else 0)
+                 | (NB_END_AT_DRIFT if end_at_drift else 0))
         nrec = int(nsteps) // int(record_every) + 1 if record_every > 0 else 0
         self._call("nb_rollout", n, _ptr(pos, "pos", 3 * n), _ptr(vel, "vel", 3 * n),
                    _ptr(mass, "mass", n), float(G), float(eps), float(dt), int(nsteps),

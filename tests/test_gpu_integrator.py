@@ -127,3 +127,36 @@ def test_momentum_conserved_fp64(cuda):
     p0 = (b.mass[:, None] * b.vel).sum(0)
     p1 = (b.mass[:, None] * v).sum(0)
     assert np.abs(p1 - p0).max() <= 1e-14
+
+
+@pytest.mark.parametrize("prec,n", [("fp64", 300), ("df64", 300), ("fp32_comp", 700), ("fp32", 9001)])
+@pytest.mark.parametrize("graph", [False, True])
+def test_rollout_that_ends_at_a_drift(cuda, prec, n, graph):
+    # the records of a whole rollout, the last one before its closing half-kick
+    from paper_1211_2292_gb300 import tune
+    b = inputs.plummer(n, seed=n)
+    m, dt = to_dev(b.mass, cuda), 1e-3
+    with nbody.NBody(n, prec) as nb:
+        tune.apply(nb)
+
+        def run(k, end):
+            x, v = to_dev(b.pos, cuda), to_dev(b.vel, cuda)
+            acc, rx, rv = torch.empty_like(x), *(torch.empty((k + 1, n, 3), dtype=x.dtype, device=cuda)
+                                                 for _ in range(2))
+            nb.rollout(x, v, m, 1.0, 0.01, dt, k, acc, 1, rx, rv, graph=graph, end_at_drift=end)
+            return [host(t) for t in (x, v, acc, rx, rv)]
+
+        for k in (1, 2, 4):
+            x, v, acc, rx, rv = run(k, False)
+            ex, ev, eacc, erx, erv = run(k, True)
+            assert np.array_equal(ex, x) and np.array_equal(erx, rx)
+            assert np.array_equal(erv[:-1], rv[:-1]) and np.array_equal(erv[-1], ev)
+            # the force before the last step, and half of its two kicks
+            want = run(k - 1, False)
+            assert np.array_equal(eacc, want[2])
+            kick = 0.5 * dt * want[2]  # (the product and the sum rounded once or twice)
+            assert (np.abs(ev - (want[1] + kick)) <= 2.0 ** -52 * (np.abs(want[1]) + np.abs(kick))).all()
+        x, v, acc, rx, rv = run(0, True)
+        assert np.array_equal(x, b.pos) and np.array_equal(v, b.vel) and np.array_equal(rx[0], b.pos)
+        assert np.array_equal(acc, run(0, False)[2])
+        nb.sync()
